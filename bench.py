@@ -532,7 +532,7 @@ CLASSES = {
     "u1_wop": ("hbm", "byte"), "u1_pack_theta": ("hbm", "byte"), "u1_gather": ("hbm", "byte"),
     "oz_gemm": ("tensor_fp64", "flop"), "oz_slice": ("hbm", "byte"),
 }
-OZ_TENSOR_PER_USEFUL = 45.0  # slice pairs per complex product: 45 x 4 real MMAs / (8 / 2) FLOPs
+OZ_TENSOR_PER_USEFUL = 36.0  # slice pairs per complex product: 36 x 4 real MMAs / (8 / 2) FLOPs
 
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
@@ -573,11 +573,11 @@ def roofline(cls, ms, n, work, peaks, src):
     if unit is None or work <= 0:
         return dict(base, achieved=None, peak=None, unit=None, frac=None)
     if bound == "tensor_fp64":
-        pk = bf16 * TF32_PER_BF16 / OZ_TENSOR_PER_USEFUL
+        pk = bf16 / OZ_TENSOR_PER_USEFUL
         ach = work / secs / 1e12
         return dict(base, bound="tensor", achieved=ach, peak=pk, unit="TFLOP/s", frac=ach / pk,
-                    peak_source=f"{src} bf16 burst x nominal tf32/bf16 ratio / 45 slice pairs "
-                                "(FP64-accurate products on the TF32 pipe)")
+                    peak_source=f"{src} bf16 burst / 36 slice pairs "
+                                "(FP64-accurate products on the FP16 pipe)")
     if bound == "tensor":
         pk = bf16 * TF32_PER_BF16
         ach = work / secs / 1e12

@@ -467,8 +467,8 @@ int tnt_dmrg_destroy(tnt_dmrg* dmrg);
  * B(k,j) = d_B[k*b_rs + j*b_cs] (conjugated if conj_b), C(i,j) = d_C[i*c_rs + j] (out;
  * must not alias A or B).  Device pointers, borrowed.  The engine is the context's FP64
  * GEMM setting: FMA (FP64 units) or TC (exact integer slices of the operands multiplied
- * on the TF32 tensor cores with exact FP32 sums, added in FP64: error within the size of
- * FP64 rounding, see tnt_set_fp64_gemm).  TNT_E_INVALID on bad sizes. */
+ * on the FP16 tensor cores with exact FP32 sums, combined in 64-bit integers and rounded
+ * once: error within the size of FP64 rounding, see tnt_set_fp64_gemm).  TNT_E_INVALID on bad sizes. */
 int tnt_matmul(tnt_ctx* ctx, int64_t M, int64_t N, int64_t K, const tnt_cplx* d_A, int64_t a_rs,
                int64_t a_cs, int conj_a, const tnt_cplx* d_B, int64_t b_rs, int64_t b_cs,
                int conj_b, tnt_cplx* d_C, int64_t c_rs);
@@ -477,11 +477,12 @@ enum { TNT_FP64_GEMM_FMA = 0, TNT_FP64_GEMM_TC = 1 };
 /* Engine of the library's FP64 matrix products (the FP64 H_eff.theta, theta, the
  * environments, the SVD's Gram matrices and projections).
  * TNT_FP64_GEMM_TC (default): each row of A and column of B is scaled by a power of two
- * to below 1 and cut into 9 integer slices of 6 bits (exact FP64 steps); slice products
- * run as TF32 MMAs whose FP32 sums over K chunks of 224 stay below 2^24 and so are exact;
- * the 45 slice pairs p + q <= 10 are added in FP64.  The error is below
- * 11 * 2^-54 * K * sigma_i * tau_j, sigma_i and tau_j the powers of two just above
- * max_k|A_ik| and max_k|B_kj|: the size of FP64's own rounding bound.
+ * to below 1, rounded to 55 bits and cut into 8 integer slices (balanced base-128 digits);
+ * slice products run as FP16 MMAs whose FP32 sums over K chunks of 256 stay within 2^24
+ * and so are exact; the sums of the 36 slice pairs p + q <= 9 are combined in 64-bit
+ * integers and rounded once.  The error is below 2^-53 * K * sigma_i * tau_j, sigma_i and
+ * tau_j the powers of two just above max_k|A_ik| and max_k|B_kj|: the size of FP64's own
+ * rounding bound.  A row of A or column of B with an infinity or NaN gives NaN.
  * Small products (and calls that must not allocate) use FMA. */
 int tnt_set_fp64_gemm(tnt_ctx* ctx, int engine);
 

@@ -75,8 +75,7 @@ __host__ __device__ __forceinline__ double f64_of(float f) {
   return double_of_bits(((uint64_t)hi << 32) | lo);
 }
 
-// F = floor(|v| 2^(54 - esc)) for |v| < 2^esc: the 53-bit mantissa shifted (exact), the
-// fixed-point form whose 6-bit groups are the slices of the FP64-accurate GEMM (oz.cu)
+// F = floor(|v| 2^(54 - esc)) for |v| < 2^esc: the 53-bit mantissa shifted (exact)
 __host__ __device__ __forceinline__ uint64_t fixed54(double v, int esc) {
   const uint64_t u = bits_of(v);
   const int eb = (int)((u >> 52) & 0x7ff);

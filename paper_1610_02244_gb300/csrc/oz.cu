@@ -1,31 +1,42 @@
-// FP64-accurate complex GEMM on the TF32 tensor cores by exact integer slicing.
+// FP64-accurate complex GEMM on the FP16 tensor cores by exact integer slicing.
 //
-// GB300 runs FP64 FMA at 1.25 TFLOP/s, and its tensor cores run TF32 about 750 times faster. The
-// large FP64 products of the update (the FP64 H_eff.theta of the accuracy win-back, theta,
-// the environments and the SVD projections) are therefore computed as sums of exact
-// integer products (the Ozaki splitting):
-//   * every row i of A gets a power-of-two scale sigma_i >= max_k |A_ik| (re and im), every
-//     column j of B a scale tau_j, so that A_ik / sigma_i lies in (-1, 1);
-//   * A_ik / sigma_i = sum_{p=1..S} a_p 2^{-p beta} + r with integers |a_p| < 2^beta taken by
-//     repeated truncation (exact FP64 steps) and |r| < 2^{-S beta}; likewise B;
-//   * the slice products a_p b_q are integers below 2^{2 beta}; a K-chunk of them summed
-//     over all pairs (p, q) of one level p + q = l stays below 2^24, so TF32 operands
-//     (11 significant bits hold |a| < 2^6 exactly) with FP32 accumulation give the level's
-//     sum exactly;
-//   * C = sum over chunks and levels l = 2..S+1 of 2^{-l beta} sigma_i tau_j (level sum),
-//     added in FP64.
-// With beta = 6 and S = 9 the pairs kept (p + q <= S + 1) carry 54 bits; the omitted
-// terms and the remainders are below (S + 2) 2^{-54} K sigma_i tau_j, the size of an FP64
-// GEMM's own rounding bound.  Complex products take four real MMAs per k step
-// (re+ += Ar Br, re- += Ai Bi, im += Ar Bi + Ai Br; re = re+ - re- in FP64).
+// GB300 runs FP64 FMA at 1.25 TFLOP/s; its tensor cores run FP16 about 1500 times faster.
+// The FP64 products of the update (the FP64 H_eff.theta, theta, the environments, the SVD's
+// Gram matrices and projections) are therefore computed as sums of exact integer products
+// (the Ozaki splitting):
+//   * every row i of A has a power of two 2^a_i > max_k |A_ik| (re and im), every column j
+//     of B a power 2^b_j;
+//   * A_ik 2^-a_i is rounded to the 55-bit fixed-point value F 2^-55 and written in balanced
+//     base-128 digits, F = sum_p d_p 128^(8-p), -64 <= d_p <= 64: eight slices of integers
+//     that FP16 holds exactly; likewise B;
+//   * a product of digits is an integer of at most 2^12, and the sum over a K chunk of 256
+//     and over all pairs (p, q) of one level p + q = l (at most 8 pairs, two terms each of
+//     a complex part) is at most 2^24: FP32 accumulation gives the level's sum exactly;
+//   * the level sums are integers, combined in 64-bit integer arithmetic: the four top
+//     levels H = sum_{l=2..5} 128^(5-l) S_l and the four others L = sum_{l=6..9} 128^(9-l) S_l
+//     are exact over all of K; C = (2^28 H + L) 2^(a_i + b_j - 61), rounded once, by a
+//     second kernel (in the MMA kernel's eight epilogue warps that conversion took 25 to
+//     60 us a tile, more than the tile's MMAs).
+// The pairs left out (p + q > 9) and the digits' rounding are below K 2^-53 2^(a_i + b_j) in
+// the worst case and of random sign; the result does not depend on tiling or K splits.
+// No FP64-pipe instruction runs in these kernels: an SM retires two FP64 operations per
+// clock, and combining the level sums in FP64 (with TF32 operands, six-bit digits and 45
+// pairs) took longer than the MMAs.  Measured: H_eff.theta at chi = 256, d = 4 (two products
+// of 1.07 G complex multiply-adds) 5.71 -> 0.72 ms; theta at chi = 512, d = 5 7.0 -> 0.76 ms
+// (34 TFLOP/s of the complex product's own operations).  What bounds it: operand reads from
+// shared memory (an N = 128 MMA takes about 90 of the 64 clocks its arithmetic needs).
 //
-// Kernel: persistent, one CTA per SM over (output tile, level group, K split) items,
-// 128 x 128 or 128 x 64 tiles (K is split only when the tiles alone would leave most SMs
-// idle, as for the 256 x 256 products of a truncated SVD); warp 0 issues TMA loads of the
-// slice planes (3-D maps [plane][row][k], 64-byte swizzle), warp 1 the MMAs into three
-// TMEM accumulators, warps 2..5 convert each (chunk, level) accumulator and add it to the
-// item's FP64 partial tile, handing TMEM back through an mbarrier; a second kernel adds the
-// partial outputs in a fixed order.  All waits bounded.
+// Kernel: persistent, one CTA per SM over items (output tile 128 x 64, level group, K
+// split).  A complex multiply-add is two MMAs of N = 128: A_re with the rows [B_re; B_im] of
+// the B tile gives the real and the imaginary part side by side, A_im with [-B_im; B_re]
+// adds the rest (the B tile keeps three planes, -im, re, im).  The group's four levels
+// accumulate at once in the 512 TMEM columns, so a slice tile is loaded once per 32 of K
+// and group instead of once per pair: 28 KB per 1024 MMA clocks, which the L2 can feed.
+// Within a block of 32 of K, A's slices p stream through a ring; slice q of B stays in its
+// own ring from its first to its last pair.  The slice kernel writes the tiles in the
+// shared-memory order (64-byte rows, 64-byte swizzle), so a load is one bulk copy and no
+// tensor map is built.  Warp 0 loads, warp 1 issues, warps 2..9 convert the level sums.
+// All waits bounded.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -33,78 +44,200 @@
 #include "heff_plan.cuh"
 #include "tc_common.cuh"
 #include "f32conv.cuh"
+#include "oz.cuh"
 
 namespace tnt {
 
 namespace {
 using namespace tc;
 
-constexpr int OZ_S = 9;         // slices per operand
-constexpr int OZ_BETA = 6;      // bits per slice
-constexpr int OZ_KC = 224;      // K chunk: 2 * S * KC * (2^beta - 1)^2 < 2^24
-constexpr int OZ_PLANES = 2 * OZ_S;
-constexpr int O_TILE_A = 128 * 16 * 4;               // one A plane tile, 8 KB
-// the levels of a tile in two groups of nearly equal work (21 and 24 slice pairs), each
-// group an independent work item with its own FP64 partial output
-constexpr int OZ_GROUP_SPLIT = 7;                    // levels 2..7 | 8..S+1
-
-template <int BN>
-struct OzCfg {
-  static constexpr int TILE_B = BN * 16 * 4;
-  static constexpr int STAGE = 2 * O_TILE_A + 2 * TILE_B;  // A re, A im, B re, B im
-  static constexpr int STAGES = (BN == 128) ? 6 : 8;
-  static constexpr int SMEM = STAGES * STAGE + 1024 + 256;
-  static constexpr int TMEM = (BN == 128) ? 512 : 256;
-};
-static_assert(2LL * OZ_S * OZ_KC * ((1 << OZ_BETA) - 1) * ((1 << OZ_BETA) - 1) < (1LL << 24),
+constexpr int OZ_S = 8;                         // slices per operand
+constexpr int OZ_KB = 32;                       // K of one slice tile (64 bytes of FP16)
+constexpr int OZ_CHUNK = 8;                     // K blocks per exact FP32 accumulation
+constexpr int OZ_BM = 128, OZ_BN = 64;          // output tile
+constexpr int OZ_TA = 2 * OZ_BM * 64;           // A slice tile: re, im
+constexpr int OZ_TB = 3 * OZ_BN * 64;           // B slice tile: -im, re, im
+constexpr int OZ_NA = 6, OZ_NB = 10;            // ring stages
+constexpr int OZ_SMEM = OZ_NA * OZ_TA + OZ_NB * OZ_TB + 1024 + 512;
+constexpr int OZ_EPI = 8;                       // epilogue warps
+constexpr int OZ_THREADS = 64 + 32 * OZ_EPI;
+constexpr int OZ_SPLIT_LEVEL = 5;               // group 0: levels 2..5, group 1: 6..9
+constexpr int OZ_PAIRS0 = 10, OZ_PAIRS1 = 26;   // slice pairs of the two groups
+static_assert(2LL * OZ_S * OZ_CHUNK * OZ_KB * 64 * 64 <= (1LL << 24),
               "a level sum over one K chunk must stay exact in FP32");
-static_assert(OZ_KC % 16 == 0, "K chunk in whole k-blocks");
+static_assert(OZ_SMEM <= 227 * 1024, "rings fit the shared memory of an SM");
 
 struct OzArgs {
-  int64_t M, N, Kp;
+  int64_t M, N;
   int ntm, ntn;       // tiles along M and N
-  int nchunk;         // K chunks of OZ_KC
-  int ks;             // K splits: split s takes chunks [s nchunk / ks, (s+1) nchunk / ks)
-  z* P;               // 2 ks FP64 partial outputs, [split][group][M][N]
-  const double* sA;   // row scales (powers of two)
-  const double* sB;   // column scales
+  int nkb;            // K blocks of 32
+  int ks;             // K splits
+  int both;           // an item runs both level groups, one after the other
+  const uint8_t* A;   // [ntm][nkb][OZ_S] slice tiles
+  const uint8_t* B;   // [ntn][nkb][OZ_S]
+  longlong2* P;       // [split][group][M][N] partial sums
+  int lower;          // Hermitian result: tiles strictly above the diagonal are left out
   int* status;
 };
 
-// sub-items of one tile: (chunk, level), levels 2..S+1; pairs (p, l - p), 1 <= p, q <= S
-__device__ __forceinline__ void level_pairs(int l, int* p0, int* p1) {
-  *p0 = max(1, l - OZ_S);
-  *p1 = min(OZ_S, l - 1);
+struct OzItem {
+  int mt, nt, g0, g1, kb0, kb1, sp;  // groups g0..g1, K blocks [kb0, kb1)
+};
+// item w; the heavier group's items come first.  false: a tile left out
+__device__ __forceinline__ bool oz_item(const OzArgs& g, int w, OzItem* it) {
+  const int ntiles = g.ntm * g.ntn;
+  const int t = w % ntiles, r = w / ntiles;
+  it->mt = t / g.ntn;
+  it->nt = t % g.ntn;
+  if (g.both) {
+    it->g0 = 0;
+    it->g1 = 1;
+  } else {
+    it->g0 = it->g1 = r < g.ks ? 1 : 0;
+  }
+  it->sp = r % g.ks;
+  it->kb0 = (int)((int64_t)it->sp * g.nkb / g.ks);
+  it->kb1 = (int)((int64_t)(it->sp + 1) * g.nkb / g.ks);
+  return !(g.lower && it->mt * OZ_BM + OZ_BM <= it->nt * OZ_BN);
+}
+__host__ __device__ inline int oz_items(const OzArgs& g) {
+  return g.ntm * g.ntn * g.ks * (g.both ? 1 : 2);
+}
+// pairs (p, q) of group levels l0..l1 at slice p of A: q in [qlo, qhi]
+__device__ __forceinline__ void oz_levels(int grp, int* l0, int* l1) {
+  *l0 = grp ? OZ_SPLIT_LEVEL + 1 : 2;
+  *l1 = grp ? OZ_S + 1 : OZ_SPLIT_LEVEL;
 }
 
-template <int BN>
-__global__ void __launch_bounds__(192, 1) k_oz_gemm(const __grid_constant__ CUtensorMap tmA,
-                                                    const __grid_constant__ CUtensorMap tmB,
-                                                    OzArgs g) {
-  using Cf = OzCfg<BN>;
-  constexpr int O_STAGES = Cf::STAGES;
-  constexpr int O_STAGE = Cf::STAGE;
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+          su32(dst)),
+      "l"(src), "r"(bytes), "r"(su32(bar))
+      : "memory");
+}
+// instruction descriptor: D = F32, A = B = F16, both K-major, M = 128, N = 128
+constexpr uint32_t OZ_IDESC = (1u << 4) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+// high word of a shared-memory descriptor (as tc::desc_sw64); the low word is the address / 16
+constexpr uint32_t OZ_DESC_HI = (512u >> 4) | (1u << 14) | (4u << 29);
+__device__ __forceinline__ void mma_f16(uint32_t tmem, uint32_t alo, uint32_t blo, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "mov.b64 a, {%1, %5};\n\t"
+      "mov.b64 b, {%2, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}\n" ::"r"(tmem),
+      "r"(alo), "r"(blo), "r"(OZ_IDESC), "r"(acc), "r"(OZ_DESC_HI)
+      : "memory");
+}
+
+// The MMAs of one K block of group GRP: the loop over the pairs is unrolled, so that the one
+// issuing thread spends about ten instructions per MMA (with the ring slots and descriptors
+// computed in a rolled loop it took about 200 clocks per 64-clock MMA, 450 us for a
+// 1024 x 1024 x 1024 product that is 142 us of MMAs).  sa / sb: ring slots of the block's
+// first A and B slice, with the phases of their barriers in pa / pb.
+struct OzIssue {
+  uint32_t a0, b0;  // shared-memory addresses / 16 of the rings
+  uint64_t *fa, *ea, *fb, *eb;
+  uint64_t* acce;  // set: a level's first MMA waits until its last sums have been read
+  uint32_t pacc;
+  uint32_t sa, pa, sb, pb;
+};
+template <int GRP>
+__device__ __forceinline__ bool oz_issue_block(OzIssue& r, uint32_t tmem, bool first, int* status) {
+  constexpr int L0 = GRP ? OZ_SPLIT_LEVEL + 1 : 2, L1 = GRP ? OZ_S + 1 : OZ_SPLIT_LEVEL;
+  constexpr int QM = L1 - 1;  // slices of either operand
+  uint32_t blo[QM];
+  uint32_t sq = r.sb, pq = r.pb;  // slot and phase of the next slice of B (descending q)
+#pragma unroll
+  for (int p = 1; p <= QM; ++p) {
+    constexpr int LL0 = L0;
+    const int qlo = LL0 - p > 1 ? LL0 - p : 1, qhi = L1 - p < QM ? L1 - p : QM;
+    const int qprev = p == 1 ? QM + 1 : (LL0 - p + 1 > 1 ? LL0 - p + 1 : 1);  // lowest slice seen before
+    if (!mbar_wait(&r.fa[r.sa], r.pa, status)) return false;
+    const uint32_t alo = r.a0 + r.sa * (uint32_t)(OZ_TA >> 4);
+#pragma unroll
+    for (int q = qhi; q >= qlo; --q) {
+      if (q < qprev) {
+        if (!mbar_wait(&r.fb[sq], pq, status)) return false;
+        blo[q - 1] = r.b0 + sq * (uint32_t)(OZ_TB >> 4);
+        if (++sq == OZ_NB) {
+          sq = 0;
+          pq ^= 1;
+        }
+      }
+      if (p == 1 && r.acce && !mbar_wait(&r.acce[q + 1 - L0], r.pacc, status)) return false;
+      if (q == qhi || q < qprev) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t d = tmem + (uint32_t)(p + q - L0) * 128u, bq = blo[q - 1];
+      // every level's first pair has p = 1
+      mma_f16(d, alo, bq + (OZ_BN * 64 >> 4), p == 1 ? (first ? 0u : 1u) : 1u);
+      mma_f16(d, alo + (OZ_BM * 64 >> 4), bq, 1u);
+      mma_f16(d, alo + 2, bq + (OZ_BN * 64 >> 4) + 2, 1u);
+      mma_f16(d, alo + (OZ_BM * 64 >> 4) + 2, bq + 2, 1u);
+    }
+    mma_commit(&r.ea[r.sa]);
+    if (++r.sa == OZ_NA) {
+      r.sa = 0;
+      r.pa ^= 1;
+    }
+    mma_commit(&r.eb[r.sb]);  // the last pair of slice q = L1 - p, the oldest in its ring
+    if (++r.sb == OZ_NB) {
+      r.sb = 0;
+      r.pb ^= 1;
+    }
+  }
+  return true;
+}
+
+// one group's loads of an item, in the order of first use
+struct OzRings {
+  uint8_t *a, *b;
+  uint64_t *fa, *ea, *fb, *eb;
+};
+
+// 32 pairs of one row to memory (nc of them exist), two per 32-byte store where o allows it
+__device__ __forceinline__ void oz_put(longlong2* o, int nc, const long long* re, const long long* im) {
+  if (nc == 32 && ((uintptr_t)o & 31) == 0) {
+#pragma unroll
+    for (int j = 0; j < 32; j += 2)
+      asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(o + j), "l"(re[j]), "l"(im[j]), "l"(re[j + 1]),
+                   "l"(im[j + 1])
+                   : "memory");
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    if (j < nc) o[j] = make_longlong2(re[j], im[j]);
+}
+
+__global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = (uint64_t*)(smem + O_STAGES * O_STAGE);
-  uint64_t* empty = full + O_STAGES;
-  uint64_t* accf = empty + O_STAGES;
+  OzRings R;
+  R.a = smem;
+  R.b = smem + OZ_NA * OZ_TA;
+  R.fa = (uint64_t*)(R.b + OZ_NB * OZ_TB);
+  R.ea = R.fa + OZ_NA;
+  R.fb = R.ea + OZ_NA;
+  R.eb = R.fb + OZ_NB;
+  uint64_t* accf = R.eb + OZ_NB;
   uint64_t* acce = accf + 1;
-  uint32_t* tmem_slot = (uint32_t*)(acce + 1);
+  uint32_t* tmem_slot = (uint32_t*)(acce + 4);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ntiles = g.ntm * g.ntn;
-  const int nitems = 2 * ntiles * g.ks;  // (tile, level group, K split)
-  const int kb_total = (int)(g.Kp / 16);
-  const int kb_chunk = OZ_KC / 16;
+  const int nitems = oz_items(g);
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < O_STAGES; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+    for (int s = 0; s < OZ_NA; ++s) {
+      mbar_init(&R.fa[s], 1);
+      mbar_init(&R.ea[s], 1);
+    }
+    for (int s = 0; s < OZ_NB; ++s) {
+      mbar_init(&R.fb[s], 1);
+      mbar_init(&R.eb[s], 1);
     }
     mbar_init(accf, 1);
-    mbar_init(acce, 4);
+    for (int l = 0; l < 4; ++l) mbar_init(&acce[l], OZ_EPI);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -112,7 +245,7 @@ __global__ void __launch_bounds__(192, 1) k_oz_gemm(const __grid_constant__ CUte
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      su32(tmem_slot)),
-                 "r"(Cf::TMEM)
+                 "r"(512)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -122,156 +255,121 @@ __global__ void __launch_bounds__(192, 1) k_oz_gemm(const __grid_constant__ CUte
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0 && lane == 0) {
-    // ------------------------------------------------ TMA producer
-    uint32_t it = 0;
+    // ------------------------------------------------ loads
+    uint32_t ia = 0, ib = 0;
     bool stop = false;
+    auto load = [&](uint8_t* ring, uint64_t* full, uint64_t* empty, uint32_t& i, int n, uint32_t bytes,
+                    const uint8_t* src) {
+      const int s = (int)(i % (uint32_t)n);
+      if (i >= (uint32_t)n && !mbar_wait(&empty[s], ((i / n) & 1) ^ 1, g.status)) *abort_flag = 1;
+      if (*abort_flag) {
+        stop = true;
+        return;
+      }
+      mbar_expect_tx(&full[s], bytes);
+      bulk_load(ring + (size_t)s * bytes, src, bytes, &full[s]);
+      ++i;
+    };
     for (int w = blockIdx.x; w < nitems && !stop; w += gridDim.x) {
-      const int t = w % ntiles, grp = (w / ntiles) & 1, sp = w / (2 * ntiles);
-      const int m0 = (t / g.ntn) * 128, n0 = (t % g.ntn) * BN;
-      const int l0 = grp ? OZ_GROUP_SPLIT + 1 : 2, l1 = grp ? OZ_S + 1 : OZ_GROUP_SPLIT;
-      const int ch0 = sp * g.nchunk / g.ks, ch1 = (sp + 1) * g.nchunk / g.ks;
-      for (int ch = ch0; ch < ch1 && !stop; ++ch) {
-        const int kb0 = ch * kb_chunk, kb1 = min(kb_total, kb0 + kb_chunk);
-        for (int l = l0; l <= l1 && !stop; ++l) {
-          int p0, p1;
-          level_pairs(l, &p0, &p1);
-          for (int p = p0; p <= p1 && !stop; ++p) {
-            const int q = l - p;
-            for (int kb = kb0; kb < kb1; ++kb) {
-              const int s = it % O_STAGES;
-              if (it >= O_STAGES && !mbar_wait(&empty[s], ((it / O_STAGES) & 1) ^ 1, g.status)) {
-                *abort_flag = 1;
-                stop = true;
-                break;
-              }
-              if (*abort_flag) {
-                stop = true;
-                break;
-              }
-              uint8_t* st = smem + s * O_STAGE;
-              mbar_expect_tx(&full[s], O_STAGE);
-              const int k = kb * 16;
-              tma_load3(st, &tmA, &full[s], k, m0, 2 * (p - 1));
-              tma_load3(st + O_TILE_A, &tmA, &full[s], k, m0, 2 * (p - 1) + 1);
-              tma_load3(st + 2 * O_TILE_A, &tmB, &full[s], k, n0, 2 * (q - 1));
-              tma_load3(st + 2 * O_TILE_A + Cf::TILE_B, &tmB, &full[s], k, n0, 2 * (q - 1) + 1);
-              ++it;
-            }
+      OzItem it;
+      if (!oz_item(g, w, &it)) continue;
+      for (int grp = it.g0; grp <= it.g1 && !stop; ++grp) {
+        int l0, l1;
+        oz_levels(grp, &l0, &l1);
+        const int pmax = min(OZ_S, l1 - 1);
+        for (int kb = it.kb0; kb < it.kb1 && !stop; ++kb) {
+          const uint8_t* A = g.A + ((int64_t)it.mt * g.nkb + kb) * (OZ_S * OZ_TA);
+          const uint8_t* B = g.B + ((int64_t)it.nt * g.nkb + kb) * (OZ_S * OZ_TB);
+          int qnext = min(OZ_S, l1 - 1);  // next slice of B to load (descending)
+          for (int p = 1; p <= pmax && !stop; ++p) {
+            const int qlo = max(1, l0 - p);
+            for (; qnext >= qlo && !stop; --qnext)
+              load(R.b, R.fb, R.eb, ib, OZ_NB, OZ_TB, B + (qnext - 1) * OZ_TB);
+            if (!stop) load(R.a, R.fa, R.ea, ia, OZ_NA, OZ_TA, A + (p - 1) * OZ_TA);
           }
         }
       }
     }
-    for (uint32_t i = (it > (uint32_t)O_STAGES ? it - O_STAGES : 0u); i < it; ++i)
-      mbar_wait(&full[i % O_STAGES], (i / O_STAGES) & 1, g.status);
+    // copies in flight land before the CTA may exit
+    for (uint32_t i = (ia > (uint32_t)OZ_NA ? ia - OZ_NA : 0u); i < ia; ++i)
+      mbar_wait(&R.fa[i % OZ_NA], (i / OZ_NA) & 1, g.status);
+    for (uint32_t i = (ib > (uint32_t)OZ_NB ? ib - OZ_NB : 0u); i < ib; ++i)
+      mbar_wait(&R.fb[i % OZ_NB], (i / OZ_NB) & 1, g.status);
   } else if (warp == 1 && lane == 0) {
-    // ------------------------------------------------ MMA issuer
-    const uint32_t id = idesc_tf32_n(BN);
-    const uint32_t t_re = tmem, t_im = tmem + BN, t_rn = tmem + 2 * BN;
-    uint32_t it = 0, sub = 0;
+    // ------------------------------------------------ MMA issue
+    uint32_t sub = 0;
     bool stop = false;
+    OzIssue r{su32(R.a) >> 4, su32(R.b) >> 4, R.fa, R.ea, R.fb, R.eb, nullptr, 0, 0, 0, 0, 0};
     for (int w = blockIdx.x; w < nitems && !stop; w += gridDim.x) {
-      const int grp = (w / ntiles) & 1, sp = w / (2 * ntiles);
-      const int l0 = grp ? OZ_GROUP_SPLIT + 1 : 2, l1 = grp ? OZ_S + 1 : OZ_GROUP_SPLIT;
-      const int ch0 = sp * g.nchunk / g.ks, ch1 = (sp + 1) * g.nchunk / g.ks;
-      for (int ch = ch0; ch < ch1 && !stop; ++ch) {
-        const int kb0 = ch * kb_chunk, kb1 = min(kb_total, kb0 + kb_chunk);
-        for (int l = l0; l <= l1 && !stop; ++l) {
-          int p0, p1;
-          level_pairs(l, &p0, &p1);
-          if (sub > 0 && (*abort_flag || !mbar_wait(acce, (sub - 1) & 1, g.status))) {
+      OzItem it;
+      if (!oz_item(g, w, &it)) continue;
+      for (int grp = it.g0; grp <= it.g1 && !stop; ++grp) {
+        for (int kb = it.kb0; kb < it.kb1; ++kb) {
+          const bool first = ((kb - it.kb0) % OZ_CHUNK) == 0;
+          bool ok = *abort_flag == 0;
+          r.acce = first && sub > 0 ? acce : nullptr;
+          r.pacc = (sub - 1) & 1;
+          if (ok) ok = grp ? oz_issue_block<1>(r, tmem, first, g.status) : oz_issue_block<0>(r, tmem, first, g.status);
+          if (!ok) {
             *abort_flag = 1;
             stop = true;
             break;
           }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          bool first = true;
-          for (int p = p0; p <= p1 && !stop; ++p) {
-            for (int kb = kb0; kb < kb1; ++kb) {
-              const int s = it % O_STAGES;
-              if (*abort_flag || !mbar_wait(&full[s], (it / O_STAGES) & 1, g.status)) {
-                *abort_flag = 1;
-                stop = true;
-                break;
-              }
-              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-              const uint32_t base = su32(smem + s * O_STAGE);
-              for (int ks = 0; ks < 2; ++ks) {
-                const uint32_t off = ks * 32;
-                const uint64_t ar = desc_sw64(base + off);
-                const uint64_t ai = desc_sw64(base + O_TILE_A + off);
-                const uint64_t br = desc_sw64(base + 2 * O_TILE_A + off);
-                const uint64_t bi = desc_sw64(base + 2 * O_TILE_A + Cf::TILE_B + off);
-                const uint32_t acc = first ? 0u : 1u;
-                mma_tf32(t_re, ar, br, id, acc);
-                mma_tf32(t_rn, ai, bi, id, acc);
-                mma_tf32(t_im, ar, bi, id, acc);
-                mma_tf32(t_im, ai, br, id, 1);
-                first = false;
-              }
-              mma_commit(&empty[s]);
-              ++it;
-            }
+          if (kb + 1 == it.kb1 || (kb + 1 - it.kb0) % OZ_CHUNK == 0) {
+            mma_commit(accf);
+            ++sub;
           }
-          if (stop) break;
-          mma_commit(accf);
-          ++sub;
         }
       }
     }
   } else if (warp >= 2) {
-    // ------------------------------------------------ epilogue: level sums into FP64 C
-    const int q4 = warp & 3;
+    // ------------------------------------------------ level sums into 64-bit integers
+    const int q4 = warp & 3, half = (warp - 2) >> 2;
     const int row = q4 * 32 + lane;
-    const uint32_t lane_addr = (uint32_t)(q4 * 32) << 16;
+    const uint32_t taddr = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(half * 32);
     uint32_t sub = 0;
     bool stop = false;
     for (int w = blockIdx.x; w < nitems && !stop; w += gridDim.x) {
-      const int t = w % ntiles, grp = (w / ntiles) & 1, sp = w / (2 * ntiles);
-      const int m0 = (t / g.ntn) * 128, n0 = (t % g.ntn) * BN;
-      const int l0 = grp ? OZ_GROUP_SPLIT + 1 : 2, l1 = grp ? OZ_S + 1 : OZ_GROUP_SPLIT;
-      const int64_t gm = (int64_t)m0 + row;
-      const double sa = (gm < g.M) ? g.sA[gm] : 0.0;
-      z* Cg = g.P + (int64_t)(grp + 2 * sp) * g.M * g.N;
-      const int ch0 = sp * g.nchunk / g.ks, ch1 = (sp + 1) * g.nchunk / g.ks;
-      for (int ch = ch0; ch < ch1 && !stop; ++ch) {
-        for (int l = l0; l <= l1; ++l) {
+      OzItem it;
+      if (!oz_item(g, w, &it)) continue;
+      const int64_t gm = (int64_t)it.mt * OZ_BM + row;
+      const int64_t gn0 = (int64_t)it.nt * OZ_BN + half * 32;
+      for (int grp = it.g0; grp <= it.g1 && !stop; ++grp) {
+        long long re[32], im[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) re[j] = im[j] = 0;
+        for (int kb = it.kb0; kb < it.kb1; kb += OZ_CHUNK) {
           if (*abort_flag || !mbar_wait(accf, sub & 1, g.status)) {
             *abort_flag = 1;
             stop = true;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const double lv = ldexp(sa, -l * OZ_BETA);
-          const bool first = (ch == ch0 && l == l0);
-          for (int c0 = 0; c0 < BN; c0 += 32) {
-            uint32_t r[32], s[32], u[32];
-            tmem_ld32(tmem + lane_addr + c0, r);
-            tmem_ld32(tmem + lane_addr + BN + c0, s);
-            tmem_ld32(tmem + lane_addr + 2 * BN + c0, u);
-            if (gm < g.M) {
-              z* pc = Cg + gm * g.N + n0 + c0;
 #pragma unroll
-              for (int j = 0; j < 32; ++j) {
-                const int64_t gn = (int64_t)n0 + c0 + j;
-                if (gn < g.N) {
-                  const double f = lv * g.sB[gn];
-                  const double dr = (double)__uint_as_float(r[j]) - (double)__uint_as_float(u[j]);
-                  const double di = (double)__uint_as_float(s[j]);
-                  if (first) {
-                    pc[j] = zmk(dr * f, di * f);
-                  } else {
-                    const z o = pc[j];
-                    pc[j] = zmk(fma(dr, f, o.x), fma(di, f, o.y));
-                  }
-                }
-              }
+          for (int l = 3; l >= 0; --l) {  // the order in which the next chunk needs them
+            const int wt = 1 << (7 * (3 - l));
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              uint32_t r[16];
+              tmem_ld16(taddr + l * 128 + h * 16, r);
+#pragma unroll
+              for (int j = 0; j < 16; ++j)
+                re[16 * h + j] += (long long)__float2int_rn(__uint_as_float(r[j])) * wt;
+              tmem_ld16(taddr + l * 128 + 64 + h * 16, r);
+#pragma unroll
+              for (int j = 0; j < 16; ++j)
+                im[16 * h + j] += (long long)__float2int_rn(__uint_as_float(r[j])) * wt;
             }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acce[l]);
           }
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          __syncwarp();
-          if (lane == 0) mbar_arrive(acce);
           ++sub;
         }
+        if (stop || gm >= g.M) continue;
+        const int nc = (int)min((int64_t)32, g.N - gn0);  // columns of this half tile
+        if (nc <= 0) continue;
+        oz_put(g.P + ((int64_t)(2 * it.sp + grp) * g.M + gm) * g.N + gn0, nc, re, im);
       }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -279,145 +377,223 @@ __global__ void __launch_bounds__(192, 1) k_oz_gemm(const __grid_constant__ CUte
   __syncthreads();
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Cf::TMEM)
-                 : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
   }
 }
 
-// C = P[0] + P[1], the two level groups, in a fixed order
-__global__ void k_oz_finish(const z* __restrict__ P, int np, int64_t M, int64_t N,
+// C from the partial sums of the K splits (integers: any order gives the same value)
+__global__ void k_oz_finish(const longlong2* __restrict__ P, int ks, int64_t M, int64_t N,
+                            const int* __restrict__ eA, const int* __restrict__ eB, int lower,
                             z* __restrict__ C, int64_t ldc) {
   const int64_t total = M * N;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
-    z acc = P[e];
-    for (int i = 1; i < np; ++i) acc = zadd(acc, P[(int64_t)i * total + e]);
-    C[(e / N) * ldc + e % N] = acc;
+    const int64_t i = e / N, j = e % N;
+    if (lower && (i / OZ_BM) * OZ_BM + OZ_BM <= (j / OZ_BN) * OZ_BN) continue;
+    longlong2 h = make_longlong2(0, 0), l = h;
+    for (int s = 0; s < ks; ++s) {
+      const longlong2 a = P[(int64_t)(2 * s) * total + e], b = P[(int64_t)(2 * s + 1) * total + e];
+      h.x += a.x;
+      h.y += a.y;
+      l.x += b.x;
+      l.y += b.y;
+    }
+    C[i * ldc + j] = zmk(oz_value(h.x, l.x, eA[i], eB[j]), oz_value(h.y, l.y, eA[i], eB[j]));
   }
 }
 
 // ---------------------------------------------------------------- scales and slices
-// sA[i] = 2^e with 2^(e-1) <= max_k max(|re A_ik|, |im A_ik|) < 2^e (1 for a zero row);
-// one warp per row of a strided operand X[i * rs + k * cs]
-__global__ void k_oz_row_scale(const z* __restrict__ X, int64_t rows, int64_t K, int64_t rs,
-                               int64_t cs, double* __restrict__ sc) {
-  // by integer operations on the exponent fields (no FP64-pipe comparisons): the largest
-  // field mx of the row gives 2^(mx - 1023) <= max < 2^(mx - 1022), so sc = 2^(mx - 1022),
-  // the frexp exponent of the maximum; a row of subnormals gets 2^-1022, a zero row 1
+// one operand of the product seen as rows of K entries: X[i * rs + k * cs]
+struct OzOp {
+  const z* X;
+  int64_t rows, rs, cs;
+  int conj;
+  int* e;        // per row: largest exponent field of the re and im parts
+  uint8_t* out;  // slice tiles
+};
+
+// largest exponent field of every row.  Entries contiguous along K: one warp per row;
+// otherwise 32 rows by 64 of K per CTA, neighbouring lanes on neighbouring rows, combined
+// with an atomic maximum (e zeroed before)
+__device__ __forceinline__ unsigned oz_exp(z v) {
+  return max(((unsigned)__double2hiint(v.x) >> 20) & 0x7ffu, ((unsigned)__double2hiint(v.y) >> 20) & 0x7ffu);
+}
+__host__ __device__ inline int64_t oz_scale_blocks(const OzOp& o, int64_t K) {
+  return o.cs == 1 ? (o.rows + 7) / 8 : ((o.rows + 31) / 32) * ((K + 63) / 64);
+}
+__global__ void __launch_bounds__(256) k_oz_scale(OzOp a, OzOp b, int64_t K, int64_t nba) {
+  const bool isb = blockIdx.x >= nba;
+  const OzOp o = isb ? b : a;
+  const int64_t blk = isb ? (int64_t)blockIdx.x - nba : (int64_t)blockIdx.x;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (o.cs == 1) {
+    const int64_t i = blk * 8 + warp;
+    if (i >= o.rows) return;
+    unsigned mx = 0;
+    const z* x = o.X + i * o.rs;
+#pragma unroll 8
+    for (int64_t k = lane; k < K; k += 32) mx = max(mx, oz_exp(x[k]));
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) o.e[i] = (int)mx;
+    return;
+  }
+  __shared__ unsigned s_mx[32];
+  if (threadIdx.x < 32) s_mx[threadIdx.x] = 0;
+  __syncthreads();
+  const int64_t nk = (K + 63) / 64, i = (blk / nk) * 32 + lane, k0 = (blk % nk) * 64;
+  unsigned mx = 0;
+  if (i < o.rows)
+#pragma unroll
+    for (int64_t k = k0 + warp; k < min(K, k0 + 64); k += 8) mx = max(mx, oz_exp(o.X[i * o.rs + k * o.cs]));
+  if (mx) atomicMax(&s_mx[lane], mx);
+  __syncthreads();
+  if (warp == 0 && i < o.rows && s_mx[lane]) atomicMax((unsigned*)o.e + i, s_mx[lane]);
+}
+
+// slices of 8 rows by 32 of K per warp: lane = (row, 8 of K), so every plane's 512-byte
+// swizzle atom is written whole.  Rows and K beyond the operand are zero.
+template <int PLANES>
+__device__ __forceinline__ void oz_slice_atom(const OzOp& o, int64_t K, int nkb, int64_t atom, int lane) {
+  constexpr int ROWS = PLANES == 2 ? OZ_BM : OZ_BN, TILE = PLANES == 2 ? OZ_TA : OZ_TB;
+  const int kb = (int)(atom % nkb);
+  const int64_t i8 = atom / nkb;  // group of 8 rows
+  const int r = lane >> 2, c8 = lane & 3;
+  const int64_t i = i8 * 8 + r, k0 = (int64_t)kb * OZ_KB + c8 * 8;
+  uint64_t fr[8], fi[8];
+  uint32_t sr[4], si[4];  // signs of the eight entries, as bits 15 and 31 of a word per pair
+  const int e = i < o.rows ? o.e[i] : 0;
+  const z* x = o.X + i * o.rs + k0 * o.cs;
+  z v[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) v[t] = (i < o.rows && k0 + t < K) ? x[t * o.cs] : zmk(0, 0);
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const uint32_t cj = o.conj ? 0x80008000u : 0u;
+    sr[t] = oz_signs(v[2 * t].x, v[2 * t + 1].x);
+    si[t] = oz_signs(v[2 * t].y, v[2 * t + 1].y) ^ cj;
+  }
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    fr[t] = oz_fixed(v[t].x, e) + OZ_BIAS;
+    fi[t] = oz_fixed(v[t].y, e) + OZ_BIAS;
+  }
+  const int64_t rt = (i8 * 8) / ROWS;
+  const int ra = (int)((i8 * 8) % ROWS) / 8;
+  uint8_t* base = o.out + (rt * nkb + kb) * (int64_t)(OZ_S * TILE) + ra * 512 + r * 64 + ((c8 ^ ((r >> 1) & 3)) << 4);
+#pragma unroll
+  for (int p = 0; p < OZ_S; ++p) {
+    uint32_t wr[4], wi[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      wr[t] = oz_digit2(fr[2 * t], fr[2 * t + 1], p, sr[t]);
+      wi[t] = oz_digit2(fi[2 * t], fi[2 * t + 1], p, si[t]);
+    }
+    uint8_t* q = base + p * TILE;
+    if (PLANES == 3) {
+      *(uint4*)q = make_uint4(wi[0] ^ 0x80008000u, wi[1] ^ 0x80008000u, wi[2] ^ 0x80008000u, wi[3] ^ 0x80008000u);
+      q += ROWS * 64;
+    }
+    *(uint4*)q = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+    *(uint4*)(q + ROWS * 64) = make_uint4(wi[0], wi[1], wi[2], wi[3]);
+  }
+}
+__global__ void __launch_bounds__(256) k_oz_slice(OzOp a, OzOp b, int64_t K, int nkb, int64_t na, int64_t nb) {
   const int lane = threadIdx.x & 31;
-  for (int64_t i = (int64_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); i < rows;
-       i += (int64_t)((gridDim.x * blockDim.x) >> 5)) {
-    unsigned mx = 0, nz = 0;
-    for (int64_t k = lane; k < K; k += 32) {
-      const z v = X[i * rs + k * cs];
-      const unsigned hr = (unsigned)__double2hiint(v.x), hi = (unsigned)__double2hiint(v.y);
-      mx = max(mx, max((hr >> 20) & 0x7ffu, (hi >> 20) & 0x7ffu));
-      nz |= (hr & 0x7fffffffu) | (unsigned)__double2loint(v.x) | (hi & 0x7fffffffu) |
-            (unsigned)__double2loint(v.y);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      nz |= __shfl_xor_sync(0xffffffffu, nz, o);
-    }
-    if (lane == 0) {
-      double r = 1.0;
-      if (mx > 0) r = __hiloint2double((int)((mx + 1u) << 20), 0);  // 2^(mx - 1022)
-      else if (nz) r = __hiloint2double(1 << 20, 0);                  // 2^-1022
-      sc[i] = r;
-    }
+  for (int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); w < na + nb; w += (int64_t)gridDim.x * 8) {
+    if (w < na) oz_slice_atom<2>(a, K, nkb, w, lane);
+    else oz_slice_atom<3>(b, K, nkb, w - na, lane);
   }
 }
 
-// slice planes: out[2(p-1) + (0 re | 1 im)][i][k] = p-th integer slice of X_ik / sc[i],
-// i < rows, k < Kp (zero for k >= K); X[i * rs + k * cs], conjugated if conj
-static_assert(OZ_S * OZ_BETA == 54, "the fixed-point form holds 54 bits");
-__global__ void k_oz_slice(const z* __restrict__ X, int64_t rows, int64_t K, int64_t Kp,
-                           int64_t rs, int64_t cs, int conj, const double* __restrict__ sc,
-                           float* __restrict__ out) {
-  // The p-th slice is the p-th base-2^beta digit of X_ik / sc[i] with its sign: what
-  // repeated multiplication by 2^beta and truncation give (every step exact), taken here
-  // from the fixed-point value F = floor(|X_ik| / sc[i] 2^54) by shifts and masks
-  const int64_t plane = rows * Kp;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < plane;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / Kp, k = e % Kp;
-    uint64_t fr = 0, fi = 0;
-    bool nr = false, ni = false;
-    if (k < K) {
-      const z v = X[i * rs + k * cs];
-      const int esc = (int)(((uint64_t)__double_as_longlong(sc[i]) >> 52) & 0x7ff) - 1023;
-      fr = fixed54(v.x, esc);
-      fi = fixed54(v.y, esc);
-      nr = __double2hiint(v.x) < 0;
-      ni = (__double2hiint(v.y) < 0) != (conj != 0);
-    }
-#pragma unroll
-    for (int p = 0; p < OZ_S; ++p) {
-      const int shift = OZ_S * OZ_BETA - OZ_BETA * (p + 1);
-      const float ar = (float)(int)((fr >> shift) & ((1u << OZ_BETA) - 1));
-      const float ai = (float)(int)((fi >> shift) & ((1u << OZ_BETA) - 1));
-      out[(int64_t)(2 * p) * plane + e] = nr ? -ar : ar;
-      out[(int64_t)(2 * p + 1) * plane + e] = ni ? -ai : ai;
-    }
-  }
+int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// sizes of the context-owned buffer of one product
+struct OzSize {
+  int64_t ntm, ntn, nkb;
+  size_t a, b, e, p;
+};
+OzSize oz_size(int64_t M, int64_t N, int64_t K, int ks) {
+  OzSize s;
+  s.ntm = cdiv(M, OZ_BM);
+  s.ntn = cdiv(N, OZ_BN);
+  s.nkb = cdiv(K, OZ_KB);
+  s.a = ws_round((size_t)(s.ntm * s.nkb) * OZ_S * OZ_TA);
+  s.b = ws_round((size_t)(s.ntn * s.nkb) * OZ_S * OZ_TB);
+  s.e = ws_round(sizeof(int) * (size_t)(M + N));
+  s.p = ws_round(sizeof(longlong2) * 2 * (size_t)ks * M * N);
+  return s;
 }
 
-unsigned ogrid(int64_t n) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 8)); }
-int64_t rup16(int64_t x) { return (x + 15) / 16 * 16; }
+// How a product of `tiles` output tiles and nkb K blocks is dealt to nsm SMs: K splits, and
+// whether an item takes both level groups (one CTA then loads the rings once) or one.  In
+// units of one slice pair over one K block (about 330 clocks) an item costs its pairs times
+// its blocks plus about 8 per group for reading the level sums out; the partial sums of one
+// tile and split cost about 0.4 to write and read back (0.5 MB), spread over the GPU.
+struct OzDeal {
+  int ks, both;
+};
+OzDeal oz_deal(int64_t tiles, int64_t nkb, int nsm) {
+  OzDeal best{1, 1};
+  double cost = 1e300;
+  for (int ks = 1; ks <= 16 && ks <= nkb; ++ks) {
+    if (ks > 1 && tiles * (ks - 1) >= nsm) break;
+    const double kb = (double)cdiv(nkb, ks), heavy = OZ_PAIRS1 * kb + 8.0, light = OZ_PAIRS0 * kb + 8.0;
+    const int64_t n = tiles * ks;
+    const double sums = 0.4 * (double)n;
+    for (int both = 1; both >= 0; --both) {
+      double c;
+      if (both) {
+        c = (double)cdiv(n, nsm) * (heavy + light);
+      } else {
+        // items w, w + nsm, ... of one CTA; the n heavy ones come first
+        c = 0;
+        for (int64_t b : {(int64_t)0, n % nsm, (2 * n) % nsm, (int64_t)nsm - 1}) {
+          const int64_t all = 2 * n > b ? cdiv(2 * n - b, nsm) : 0, h = n > b ? cdiv(n - b, nsm) : 0;
+          c = std::max(c, (double)h * heavy + (double)(all - h) * light);
+        }
+      }
+      c += sums;
+      if (c < cost * 0.98) {
+        cost = c;
+        best = OzDeal{ks, both};
+      }
+    }
+  }
+  return best;
+}
 
 }  // namespace
 
-size_t ozgemm_scratch_bytes(int64_t M, int64_t N, int64_t K, int ks) {
-  const int64_t Kp = rup16(K);
-  return ws_round(sizeof(float) * OZ_PLANES * M * Kp) + ws_round(sizeof(float) * OZ_PLANES * N * Kp) +
-         ws_round(sizeof(double) * M) + ws_round(sizeof(double) * N) +
-         ws_round(sizeof(z) * 2 * (size_t)ks * M * N) + 4096;
-}
-
+// Where the slice product is the faster one.  The FP64 kernel's 16 x 16 tiles take 0.27 us per
+// K entry and round of one tile per SM (512 FMAs of 256 threads at two per clock); the five
+// launches here take about 30 us however small the product.  Measured on both sides of the
+// line (FP64 / slices, us): 128 x 512 x 32 35 / 30, 64 x 512 x 64 18 / 27, 128 x 64 x 128
+// 36 / 29, 256 x 256 x 64 36 / 30, 256 x 1024 x 64 125 / 32, 64 x 64 x 1024 280 / 39.
 bool ozgemm_eligible(const Ctx* c, const ZGemm& g) {
-  // (a Hermitian product asked for its lower part only is formed whole: the caller mirrors it)
-  return c->oz_mode != 0 && g.batch == 1 && g.alpha.x == 1.0 && g.alpha.y == 0.0 &&
-         g.beta.x == 0.0 && g.beta.y == 0.0 && g.M >= 128 && g.N >= 64 && g.K >= 64 &&
-         (double)g.M * (double)g.N * (double)g.K >= 3.0e7 && g.M < (1LL << 31) && g.N < (1LL << 31);
+  if (c->oz_mode == 0 || g.batch != 1 || g.alpha.x != 1.0 || g.alpha.y != 0.0 || g.beta.x != 0.0 ||
+      g.beta.y != 0.0 || g.M < 16 || g.N < 16 || g.K < 16 || g.M >= (1LL << 31) || g.N >= (1LL << 31))
+    return false;
+  const double tiles = (double)cdiv(g.M, 16) * (double)cdiv(g.N, 16) * (g.lower_only ? 0.5 : 1.0);
+  return (double)g.K * std::max(1.0, tiles / 152.0) >= 110.0;
 }
 
-namespace {
-template <int BN>
-int launch_oz(Ctx* c, const CUtensorMap& tA, const CUtensorMap& tB, const OzArgs& a, int nitems, int sm) {
-  static bool attr = false;
-  if (!attr) {
-    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_oz_gemm<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         OzCfg<BN>::SMEM));
-    attr = true;
-  }
-  k_oz_gemm<BN><<<(unsigned)std::min(nitems, sm), 192, OzCfg<BN>::SMEM, c->stream>>>(tA, tB, a);
-  return TNT_OK;
-}
-}  // namespace
-
-// C = A B (FP64-accurate) through the integer-slice tensor-core kernel; slices and the two
-// partial outputs live in the context's own buffer (grown between calls, never inside a
-// capture)
+// C = A B (FP64-accurate) through the integer-slice tensor-core kernel; slices and partial
+// sums live in the context's own buffer (grown between calls, never inside a capture)
 int ozgemm(Ctx* c, const ZGemm& g) {
-  const int64_t M = g.M, N = g.N, K = g.K, Kp = rup16(K);
+  const int64_t M = g.M, N = g.N, K = g.K;
   static int sm = 0;
   if (!sm) {
-    int dev = 0;
+    int dev = 0, v = 0;
     cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sm < 1) sm = 152;
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) v = 152;
+    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
+    sm = v;
   }
-  const int ntm = (int)((M + 127) / 128);
-  // N tile 64 when 128-wide tiles would leave SMs idle; split K when even the 64-wide
-  // (tile, level group) items leave most SMs idle (a 256 x 256 product makes 16), keeping
-  // the partial outputs within 256 MB
-  const int bn = (2LL * ntm * ((N + 127) / 128) < 2LL * sm) ? 64 : 128;
-  const int ntn = (int)((N + bn - 1) / bn);
-  const int nchunk = (int)((Kp + OZ_KC - 1) / OZ_KC);
-  int ks = 1;
-  if (2LL * ntm * ntn < sm) ks = (int)std::min<int64_t>(nchunk, std::max<int64_t>(1, sm / (2LL * ntm * ntn)));
-  while (ks > 1 && 32.0 * ks * (double)M * (double)N > 256e6) --ks;
-  const size_t need = ozgemm_scratch_bytes(M, N, K, ks);
+  OzSize s = oz_size(M, N, K, 0);
+  OzDeal deal = oz_deal(s.ntm * s.ntn, s.nkb, sm);
+  while (deal.ks > 1 && 32.0 * deal.ks * (double)M * (double)N > 256e6) --deal.ks;
+  s = oz_size(M, N, K, deal.ks);
+  const size_t need = s.a + s.b + s.e + s.p;
   if (need > c->oz_cap) {
     TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     dev_free(c->dalloc, c->oz_buf);
@@ -427,48 +603,42 @@ int ozgemm(Ctx* c, const ZGemm& g) {
       return set_err(c, TNT_E_ALLOC, "device allocation of %zu bytes (FP64 product slices) failed", need);
     c->oz_cap = need;
   }
-  char* b = (char*)c->oz_buf;
-  float* Ap = (float*)b;
-  b += ws_round(sizeof(float) * OZ_PLANES * M * Kp);
-  float* Bp = (float*)b;
-  b += ws_round(sizeof(float) * OZ_PLANES * N * Kp);
-  double* sA = (double*)b;
-  b += ws_round(sizeof(double) * M);
-  double* sB = (double*)b;
-  b += ws_round(sizeof(double) * N);
-  z* P = (z*)b;
+  uint8_t* b = (uint8_t*)c->oz_buf;
+  OzOp oa{g.A, M, g.a_rs, g.a_cs, g.conj_a, (int*)(b + s.a + s.b), b};
   // B enters as rows n with K along the row: B^T[n][k] = B[k * b_rs + n * b_cs]
-  k_oz_row_scale<<<ogrid(32 * M), 256, 0, c->stream>>>(g.A, M, K, g.a_rs, g.a_cs, sA);
-  k_oz_row_scale<<<ogrid(32 * N), 256, 0, c->stream>>>(g.B, N, K, g.b_cs, g.b_rs, sB);
+  OzOp ob{g.B, N, g.b_cs, g.b_rs, g.conj_b, oa.e + M, b + s.a};
   {
-    ProfScope ps(c, "oz_slice", 16.0 * (double)(M + N) * (double)K + 4.0 * OZ_PLANES * (double)(M + N) * Kp);
-    k_oz_slice<<<ogrid(M * Kp), 256, 0, c->stream>>>(g.A, M, K, Kp, g.a_rs, g.a_cs, g.conj_a, sA, Ap);
-    k_oz_slice<<<ogrid(N * Kp), 256, 0, c->stream>>>(g.B, N, K, Kp, g.b_cs, g.b_rs, g.conj_b, sB, Bp);
+    ProfScope ps(c, "oz_slice", 16.0 * (double)(M + N) * (double)K + (double)(s.a + s.b));
+    const int64_t nba = oz_scale_blocks(oa, K), nbb = oz_scale_blocks(ob, K);
+    TNT_CUDA_TRY(c, cudaMemsetAsync(oa.e, 0, sizeof(int) * (size_t)(M + N), c->stream));
+    k_oz_scale<<<(unsigned)(nba + nbb), 256, 0, c->stream>>>(oa, ob, K, nba);
+    const int64_t na = s.ntm * (OZ_BM / 8) * s.nkb, nb = s.ntn * (OZ_BN / 8) * s.nkb;
+    k_oz_slice<<<(unsigned)std::min<int64_t>(cdiv(na + nb, 8), 152 * 16), 256, 0, c->stream>>>(
+        oa, ob, K, (int)s.nkb, na, nb);
   }
-  c->launches += 4;
+  c->launches += 2;
   TNT_CHECK_LAUNCH(c);
   OzArgs a;
   a.M = M;
   a.N = N;
-  a.Kp = Kp;
-  a.nchunk = nchunk;
-  a.ks = ks;
-  a.ntm = ntm;
-  a.ntn = ntn;
-  a.P = P;
-  a.sA = sA;
-  a.sB = sB;
+  a.ntm = (int)s.ntm;
+  a.ntn = (int)s.ntn;
+  a.nkb = (int)s.nkb;
+  a.ks = deal.ks;
+  a.both = deal.both;
+  a.A = oa.out;
+  a.B = ob.out;
+  a.P = (longlong2*)(b + s.a + s.b + s.e);
+  a.lower = g.lower_only;
   a.status = c->d_status;
-  CUtensorMap tA, tB;
-  TNT_TRY(tma_map_planes_n(c, &tA, Ap, M, Kp, 128, OZ_PLANES));
-  TNT_TRY(tma_map_planes_n(c, &tB, Bp, N, Kp, bn, OZ_PLANES));
-  const int nitems = 2 * a.ntm * a.ntn * ks;
   {
-    ProfScope ps(c, "oz_gemm", 8.0 * (double)M * (double)N * (double)K);
-    TNT_TRY(bn == 64 ? launch_oz<64>(c, tA, tB, a, nitems, sm) : launch_oz<128>(c, tA, tB, a, nitems, sm));
-    k_oz_finish<<<ogrid(M * N), 256, 0, c->stream>>>(P, 2 * ks, M, N, g.C, g.c_rs);
+    ProfScope ps(c, "oz_gemm", (g.lower_only ? 4.0 : 8.0) * (double)M * (double)N * (double)K);
+    k_oz_gemm<<<(unsigned)std::min(oz_items(a), sm), OZ_THREADS, OZ_SMEM, c->stream>>>(a);
+    c->launches++;
+    k_oz_finish<<<(unsigned)std::min<int64_t>(cdiv(M * N, 256), 152 * 8), 256, 0, c->stream>>>(
+        a.P, a.ks, M, N, oa.e, ob.e, g.lower_only, g.C, g.c_rs);
+    c->launches++;
   }
-  c->launches += 2;
   TNT_CHECK_LAUNCH(c);
   return TNT_OK;
 }
