@@ -2,6 +2,7 @@
 // primitive of App. B.1.1: reorder indices, one matrix product -- here the reorder is
 // folded into the strides), a sparse small-operator kernel for the MPO and gate legs,
 // the Lanczos vector operations and the tridiagonal eigensolve.
+#include <algorithm>
 #include <cstdarg>
 #include <cmath>
 
@@ -202,20 +203,13 @@ namespace {
 constexpr int OP_MAX_NNZ = 2048;
 constexpr int OP_MAX_LEG = 256;
 
-__global__ void __launch_bounds__(256) k_op_apply(OpApply a, int nnz) {
-  __shared__ int s_row[OP_MAX_LEG + 1];
-  __shared__ int s_col[OP_MAX_NNZ];
-  __shared__ z s_val[OP_MAX_NNZ];
-  __shared__ int64_t s_in[OP_MAX_LEG];
-  __shared__ int64_t s_out[OP_MAX_LEG];
-  for (int t = threadIdx.x; t <= a.nI; t += blockDim.x) s_row[t] = a.row_ptr[t];
-  for (int t = threadIdx.x; t < nnz; t += blockDim.x) {
-    s_col[t] = a.col[t];
-    s_val[t] = a.val[t];
-  }
-  for (int t = threadIdx.x; t < a.nJ; t += blockDim.x) s_in[t] = a.in_off[t];
-  for (int t = threadIdx.x; t < a.nI; t += blockDim.x) s_out[t] = a.out_off[t];
-  __syncthreads();
+// One thread per batch element and group of `rows` output indices (blockIdx.y): with all
+// output indices in one thread a small batch (chi = 64: 4096 elements) kept 16 SMs busy, 48
+// us for an operator of 64 outputs.  Operators with real entries (every MPO and bond term of
+// the models here) take two FMAs per entry instead of four on the FP64 pipe.
+template <bool REAL>
+__device__ __forceinline__ void op_rows(const OpApply& a, int i0, int i1, const int* s_row, const int* s_col,
+                                        const z* s_val, const int64_t* s_in, const int64_t* s_out) {
   const int64_t total = a.B0 * a.B1 * a.B2;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -225,14 +219,45 @@ __global__ void __launch_bounds__(256) k_op_apply(OpApply a, int nnz) {
     int64_t b0 = r / a.B1;
     const z* in = a.in + b0 * a.is0 + b1 * a.is1 + b2 * a.is2;
     z* out = a.out + b0 * a.os0 + b1 * a.os1 + b2 * a.os2;
-    for (int i = 0; i < a.nI; ++i) {
+    for (int i = i0; i < i1; ++i) {
       z acc = zmk(0, 0);
-      for (int t = s_row[i]; t < s_row[i + 1]; ++t) zfma(acc, s_val[t], in[s_in[s_col[t]]]);
+      for (int t = s_row[i]; t < s_row[i + 1]; ++t) {
+        const z x = in[s_in[s_col[t]]];
+        if (REAL) {
+          acc.x = fma(s_val[t].x, x.x, acc.x);
+          acc.y = fma(s_val[t].x, x.y, acc.y);
+        } else {
+          zfma(acc, s_val[t], x);
+        }
+      }
       z* p = out + s_out[i];
       if (a.accumulate) acc = zadd(acc, *p);
       *p = acc;
     }
   }
+}
+
+__global__ void __launch_bounds__(256) k_op_apply(OpApply a, int rows) {
+  __shared__ int s_row[OP_MAX_LEG + 1];
+  __shared__ int s_col[OP_MAX_NNZ];
+  __shared__ z s_val[OP_MAX_NNZ];
+  __shared__ int64_t s_in[OP_MAX_LEG];
+  __shared__ int64_t s_out[OP_MAX_LEG];
+  const int i0 = blockIdx.y * rows, i1 = min(a.nI, i0 + rows);
+  for (int t = threadIdx.x; t <= a.nI; t += blockDim.x) s_row[t] = a.row_ptr[t];
+  for (int t = threadIdx.x; t < a.nJ; t += blockDim.x) s_in[t] = a.in_off[t];
+  for (int t = threadIdx.x; t < a.nI; t += blockDim.x) s_out[t] = a.out_off[t];
+  __syncthreads();
+  int cplx = 0;
+  for (int t = s_row[i0] + threadIdx.x; t < s_row[i1]; t += blockDim.x) {
+    s_col[t] = a.col[t];
+    const z v = a.val[t];
+    s_val[t] = v;
+    cplx |= v.y != 0.0;
+  }
+  cplx = __syncthreads_or(cplx);
+  if (cplx) op_rows<false>(a, i0, i1, s_row, s_col, s_val, s_in, s_out);
+  else op_rows<true>(a, i0, i1, s_row, s_col, s_val, s_in, s_out);
 }
 }  // namespace
 
@@ -295,9 +320,11 @@ int op_apply(Ctx* c, const OpApply& a) {
   if (total <= 0) return TNT_OK;
   int64_t blocks = (total + 255) / 256;
   if (blocks > 152 * 16) blocks = 152 * 16;
-  int nnz = a.nnz > 0 ? a.nnz : 1;
   ProfScope ps(c, "op_apply", 8.0 * (double)a.nnz * (double)total);
-  k_op_apply<<<(unsigned)blocks, 256, 0, c->stream>>>(a, nnz);
+  // at least four blocks per SM where the output indices allow it
+  const int64_t want = std::min<int64_t>(a.nI, (152 * 4 + blocks - 1) / blocks);
+  const int rows = (int)((a.nI + want - 1) / want);
+  k_op_apply<<<dim3((unsigned)blocks, (unsigned)((a.nI + rows - 1) / rows)), 256, 0, c->stream>>>(a, rows);
   c->launches++;
   TNT_CHECK_LAUNCH(c);
   return TNT_OK;
@@ -816,10 +843,305 @@ int vec_normalize(Ctx* c, const z* x, z* y, int64_t n, const double* d_norm2) {
   return TNT_OK;
 }
 
+// ============================================================ one Gram-Schmidt step
+// The vector work of one FP64 Krylov step in one cooperative launch: two classical
+// Gram-Schmidt passes of w against V[0..k), the norm, and the next basis vector.
+//   phase 1: c = V^H w           | grid barrier
+//   phase 2: w -= V c, c' = V^H w | grid barrier
+//   phase 3: w -= V c', |w|^2     | grid barrier;  v_k = w / |w|
+// CTA b keeps elements [b S, (b + 1) S) of w in shared memory, and of the basis too where
+// they fit (k S 16 bytes), so that V is read from L2 once.  Each warp takes whole vectors
+// (v = warp, warp + 8, ...) of its CTA's slice: the lanes' sums are combined by a transposed
+// butterfly over four vectors' eight sums (nine FP64 adds instead of 40).  The partial sums
+// of all CTAs are added in CTA order by every CTA, so all hold the same c, and the result is
+// deterministic.
+// What bounds it: the FP64 pipe, 16 k n FMAs at two per SM and clock (27 us at n = 65536,
+// k = 16), and three grid barriers of about 1.5 us.  The separate launches it replaces took
+// 160 us there (four dot-product launches of eight vectors at 27 to 30 us, whatever n: with
+// one element per thread each spent its time reducing 16 sums per thread), 115 us at
+// n = 5000.
+namespace {
+constexpr int GS_THREADS = 256, GS_WARPS = GS_THREADS / 32;
+constexpr int GS_SMEM = 208 * 1024;
+constexpr int64_t GS_MAX_N = 1 << 18;
+
+struct GsArgs {
+  const z* V;
+  int64_t n;
+  int k;
+  const z* w;
+  z* vnext;  // v_k; nullptr: not wanted
+  double* alpha;  // alpha[k - 1] and beta[k - 1] of the step
+  double* beta;
+  z* part;       // 2 x 64 x gridDim.x
+  double* npart; // gridDim.x
+  unsigned* bar; // arrivals, generation, abort flag
+  int* status;
+  int S;
+  int keep;      // V slices in shared memory
+};
+
+// false: a wait expired here or elsewhere, the CTA must stop
+__device__ bool gs_barrier(const GsArgs& a) {
+  __shared__ int s_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    volatile unsigned* gen = a.bar + 1;
+    const unsigned g = *gen;
+    __threadfence();
+    int ok = 1;
+    if (atomicAdd(a.bar, 1u) == gridDim.x - 1) {
+      a.bar[0] = 0;
+      __threadfence();
+      atomicAdd(a.bar + 1, 1u);
+    } else {
+      uint64_t t0, t1;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+      while (*gen == g) {
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
+        if (*(volatile unsigned*)(a.bar + 2)) break;
+        if (t1 - t0 > 2000000000ull) {
+          atomicOr(a.status, 2);
+          atomicExch(a.bar + 2, 1u);
+          break;
+        }
+      }
+    }
+    __threadfence();
+    if (*(volatile unsigned*)(a.bar + 2)) ok = 0;
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
+// eight sums over the warp: lane l returns the total of s[l & 7]
+__device__ __forceinline__ double sum8(double* s) {
+  const int l = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 4; o >= 1; o >>= 1) {  // lanes whose bit o is set keep the upper half
+    const bool up = (l & o) != 0;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const double give = up ? s[i] : s[i + o], keep = up ? s[i + o] : s[i];
+      s[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  double r = s[0];
+  r += __shfl_xor_sync(0xffffffffu, r, 8);
+  r += __shfl_xor_sync(0xffffffffu, r, 16);
+  return r;
+}
+
+// the CTA's share of V^H w to part[v][blockIdx.x]
+template <bool STORE>
+__device__ void gs_dots(const GsArgs& a, const z* sw, z* sv, const z* V0, int64_t ld, int cnt, z* part) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int v0 = warp; v0 < a.k; v0 += 4 * GS_WARPS) {
+    double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    const int nv = min(4, (a.k - v0 + GS_WARPS - 1) / GS_WARPS);
+    const z* p0 = V0 + (int64_t)v0 * ld;
+    const int64_t st = (int64_t)GS_WARPS * ld;
+    if (nv == 4) {
+#pragma unroll 2
+      for (int e = lane; e < cnt; e += 32) {
+        const z x = sw[e];
+        z u[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) u[q] = p0[q * st + e];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (STORE) sv[(int64_t)(v0 + q * GS_WARPS) * a.S + e] = u[q];
+          s[2 * q] = fma(u[q].x, x.x, fma(u[q].y, x.y, s[2 * q]));
+          s[2 * q + 1] = fma(u[q].x, x.y, fma(-u[q].y, x.x, s[2 * q + 1]));
+        }
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        if (q >= nv) break;
+#pragma unroll 4
+        for (int e = lane; e < cnt; e += 32) {
+          const z x = sw[e], u = p0[q * st + e];
+          if (STORE) sv[(int64_t)(v0 + q * GS_WARPS) * a.S + e] = u;
+          s[2 * q] = fma(u.x, x.x, fma(u.y, x.y, s[2 * q]));
+          s[2 * q + 1] = fma(u.x, x.y, fma(-u.y, x.x, s[2 * q + 1]));
+        }
+      }
+    }
+    const double r = sum8(s);
+    if (lane < 2 * nv)
+      ((double*)(part + (int64_t)(v0 + (lane >> 1) * GS_WARPS) * gridDim.x + blockIdx.x))[lane & 1] = r;
+  }
+}
+
+// c[v] = the sum over the CTAs, in shared memory
+__device__ void gs_total(const GsArgs& a, const z* part, z* sc) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int v0 = warp; v0 < a.k; v0 += 4 * GS_WARPS) {
+    double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    const int nv = min(4, (a.k - v0 + GS_WARPS - 1) / GS_WARPS);
+    for (int b = lane; b < (int)gridDim.x; b += 32)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (q < nv) {
+          const z p = __ldcg(part + (int64_t)(v0 + q * GS_WARPS) * gridDim.x + b);
+          s[2 * q] += p.x;
+          s[2 * q + 1] += p.y;
+        }
+    const double r = sum8(s);
+    if (lane < 2 * nv) ((double*)(sc + v0 + (lane >> 1) * GS_WARPS))[lane & 1] = r;
+  }
+  __syncthreads();
+}
+
+// w -= V c over the CTA's slice; returns the thread's share of |w|^2
+__device__ double gs_update(const GsArgs& a, z* sw, const z* V0, int64_t ld, int cnt, const z* sc) {
+  double acc = 0;
+  for (int e = threadIdx.x; e < cnt; e += GS_THREADS) {
+    z x = sw[e];
+    int v = 0;
+    for (; v + 8 <= a.k; v += 8) {
+      z u[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) u[q] = V0[(int64_t)(v + q) * ld + e];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const z c = sc[v + q];
+        x.x = fma(-c.x, u[q].x, fma(c.y, u[q].y, x.x));
+        x.y = fma(-c.x, u[q].y, fma(-c.y, u[q].x, x.y));
+      }
+    }
+    for (; v < a.k; ++v) {
+      const z u = V0[(int64_t)v * ld + e], c = sc[v];
+      x.x = fma(-c.x, u.x, fma(c.y, u.y, x.x));
+      x.y = fma(-c.x, u.y, fma(-c.y, u.x, x.y));
+    }
+    sw[e] = x;
+    acc = fma(x.x, x.x, fma(x.y, x.y, acc));
+  }
+  return acc;
+}
+
+__global__ void __launch_bounds__(GS_THREADS, 1) k_gs_step(GsArgs a) {
+  extern __shared__ z sm_gs[];
+  __shared__ z sc[64];
+  __shared__ double sh[32];
+  __shared__ double s_rn;
+  z* sw = sm_gs;
+  z* sv = sm_gs + a.S;
+  const int64_t lo = (int64_t)blockIdx.x * a.S;
+  const int cnt = (int)max((int64_t)0, min((int64_t)a.S, a.n - lo));
+  const int tid = threadIdx.x;
+  for (int e = tid; e < cnt; e += GS_THREADS) sw[e] = a.w[lo + e];
+  __syncthreads();
+  z* p1 = a.part;
+  z* p2 = a.part + (int64_t)64 * gridDim.x;
+  const z* Vg = a.V + lo;
+  if (a.keep) gs_dots<true>(a, sw, sv, Vg, a.n, cnt, p1);
+  else gs_dots<false>(a, sw, sv, Vg, a.n, cnt, p1);
+  const z* V = a.keep ? sv : Vg;
+  const int64_t ld = a.keep ? a.S : a.n;
+  bool ok = gs_barrier(a);
+  if (ok) {
+    gs_total(a, p1, sc);
+    if (blockIdx.x == 0 && tid == 0) a.alpha[a.k - 1] = sc[a.k - 1].x;
+    gs_update(a, sw, V, ld, cnt, sc);
+    __syncthreads();
+    gs_dots<false>(a, sw, sv, V, ld, cnt, p2);
+    ok = gs_barrier(a);
+  }
+  if (ok) {
+    gs_total(a, p2, sc);
+    double acc = gs_update(a, sw, V, ld, cnt, sc);
+    acc = block_sum(acc, sh);
+    if (tid == 0) a.npart[blockIdx.x] = acc;
+    ok = gs_barrier(a);
+  }
+  if (!ok) {  // the host reads a NaN beta, and the status word names the wait
+    if (blockIdx.x == 0 && tid == 0) a.beta[a.k - 1] = __longlong_as_double(0x7ff8000000000000ll);
+    return;
+  }
+  if (tid < 32) {
+    double r = 0;
+    for (int b = tid; b < (int)gridDim.x; b += 32) r += __ldcg(a.npart + b);
+    r = warp_sum(r);
+    if (tid == 0) {
+      const double nr = sqrt(r);
+      s_rn = 1.0 / nr;
+      if (blockIdx.x == 0) a.beta[a.k - 1] = nr;
+    }
+  }
+  __syncthreads();
+  const double rn = s_rn;
+  if (a.vnext)
+    for (int e = tid; e < cnt; e += GS_THREADS) a.vnext[lo + e] = zscale(sw[e], rn);
+}
+}  // namespace
+
+// Elements of w per CTA, and whether the basis slice is kept: as many CTAs as SMs, down to 64
+// elements each
+bool vec_gs_eligible(int64_t n) { return n <= GS_MAX_N; }
+
+int vec_gs_reset(Ctx* c) {
+  TNT_CUDA_TRY(c, cudaMemsetAsync(c->d_count + 16, 0, 3 * sizeof(unsigned), c->stream));
+  return TNT_OK;
+}
+
+int vec_gs_step(Ctx* c, const z* V, int k, const z* w, int64_t n, z* vnext, double* d_alpha, double* d_beta) {
+  if (k < 1 || k > 64) return set_err(c, TNT_E_UNSUPPORTED, "Gram-Schmidt step with k = %d", k);
+  static int nsm = 0;
+  if (!nsm) {
+    int v = 0;
+    TNT_CUDA_TRY(c, cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, c->device));
+    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_gs_step, cudaFuncAttributeMaxDynamicSharedMemorySize, GS_SMEM));
+    nsm = v;
+  }
+  const size_t top = c->ws.top;
+  z* part = (z*)ws_alloc(c, ws_round(sizeof(z) * 2 * 64 * (size_t)nsm));
+  double* npart = (double*)ws_alloc(c, ws_round(sizeof(double) * (size_t)nsm));
+  c->ws.top = top;  // used by this launch only (stream order serialises its reuse)
+  if (!part || !npart) return set_err(c, TNT_E_ALLOC, "scratch exhausted (Gram-Schmidt step)");
+  GsArgs a;
+  a.V = V; a.n = n; a.k = k; a.w = w; a.vnext = vnext;
+  a.alpha = d_alpha; a.beta = d_beta;
+  a.part = part; a.npart = npart;
+  a.bar = c->d_count + 16;
+  a.status = c->d_status;
+  a.S = (int)std::max<int64_t>(64, (n + nsm - 1) / nsm);
+  const int grid = (int)((n + a.S - 1) / a.S);
+  const size_t sw = sizeof(z) * (size_t)a.S, all = sw * (size_t)(k + 1);
+  a.keep = all <= (size_t)GS_SMEM;
+  const size_t smem = a.keep ? all : sw;
+  if (smem > (size_t)GS_SMEM) return set_err(c, TNT_E_UNSUPPORTED, "Gram-Schmidt step with n = %lld", (long long)n);
+  void* args[] = {&a};
+  {
+    ProfScope ps(c, "gs_step", (32.0 * (double)k + 6.0) * (double)n);  // FP64 FLOPs
+    TNT_CUDA_TRY(c, cudaLaunchCooperativeKernel((void*)k_gs_step, dim3((unsigned)grid), dim3(GS_THREADS), args,
+                                                smem, c->stream));
+  }
+  c->launches++;
+  TNT_CHECK_LAUNCH(c);
+  return TNT_OK;
+}
+
 // ============================================================ tridiagonal eigensolve
-// Lowest eigenpair of the Lanczos matrix T (k <= 64): multisection on the Sturm count by
-// one warp (33 sub-intervals per step), then inverse iteration with a pivoted tridiagonal
-// LU (thread 0).  out[0] = E, out[1] = |y_{k-1}|.
+// Lowest eigenpair of the Lanczos matrix T (k <= 64), one warp per problem.  out[0] = E,
+// out[1] = |y_{k-1}|.  On GB300 an FP64 instruction holds a sub-partition's FP64 pipe for 64
+// clocks however few lanes are active, so what counts is the number of FP64 instructions in
+// sequence:
+//   * the lowest eigenvalue to ~1e-7 |T| by multisection on Sturm counts in FP32;
+//   * Rayleigh quotient iteration from there (two or three rounds, cubic): the vector of the
+//     shift by the three-term recurrences from both ends (lane 0 from the top, lane 1 from
+//     the bottom, two FP64 instructions a row), joined at the row r whose residual
+//     gamma_r = ((T - lam) y)_r is smallest, all rows' residuals and the norm in parallel;
+//     the next shift is lam + gamma_r / |y|^2;
+//   * the quotients of neighbouring entries are the pivots of the twisted factorisation of
+//     T - lam: all of them (but gamma_r) positive says that no eigenvalue lies below, so the
+//     pair found is the lowest.
+// If that check or the convergence fails (a zero beta, eigenvalues closer than rounding), the
+// pair comes from FP64 multisection and inverse iteration.  That form alone took 95 to 105
+// us at k = 20..32, more than the rest of a small problem's Krylov step.
 namespace {
 // number of eigenvalues < x: sign changes of the leading principal minors
 // p_i = (a_i - x) p_{i-1} - b_{i-1}^2 p_{i-2} (division-free Sturm sequence; a zero minor
@@ -848,37 +1170,14 @@ __device__ int sturm_count(const double* a, const double* b, int k, double x) {
   return cnt;
 }
 
-// one block per problem: problem p's alpha, beta, y at p * 64, out at p * 2 (skipped
-// where skip[p] is set)
-__global__ void k_tridiag_lowest(const double* __restrict__ alpha,
-                                 const double* __restrict__ beta, int k,
-                                 double* __restrict__ out, double* __restrict__ y,
-                                 const int* __restrict__ skip) {
-  const int pb = blockIdx.x;
-  if (skip && skip[pb]) return;
-  alpha += 64 * pb;
-  beta += 64 * pb;
-  out += 2 * pb;
-  y += 64 * pb;
-  __shared__ double a[64], b[64];
-  __shared__ double lo_s, hi_s;
-  const int l = threadIdx.x;
-  for (int i = l; i < k; i += 32) a[i] = alpha[i];
-  for (int i = l; i < k - 1; i += 32) b[i] = beta[i];
-  __syncwarp();
-  if (l == 0) {
-    double lo = a[0], hi = a[0];
-    for (int i = 0; i < k; ++i) {
-      double r = (i > 0 ? fabs(b[i - 1]) : 0.0) + (i < k - 1 ? fabs(b[i]) : 0.0);
-      lo = fmin(lo, a[i] - r);
-      hi = fmax(hi, a[i] + r);
-    }
-    double pad = 1e-12 * fmax(fabs(lo), fabs(hi)) + 1e-300;
-    lo_s = lo - pad;
-    hi_s = hi + pad;
-  }
-  __syncwarp();
-  double lo = lo_s, hi = hi_s;
+// FP64 multisection (33 sub-intervals per step) from the Gershgorin interval [lo, hi], then
+// inverse iteration with a pivoted tridiagonal LU (lane 0)
+__device__ __noinline__ void tridiag_bisect(const double* a, const double* b, int k, double lo, double hi,
+                                            double* __restrict__ out, double* __restrict__ y) {
+  const int l = threadIdx.x & 31;
+  const double pad = 1e-12 * fmax(fabs(lo), fabs(hi)) + 1e-300;
+  lo -= pad;
+  hi += pad;
   for (int it = 0; it < 64; ++it) {
     double width = hi - lo;
     if (width <= 4.0 * 2.220446049250313e-16 * fmax(fabs(lo), fabs(hi)) || width <= 1e-300)
@@ -976,6 +1275,236 @@ __global__ void k_tridiag_lowest(const double* __restrict__ alpha,
     out[0] = lam;
     out[1] = fabs(v[k - 1]);
   }
+}
+
+// the vector of one shift: entries of the recurrences from the top (f) and from the bottom
+// (h) with their powers of two, as (value, exponent); s_P, s_Q hold per row the factors of
+// the two recurrences (top first)
+struct TwistShared {
+  double a[64], b[64];
+  double P[2][64], Q[2][64];  // y_{i+1} = P y_i - Q y_{i-1} (top), y_{i-1} = P y_i - Q y_{i+1} (bottom)
+  double v[2][64];
+  int ex[2][64];
+};
+
+__device__ bool tridiag_twisted(TwistShared& S, int k, double lo, double hi, double* __restrict__ out,
+                                double* __restrict__ y) {
+  const int l = threadIdx.x & 31;
+  const unsigned full = 0xffffffffu;
+  const double width = hi - lo;
+  if (!(width > 1e-290) || !(width < 1e290)) return false;
+  // FP32 multisection on (T - lo) / width, eigenvalues in [0, 1]
+  __shared__ float s_a[64], s_b2[64];
+  {
+    const double inv = 1.0 / width;
+    bool bad = false;
+    for (int i = l; i < k; i += 32) {
+      s_a[i] = (float)((S.a[i] - lo) * inv);
+      if (i < k - 1) {
+        const float bf = (float)(S.b[i] * inv);
+        s_b2[i] = bf * bf;
+        bad |= !(fabs(S.b[i]) >= 1e-140 * width);
+      }
+    }
+    if (__any_sync(full, bad)) return false;
+  }
+  __syncwarp();
+  float xl = 0.f, xw = 1.f;
+  for (int it = 0; it < 6 && xw > 6e-8f; ++it) {
+    const float x = xl + xw * (float)(l + 1) * (1.f / 33.f);
+    bool neg = false;
+    float q = s_a[0] - x;
+    for (int i = 1;; ++i) {
+      if (fabsf(q) < 1e-20f) q = -1e-20f;
+      neg |= q < 0.f;
+      if (i >= k) break;
+      q = s_a[i] - x - __fdividef(s_b2[i - 1], q);
+    }
+    const unsigned m = __ballot_sync(full, neg);
+    const int first = m ? __ffs((int)m) - 1 : 32;
+    xl += xw * (float)first * (1.f / 33.f);
+    xw *= 1.f / 33.f;
+  }
+  double lam = lo + width * (double)(xl + 0.5f * xw);
+  const double tiny = 4.0 * 2.220446049250313e-16 * fmax(fabs(lo), fabs(hi));
+  // per row: 1 / b of the row's own and the previous off-diagonal
+  double rb[2], rbm[2];
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    const int i = l + 32 * t;
+    rb[t] = i < k - 1 ? 1.0 / S.b[i] : 0.0;
+    rbm[t] = __shfl_up_sync(full, rb[t], 1);
+    if (l == 0) rbm[t] = 0.0;
+  }
+  {  // row 32's previous off-diagonal is lane 31's first
+    const double r31 = __shfl_sync(full, rb[0], 31);
+    if (l == 0) rbm[1] = r31;
+  }
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    const int i = l + 32 * t;
+    if (i < k) {
+      S.Q[0][i] = i > 0 ? S.b[i - 1] * rb[t] : 0.0;
+      S.Q[1][i] = i < k - 1 ? S.b[i] * rbm[t] : 0.0;
+    }
+  }
+  double gam = 0, nrm = 1;
+  double yv[2] = {0, 0};
+  bool done = false;
+  for (int it = 0; it < 6; ++it) {
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const int i = l + 32 * t;
+      if (i < k) {
+        const double g = lam - S.a[i];
+        S.P[0][i] = g * rb[t];
+        S.P[1][i] = g * rbm[t];
+      }
+    }
+    __syncwarp();
+    if (l < 2) {  // lane 0 from the top, lane 1 from the bottom
+      double y1 = 1.0, y0 = 0.0;  // the last two entries
+      int ex = 0;
+      int i = l ? k - 1 : 0;
+      const int d = l ? -1 : 1;
+      S.v[l][i] = 1.0;
+      S.ex[l][i] = 0;
+      for (int st = 1; st < k; ++st) {
+        const double yn = fma(S.P[l][i], y1, -S.Q[l][i] * y0);
+        i += d;
+        y0 = y1;
+        y1 = yn;
+        const int e = (__double2hiint(yn) >> 20) & 0x7ff;
+        if (e > 1023 + 300 || (e < 1023 - 300 && e > 0)) {  // exact scaling of the pair
+          const double f = __hiloint2double((2046 - e) << 20, 0);
+          y0 *= f;
+          y1 *= f;
+          ex += e - 1023;
+        }
+        S.v[l][i] = y1;
+        S.ex[l][i] = ex;
+      }
+    }
+    __syncwarp();
+    // residual of the vector joined at row i, and the signs of the neighbours' quotients
+    double gi[2];
+    unsigned nf[2], nh[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const int i = l + 32 * t;
+      double g = 0;
+      bool pf = false, ph = false;  // quotient f_{i+1} / f_i, h_{i-1} / h_i not of the right sign
+      if (i < k) {
+        g = S.a[i] - lam;
+        const double f = S.v[0][i], h = S.v[1][i];
+        if (i > 0) {
+          const int e = S.ex[0][i - 1] - S.ex[0][i];
+          const double q = S.v[0][i - 1] / f;
+          g = fma(S.b[i - 1], e ? ldexp(q, e) : q, g);
+          ph = !((S.v[1][i - 1] < 0) != ((h < 0) != (S.b[i - 1] < 0))) || S.v[1][i - 1] == 0.0;
+        }
+        if (i < k - 1) {
+          const int e = S.ex[1][i + 1] - S.ex[1][i];
+          const double q = S.v[1][i + 1] / h;
+          g = fma(S.b[i], e ? ldexp(q, e) : q, g);
+          pf = !((S.v[0][i + 1] < 0) != ((f < 0) != (S.b[i] < 0))) || S.v[0][i + 1] == 0.0;
+        }
+        if (!isfinite(g)) g = INFINITY;
+      } else {
+        g = INFINITY;
+      }
+      gi[t] = g;
+      nf[t] = __ballot_sync(full, pf);
+      nh[t] = __ballot_sync(full, ph);
+    }
+    // the row of the smallest residual: on the bits of |g| rounded to its upper half
+    unsigned key = min(((unsigned)__double2hiint(fabs(gi[0])) & ~63u) | (unsigned)l,
+                       ((unsigned)__double2hiint(fabs(gi[1])) & ~63u) | (unsigned)(l + 32));
+    key = __reduce_min_sync(full, key);
+    const int r = (int)(key & 63u);
+    gam = __shfl_sync(full, r < 32 ? gi[0] : gi[1], r & 31);
+    if (!isfinite(gam)) return false;
+    const uint64_t F = ((uint64_t)nf[1] << 32) | nf[0], H = ((uint64_t)nh[1] << 32) | nh[0];
+    const uint64_t below = r ? (~0ull >> (64 - r)) : 0ull;  // rows above the join
+    const uint64_t above = r < 63 ? ~0ull << (r + 1) : 0ull;
+    const bool lowest = (F & below) == 0 && (H & above) == 0;
+    const double rf = 1.0 / S.v[0][r], rh = 1.0 / S.v[1][r];
+    double s2 = 0;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const int i = l + 32 * t;
+      double v = 0;
+      if (i < k) {
+        const int o = i <= r ? 0 : 1;
+        v = S.v[o][i] * (o ? rh : rf);
+        const int e = S.ex[o][i] - S.ex[o][r];
+        if (e) v = ldexp(v, e);
+        if (i == r) v = 1.0;
+      }
+      yv[t] = v;
+      s2 = fma(v, v, s2);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(full, s2, o);
+    nrm = s2;
+    if (!isfinite(nrm)) return false;
+    const double step = gam / nrm;
+    lam += step;
+    if (fabs(step) <= tiny) {
+      if (!lowest) return false;
+      done = true;
+      break;
+    }
+  }
+  if (!done) return false;
+  // |y| = 1, first non-zero entry positive
+  const double rn = 1.0 / sqrt(nrm);
+  const unsigned z0 = __ballot_sync(full, yv[0] != 0.0), z1 = __ballot_sync(full, yv[1] != 0.0);
+  const double first = z0 ? __shfl_sync(full, yv[0], __ffs((int)z0) - 1) : __shfl_sync(full, yv[1], z1 ? __ffs((int)z1) - 1 : 0);
+  const double sc = first < 0 ? -rn : rn;
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    const int i = l + 32 * t;
+    if (i < k) {
+      y[i] = yv[t] * sc;
+      if (i == k - 1) out[1] = fabs(yv[t] * sc);
+    }
+  }
+  if (l == 0) out[0] = lam;
+  return true;
+}
+
+// one block per problem: problem p's alpha, beta, y at p * 64, out at p * 2 (skipped
+// where skip[p] is set)
+__global__ void __launch_bounds__(32) k_tridiag_lowest(const double* __restrict__ alpha,
+                                                       const double* __restrict__ beta, int k,
+                                                       double* __restrict__ out, double* __restrict__ y,
+                                                       const int* __restrict__ skip) {
+  const int pb = blockIdx.x;
+  if (skip && skip[pb]) return;
+  alpha += 64 * pb;
+  beta += 64 * pb;
+  out += 2 * pb;
+  y += 64 * pb;
+  __shared__ TwistShared S;
+  const int l = threadIdx.x;
+  for (int i = l; i < k; i += 32) S.a[i] = alpha[i];
+  for (int i = l; i < k - 1; i += 32) S.b[i] = beta[i];
+  __syncwarp();
+  // Gershgorin interval
+  double lo = INFINITY, hi = -INFINITY;
+  for (int i = l; i < k; i += 32) {
+    const double r = (i > 0 ? fabs(S.b[i - 1]) : 0.0) + (i < k - 1 ? fabs(S.b[i]) : 0.0);
+    lo = fmin(lo, S.a[i] - r);
+    hi = fmax(hi, S.a[i] + r);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if (!tridiag_twisted(S, k, lo, hi, out, y)) tridiag_bisect(S.a, S.b, k, lo, hi, out, y);
 }
 }  // namespace
 

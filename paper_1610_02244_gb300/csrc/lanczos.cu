@@ -81,6 +81,8 @@ static int lanczos_cycle_loop(Ctx* c, const MatVec& A, z* theta, int precision,
   // u_32 |V c|, stays below the matvec's own ~2^-22 error); the Ritz vector is assembled
   // in FP64, as its norm enters the FP64 Rayleigh quotient
   const bool f32_gs = (precision == TNT_PREC_MIXED);
+  const bool fused_gs = !f32_gs && vec_gs_eligible(n);
+  if (fused_gs) TNT_TRY(vec_gs_reset(c));
   double* hp = c->h_pinned;
   // v_0 = theta / |theta| (a zero or non-finite start vector is reported, not iterated)
   TNT_TRY(vec_norm2(c, theta, n, norm2));
@@ -123,6 +125,15 @@ static int lanczos_cycle_loop(Ctx* c, const MatVec& A, z* theta, int precision,
     *cv = (resid_only || (have_prev && std::fabs(E - E_prev) <= tol * std::fabs(E))) &&
           resid <= rtol * std::fabs(E);
     if (bk <= rtol * std::fabs(E) * 1e-3 || bk == 0.0) *cv = true;
+    if (fused_gs && !std::isfinite(bk)) {  // a grid barrier's expired wait, or the numbers?
+      int st = 0;
+      TNT_CUDA_TRY(c, cudaMemcpyAsync(&st, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+      TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+      if (st & 2) {
+        cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
+        return set_err(c, TNT_E_TIMEOUT, "Gram-Schmidt step: a grid barrier wait expired");
+      }
+    }
     if (!std::isfinite(E) || !std::isfinite(bk))
       return set_err(c, TNT_E_NAN, "Lanczos produced a non-finite value at step %d (E = %g, beta = %g, %s matvec)",
                      total, E, bk, precision == TNT_PREC_MIXED ? "split-TF32" : "FP64");
@@ -137,25 +148,31 @@ static int lanczos_cycle_loop(Ctx* c, const MatVec& A, z* theta, int precision,
       z* vk = V + (int64_t)k * n;
       TNT_TRY(A.apply(c, vk, w, precision));
       ++total;
-      if (f32_gs) {
-        TNT_TRY(vec_multidot_f32(c, V, n, k + 1, w, n, dots));
-        TNT_TRY(vec_multiaxpy_norm_f32(c, V, n, k + 1, dots, w, n, norm2));
+      if (fused_gs) {
+        // v_{k+1} belongs to the next step; the last step of a cycle has none
+        const bool last = k + 1 == cap || total >= max_matvec;
+        TNT_TRY(vec_gs_step(c, V, k + 1, w, n, last ? nullptr : V + (int64_t)(k + 1) * n, alpha, beta));
       } else {
-        TNT_TRY(vec_multidot(c, V, n, k + 1, w, n, dots));
-        TNT_TRY(vec_multiaxpy_norm(c, V, n, k + 1, dots, w, n, norm2));
+        if (f32_gs) {
+          TNT_TRY(vec_multidot_f32(c, V, n, k + 1, w, n, dots));
+          TNT_TRY(vec_multiaxpy_norm_f32(c, V, n, k + 1, dots, w, n, norm2));
+        } else {
+          TNT_TRY(vec_multidot(c, V, n, k + 1, w, n, dots));
+          TNT_TRY(vec_multiaxpy_norm(c, V, n, k + 1, dots, w, n, norm2));
+        }
+        k_lz_scalars<<<1, 32, 0, c->stream>>>(dots, k, norm2, alpha, beta);  // alpha_k from pass 1
+        c->launches += 1;
+        if (f32_gs) {
+          TNT_TRY(vec_multidot_f32(c, V, n, k + 1, w, n, coef));
+          TNT_TRY(vec_multiaxpy_norm_f32(c, V, n, k + 1, coef, w, n, norm2));
+        } else {
+          TNT_TRY(vec_multidot(c, V, n, k + 1, w, n, coef));
+          TNT_TRY(vec_multiaxpy_norm(c, V, n, k + 1, coef, w, n, norm2));
+        }
+        // beta_k from pass 2 (overwrite), then the tridiagonal eigenpair of T_k on the side
+        k_lz_scalars<<<1, 32, 0, c->stream>>>(dots, k, norm2, alpha, beta);
+        c->launches++;
       }
-      k_lz_scalars<<<1, 32, 0, c->stream>>>(dots, k, norm2, alpha, beta);  // alpha_k from pass 1
-      c->launches += 1;
-      if (f32_gs) {
-        TNT_TRY(vec_multidot_f32(c, V, n, k + 1, w, n, coef));
-        TNT_TRY(vec_multiaxpy_norm_f32(c, V, n, k + 1, coef, w, n, norm2));
-      } else {
-        TNT_TRY(vec_multidot(c, V, n, k + 1, w, n, coef));
-        TNT_TRY(vec_multiaxpy_norm(c, V, n, k + 1, coef, w, n, norm2));
-      }
-      // beta_k from pass 2 (overwrite), then the tridiagonal eigenpair of T_k on the side
-      k_lz_scalars<<<1, 32, 0, c->stream>>>(dots, k, norm2, alpha, beta);
-      c->launches++;
       TNT_TRY(launch_tk(k));
       if (k > 0) {
         bool cv = false;
@@ -177,7 +194,7 @@ static int lanczos_cycle_loop(Ctx* c, const MatVec& A, z* theta, int precision,
       }
       // v_{k+1}, except after the last step of a cycle: the basis holds cap vectors, and
       // the restart begins from the Ritz vector instead
-      TNT_TRY(vec_normalize(c, w, V + (int64_t)(k + 1) * n, n, norm2));
+      if (!fused_gs) TNT_TRY(vec_normalize(c, w, V + (int64_t)(k + 1) * n, n, norm2));
     }
     // the side stream's work is done before the main stream reuses its buffers
     TNT_CUDA_TRY(c, cudaStreamWaitEvent(c->stream, c->ev_side[last_side], 0));

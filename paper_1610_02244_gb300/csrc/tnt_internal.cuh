@@ -210,6 +210,16 @@ int vec_normalize(Ctx* c, const z* x, z* y, int64_t n, const double* d_norm2);
 int vec_norm2(Ctx* c, const z* x, int64_t n, double* d_norm2);
 int vec_dot(Ctx* c, const z* x, const z* y, int64_t n, z* d_dot);
 
+// Both FP64 Gram-Schmidt passes of one Krylov step in one launch (n up to the bound of
+// vec_gs_eligible): w against V[0..k) (leading dimension n) twice, alpha[k-1] = Re <V_{k-1}|w>
+// of the first pass, beta[k-1] = |w| after the second, vnext = w / |w| (none if null); w
+// itself is left as it was.  vec_gs_reset before the first step of a solve: the grid barrier's
+// words (a barrier whose wait expired leaves them set).
+bool vec_gs_eligible(int64_t n);
+int vec_gs_reset(Ctx* c);
+int vec_gs_step(Ctx* c, const z* V, int k, const z* w, int64_t n, z* vnext, double* d_alpha,
+                double* d_beta);
+
 // Lanczos tridiagonal: lowest eigenpair of T (k x k) given alpha[0..k-1], beta[0..k-2];
 // writes out[0] = E, out[1] = |y_{k-1}|, and y[0..k-1].
 int tridiag_lowest(Ctx* c, const double* d_alpha, const double* d_beta, int k, double* d_out,
