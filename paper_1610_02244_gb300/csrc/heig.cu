@@ -14,7 +14,8 @@
 //   5. Two Newton-Schulz steps U <- U (3 I - U^H U) / 2 in FP64 to restore orthonormality
 //      lost to close eigenvalues.
 // All arithmetic is FP64.  The cost is O(n^3) once, against O(sweeps n^3) for a Jacobi
-// eigensolver.  Blocks of up to 256 rows are reduced together, one CTA each.
+// eigensolver.  Blocks of up to 1216 rows go through every stage together (heig_blocks).
+#include <algorithm>
 #include <cmath>
 
 #include "heff_plan.cuh"
@@ -355,34 +356,95 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tridiag_persistent(TriArgs a) {
 }
 
 // ---------------------------------------------------------------- rows in shared memory
-// The same column-by-column reduction for n <= TRI_ROWS_NMAX with each block's rows of the
-// matrix (row g belongs to block g mod nb) resident in its shared memory for the whole
-// reduction: the trailing update and the product with the next reflector touch shared
-// memory only, and per column the global memory carries p (n entries), the per-block
-// partial sums and the one row that is the source of the next reflector.
+// The same column-by-column reduction for blocks of n <= TRI_ROWS_NMAX rows, several blocks
+// (the charge blocks of one truncated SVD) in one cooperative launch.  A block gets a group of
+// CTAs in proportion to its work (tri_deal); row g of the block belongs to CTA g mod nb of
+// its group and stays in that CTA's shared memory for the whole reduction: the trailing
+// update and the product with the next reflector touch shared memory only, and per column
+// the global memory carries p (n entries), the per-CTA partial sums and the one row that is
+// the source of the next reflector.  The group's own barrier, once per column; a group of
+// one CTA needs none, and keeps p in shared memory.
 // Reflector j is v_j = (1, conj(x_c) s_j for c > j+1) with x row j of the updated matrix
 // and s_j its scale; p_j = tau_j T_j v_j is formed without v_j as
 // tau_j (T(g, j+1) + s_j sum_{c > j+1} T(g, c) conj(x_c)), so that the reflector's
-// scalars (a block sum and one thread's square root and divisions) are computed while the
-// rows are updated, and v_j is written out at the start of the next column.  Entering
-// column j every block holds x (in sx, the entry j+1 zeroed), tau_j and s_j, and p_j with
-// the per-block partial sums of p_j^H v_j is in global memory:
-//   every block, one pass over the columns c > j with its loads issued first: v_j(c);
-//     w_j(c) = p_j(c) + cf v_j(c), cf = -(tau_j / 2) p_j^H v_j; and
+// scalars are computed by a warp of their own (TRI_WARPS, a square root and two divisions:
+// about 100 FP64 instructions in sequence, 3 us) while the others update the rows.
+// Entering column j every CTA holds x (in sx, the entry j+1 zeroed), tau_j and s_j, and p_j
+// with the per-CTA partial sums of p_j^H v_j is in global memory:
+//   the scalar warp: cf = -(tau_j / 2) p_j^H v_j; the others: v_j(c), and loads of p_j and
+//     row j+1;
+//   one pass over the columns c > j: w_j(c) = p_j(c) + cf v_j(c), and
 //     x'(c) = T_j(j+1, c) - conj(w_j(c)) - w_j(j+1) conj(v_j(c)), row j+1 after the
 //     update (v_j(j+1) = 1), into sx, with the sum of |x'(c)|^2 over c > j+2;
-//   each block, its rows g > j+1 of T_j, split evenly over its warps (a warp spans at most
-//     two rows): T <- T - v_j w_j^H - w_j v_j^H and sum_c T(g, c) conj(x'(c)); the owner
-//     of row j+2 also stores it in global memory for the next column;
-//   warp 0: reflector j+1 (alpha = conj(x'(j+2))), then p_{j+1}(g) for the block's rows
-//     and the block's share of p_{j+1}^H v_{j+1};
-//   grid barrier.
-// Vectors are indexed by global row.  Per column a block spends 16 FP64 operations per
+//   the scalar warp: reflector j+1; the others, the CTA's rows g > j+1 of T_j, flattened over
+//     (row, column) and split evenly over the warps: T <- T - v_j w_j^H - w_j v_j^H and
+//     sum_c T(g, c) conj(x'(c)); the owner of row j+2 also stores it in global memory;
+//   warp 0: p_{j+1}(g) for the CTA's rows and its share of p_{j+1}^H v_{j+1};
+//   group barrier.
+// Reflector j replaces row j of the block in global memory (columns 0 .. n-j-2), the layout
+// the back-transformation reads: no CTA reads row j after its barrier j.
+// Vectors are indexed by row of the block.  Per column a CTA spends 16 FP64 operations per
 // trailing entry on the shared vectors and 12 per entry of its rows.
-constexpr int TRI_ROWS_MAX = 8;         // rows per block
+// Before, blocks of up to 256 rows were reduced on one SM each (a 200-row block: 3.8 ms,
+// the FP64 pipe of one SM) and larger ones one after the other across the GPU (500 rows
+// 4.5 ms, 1024 rows 24.4 ms with the scalars between two barriers of the CTA).
 static_assert(TRI_WARPS == 16, "the flattened row split divides by 16 with shifts");
 constexpr int TRI_VEC = 3;              // vector entries per thread
 constexpr int64_t TRI_ROWS_NMAX = 1216; // <= TRI_VEC * TRI_THREADS; (8 + 3) n entries fit
+constexpr int TRI_RMAX = 128;           // rows per CTA
+constexpr int TRI_GTHREADS = TRI_THREADS + 32;
+constexpr int TRI_MAXB = 48;            // blocks of one launch
+
+struct TriBlk {
+  z* G;          // the block, n x n; its rows become the reflectors
+  z* tau;
+  double* d;
+  double* e;
+  z* p;          // 2 x n: p of even / odd columns
+  z* part;       // 2 x nb partial sums of p^H v
+  int n, c0, nb; // CTAs [c0, c0 + nb)
+};
+struct TriGroup {
+  int nblk;
+  unsigned* bar;   // 32 words per block: arrivals, generation
+  int* abort_flag;
+  int* status;
+  TriBlk b[TRI_MAXB];
+};
+
+// false: a wait expired here or elsewhere, the CTA must stop
+__device__ bool group_barrier(const TriGroup& t, int grp, int nb) {
+  __shared__ int s_ok;
+  __syncthreads();
+  if (nb == 1) return true;
+  if (threadIdx.x == 0) {
+    unsigned* bar = t.bar + 32 * grp;
+    volatile unsigned* gen = bar + 1;
+    const unsigned g = *gen;
+    __threadfence();
+    int ok = 1;
+    if (atomicAdd(bar, 1u) == (unsigned)nb - 1u) {
+      bar[0] = 0;
+      __threadfence();
+      atomicAdd(bar + 1, 1u);
+    } else {
+      const uint64_t t0 = gtime();
+      while (*gen == g) {
+        if (*(volatile int*)t.abort_flag) break;
+        if (gtime() - t0 > 2000000000ull) {
+          atomicOr(t.status, 2);
+          atomicExch(t.abort_flag, 1);
+          break;
+        }
+      }
+    }
+    __threadfence();
+    if (*(volatile int*)t.abort_flag) ok = 0;
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
 
 // (a, b) summed over the warp with five FP64 adds (the two sums share each step); every
 // lane returns both
@@ -396,170 +458,220 @@ __device__ __forceinline__ void warp_sum_pair(double& a, double& b) {
 }
 
 struct RowsShared {
-  double br[TRI_WARPS][2], bi[TRI_WARPS][2];  // per warp, per row segment: sum T conj(x)
-  double nrm[TRI_WARPS];                       // per warp: sum |x|^2
-  Refl rf;                                     // reflector of the column being finished
-  z cf, alpha;
+  double br[TRI_WARPS][2], bi[TRI_WARPS][2];  // few rows: per warp and row segment, sum T conj(x)
+  z q0[TRI_RMAX], q1[TRI_RMAX];               // many rows: per row, from its start / its second warp
+  double nrm[TRI_WARPS];                      // per warp: sum |x|^2
+  Refl rf[2];                                 // reflectors of even / odd columns
+  z cf, alpha, part;
 };
 
-// Rows g >= lo of this block (rows[i] = row b + nb i, R of them), flattened over
-// (row, column) and split evenly over the warps: with UPD,
-// T(g, c) -= v(g) conj(w(c)) + w(g) conj(v(c)) for c >= lo (the row g == lo also to
-// grow); the sum over c >= lo of T(g, c) conj(x(c)) into S.br/bi[warp][segment].
+// Reflector parameters by one warp (refl_params with the two divisions side by side)
+__device__ Refl refl_warp(z alpha, double xn2, bool empty) {
+  Refl R;
+  if (empty || (xn2 == 0.0 && alpha.y == 0.0)) {
+    R.tau = zmk(0, 0);
+    R.beta = alpha.x;
+    R.scale = zmk(0, 0);
+    return R;
+  }
+  const double nrm = sqrt(fma(alpha.x, alpha.x, fma(alpha.y, alpha.y, xn2)));
+  R.beta = alpha.x >= 0 ? -nrm : nrm;
+  const z den = zmk(alpha.x - R.beta, alpha.y);  // scale = 1 / (alpha - beta)
+  const double dd = fma(den.x, den.x, den.y * den.y);
+  const double r = 1.0 / ((threadIdx.x & 1) ? dd : R.beta);
+  const double rb = __shfl_sync(0xffffffffu, r, 0), rd = __shfl_sync(0xffffffffu, r, 1);
+  R.tau = zmk(-den.x * rb, -alpha.y * rb);
+  R.scale = zmk(den.x * rd, -den.y * rd);
+  return R;
+}
+
+// one segment of a row: T(g, c) -= v(g) conj(w(c)) + w(g) conj(v(c)) (with UPD; also to gout)
+// for c0 <= c < c1, and the sum of T(g, c) conj(x(c)); every lane returns it
 template <bool UPD>
-__device__ void rows_update(z* rows, int R, int b, int nb, int64_t n, int64_t lo,
-                            const z* v, const z* w, const z* x, z* grow, RowsShared& S) {
+__device__ __forceinline__ z row_segment(z* rw, int c0, int c1, z vr, z wr, const z* v, const z* w, const z* x,
+                                         z* gout) {
+  double sr = 0, si = 0;
+#pragma unroll 2
+  for (int c = c0 + (threadIdx.x & 31); c < c1; c += 32) {
+    z t = rw[c];
+    if (UPD) {
+      zsub_mul_conj(t, vr, w[c]);
+      zsub_mul_conj(t, wr, v[c]);
+      rw[c] = t;
+      if (gout) gout[c] = t;
+    }
+    const z y = x[c];  // t conj(y)
+    sr = fma(t.x, y.x, fma(t.y, y.y, sr));
+    si = fma(t.y, y.x, fma(-t.x, y.y, si));
+  }
+  warp_sum_pair(sr, si);
+  return zmk(sr, si);
+}
+
+// Rows g >= lo of this CTA (rows[i] = row b + nb i, R of them) over the 16 row warps: warp w
+// covers [f0, f1) of the flattened (row, column) range, f0 = ract L w / 16, and starts in row
+// floor(ract w / 16) (exact: floor(floor(x) / L) = floor(x / L)).  Fewer than 16 rows: a warp
+// meets at most two rows, a row several warps.  16 and more: a row meets at most two warps.
+template <bool UPD>
+__device__ void rows_update(z* rows, int R, int b, int nb, int n, int lo, const z* v, const z* w, const z* x,
+                            z* grow, RowsShared& S) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i0 = (lo > b) ? (int)((lo - b + nb - 1) / nb) : 0;
+  const int i0 = (lo > b) ? (lo - b + nb - 1) / nb : 0;
   const int ract = R - i0 > 0 ? R - i0 : 0;
-  // warp w covers [f0, f1) of the flattened (row, column) range, f0 = ract L w / 16, and
-  // starts in row floor(ract w / 16) (exact: floor(floor(x) / L) = floor(x / L)); all in
-  // 32-bit multiplies and shifts (ract L <= 8 * 1216)
   const unsigned L = (unsigned)(n - lo), total = (unsigned)ract * L;
   const unsigned f0 = (total * (unsigned)warp) >> 4, f1 = (total * (unsigned)(warp + 1)) >> 4;
   const int r0 = (ract * warp) >> 4;
+  if (ract < 16) {
 #pragma unroll
-  for (int seg = 0; seg < 2; ++seg) {
-    double sr = 0, si = 0;
-    const int ri = r0 + seg;  // row of this segment
-    const int64_t s0 = (seg == 0) ? (int64_t)f0 - (int64_t)ri * L : 0;
-    const int64_t s1 = min((int64_t)L, (int64_t)f1 - (int64_t)ri * L);
-    if (ri < ract && s0 < s1) {
-      const int i = i0 + ri;
-      const int64_t g = b + (int64_t)nb * i;
-      z* rw = rows + (int64_t)i * n;
-      z vr = zmk(0, 0), wr = zmk(0, 0);
-      if (UPD) {
-        vr = v[g];
-        wr = w[g];
+    for (int seg = 0; seg < 2; ++seg) {
+      const int ri = r0 + seg;  // row of this segment
+      const int s0 = (seg == 0) ? (int)f0 - ri * (int)L : 0;
+      const int s1 = min((int)L, (int)f1 - ri * (int)L);
+      z s = zmk(0, 0);
+      if (ri < ract && s0 < s1) {
+        const int i = i0 + ri, g = b + nb * i;
+        s = row_segment<UPD>(rows + (int64_t)i * n, lo + s0, lo + s1, UPD ? v[g] : zmk(0, 0), UPD ? w[g] : zmk(0, 0),
+                             v, w, x, (UPD && g == lo) ? grow : nullptr);
       }
-      z* gout = (UPD && g == lo) ? grow : nullptr;
-#pragma unroll 2
-      for (int64_t c = lo + s0 + lane; c < lo + s1; c += 32) {
-        z t = rw[c];
-        if (UPD) {
-          zsub_mul_conj(t, vr, w[c]);
-          zsub_mul_conj(t, wr, v[c]);
-          rw[c] = t;
-          if (gout) gout[c] = t;
-        }
-        const z y = x[c];  // t conj(y)
-        sr = fma(t.x, y.x, fma(t.y, y.y, sr));
-        si = fma(t.y, y.x, fma(-t.x, y.y, si));
+      if (lane == 0) {
+        S.br[warp][seg] = s.x;
+        S.bi[warp][seg] = s.y;
       }
     }
-    warp_sum_pair(sr, si);
+    return;
+  }
+  for (int ri = r0; ri < ract && (unsigned)ri * L < f1; ++ri) {
+    const int s0 = max(0, (int)f0 - ri * (int)L), s1 = min((int)L, (int)f1 - ri * (int)L);
+    if (s0 >= s1) continue;
+    const int i = i0 + ri, g = b + nb * i;
+    const z s = row_segment<UPD>(rows + (int64_t)i * n, lo + s0, lo + s1, UPD ? v[g] : zmk(0, 0),
+                                 UPD ? w[g] : zmk(0, 0), v, w, x, (UPD && g == lo) ? grow : nullptr);
     if (lane == 0) {
-      S.br[warp][seg] = sr;
-      S.bi[warp][seg] = si;
+      if (s0 == 0) S.q0[ri] = s;
+      else S.q1[ri] = s;
     }
   }
 }
 
-// Warp 0 after rows_update: reflector from (alpha, the block's sum of |x|^2 in S.nrm) for
-// the column whose trailing block starts at lo; p(g) = tau (T(g, lo) + s sum) for the
-// block's rows g >= lo into pout, the block's sum of conj(p(g)) v(g) into *partout
-// (v(lo) = 1, v(c) = conj(x(c)) s).  Lane 0 returns the reflector in S.rf.
-__device__ void rows_finish(const z* rows, int R, int b, int nb, int64_t n, int64_t lo,
-                            const z* x, bool empty, z* pout, z* partout, RowsShared& S) {
+// Warp 0 after rows_update, with reflector rf of the column whose trailing block starts at lo:
+// p(g) = tau (T(g, lo) + s sum) for the CTA's rows g >= lo into pout, the CTA's sum of
+// conj(p(g)) v(g) into *partout (v(lo) = 1, v(c) = conj(x(c)) s).
+__device__ void rows_finish(const z* rows, int R, int b, int nb, int n, int lo, const z* x, const Refl& rf, z* pout,
+                            z* partout, RowsShared& S) {
   const int lane = threadIdx.x & 31;
-  double nr = lane < TRI_WARPS ? S.nrm[lane] : 0.0;
-  nr = warp_sum_d(nr);
-  if (lane == 0) S.rf = refl_params(empty ? zmk(0, 0) : S.alpha, nr, empty);
-  __syncwarp();
-  const Refl rf = S.rf;
-  const int i0 = (lo > b) ? (int)((lo - b + nb - 1) / nb) : 0;
+  const int i0 = (lo > b) ? (lo - b + nb - 1) / nb : 0;
   const int ract = R - i0 > 0 ? R - i0 : 0;
   const unsigned L = (unsigned)(n - lo), total = (unsigned)ract * L;
   double pr = 0, pi = 0;
-  if (lane < ract) {
+  for (int r = lane; r < ract; r += 32) {
     double sr = 0, si = 0;
-    for (int w = 0; w < TRI_WARPS; ++w) {  // the warps whose range meets row `lane`, in order
-      const unsigned f0 = (total * (unsigned)w) >> 4, f1 = (total * (unsigned)(w + 1)) >> 4;
-      const int r0 = (ract * w) >> 4;
-      if (f0 < f1 && r0 == lane) {
-        sr += S.br[w][0];
-        si += S.bi[w][0];
-      } else if (f0 < f1 && r0 + 1 == lane && f1 > (unsigned)lane * L) {
-        sr += S.br[w][1];
-        si += S.bi[w][1];
+    if (ract < 16) {
+      for (int w = 0; w < TRI_WARPS; ++w) {  // the warps whose range meets row r, in order
+        const unsigned f0 = (total * (unsigned)w) >> 4, f1 = (total * (unsigned)(w + 1)) >> 4;
+        const int r0 = (ract * w) >> 4;
+        if (f0 < f1 && r0 == r) {
+          sr += S.br[w][0];
+          si += S.bi[w][0];
+        } else if (f0 < f1 && r0 + 1 == r && f1 > (unsigned)r * L) {
+          sr += S.br[w][1];
+          si += S.bi[w][1];
+        }
+      }
+    } else {
+      sr = S.q0[r].x;
+      si = S.q0[r].y;
+      // the first warp boundary after the row's start, if it falls inside the row
+      const unsigned rl = (unsigned)r * L, w = (16u * (rl + 1u) + total - 1u) / total;
+      if (w < 16u && ((total * w) >> 4) < rl + L) {
+        sr += S.q1[r].x;
+        si += S.q1[r].y;
       }
     }
-    const int64_t g = b + (int64_t)nb * (i0 + lane);
-    const z t0 = rows[(int64_t)(i0 + lane) * n + lo];
+    const int g = b + nb * (i0 + r);
+    const z t0 = rows[(int64_t)(i0 + r) * n + lo];
     const z q = zmk(t0.x + rf.scale.x * sr - rf.scale.y * si, t0.y + rf.scale.x * si + rf.scale.y * sr);
     const z pv = zmul(rf.tau, q);
     pout[g] = pv;
     const z vg = (g == lo) ? zmk(1, 0) : zmul(zconj(x[g]), rf.scale);
-    pr = pv.x * vg.x + pv.y * vg.y;
-    pi = pv.x * vg.y - pv.y * vg.x;
+    pr = fma(pv.x, vg.x, fma(pv.y, vg.y, pr));
+    pi = fma(pv.x, vg.y, fma(-pv.y, vg.x, pi));
   }
   warp_sum_pair(pr, pi);
   if (lane == 0) *partout = zmk(pr, pi);
 }
 
-__global__ void __launch_bounds__(TRI_THREADS) k_tridiag_rows(TriArgs a) {
+__global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_constant__ TriGroup T) {
   extern __shared__ z sm_tri[];
   __shared__ RowsShared S;
-  const int64_t n = a.n;
-  const int nb = gridDim.x, b = blockIdx.x;
+  int grp = 0;
+  while (grp + 1 < T.nblk && T.b[grp + 1].c0 <= (int)blockIdx.x) ++grp;
+  const TriBlk& a = T.b[grp];
+  const int n = a.n, nb = a.nb, b = (int)blockIdx.x - a.c0;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int rmax = (int)((n + nb - 1) / nb);
-  const int R = (b < n) ? (int)((n - b + nb - 1) / nb) : 0;
+  const bool scalar = warp == TRI_WARPS;  // the warp of the scalars
+  const int rmax = (n + nb - 1) / nb;
+  const int R = (b < n) ? (n - b + nb - 1) / nb : 0;
   z* rows = sm_tri;
   z* sv = rows + (int64_t)rmax * n;  // v_j
   z* sw = sv + n;                    // w_j
   z* sx = sw + n;                    // x of the next reflector (its first entry zeroed)
+  z* sp = sx + n;                    // p, in a group of one CTA
+  const bool one = nb == 1;
   for (int i = 0; i < R; ++i) {
     const z* src = a.G + (b + (int64_t)nb * i) * n;
-    for (int64_t c = tid; c < n; c += TRI_THREADS) rows[(int64_t)i * n + c] = __ldcg(src + c);
+    for (int c = tid; c < n; c += TRI_GTHREADS) rows[(int64_t)i * n + c] = __ldcg(src + c);
   }
   {  // reflector 0 from row 0 (columns 1..n-1), and p_0
     double acc = 0;
+    if (!scalar) {
 #pragma unroll
-    for (int k = 0; k < TRI_VEC; ++k) {
-      const int64_t c = 1 + tid + (int64_t)k * TRI_THREADS;
-      if (c < n) {
-        const z xc = __ldcg(a.G + c);
-        if (c == 1) S.alpha = zconj(xc);
-        else acc = fma(xc.x, xc.x, fma(xc.y, xc.y, acc));
-        sx[c] = (c == 1) ? zmk(0, 0) : xc;
+      for (int k = 0; k < TRI_VEC; ++k) {
+        const int c = 1 + tid + k * TRI_THREADS;
+        if (c < n) {
+          const z xc = __ldcg(a.G + c);
+          if (c == 1) S.alpha = zconj(xc);
+          else acc = fma(xc.x, xc.x, fma(xc.y, xc.y, acc));
+          sx[c] = (c == 1) ? zmk(0, 0) : xc;
+        }
       }
+      acc = warp_sum_d(acc);
+      if (lane == 0) S.nrm[warp] = acc;
     }
-    acc = warp_sum_d(acc);
-    if (lane == 0) S.nrm[warp] = acc;
     __syncthreads();
-    rows_update<false>(rows, R, b, nb, n, 1, sv, sw, sx, nullptr, S);
-    __syncthreads();
-    if (warp == 0) {
-      rows_finish(rows, R, b, nb, n, 1, sx, n < 2, a.p, a.part + b, S);
-      if (b == 0 && lane == 0) {
-        a.tau[0] = S.rf.tau;
-        a.d[0] = __ldcg(a.G).x;
-        if (n > 1) a.e[0] = S.rf.beta;
+    if (scalar) {
+      double nr = lane < TRI_WARPS ? S.nrm[lane] : 0.0;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
+      nr = __shfl_sync(0xffffffffu, nr, 0);
+      const Refl rf = refl_warp(n > 1 ? S.alpha : zmk(0, 0), nr, n < 2);
+      if (lane == 0) {
+        S.rf[0] = rf;
+        if (b == 0) {
+          a.tau[0] = rf.tau;
+          a.d[0] = __ldcg(a.G).x;
+          if (n > 1) a.e[0] = rf.beta;
+        }
       }
+    } else {
+      rows_update<false>(rows, R, b, nb, n, 1, sv, sw, sx, nullptr, S);
     }
+    __syncthreads();
+    if (warp == 0) rows_finish(rows, R, b, nb, n, 1, sx, S.rf[0], one ? sp : a.p, one ? &S.part : a.part + b, S);
   }
-  for (int64_t j = 0; j + 1 < n; ++j) {
-    if (!grid_barrier(a)) return;
-    const Refl rf = S.rf;  // reflector j
-    const z* pj = a.p + (j & 1) * n;
-    z* pn = a.p + ((j + 1) & 1) * n;
-    const z* partj = a.part + (j & 1) * nb;
-    z* partn = a.part + ((j + 1) & 1) * nb;
-    const z* grow = a.G + (j + 1) * n;
+  for (int j = 0; j + 1 < n; ++j) {
+    if (!group_barrier(T, grp, nb)) return;
+    const Refl rf = S.rf[j & 1];  // reflector j
+    const z* pj = one ? sp : a.p + (j & 1) * n;
+    z* pn = one ? sp : a.p + ((j + 1) & 1) * n;
+    const z* partj = one ? &S.part : a.part + (j & 1) * nb;
+    z* partn = one ? &S.part : a.part + ((j + 1) & 1) * nb;
+    const z* grow = one ? rows + (int64_t)(j + 1) * n : a.G + (int64_t)(j + 1) * n;
     z pc[TRI_VEC], rc[TRI_VEC], vc[TRI_VEC];
-#pragma unroll
-    for (int k = 0; k < TRI_VEC; ++k) {
-      const int64_t c = j + 1 + tid + (int64_t)k * TRI_THREADS;
-      pc[k] = c < n ? __ldcg(pj + c) : zmk(0, 0);
-      rc[k] = c < n ? __ldcg(grow + c) : zmk(0, 0);
-    }
-    const z p1 = __ldcg(pj + j + 1);
-    if (warp == 0) {  // the nb partials, loaded by 32 lanes at once and summed by shuffles
+    z p1 = zmk(0, 0);
+    if (scalar) {  // the group's partial sums, by 32 lanes at once
       double sa = 0, sb = 0;
       for (int q = lane; q < nb; q += 32) {
-        const z pq = __ldcg(partj + q);
+        const z pq = one ? partj[q] : __ldcg(partj + q);
         sa += pq.x;
         sb += pq.y;
       }
@@ -568,226 +680,143 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tridiag_rows(TriArgs a) {
         const z ts = zmul(rf.tau, zmk(sa, sb));
         S.cf = zmk(-0.5 * ts.x, -0.5 * ts.y);
       }
-    }
+    } else {
 #pragma unroll
-    for (int k = 0; k < TRI_VEC; ++k) {  // v_j, written out for the back-transformation
-      const int64_t c = j + 1 + tid + (int64_t)k * TRI_THREADS;
-      if (c < n) {
-        vc[k] = (c == j + 1) ? zmk(1, 0) : zmul(zconj(sx[c]), rf.scale);
-        sv[c] = vc[k];
-        if (b == 0) a.Hv[j * n + (c - j - 1)] = vc[k];
+      for (int k = 0; k < TRI_VEC; ++k) {
+        const int c = j + 1 + tid + k * TRI_THREADS;
+        pc[k] = rc[k] = zmk(0, 0);
+        if (c < n) {
+          pc[k] = one ? pj[c] : __ldcg(pj + c);
+          rc[k] = one ? grow[c] : __ldcg(grow + c);
+        }
       }
-    }
-    __syncthreads();
-    const z cf = S.cf;
-    const z w1 = zmk(p1.x + cf.x, p1.y + cf.y);  // w_j(j+1), as v_j(j+1) = 1
-    double acc = 0;
-    double d1 = 0;
+      p1 = one ? pj[j + 1] : __ldcg(pj + j + 1);
 #pragma unroll
-    for (int k = 0; k < TRI_VEC; ++k) {
-      const int64_t c = j + 1 + tid + (int64_t)k * TRI_THREADS;
-      if (c < n) {
-        const z vv = vc[k];
-        const z wv = zmk(fma(cf.x, vv.x, fma(-cf.y, vv.y, pc[k].x)),
-                         fma(cf.x, vv.y, fma(cf.y, vv.x, pc[k].y)));
-        sw[c] = wv;
-        z xn = zmk(rc[k].x - wv.x, rc[k].y + wv.y);
-        zsub_mul_conj(xn, w1, vv);
-        if (c == j + 1) {
-          d1 = xn.x;
-        } else if (c == j + 2) {
-          S.alpha = zconj(xn);
-          sx[c] = zmk(0, 0);
-        } else {
-          acc = fma(xn.x, xn.x, fma(xn.y, xn.y, acc));
-          sx[c] = xn;
+      for (int k = 0; k < TRI_VEC; ++k) {  // v_j, written out for the back-transformation
+        const int c = j + 1 + tid + k * TRI_THREADS;
+        if (c < n) {
+          vc[k] = (c == j + 1) ? zmk(1, 0) : zmul(zconj(sx[c]), rf.scale);
+          sv[c] = vc[k];
+          if (b == 0) a.G[(int64_t)j * n + (c - j - 1)] = vc[k];
         }
       }
     }
-    acc = warp_sum_d(acc);
-    if (lane == 0) S.nrm[warp] = acc;
     __syncthreads();
-    rows_update<true>(rows, R, b, nb, n, j + 2, sv, sw, sx, a.G + (j + 2) * n, S);
-    __syncthreads();
-    if (warp == 0) {
-      const int64_t m2 = n - j - 2;  // length of reflector j+1
-      rows_finish(rows, R, b, nb, n, j + 2, sx, m2 <= 0, pn, partn + b, S);
-      if (b == 0 && lane == 0) {  // thread 0 holds column j+1
-        a.tau[j + 1] = S.rf.tau;
-        a.d[j + 1] = d1;
-        if (m2 > 0) a.e[j + 1] = S.rf.beta;
+    double d1 = 0;
+    if (!scalar) {
+      const z cf = S.cf;
+      const z w1 = zmk(p1.x + cf.x, p1.y + cf.y);  // w_j(j+1), as v_j(j+1) = 1
+      double acc = 0;
+#pragma unroll
+      for (int k = 0; k < TRI_VEC; ++k) {
+        const int c = j + 1 + tid + k * TRI_THREADS;
+        if (c < n) {
+          const z vv = vc[k];
+          const z wv = zmk(fma(cf.x, vv.x, fma(-cf.y, vv.y, pc[k].x)),
+                           fma(cf.x, vv.y, fma(cf.y, vv.x, pc[k].y)));
+          sw[c] = wv;
+          z xn = zmk(rc[k].x - wv.x, rc[k].y + wv.y);
+          zsub_mul_conj(xn, w1, vv);
+          if (c == j + 1) {
+            d1 = xn.x;
+          } else if (c == j + 2) {
+            S.alpha = zconj(xn);
+            sx[c] = zmk(0, 0);
+          } else {
+            acc = fma(xn.x, xn.x, fma(xn.y, xn.y, acc));
+            sx[c] = xn;
+          }
+        }
       }
+      acc = warp_sum_d(acc);
+      if (lane == 0) S.nrm[warp] = acc;
+      if (b == 0 && tid == 0) a.d[j + 1] = d1;  // thread 0 holds column j+1
     }
+    __syncthreads();
+    const bool empty = n - j - 2 <= 0;  // length of reflector j+1
+    if (scalar) {
+      double nr = lane < TRI_WARPS ? S.nrm[lane] : 0.0;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
+      nr = __shfl_sync(0xffffffffu, nr, 0);
+      const Refl r2 = refl_warp(empty ? zmk(0, 0) : S.alpha, nr, empty);
+      if (lane == 0) {
+        S.rf[(j + 1) & 1] = r2;
+        if (b == 0) {
+          a.tau[j + 1] = r2.tau;
+          if (!empty) a.e[j + 1] = r2.beta;
+        }
+      }
+    } else {
+      rows_update<true>(rows, R, b, nb, n, j + 2, sv, sw, sx, one ? nullptr : a.G + (int64_t)(j + 2) * n, S);
+    }
+    __syncthreads();
+    if (warp == 0) rows_finish(rows, R, b, nb, n, j + 2, sx, S.rf[(j + 1) & 1], pn, partn + (one ? 0 : b), S);
   }
 }
 
-// ---------------------------------------------------------------- one block per CTA
-// The same Householder reduction for many small Hermitian blocks (the charge blocks of a
-// truncated SVD), one CTA per block and all blocks in one launch: no grid barrier, the
-// block (<= TRI_CTA_MAX rows) stays in L2 and the reflector and p live in shared memory.
-// On GB300 an SM retires two FP64 FMAs per clock, so a 115-row block takes about a
-// millisecond on its SM while the others reduce the other blocks.  Reflector j is kept in
-// row j of the block itself (columns 0..m-1), the layout the back-transformation reads:
-// after column j is eliminated, row j is read no more.
-constexpr int TRI_CTA_MAX = 256;
-constexpr int TRI_CTA_THREADS = 256;
-
-struct CtaBlk {
-  int64_t goff;  // block (row-major, n x n) offset in the Gram buffer
-  int64_t off;   // offset of its d, e, tau
+// Reflectors as the columns of V: column i of a panel starting at reflector j0 is element
+// (rho, i) = Hv[j0 n + i (n - 1) + rho], which for rho < i falls in the part of row j0 + i - 1
+// right of its reflector.  That part is zeroed here, and so is a reflector with tau = 0.
+struct CleanBlk {
+  z* G;
+  z* tau;  // a zero becomes 1 (the inverse of T's diagonal entry)
   int n;
 };
-
-// Rows g >= lo of A (one warp per row): with UPD, T(g, c) -= v(g) conj(w(c)) + w(g) conj(v(c))
-// for c >= lo; p(g) = tq sum_{c >= lo} T(g, c) q(c); each warp's sum of conj(p(g)) q(g) to
-// s_part[.][warp].
-template <bool UPD>
-__device__ void cta_rows_pass(z* A, int64_t n, int64_t lo, const z* v, const z* w, const z* q,
-                              z tq, z* p, double (*s_part)[TRI_CTA_THREADS / 32]) {
-  constexpr int NW = TRI_CTA_THREADS / 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double pr = 0, pi = 0;
-  for (int64_t g = lo + warp; g < n; g += NW) {
-    z* row = A + g * n;
-    z vr = zmk(0, 0), wr = zmk(0, 0);
-    if (UPD) {
-      vr = v[g];
-      wr = w[g];
-    }
-    double sr = 0, si = 0;
-    for (int64_t c = lo + lane; c < n; c += 32) {
-      z x = row[c];
-      if (UPD) {
-        zsub_mul_conj(x, vr, w[c]);
-        zsub_mul_conj(x, wr, v[c]);
-        row[c] = x;
-      }
-      const z y = q[c];
-      sr = fma(x.x, y.x, fma(-x.y, y.y, sr));
-      si = fma(x.x, y.y, fma(x.y, y.x, si));
-    }
-    sr = warp_sum_d(sr);
-    si = warp_sum_d(si);
-    if (lane == 0) {
-      const z pv = zmul(tq, zmk(sr, si));
-      p[g] = pv;
-      const z qq = q[g];
-      pr += pv.x * qq.x + pv.y * qq.y;
-      pi += pv.x * qq.y - pv.y * qq.x;
-    }
-  }
-  if (lane == 0) {
-    s_part[0][warp] = pr;
-    s_part[1][warp] = pi;
+struct CleanGroup {
+  int nblk;
+  CleanBlk b[TRI_MAXB];
+};
+__global__ void __launch_bounds__(256) k_clean_reflectors(const __grid_constant__ CleanGroup T) {
+  const CleanBlk& a = T.b[blockIdx.y];
+  for (int j = blockIdx.x; j + 1 < a.n; j += gridDim.x) {
+    const z t = a.tau[j];
+    const bool none = t.x == 0.0 && t.y == 0.0;
+    z* row = a.G + (int64_t)j * a.n;
+    for (int c = (none ? 0 : a.n - j - 1) + threadIdx.x; c < a.n; c += 256) row[c] = zmk(0, 0);
+    __syncthreads();
+    if (none && threadIdx.x == 0) a.tau[j] = zmk(1, 0);
   }
 }
 
-// Column j: entering, v_j and p_j = tau_j T_j v_j are in shared memory with the warps'
-// partial sums of p_j^H v_j.  One pass over the columns c > j gives w_j and row j+1 after
-// the update (x), whose entries past j+1 give reflector j+1 (stored in row j+1 of the
-// block, which is read no more); then one pass over the rows g > j+1 updates them and
-// forms p_{j+1} (the trailing block is read and written once per column).  Vectors are
-// indexed by row of the block; one entry per thread (n <= TRI_CTA_MAX = threads).
-__global__ void __launch_bounds__(TRI_CTA_THREADS) k_tridiag_cta(z* __restrict__ G,
-                                                                 const CtaBlk* __restrict__ blks,
-                                                                 double* __restrict__ dAll,
-                                                                 double* __restrict__ eAll,
-                                                                 z* __restrict__ tauAll) {
-  constexpr int NW = TRI_CTA_THREADS / 32;
-  __shared__ z s_v[TRI_CTA_MAX], s_v2[TRI_CTA_MAX], s_w[TRI_CTA_MAX], s_p[TRI_CTA_MAX];
-  __shared__ double sh[32];
-  __shared__ double s_part[2][NW];
-  __shared__ z s_cf, s_alpha;
-  __shared__ Refl s_refl;
-  const CtaBlk B = blks[blockIdx.x];
-  const int64_t n = B.n;
-  z* A = G + B.goff;
-  double* d = dAll + B.off;
-  double* e = eAll + B.off;
-  z* tau = tauAll + B.off;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  z* v = s_v;
-  z* v2 = s_v2;
-  z t;
-  {  // reflector 0 from row 0 (thread tid holds column 1 + tid), kept in row 0
-    const int64_t c = 1 + tid;
-    const z x = c < n ? A[c] : zmk(0, 0);
-    double acc = (c >= 2 && c < n) ? fma(x.x, x.x, x.y * x.y) : 0.0;
-    acc = block_sum0(acc, sh);
-    if (tid == 0) {
-      const Refl rf = refl_params(zconj(x), acc, n < 2);
-      s_refl = rf;
-      tau[0] = rf.tau;
-      d[0] = A[0].x;
-      if (n > 1) e[0] = rf.beta;
-    }
+// T of a panel of reflectors, H_0 ... H_{b-1} = I - V T V^H: T^-1 is the strict upper triangle
+// of V^H V plus diag(1 / tau).  One CTA per diagonal sub-block of up to WY_SUB reflectors,
+// four threads per column of T: T(i, i) = tau_i, then T(r, i) = -tau_r sum_q S(r, q) T(q, i)
+// upwards.  The off-diagonal blocks, -T_1 S_12 T_2, come from products (32 -> 64 -> 128).
+constexpr int WY_SUB = 32, WY_PANEL = 4 * WY_SUB;
+struct WySub {
+  const z* S;   // the sub-block's diagonal block of V^H V
+  const z* tau;
+  z* T;         // zero before
+  int n, ld;
+};
+__global__ void __launch_bounds__(4 * WY_SUB) k_wy_t(const WySub* __restrict__ subs) {
+  __shared__ z s_t[WY_SUB][WY_SUB + 1];  // column i in s_t[i]
+  const WySub a = subs[blockIdx.x];
+  const int i = threadIdx.x >> 2, part = threadIdx.x & 3;
+  if (part == 0 && i < a.n) s_t[i][i] = a.tau[i];
+  for (int r = a.n - 2; r >= 0; --r) {
     __syncthreads();
-    const Refl rf = s_refl;
-    t = rf.tau;
-    if (c < n) {
-      const z vc = (c == 1) ? zmk(1, 0) : zmul(zconj(x), rf.scale);
-      v[c] = vc;
-      A[c - 1] = vc;
-    }
-    __syncthreads();
-    cta_rows_pass<false>(A, n, 1, v, s_w, v, t, s_p, s_part);
-  }
-  for (int64_t j = 0; j + 1 < n; ++j) {
-    __syncthreads();
-    const int64_t c = j + 1 + tid;
-    z pc = zmk(0, 0), rc = zmk(0, 0);
-    if (c < n) {
-      pc = s_p[c];
-      rc = A[(j + 1) * n + c];
-    }
-    const z p1 = s_p[j + 1];
-    if (warp == 0) {
-      double sa = lane < NW ? s_part[0][lane] : 0.0;
-      double sb = lane < NW ? s_part[1][lane] : 0.0;
-      sa = warp_sum_d(sa);
-      sb = warp_sum_d(sb);
-      if (lane == 0) {
-        const z ts = zmul(t, zmk(sa, sb));
-        s_cf = zmk(-0.5 * ts.x, -0.5 * ts.y);
+    double sr = 0, si = 0;
+    if (i > r && i < a.n)
+      for (int q = r + 1 + part; q <= i; q += 4) {
+        const z s = a.S[(int64_t)r * a.ld + q], t = s_t[i][q];
+        sr = fma(s.x, t.x, fma(-s.y, t.y, sr));
+        si = fma(s.x, t.y, fma(s.y, t.x, si));
       }
+#pragma unroll
+    for (int o = 1; o <= 2; o <<= 1) {
+      sr += __shfl_xor_sync(0xffffffffu, sr, o);
+      si += __shfl_xor_sync(0xffffffffu, si, o);
     }
-    __syncthreads();
-    const z cf = s_cf;
-    const z w1 = zmk(p1.x + cf.x, p1.y + cf.y);  // w_j(j+1), as v_j(j+1) = 1
-    z x = zmk(0, 0);
-    double acc = 0;
-    if (c < n) {
-      const z vv = v[c];
-      const z wv = zmk(fma(cf.x, vv.x, fma(-cf.y, vv.y, pc.x)), fma(cf.x, vv.y, fma(cf.y, vv.x, pc.y)));
-      s_w[c] = wv;
-      x = zmk(rc.x - wv.x, rc.y + wv.y);
-      zsub_mul_conj(x, w1, vv);
-      if (c >= j + 3) acc = fma(x.x, x.x, x.y * x.y);
-      if (c == j + 2) s_alpha = zconj(x);
+    if (part == 0 && i > r && i < a.n) {
+      const z t = a.tau[r];
+      s_t[i][r] = zmk(fma(-t.x, sr, t.y * si), fma(-t.x, si, -t.y * sr));
     }
-    acc = block_sum0(acc, sh);
-    const int64_t m2 = n - j - 2;
-    if (tid == 0) {  // thread 0 holds column j+1
-      const Refl rf = refl_params(m2 > 0 ? s_alpha : zmk(0, 0), acc, m2 <= 0);
-      s_refl = rf;
-      tau[j + 1] = rf.tau;
-      d[j + 1] = x.x;
-      if (m2 > 0) e[j + 1] = rf.beta;
-    }
-    __syncthreads();
-    const Refl rf = s_refl;
-    if (c >= j + 2 && c < n) {
-      const z vc = (c == j + 2) ? zmk(1, 0) : zmul(zconj(x), rf.scale);
-      v2[c] = vc;
-      A[(j + 1) * n + (c - j - 2)] = vc;
-    }
-    __syncthreads();
-    cta_rows_pass<true>(A, n, j + 2, v, s_w, v2, rf.tau, s_p, s_part);
-    z* tmp = v;
-    v = v2;
-    v2 = tmp;
-    t = rf.tau;
   }
+  __syncthreads();
+  if (i < a.n)
+    for (int r = part; r <= i; r += 4) a.T[(int64_t)r * a.ld + i] = s_t[i][r];
 }
 
 // Number of eigenvalues of T below x from the signs of the leading principal minors
@@ -1191,54 +1220,32 @@ __global__ void __launch_bounds__(256) k_backtransform(const double* __restrict_
     for (int64_t r = threadIdx.x; r < n; r += blockDim.x) U[r * k + i0 + q] = y[q * n + r];
 }
 
-// Small complex GEMMs of many problems in one launch (the Newton-Schulz steps of the
-// eigen phase): task t computes C = op(A) B, op(A)(i, l) = A[i a_rs + l a_cs] (conjugated
-// if conj_a), B(l, j) = B[l b_rs + j b_cs], C(i, j) = C[i c_rs + j]; one 16 x 16 output
-// tile per CTA iteration, tiles[g] = (task, m0, n0).  coef != 0 instead writes
-// C = 1.5 I - 0.5 op(A) B (the Newton-Schulz coefficient matrix).
-struct NsTask {
-  int64_t M, N, K;
-  const z* A;
-  int64_t a_rs, a_cs;
-  const z* B;
-  int64_t b_rs, b_cs;
-  z* C;
-  int64_t c_rs;
-  int conj_a, coef;
-};
-__global__ void __launch_bounds__(256) k_gemm_tasks(const NsTask* __restrict__ tasks,
-                                                    const int4* __restrict__ tiles, int ntiles) {
-  __shared__ z As[16][17];
-  __shared__ z Bs[16][17];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const int4 tl = tiles[t];
-    const NsTask tk = tasks[tl.x];
-    z acc = zmk(0, 0);
-    for (int64_t k0 = 0; k0 < tk.K; k0 += 16) {
-      {
-        const int64_t gi = tl.y + ty, gk = k0 + tx;
-        z v = (gi < tk.M && gk < tk.K) ? tk.A[gi * tk.a_rs + gk * tk.a_cs] : zmk(0, 0);
-        if (tk.conj_a) v.y = -v.y;
-        As[ty][tx] = v;
-      }
-      {
-        const int64_t gk = k0 + ty, gj = tl.z + tx;
-        Bs[ty][tx] = (gj < tk.N && gk < tk.K) ? tk.B[gk * tk.b_rs + gj * tk.b_cs] : zmk(0, 0);
-      }
-      __syncthreads();
-#pragma unroll
-      for (int kk = 0; kk < 16; ++kk) zfma(acc, As[ty][kk], Bs[kk][tx]);
-      __syncthreads();
-    }
-    const int64_t gi = tl.y + ty, gj = tl.z + tx;
-    if (gi < tk.M && gj < tk.N) {
-      if (tk.coef) {
-        acc = zscale(acc, -0.5);
-        if (gi == gj) acc.x += 1.5;
-      }
-      tk.C[gi * tk.c_rs + gj] = acc;
-    }
+// per eigenproblem: U0 (n x k) = Y as complex numbers (U0 at Y's offset)
+__global__ void __launch_bounds__(256) k_complex_cols(const double* __restrict__ YAll, const EBlk* __restrict__ blks,
+                                                      z* __restrict__ U0All) {
+  __shared__ double s[32][33];
+  const EBlk B = blks[blockIdx.y];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int64_t nt = (B.n + 31) / 32, kt = (B.k + 31) / 32;
+  for (int64_t w = blockIdx.x; w < nt * kt; w += gridDim.x) {
+    const int64_t r0 = (w % nt) * 32, i0 = (w / nt) * 32;
+    for (int q = ty; q < 32; q += 8)
+      if (i0 + q < B.k && r0 + tx < B.n) s[q][tx] = YAll[B.yo + (i0 + q) * B.n + r0 + tx];
+    __syncthreads();
+    for (int q = ty; q < 32; q += 8)
+      if (r0 + q < B.n && i0 + tx < B.k) U0All[B.yo + (r0 + q) * B.k + i0 + tx] = zmk(s[tx][q], 0);
+    __syncthreads();
+  }
+}
+
+// S <- 1.5 I - 0.5 S for every problem's k x k block (at so[problem])
+__global__ void k_ns_coef_all(z* __restrict__ SAll, const EBlk* __restrict__ blks, const int64_t* __restrict__ so) {
+  const int64_t k = blks[blockIdx.y].k;
+  z* S = SAll + so[blockIdx.y];
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < k * k; e += (int64_t)gridDim.x * blockDim.x) {
+    z v = zscale(S[e], -0.5);
+    if (e / k == e % k) v.x += 1.5;
+    S[e] = v;
   }
 }
 
@@ -1387,42 +1394,24 @@ int heig_top(Ctx* c, z* G, int64_t n, int64_t k, z* U, int64_t ldu, double* ev) 
     // multiply-add, two rank-2 updates of the trailing block and its matrix-vector product)
     ProfScope ps(c, "heig_tridiag", 16.0 / 3.0 * nn * nn * nn);
     const size_t tri_smem = 4 * TRI_CACHE * sizeof(z);
-    static int nsm = 0, occ = 0, rows_dyn_max = 0;
+    static int nsm = 0, occ = 0;
     if (!nsm) {
+      int v = 0;
       TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_tridiag_persistent,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri_smem));
-      TNT_CUDA_TRY(c, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
+      TNT_CUDA_TRY(c, cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, c->device));
       TNT_CUDA_TRY(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tridiag_persistent,
                                                                     TRI_THREADS, tri_smem));
-      int optin = 0;
-      cudaFuncAttributes fa{};
-      TNT_CUDA_TRY(c, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
-      TNT_CUDA_TRY(c, cudaFuncGetAttributes(&fa, k_tridiag_rows));
-      rows_dyn_max = optin - (int)fa.sharedSizeBytes;
-      TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_tridiag_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           rows_dyn_max));
+      nsm = v;
     }
     if (occ < 1) return set_err(c, TNT_E_UNSUPPORTED, "tridiagonal kernel cannot be resident");
     TNT_CUDA_TRY(c, cudaMemsetAsync(bar, 0, 256, st));
     TriArgs ta{G, n, Hv, tau, d, e, p, part, (unsigned*)bar, (int*)(bar + 16), c->d_status,
                gws};
     void* args[] = {&ta};
-    // rows resident in shared memory when each block's share and the three vectors fit
-    const int nbr = (int)std::min<int64_t>(std::min(nsm, TRI_MAX_BLOCKS), n);
-    const int64_t rmax = (n + nbr - 1) / nbr;
-    const size_t rows_smem = (size_t)(rmax + 3) * n * sizeof(z);
-    int occ_rows = 0;
-    if (n <= TRI_ROWS_NMAX && rmax <= TRI_ROWS_MAX && rows_smem <= (size_t)rows_dyn_max)
-      TNT_CUDA_TRY(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_rows, k_tridiag_rows,
-                                                                    TRI_THREADS, rows_smem));
-    if (occ_rows >= 1) {
-      TNT_CUDA_TRY(c, cudaLaunchCooperativeKernel((void*)k_tridiag_rows, dim3(nbr),
-                                                  dim3(TRI_THREADS), args, rows_smem, st));
-    } else {
-      const int nb = std::min(nsm, TRI_MAX_BLOCKS);
-      TNT_CUDA_TRY(c, cudaLaunchCooperativeKernel((void*)k_tridiag_persistent, dim3(nb),
-                                                  dim3(TRI_THREADS), args, tri_smem, st));
-    }
+    const int nb = std::min(nsm, TRI_MAX_BLOCKS);
+    TNT_CUDA_TRY(c, cudaLaunchCooperativeKernel((void*)k_tridiag_persistent, dim3(nb),
+                                                dim3(TRI_THREADS), args, tri_smem, st));
     c->launches += 1;
   }
   {
@@ -1440,46 +1429,226 @@ int heig_top(Ctx* c, z* G, int64_t n, int64_t k, z* U, int64_t ldu, double* ev) 
   return r;
 }
 
-// Many small blocks (n <= 256 each): every stage of the eigensolve is one launch over all
-// blocks.  blocks[i] = {offset of the n x n block in G (and of its eigenvector columns in
-// U, leading dimension n), n, k}; the reduction keeps the reflectors in the blocks' rows.
-// ev (device) receives the eigenvalues of all blocks back to back.
-int heig_small_blocks(Ctx* c, z* G, const std::vector<SmallEig>& blocks, z* U, double* ev) {
+namespace {
+// CTAs of each block's group (in the order of `n`, descending) for one launch on nsm SMs of
+// smem bytes: the shortest common time by the model
+//   t(n, nb) = n t_col + (2 n^3 / nb + 4 n^2) / f,
+// 12 FP64 operations per trailing entry of a CTA's rows and 16 per entry of its vectors at two
+// per SM and clock, and a column's latency t_col (barrier, loads, scalars: 2.5 us in a group
+// of one CTA, 6 us with a barrier).  Returns how many of the blocks fit the launch.
+int tri_deal(const std::vector<int64_t>& n, int nsm, size_t smem, std::vector<int>* nb) {
+  auto fits = [&](int64_t m, int64_t q) {
+    const int64_t rows = (m + q - 1) / q;
+    return rows <= TRI_RMAX && (size_t)(rows + 3 + (q == 1)) * m * sizeof(z) <= smem;
+  };
+  auto time = [](double m, double q) { return m * (q > 1 ? 6.0 : 2.5) + (2.0 * m * m * m / q + 4.0 * m * m) / 2070.0; };
+  std::vector<int> lo;
+  int used = 0;
+  for (int64_t m : n) {  // the least group that holds each block
+    int q = 1;
+    while (q < m && !fits(m, q)) ++q;
+    if (!fits(m, q) || used + q > nsm || (int)lo.size() == TRI_MAXB) break;
+    lo.push_back(q);
+    used += q;
+  }
+  const int cnt = (int)lo.size();
+  // more CTAs to the block that takes longest, as long as that shortens it
+  std::vector<int> q = lo;
+  while (cnt > 0) {
+    int w = 0;
+    for (int i = 1; i < cnt; ++i)
+      if (time((double)n[(size_t)i], q[(size_t)i]) > time((double)n[(size_t)w], q[(size_t)w])) w = i;
+    const double m = (double)n[(size_t)w], now = time(m, q[(size_t)w]);
+    // the next size worth having: a second CTA brings the barrier's cost with it
+    int next = q[(size_t)w] + 1;
+    while (next - q[(size_t)w] <= nsm - used && next < (int)m && time(m, next) >= now) ++next;
+    if (next - q[(size_t)w] > nsm - used || next > (int)m || time(m, next) >= now) break;
+    used += next - q[(size_t)w];
+    q[(size_t)w] = next;
+  }
+  *nb = q;
+  return cnt;
+}
+}  // namespace
+
+// Above this many rows the panels' products are the faster back-transformation: a set of
+// grouped products costs about 35 us, so a 128-reflector panel about 70 and the T factors
+// 150 in all, where the one-CTA form takes about 2.5 us per reflector (two vectors a CTA:
+// 200 rows 0.5 ms, 500 rows 2.2 ms, 1024 rows and 256 vectors 5.6 ms).
+constexpr int64_t WY_MIN = 192;
+
+// U0 <- H_0 ... H_{n-2} Y for the first nl blocks, by panels of WY_PANEL reflectors:
+// U0 <- (I - V T V^H) U0 from the last panel to the first, all blocks' panels of one index
+// together.  V is read from the reflector rows through its strides (k_clean_reflectors).
+static int wy_backtransform(Ctx* c, z* G, const std::vector<SmallEig>& blocks, int nl, const std::vector<EBlk>& he,
+                            const std::vector<int64_t>& po, const std::vector<int64_t>& vo,
+                            const std::vector<int64_t>& wo, int64_t npan, z* tau, const EBlk* dblk,
+                            const WySub* dsub, int nsub, const double* Y, z* U0, z* PS, z* PT, z* PX, z* VT, z* W) {
+  cudaStream_t st = c->stream;
+  const size_t pp = (size_t)WY_PANEL * WY_PANEL;
+  for (int i0 = 0; i0 < nl; i0 += TRI_MAXB) {
+    CleanGroup T;
+    T.nblk = std::min(TRI_MAXB, nl - i0);
+    for (int i = 0; i < T.nblk; ++i) {
+      const SmallEig& b = blocks[(size_t)(i0 + i)];
+      T.b[i] = CleanBlk{G + b.goff, tau + he[(size_t)(i0 + i)].off, (int)b.n};
+    }
+    k_clean_reflectors<<<dim3(64, (unsigned)T.nblk), 256, 0, st>>>(T);
+    c->launches++;
+  }
+  k_complex_cols<<<dim3(64, (unsigned)nl), 256, 0, st>>>(Y, dblk, U0);
+  TNT_CUDA_TRY(c, cudaMemsetAsync(PT, 0, sizeof(z) * pp * (size_t)npan, st));
+  c->launches++;
+  auto task = [](int64_t M, int64_t N, int64_t K, const z* A, int64_t a_rs, int64_t a_cs, int conj_a, const z* B,
+                 int64_t b_rs, z* C, int64_t c_rs, int herm, int sub) {
+    GemmTask t{};
+    t.g.batch = 1;
+    t.g.alpha = zmk(1, 0);
+    t.g.M = M; t.g.N = N; t.g.K = K;
+    t.g.A = A; t.g.a_rs = a_rs; t.g.a_cs = a_cs; t.g.conj_a = conj_a;
+    t.g.B = B; t.g.b_rs = b_rs; t.g.b_cs = 1;
+    t.g.C = C; t.g.c_rs = c_rs;
+    t.herm = herm; t.sub = sub;
+    return t;
+  };
+  struct Panel {
+    int blk;
+    int64_t j0, b, m, s;
+  };
+  std::vector<Panel> pan;
+  int64_t steps = 0;
+  for (int i = 0; i < nl; ++i)
+    for (int64_t j0 = 0, s = 0; j0 < blocks[(size_t)i].n - 1; j0 += WY_PANEL, ++s) {
+      const int64_t n = blocks[(size_t)i].n;
+      pan.push_back(Panel{i, j0, std::min<int64_t>(WY_PANEL, n - 1 - j0), n - 1 - j0, s});
+      steps = std::max(steps, s + 1);
+    }
+  std::vector<GemmTask> t;
+  for (const Panel& q : pan) {  // V^H V
+    const SmallEig& b = blocks[(size_t)q.blk];
+    const z* V = G + b.goff + q.j0 * b.n;
+    GemmTask g = task(q.b, q.b, q.m, V, b.n - 1, 1, 1, V, 1, PS + pp * (size_t)(po[(size_t)q.blk] + q.s), WY_PANEL, 1, 0);
+    g.g.b_cs = b.n - 1;
+    t.push_back(g);
+  }
+  TNT_TRY(zgemm_tasks(c, t));
+  k_wy_t<<<(unsigned)nsub, 4 * WY_SUB, 0, st>>>(dsub);
+  c->launches++;
+  for (int64_t h = WY_SUB; h < WY_PANEL; h *= 2) {  // off-diagonal blocks of T, -T_1 (S_12 T_2)
+    std::vector<GemmTask> ta, tb;
+    for (const Panel& q : pan) {
+      const size_t o = pp * (size_t)(po[(size_t)q.blk] + q.s);
+      for (int64_t r = 0; r + h < q.b; r += 2 * h) {
+        const int64_t n2 = std::min(h, q.b - r - h);
+        const size_t d12 = o + (size_t)(r * WY_PANEL + r + h), d11 = o + (size_t)(r * (WY_PANEL + 1)),
+                     d22 = o + (size_t)((r + h) * (WY_PANEL + 1));
+        ta.push_back(task(h, n2, n2, PS + d12, WY_PANEL, 1, 0, PT + d22, WY_PANEL, PX + d12, WY_PANEL, 0, 0));
+        tb.push_back(task(h, n2, h, PT + d11, WY_PANEL, 1, 0, PX + d12, WY_PANEL, PT + d12, WY_PANEL, 0, 1));
+      }
+    }
+    TNT_TRY(zgemm_tasks(c, ta));
+    TNT_TRY(zgemm_tasks(c, tb));
+  }
+  t.clear();
+  for (const Panel& q : pan) {  // V T (m x b, at the panel's columns of the block's n x n area)
+    const SmallEig& b = blocks[(size_t)q.blk];
+    GemmTask g = task(q.m, q.b, q.b, G + b.goff + q.j0 * b.n, 1, b.n - 1, 0,
+                      PT + pp * (size_t)(po[(size_t)q.blk] + q.s), WY_PANEL, VT + vo[(size_t)q.blk] + q.j0, b.n, 0, 0);
+    t.push_back(g);
+  }
+  TNT_TRY(zgemm_tasks(c, t));
+  for (int64_t s = steps - 1; s >= 0; --s) {
+    std::vector<GemmTask> ta, tb;
+    for (const Panel& q : pan) {
+      if (q.s != s) continue;
+      const SmallEig& b = blocks[(size_t)q.blk];
+      z* Us = U0 + he[(size_t)q.blk].yo + (q.j0 + 1) * b.k;
+      z* Wq = W + wo[(size_t)q.blk];
+      ta.push_back(task(q.b, b.k, q.m, G + b.goff + q.j0 * b.n, b.n - 1, 1, 1, Us, b.k, Wq, b.k, 0, 0));
+      tb.push_back(task(q.m, b.k, q.b, VT + vo[(size_t)q.blk] + q.j0, b.n, 1, 0, Wq, b.k, Us, b.k, 0, 1));
+    }
+    TNT_TRY(zgemm_tasks(c, ta));
+    TNT_TRY(zgemm_tasks(c, tb));
+  }
+  return TNT_OK;
+}
+
+size_t heig_blocks_scratch(int64_t n, int64_t k) {
+  const size_t nn = (size_t)n, kk = (size_t)k;
+  return sizeof(z) * (nn * nn + 2 * nn * kk + kk * kk + 5 * (nn + WY_PANEL) * WY_PANEL + WY_PANEL * kk) +
+         sizeof(double) * 7 * nn * kk + 64 * (2 * nn + 4096) + 256 * nn + (size_t)(2 << 20);
+}
+
+// Eigenvectors of the k largest eigenvalues of many Hermitian blocks: every stage of the
+// eigensolve is one launch (or a few) over all blocks of up to TRI_ROWS_NMAX rows.
+// blocks[i] = {offset of the n x n block in G (and of its eigenvector columns in U, leading
+// dimension n), n, k}; the reflectors replace the blocks' rows.  ev (device) receives
+// the eigenvalues of all blocks back to back.
+int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& all, z* U, double* ev) {
+  if (all.empty()) return TNT_OK;
+  const size_t top = c->ws.top;
+  cudaStream_t st = c->stream;
+  std::vector<SmallEig> blocks;
+  for (const SmallEig& b : all) {
+    if (b.n < 1 || b.k < 1 || b.k > b.n)
+      return set_err(c, TNT_E_INVALID, "eigensolve block n=%lld k=%lld", (long long)b.n, (long long)b.k);
+    if (b.n <= TRI_ROWS_NMAX) {
+      blocks.push_back(b);
+      continue;
+    }
+    TNT_TRY(heig_top(c, G + b.goff, b.n, b.k, U + b.goff, b.n, ev));
+    ev += b.k;
+  }
   if (blocks.empty()) return TNT_OK;
-  int64_t tot = 0, kt = 0, nk = 0, k2 = 0, nmax = 0;
-  for (const SmallEig& b : blocks) {
-    if (b.n < 1 || b.n > TRI_CTA_MAX || b.k < 1 || b.k > b.n)
-      return set_err(c, TNT_E_INVALID, "small eigensolve block n=%lld k=%lld", (long long)b.n, (long long)b.k);
+  std::stable_sort(blocks.begin(), blocks.end(), [](const SmallEig& a, const SmallEig& b) { return a.n > b.n; });
+  const int nb = (int)blocks.size();
+  static int nsm = 0;
+  static size_t smem_max = 0;
+  if (!nsm) {
+    int v = 0, optin = 0;
+    cudaFuncAttributes fa{};
+    TNT_CUDA_TRY(c, cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, c->device));
+    TNT_CUDA_TRY(c, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
+    TNT_CUDA_TRY(c, cudaFuncGetAttributes(&fa, k_tridiag_group));
+    smem_max = (size_t)optin - fa.sharedSizeBytes;
+    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_tridiag_group, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
+    nsm = v;
+  }
+  // large blocks (the first nl): back-transformation by panels of reflectors
+  int nl = 0;
+  while (nl < nb && blocks[(size_t)nl].n > WY_MIN) ++nl;
+  int64_t tot = 0, nk = 0, k2 = 0, nn = 0, npan = 0, kt = 0, kw = 0;
+  std::vector<EBlk> he((size_t)nb);
+  std::vector<int64_t> so((size_t)nb), vo((size_t)nb), po((size_t)nb), wo2((size_t)nb);
+  std::vector<int2> heig, hbt;
+  const int cols = BT_COLS;
+  for (int i = 0; i < nb; ++i) {
+    const SmallEig& b = blocks[(size_t)i];
+    he[(size_t)i] = EBlk{b.n, b.k, tot, b.goff, kt, nk, 6 * nk};
+    so[(size_t)i] = k2;
+    for (int64_t q = 0; q < b.k; ++q) heig.push_back(make_int2(i, (int)q));
+    if (i >= nl)
+      for (int64_t q = 0; q < b.k; q += cols) hbt.push_back(make_int2(i, (int)q));
     tot += b.n;
     kt += b.k;
     nk += b.n * b.k;
     k2 += b.k * b.k;
-    nmax = std::max(nmax, b.n);
+    if (i < nl) {
+      vo[(size_t)i] = nn;
+      po[(size_t)i] = npan;
+      wo2[(size_t)i] = kw;
+      nn += b.n * b.n;
+      npan += (b.n - 2 + WY_PANEL) / WY_PANEL;
+      kw += WY_PANEL * b.k;
+    }
   }
-  const int nb = (int)blocks.size();
-  const int cols = BT_COLS;  // sizeof(z) * 256 * 2 fits shared memory
-  // host tables: reduction blocks, eigen problems, eigenvalue and back-transformation
-  // indices, and the Newton-Schulz task lists with their 16 x 16 tiles
-  std::vector<CtaBlk> hc((size_t)nb);
-  std::vector<EBlk> he((size_t)nb);
-  std::vector<int2> heig, hbt;
-  int64_t off = 0, evo = 0, yo = 0, wo = 0, so = 0;
-  for (int i = 0; i < nb; ++i) {
-    const SmallEig& b = blocks[(size_t)i];
-    hc[(size_t)i] = CtaBlk{b.goff, off, (int)b.n};
-    he[(size_t)i] = EBlk{b.n, b.k, off, b.goff, evo, yo, wo};
-    for (int64_t q = 0; q < b.k; ++q) heig.push_back(make_int2(i, (int)q));
-    for (int64_t q = 0; q < b.k; q += cols) hbt.push_back(make_int2(i, (int)q));
-    off += b.n;
-    evo += b.k;
-    yo += b.n * b.k;
-    wo += 6 * b.n * b.k;
-    so += b.k * b.k;
-  }
-  const size_t top = c->ws.top;
+  const size_t pp = (size_t)WY_PANEL * WY_PANEL;
   double* d = (double*)ws_alloc(c, ws_round(sizeof(double) * tot));
   double* e = (double*)ws_alloc(c, ws_round(sizeof(double) * tot));
   z* tau = (z*)ws_alloc(c, ws_round(sizeof(z) * tot));
+  z* p = (z*)ws_alloc(c, ws_round(sizeof(z) * 2 * tot));
+  z* part = (z*)ws_alloc(c, ws_round(sizeof(z) * 2 * (size_t)nsm));
+  unsigned* bar = (unsigned*)ws_alloc(c, ws_round(sizeof(unsigned) * 32 * (TRI_MAXB + 1)));
   double* tn = (double*)ws_alloc(c, ws_round(sizeof(double) * nb));
   int64_t* nr = (int64_t*)ws_alloc(c, ws_round(sizeof(int64_t) * nb));
   double* work = (double*)ws_alloc(c, ws_round(sizeof(double) * 6 * nk));
@@ -1487,110 +1656,138 @@ int heig_small_blocks(Ctx* c, z* G, const std::vector<SmallEig>& blocks, z* U, d
   z* U0 = (z*)ws_alloc(c, ws_round(sizeof(z) * nk));
   z* U1 = (z*)ws_alloc(c, ws_round(sizeof(z) * nk));
   z* S = (z*)ws_alloc(c, ws_round(sizeof(z) * k2));
-  CtaBlk* dc = (CtaBlk*)ws_alloc(c, ws_round(sizeof(CtaBlk) * nb));
-  EBlk* dbl = (EBlk*)ws_alloc(c, ws_round(sizeof(EBlk) * nb));
-  int2* deig = (int2*)ws_alloc(c, ws_round(sizeof(int2) * (heig.size() + hbt.size())));
-  NsTask* dtask = (NsTask*)ws_alloc(c, ws_round(sizeof(NsTask) * 4 * nb));
-  // tiles of the four task lists (S = X^H X and X S, twice)
-  std::vector<NsTask> ht;
-  std::vector<int4> htile[4];
-  for (int step = 0; step < 2; ++step) {
-    for (int i = 0; i < nb; ++i) {
-      const SmallEig& b = blocks[(size_t)i];
-      const EBlk& B = he[(size_t)i];
-      z* X = (step == 0 ? U0 : U1) + B.yo;                      // n x k, ld k
-      z* Xn = (step == 0) ? U1 + B.yo : U + b.goff;             // next X
-      const int64_t ldn = (step == 0) ? b.k : b.n;
-      NsTask ts{b.k, b.k, b.n, X, 1, b.k, X, b.k, 1, nullptr, b.k, 1, 1};
-      NsTask tx{b.n, b.k, b.k, X, b.k, 1, nullptr, b.k, 1, Xn, ldn, 0, 0};
-      ht.push_back(ts);
-      ht.push_back(tx);
-    }
-  }
-  {  // S offsets per block
-    int64_t o = 0;
-    for (int i = 0; i < nb; ++i) {
-      const int64_t kb = blocks[(size_t)i].k;
-      for (int step = 0; step < 2; ++step) {
-        ht[(size_t)(step * 2 * nb + 2 * i)].C = S + o;
-        ht[(size_t)(step * 2 * nb + 2 * i + 1)].B = S + o;
+  // panels of the large blocks: V^H V, T, a product's left half, V T and V^H U
+  z* PS = (z*)ws_alloc(c, ws_round(sizeof(z) * pp * (size_t)npan));
+  z* PT = (z*)ws_alloc(c, ws_round(sizeof(z) * pp * (size_t)npan));
+  z* PX = (z*)ws_alloc(c, ws_round(sizeof(z) * pp * (size_t)npan));
+  z* VT = (z*)ws_alloc(c, ws_round(sizeof(z) * (size_t)nn));
+  z* W = (z*)ws_alloc(c, ws_round(sizeof(z) * (size_t)kw));
+  // one upload: problem table, eigenvalue and back-transformation indices, S offsets, T blocks
+  std::vector<WySub> subs;
+  for (int i = 0; i < nl; ++i)
+    for (int64_t j0 = 0, s = 0; j0 < blocks[(size_t)i].n - 1; j0 += WY_PANEL, ++s)
+      for (int64_t q = 0; q < WY_PANEL && j0 + q < blocks[(size_t)i].n - 1; q += WY_SUB) {
+        const size_t o = pp * (size_t)(po[(size_t)i] + s) + (size_t)q * (WY_PANEL + 1);
+        subs.push_back(WySub{PS + o, tau + he[(size_t)i].off + j0 + q, PT + o,
+                             (int)std::min<int64_t>(WY_SUB, blocks[(size_t)i].n - 1 - j0 - q), WY_PANEL});
       }
-      o += kb * kb;
-    }
-  }
-  for (int step = 0; step < 2; ++step)
-    for (int which = 0; which < 2; ++which) {
-      std::vector<int4>& tl = htile[2 * step + which];
-      for (int i = 0; i < nb; ++i) {
-        const int ti = step * 2 * nb + 2 * i + which;
-        const NsTask& t = ht[(size_t)ti];
-        for (int64_t m0 = 0; m0 < t.M; m0 += 16)
-          for (int64_t n0 = 0; n0 < t.N; n0 += 16) tl.push_back(make_int4(ti, (int)m0, (int)n0, 0));
-      }
-    }
-  size_t ntile_all = 0;
-  for (auto& v : htile) ntile_all += v.size();
-  int4* dtile = (int4*)ws_alloc(c, ws_round(sizeof(int4) * ntile_all));
-  if (!d || !e || !tau || !tn || !nr || !work || !Y || !U0 || !U1 || !S || !dc || !dbl || !deig || !dtask || !dtile) {
+  const size_t b_blk = ws_round(sizeof(EBlk) * nb), b_eig = ws_round(sizeof(int2) * heig.size()),
+               b_bt = ws_round(sizeof(int2) * hbt.size()), b_so = ws_round(sizeof(int64_t) * nb),
+               b_sub = ws_round(sizeof(WySub) * subs.size());
+  char* tab = (char*)ws_alloc(c, b_blk + b_eig + b_bt + b_so + b_sub + 256);
+  if (!d || !e || !tau || !p || !part || !bar || !tn || !nr || !work || !Y || !U0 || !U1 || !S || !tab ||
+      (nl > 0 && (!PS || !PT || !PX || !VT || !W))) {
     c->ws.top = top;
-    return set_err(c, TNT_E_ALLOC, "scratch exhausted (small eigensolves)");
+    return set_err(c, TNT_E_ALLOC, "scratch exhausted (eigensolves)");
   }
-  cudaStream_t st = c->stream;
-  heig.insert(heig.end(), hbt.begin(), hbt.end());
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(dc, hc.data(), sizeof(CtaBlk) * nb, cudaMemcpyHostToDevice, st));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(dbl, he.data(), sizeof(EBlk) * nb, cudaMemcpyHostToDevice, st));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(deig, heig.data(), sizeof(int2) * heig.size(), cudaMemcpyHostToDevice, st));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(dtask, ht.data(), sizeof(NsTask) * ht.size(), cudaMemcpyHostToDevice, st));
-  {
-    size_t o = 0;
-    for (auto& v : htile) {
-      if (!v.empty())
-        TNT_CUDA_TRY(c, cudaMemcpyAsync(dtile + o, v.data(), sizeof(int4) * v.size(), cudaMemcpyHostToDevice, st));
-      o += v.size();
-    }
-  }
+  // (memory a pageable copy reads is staged before the call returns)
+  std::vector<char> host(b_blk + b_eig + b_bt + b_so + b_sub, 0);
+  memcpy(host.data(), he.data(), sizeof(EBlk) * nb);
+  memcpy(host.data() + b_blk, heig.data(), sizeof(int2) * heig.size());
+  if (!hbt.empty()) memcpy(host.data() + b_blk + b_eig, hbt.data(), sizeof(int2) * hbt.size());
+  memcpy(host.data() + b_blk + b_eig + b_bt, so.data(), sizeof(int64_t) * nb);
+  if (!subs.empty()) memcpy(host.data() + b_blk + b_eig + b_bt + b_so, subs.data(), sizeof(WySub) * subs.size());
+  TNT_CUDA_TRY(c, cudaMemcpyAsync(tab, host.data(), host.size(), cudaMemcpyHostToDevice, st));
+  const EBlk* dblk = (const EBlk*)tab;
+  const int2* deig = (const int2*)(tab + b_blk);
+  const int2* dbt = (const int2*)(tab + b_blk + b_eig);
+  const int64_t* dso = (const int64_t*)(tab + b_blk + b_eig + b_bt);
+  const WySub* dsub = (const WySub*)(tab + b_blk + b_eig + b_bt + b_so);
   {
     double fl = 0;
     for (const SmallEig& b : blocks) fl += 16.0 / 3.0 * (double)b.n * b.n * b.n;
     ProfScope ps(c, "heig_tridiag", fl);
-    k_tridiag_cta<<<(unsigned)nb, TRI_CTA_THREADS, 0, st>>>(G, dc, d, e, tau);
-    c->launches++;
-    TNT_CHECK_LAUNCH(c);
+    for (int i0 = 0; i0 < nb;) {
+      std::vector<int64_t> ns;
+      for (int i = i0; i < nb; ++i) ns.push_back(blocks[(size_t)i].n);
+      std::vector<int> q;
+      const int cnt = tri_deal(ns, nsm, smem_max, &q);
+      if (cnt < 1) {
+        c->ws.top = top;
+        return set_err(c, TNT_E_UNSUPPORTED, "tridiagonal kernel cannot hold a block of %lld rows", (long long)ns[0]);
+      }
+      TriGroup T;
+      T.nblk = cnt;
+      T.bar = bar;
+      T.abort_flag = (int*)(bar + 32 * TRI_MAXB);
+      T.status = c->d_status;
+      int ctas = 0;
+      size_t smem = 0;
+      for (int i = 0; i < cnt; ++i) {
+        const SmallEig& b = blocks[(size_t)(i0 + i)];
+        const EBlk& E = he[(size_t)(i0 + i)];
+        const int64_t rows = (b.n + q[(size_t)i] - 1) / q[(size_t)i];
+        T.b[i] = TriBlk{G + b.goff, tau + E.off, d + E.off, e + E.off, p + 2 * E.off, part + 2 * ctas,
+                        (int)b.n, ctas, q[(size_t)i]};
+        ctas += q[(size_t)i];
+        smem = std::max(smem, (size_t)(rows + 3 + (q[(size_t)i] == 1)) * b.n * sizeof(z));
+      }
+      TNT_CUDA_TRY(c, cudaMemsetAsync(bar, 0, sizeof(unsigned) * 32 * (TRI_MAXB + 1), st));
+      void* args[] = {&T};
+      TNT_CUDA_TRY(c, cudaLaunchCooperativeKernel((void*)k_tridiag_group, dim3((unsigned)ctas), dim3(TRI_GTHREADS),
+                                                  args, smem, st));
+      c->launches++;
+      i0 += cnt;
+    }
   }
   {
     ProfScope ps(c, "heig_tridiag_eig");
-    k_split<<<(unsigned)nb, 32, 0, st>>>(d, e, dbl, tn, nr);
-    k_bisect<<<(unsigned)kt, 32, 0, st>>>(d, e, dbl, deig, nr, tn, ev);
-    k_inviter<<<(unsigned)kt, IV_THREADS, 0, st>>>(d, e, dbl, deig, nr, ev, tn, work, Y);
-    c->launches += 2;
+    k_split<<<(unsigned)nb, 32, 0, st>>>(d, e, dblk, tn, nr);
+    k_bisect<<<(unsigned)kt, 32, 0, st>>>(d, e, dblk, deig, nr, tn, ev);
+    k_inviter<<<(unsigned)kt, IV_THREADS, 0, st>>>(d, e, dblk, deig, nr, ev, tn, work, Y);
+    c->launches += 3;
     TNT_CHECK_LAUNCH(c);
   }
+  int r = TNT_OK;
   {
     double fl = 0;
     for (const SmallEig& b : blocks) fl += 8.0 * (double)b.n * b.n * b.k;
     ProfScope ps(c, "heig_backtransform", fl);
-    const size_t smem = sizeof(z) * nmax * cols;
-    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_backtransform, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_backtransform<<<(unsigned)hbt.size(), 256, smem, st>>>(Y, G, tau, dbl, deig + kt, cols, U0);
-    c->launches++;
-    TNT_CHECK_LAUNCH(c);
-  }
-  {  // two Newton-Schulz steps over all blocks: U0 -> U1 -> U
-    size_t o = 0;
-    for (int q = 0; q < 4; ++q) {
-      const int nt = (int)htile[q].size();
-      if (nt > 0) {
-        k_gemm_tasks<<<(unsigned)std::min(nt, 152 * 8), 256, 0, st>>>(dtask, dtile + o, nt);
-        c->launches++;
-        TNT_CHECK_LAUNCH(c);
-      }
-      o += htile[q].size();
+    if (!hbt.empty()) {
+      const size_t smem = sizeof(z) * (size_t)blocks[(size_t)nl].n * cols;
+      TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_backtransform, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      k_backtransform<<<(unsigned)hbt.size(), 256, smem, st>>>(Y, G, tau, dblk, dbt, cols, U0);
+      c->launches++;
     }
+    if (nl > 0) r = wy_backtransform(c, G, blocks, nl, he, po, vo, wo2, npan, tau, dblk, dsub, (int)subs.size(), Y, U0,
+                                     PS, PT, PX, VT, W);
   }
-  // the host tables die at return: the uploads above must have completed
-  TNT_CUDA_TRY(c, cudaStreamSynchronize(st));
+  // two Newton-Schulz steps over all blocks: S = X^H X; S <- 1.5 I - 0.5 S; X <- X S
+  for (int step = 0; step < 2 && r == TNT_OK; ++step) {
+    std::vector<GemmTask> ts, tx;
+    for (int i = 0; i < nb; ++i) {
+      const SmallEig& b = blocks[(size_t)i];
+      z* X = (step == 0 ? U0 : U1) + he[(size_t)i].yo;  // n x k, ld k
+      GemmTask t{};
+      t.g.batch = 1;
+      t.g.alpha = zmk(1, 0);
+      t.g.M = b.k; t.g.N = b.k; t.g.K = b.n;
+      t.g.A = X; t.g.a_rs = 1; t.g.a_cs = b.k; t.g.conj_a = 1;
+      t.g.B = X; t.g.b_rs = b.k; t.g.b_cs = 1;
+      t.g.C = S + so[(size_t)i]; t.g.c_rs = b.k;
+      t.herm = 1;
+      ts.push_back(t);
+      GemmTask u{};
+      u.g.batch = 1;
+      u.g.alpha = zmk(1, 0);
+      u.g.M = b.n; u.g.N = b.k; u.g.K = b.k;
+      u.g.A = X; u.g.a_rs = b.k; u.g.a_cs = 1;
+      u.g.B = S + so[(size_t)i]; u.g.b_rs = b.k; u.g.b_cs = 1;
+      u.g.C = (step == 0) ? U1 + he[(size_t)i].yo : U + b.goff;
+      u.g.c_rs = (step == 0) ? b.k : b.n;
+      tx.push_back(u);
+    }
+    r = zgemm_tasks(c, ts);
+    if (r != TNT_OK) break;
+    const int64_t kmax = blocks[0].n;
+    k_ns_coef_all<<<dim3((unsigned)std::min<int64_t>((kmax * kmax + 255) / 256, 64), (unsigned)nb), 256, 0, st>>>(
+        S, dblk, dso);
+    c->launches++;
+    r = zgemm_tasks(c, tx);
+  }
+  TNT_CHECK_LAUNCH(c);
   c->ws.top = top;
-  return TNT_OK;
+  return r;
 }
 
 }  // namespace tnt

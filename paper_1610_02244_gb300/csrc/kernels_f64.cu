@@ -179,6 +179,93 @@ int zgemm(Ctx* c, const ZGemm& g) {
 }
 
 namespace {
+// The same 16 x 16 tiles for a set of products in one launch; the products travel as a kernel
+// argument (no table upload)
+constexpr int FT_MAX = 48;
+struct FmaTask {
+  const z *A, *B;
+  z* C;
+  int64_t a_rs, a_cs, b_rs, b_cs, c_rs;
+  int M, N, K, conj_a, conj_b, herm, sub, tile0;
+};
+struct FmaTasks {
+  int n, tiles;
+  FmaTask t[FT_MAX];
+};
+__global__ void __launch_bounds__(256) k_zgemm16_tasks(const __grid_constant__ FmaTasks T) {
+  __shared__ z As[16][17];
+  __shared__ z Bs[16][17];
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  for (int w = blockIdx.x; w < T.tiles; w += gridDim.x) {
+    int lo = 0, hi = T.n;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (T.t[mid].tile0 <= w) lo = mid;
+      else hi = mid;
+    }
+    const FmaTask& g = T.t[lo];
+    const int ntn = (g.N + 15) / 16, tile = w - g.tile0;
+    const int64_t m0 = (int64_t)(tile / ntn) * 16, n0 = (int64_t)(tile % ntn) * 16;
+    if (g.herm && n0 > m0) continue;
+    z acc = zmk(0, 0);
+    for (int64_t k0 = 0; k0 < g.K; k0 += 16) {
+      {
+        const int64_t gi = m0 + ty, gk = k0 + tx;
+        z v = (gi < g.M && gk < g.K) ? g.A[gi * g.a_rs + gk * g.a_cs] : zmk(0, 0);
+        if (g.conj_a) v.y = -v.y;
+        As[ty][tx] = v;
+      }
+      {
+        const int64_t gk = k0 + ty, gj = n0 + tx;
+        z v = (gj < g.N && gk < g.K) ? g.B[gk * g.b_rs + gj * g.b_cs] : zmk(0, 0);
+        if (g.conj_b) v.y = -v.y;
+        Bs[ty][tx] = v;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int kk = 0; kk < 16; ++kk) zfma(acc, As[ty][kk], Bs[kk][tx]);
+      __syncthreads();
+    }
+    const int64_t gi = m0 + ty, gj = n0 + tx;
+    if (gi < g.M && gj < g.N && !(g.herm && gj > gi)) {
+      z* p = g.C + gi * g.c_rs + gj;
+      if (g.sub) acc = zsub(*p, acc);
+      *p = acc;
+      if (g.herm && gj < gi) g.C[gj * g.c_rs + gi] = zconj(acc);
+    }
+  }
+}
+}  // namespace
+
+int zgemm_fma_tasks(Ctx* c, const GemmTask* const* tasks, int n) {
+  for (int i0 = 0; i0 < n; i0 += FT_MAX) {
+    FmaTasks T;
+    T.n = std::min(FT_MAX, n - i0);
+    int64_t tiles = 0;
+    double flop = 0;
+    for (int i = 0; i < T.n; ++i) {
+      const ZGemm& g = tasks[i0 + i]->g;
+      FmaTask& o = T.t[i];
+      o.A = g.A; o.B = g.B; o.C = g.C;
+      o.a_rs = g.a_rs; o.a_cs = g.a_cs; o.b_rs = g.b_rs; o.b_cs = g.b_cs; o.c_rs = g.c_rs;
+      o.M = (int)g.M; o.N = (int)g.N; o.K = (int)g.K;
+      o.conj_a = g.conj_a; o.conj_b = g.conj_b;
+      o.herm = tasks[i0 + i]->herm; o.sub = tasks[i0 + i]->sub;
+      o.tile0 = (int)tiles;
+      tiles += ((g.M + 15) / 16) * ((g.N + 15) / 16);
+      flop += (o.herm ? 4.0 : 8.0) * (double)g.M * (double)g.N * (double)g.K;
+    }
+    if (tiles > INT32_MAX) return set_err(c, TNT_E_UNSUPPORTED, "grouped FP64 products: too many tiles");
+    T.tiles = (int)tiles;
+    ProfScope ps(c, "zgemm_f64", flop);
+    k_zgemm16_tasks<<<(unsigned)std::min<int64_t>(tiles, 152 * 8), 256, 0, c->stream>>>(T);
+    c->launches++;
+  }
+  TNT_CHECK_LAUNCH(c);
+  return TNT_OK;
+}
+
+namespace {
 __global__ void k_herm_mirror(z* G, int64_t n) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n * n;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -863,7 +950,10 @@ int vec_normalize(Ctx* c, const z* x, z* y, int64_t n, const double* d_norm2) {
 namespace {
 constexpr int GS_THREADS = 256, GS_WARPS = GS_THREADS / 32;
 constexpr int GS_SMEM = 208 * 1024;
-constexpr int64_t GS_MAX_N = 1 << 18;
+// Above this the slice of w alone nears the shared memory of an SM, and both forms are bound
+// by the FP64 pipe.  FP64 solves of this size, fused / separate launches: n = 2^12 9.7 / 27
+// ms, 2^16 28 / 50, 2^18 60 / 80, 2^20 232 / 239.
+constexpr int64_t GS_MAX_N = 1 << 20;
 
 struct GsArgs {
   const z* V;
@@ -1545,26 +1635,8 @@ int tridiag_lowest_batched(Ctx* c, const double* d_alpha, const double* d_beta, 
   return TNT_OK;
 }
 
-// ============================================================ gather / fill / scale
+// ============================================================ fill / scale
 namespace {
-__global__ void k_gather2d(const z* __restrict__ src, int64_t src_ld,
-                           const int64_t* __restrict__ rows, int64_t nr,
-                           const int64_t* __restrict__ cols, int64_t nc, z* __restrict__ dst,
-                           int64_t dst_ld, int conj_t) {
-  const int64_t total = nr * nc;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    int64_t i = e / nc, j = e % nc;
-    z v = src[rows[i] * src_ld + cols[j]];
-    if (conj_t) {
-      v.y = -v.y;
-      dst[j * dst_ld + i] = v;
-    } else {
-      dst[i * dst_ld + j] = v;
-    }
-  }
-}
-
 __global__ void k_zfill(z* p, int64_t n, z v) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * blockDim.x)
@@ -1589,16 +1661,6 @@ unsigned grid_for(int64_t n) {
   return (unsigned)b;
 }
 }  // namespace
-
-int gather2d(Ctx* c, const z* src, int64_t src_ld, const int64_t* d_rows, int64_t nr,
-             const int64_t* d_cols, int64_t nc, z* dst, int64_t dst_ld, int conj_t) {
-  if (nr <= 0 || nc <= 0) return TNT_OK;
-  k_gather2d<<<grid_for(nr * nc), 256, 0, c->stream>>>(src, src_ld, d_rows, nr, d_cols, nc,
-                                                        dst, dst_ld, conj_t);
-  c->launches++;
-  TNT_CHECK_LAUNCH(c);
-  return TNT_OK;
-}
 
 int zfill(Ctx* c, z* p, int64_t n, z v) {
   if (n <= 0) return TNT_OK;

@@ -67,24 +67,53 @@ static_assert(2LL * OZ_S * OZ_CHUNK * OZ_KB * 64 * 64 <= (1LL << 24),
               "a level sum over one K chunk must stay exact in FP32");
 static_assert(OZ_SMEM <= 227 * 1024, "rings fit the shared memory of an SM");
 
-struct OzArgs {
-  int64_t M, N;
-  int ntm, ntn;       // tiles along M and N
-  int nkb;            // K blocks of 32
-  int ks;             // K splits
-  int both;           // an item runs both level groups, one after the other
-  const uint8_t* A;   // [ntm][nkb][OZ_S] slice tiles
-  const uint8_t* B;   // [ntn][nkb][OZ_S]
-  longlong2* P;       // [split][group][M][N] partial sums
-  int lower;          // Hermitian result: tiles strictly above the diagonal are left out
-  int* status;
+// one product of a launch; offsets are bytes into the context's buffer
+struct OzTask {
+  const z *A, *B;
+  z* C;
+  int64_t a_rs, a_ks, b_rs, b_ks, c_rs;  // A(i, k) = A[i a_rs + k a_ks], B(k, j) = B[j b_rs + k b_ks]
+  int64_t offA, offB, offE, offP;        // slice tiles, exponent fields (M then N), partial sums
+  int64_t atom0;                         // first slice atom of the task among all tasks'
+  int M, N, K;
+  int ntm, ntn, nkb;                     // tiles along M and N, K blocks of 32
+  int ks, both;                          // K splits; an item runs both level groups, or one
+  int conj_a, conj_b;
+  int herm;  // C = A B is Hermitian: tiles strictly above the diagonal are mirrored, not computed
+  int sub;   // C -= A B
+  int item0, scale0, fin0;               // first item / scale block / finish block
 };
+// The products of one launch travel as a kernel argument: no table upload.
+constexpr int OZ_MAXT = 40;
+template <int CAP>
+struct OzTasks {
+  int n, items, scale_blocks, fin_blocks;
+  int64_t atoms;
+  uint8_t* buf;
+  int* status;
+  OzTask t[CAP];
+};
+// the last task whose first index (by FIRST) is at most w
+template <int CAP, typename F>
+__device__ __forceinline__ int oz_find(const OzTasks<CAP>& T, F first, int64_t w) {
+  if (CAP == 1) return 0;
+  int lo = 0, hi = T.n;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if ((int64_t)first(T.t[mid]) <= w) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
 
 struct OzItem {
-  int mt, nt, g0, g1, kb0, kb1, sp;  // groups g0..g1, K blocks [kb0, kb1)
+  int task, mt, nt, g0, g1, kb0, kb1, sp;  // groups g0..g1, K blocks [kb0, kb1)
 };
-// item w; the heavier group's items come first.  false: a tile left out
-__device__ __forceinline__ bool oz_item(const OzArgs& g, int w, OzItem* it) {
+// item w of the launch; a task's heavier groups come first.  false: a tile left out
+template <int CAP>
+__device__ __forceinline__ bool oz_item(const OzTasks<CAP>& T, int w, OzItem* it) {
+  it->task = oz_find(T, [](const OzTask& t) { return t.item0; }, w);
+  const OzTask& g = T.t[it->task];
+  w -= g.item0;
   const int ntiles = g.ntm * g.ntn;
   const int t = w % ntiles, r = w / ntiles;
   it->mt = t / g.ntn;
@@ -98,10 +127,7 @@ __device__ __forceinline__ bool oz_item(const OzArgs& g, int w, OzItem* it) {
   it->sp = r % g.ks;
   it->kb0 = (int)((int64_t)it->sp * g.nkb / g.ks);
   it->kb1 = (int)((int64_t)(it->sp + 1) * g.nkb / g.ks);
-  return !(g.lower && it->mt * OZ_BM + OZ_BM <= it->nt * OZ_BN);
-}
-__host__ __device__ inline int oz_items(const OzArgs& g) {
-  return g.ntm * g.ntn * g.ks * (g.both ? 1 : 2);
+  return !(g.herm && it->mt * OZ_BM + OZ_BM <= it->nt * OZ_BN);
 }
 // pairs (p, q) of group levels l0..l1 at slice p of A: q in [qlo, qhi]
 __device__ __forceinline__ void oz_levels(int grp, int* l0, int* l1) {
@@ -210,7 +236,8 @@ __device__ __forceinline__ void oz_put(longlong2* o, int nc, const long long* re
     if (j < nc) o[j] = make_longlong2(re[j], im[j]);
 }
 
-__global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
+template <int CAP>
+__global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(const __grid_constant__ OzTasks<CAP> T) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   OzRings R;
@@ -225,7 +252,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
   uint32_t* tmem_slot = (uint32_t*)(acce + 4);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nitems = oz_items(g);
+  const int nitems = T.items;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < OZ_NA; ++s) {
@@ -261,7 +288,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
     auto load = [&](uint8_t* ring, uint64_t* full, uint64_t* empty, uint32_t& i, int n, uint32_t bytes,
                     const uint8_t* src) {
       const int s = (int)(i % (uint32_t)n);
-      if (i >= (uint32_t)n && !mbar_wait(&empty[s], ((i / n) & 1) ^ 1, g.status)) *abort_flag = 1;
+      if (i >= (uint32_t)n && !mbar_wait(&empty[s], ((i / n) & 1) ^ 1, T.status)) *abort_flag = 1;
       if (*abort_flag) {
         stop = true;
         return;
@@ -272,14 +299,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
     };
     for (int w = blockIdx.x; w < nitems && !stop; w += gridDim.x) {
       OzItem it;
-      if (!oz_item(g, w, &it)) continue;
+      if (!oz_item(T, w, &it)) continue;
+      const OzTask& g = T.t[it.task];
       for (int grp = it.g0; grp <= it.g1 && !stop; ++grp) {
         int l0, l1;
         oz_levels(grp, &l0, &l1);
         const int pmax = min(OZ_S, l1 - 1);
         for (int kb = it.kb0; kb < it.kb1 && !stop; ++kb) {
-          const uint8_t* A = g.A + ((int64_t)it.mt * g.nkb + kb) * (OZ_S * OZ_TA);
-          const uint8_t* B = g.B + ((int64_t)it.nt * g.nkb + kb) * (OZ_S * OZ_TB);
+          const uint8_t* A = T.buf + g.offA + ((int64_t)it.mt * g.nkb + kb) * (OZ_S * OZ_TA);
+          const uint8_t* B = T.buf + g.offB + ((int64_t)it.nt * g.nkb + kb) * (OZ_S * OZ_TB);
           int qnext = min(OZ_S, l1 - 1);  // next slice of B to load (descending)
           for (int p = 1; p <= pmax && !stop; ++p) {
             const int qlo = max(1, l0 - p);
@@ -292,9 +320,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
     }
     // copies in flight land before the CTA may exit
     for (uint32_t i = (ia > (uint32_t)OZ_NA ? ia - OZ_NA : 0u); i < ia; ++i)
-      mbar_wait(&R.fa[i % OZ_NA], (i / OZ_NA) & 1, g.status);
+      mbar_wait(&R.fa[i % OZ_NA], (i / OZ_NA) & 1, T.status);
     for (uint32_t i = (ib > (uint32_t)OZ_NB ? ib - OZ_NB : 0u); i < ib; ++i)
-      mbar_wait(&R.fb[i % OZ_NB], (i / OZ_NB) & 1, g.status);
+      mbar_wait(&R.fb[i % OZ_NB], (i / OZ_NB) & 1, T.status);
   } else if (warp == 1 && lane == 0) {
     // ------------------------------------------------ MMA issue
     uint32_t sub = 0;
@@ -302,14 +330,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
     OzIssue r{su32(R.a) >> 4, su32(R.b) >> 4, R.fa, R.ea, R.fb, R.eb, nullptr, 0, 0, 0, 0, 0};
     for (int w = blockIdx.x; w < nitems && !stop; w += gridDim.x) {
       OzItem it;
-      if (!oz_item(g, w, &it)) continue;
+      if (!oz_item(T, w, &it)) continue;
       for (int grp = it.g0; grp <= it.g1 && !stop; ++grp) {
         for (int kb = it.kb0; kb < it.kb1; ++kb) {
           const bool first = ((kb - it.kb0) % OZ_CHUNK) == 0;
           bool ok = *abort_flag == 0;
           r.acce = first && sub > 0 ? acce : nullptr;
           r.pacc = (sub - 1) & 1;
-          if (ok) ok = grp ? oz_issue_block<1>(r, tmem, first, g.status) : oz_issue_block<0>(r, tmem, first, g.status);
+          if (ok) ok = grp ? oz_issue_block<1>(r, tmem, first, T.status) : oz_issue_block<0>(r, tmem, first, T.status);
           if (!ok) {
             *abort_flag = 1;
             stop = true;
@@ -331,7 +359,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
     bool stop = false;
     for (int w = blockIdx.x; w < nitems && !stop; w += gridDim.x) {
       OzItem it;
-      if (!oz_item(g, w, &it)) continue;
+      if (!oz_item(T, w, &it)) continue;
+      const OzTask& g = T.t[it.task];
       const int64_t gm = (int64_t)it.mt * OZ_BM + row;
       const int64_t gn0 = (int64_t)it.nt * OZ_BN + half * 32;
       for (int grp = it.g0; grp <= it.g1 && !stop; ++grp) {
@@ -339,7 +368,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
 #pragma unroll
         for (int j = 0; j < 32; ++j) re[j] = im[j] = 0;
         for (int kb = it.kb0; kb < it.kb1; kb += OZ_CHUNK) {
-          if (*abort_flag || !mbar_wait(accf, sub & 1, g.status)) {
+          if (*abort_flag || !mbar_wait(accf, sub & 1, T.status)) {
             *abort_flag = 1;
             stop = true;
             break;
@@ -367,9 +396,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
           ++sub;
         }
         if (stop || gm >= g.M) continue;
-        const int nc = (int)min((int64_t)32, g.N - gn0);  // columns of this half tile
+        const int nc = (int)min((int64_t)32, (int64_t)g.N - gn0);  // columns of this half tile
         if (nc <= 0) continue;
-        oz_put(g.P + ((int64_t)(2 * it.sp + grp) * g.M + gm) * g.N + gn0, nc, re, im);
+        oz_put((longlong2*)(T.buf + g.offP) + ((int64_t)(2 * it.sp + grp) * g.M + gm) * g.N + gn0, nc, re, im);
       }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -381,29 +410,38 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
   }
 }
 
-// C from the partial sums of the K splits (integers: any order gives the same value)
-__global__ void k_oz_finish(const longlong2* __restrict__ P, int ks, int64_t M, int64_t N,
-                            const int* __restrict__ eA, const int* __restrict__ eB, int lower,
-                            z* __restrict__ C, int64_t ldc) {
-  const int64_t total = M * N;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / N, j = e % N;
-    if (lower && (i / OZ_BM) * OZ_BM + OZ_BM <= (j / OZ_BN) * OZ_BN) continue;
+// C from the partial sums of the K splits (integers: any order gives the same value); one
+// element per thread, a block's 256 elements in one task.  Hermitian results: the lower
+// triangle, mirrored.
+template <int CAP>
+__global__ void __launch_bounds__(256) k_oz_finish(const __grid_constant__ OzTasks<CAP> T) {
+  for (int fb = blockIdx.x; fb < T.fin_blocks; fb += gridDim.x) {
+    const OzTask& g = T.t[oz_find(T, [](const OzTask& t) { return t.fin0; }, fb)];
+    const int64_t total = (int64_t)g.M * g.N, e = (int64_t)(fb - g.fin0) * 256 + threadIdx.x;
+    if (e >= total) continue;
+    const int64_t i = e / g.N, j = e % g.N;
+    if (g.herm && j > i) continue;
+    const longlong2* P = (const longlong2*)(T.buf + g.offP) + e;
     longlong2 h = make_longlong2(0, 0), l = h;
-    for (int s = 0; s < ks; ++s) {
-      const longlong2 a = P[(int64_t)(2 * s) * total + e], b = P[(int64_t)(2 * s + 1) * total + e];
+    for (int s = 0; s < g.ks; ++s) {
+      const longlong2 a = P[(int64_t)(2 * s) * total], b = P[(int64_t)(2 * s + 1) * total];
       h.x += a.x;
       h.y += a.y;
       l.x += b.x;
       l.y += b.y;
     }
-    C[i * ldc + j] = zmk(oz_value(h.x, l.x, eA[i], eB[j]), oz_value(h.y, l.y, eA[i], eB[j]));
+    const int* ex = (const int*)(T.buf + g.offE);
+    const int ea = ex[i], eb = ex[g.M + j];
+    z v = zmk(oz_value(h.x, l.x, ea, eb), oz_value(h.y, l.y, ea, eb));
+    z* o = g.C + i * g.c_rs + j;
+    if (g.sub) v = zsub(*o, v);
+    *o = v;
+    if (g.herm && j < i) g.C[j * g.c_rs + i] = zconj(v);
   }
 }
 
 // ---------------------------------------------------------------- scales and slices
-// one operand of the product seen as rows of K entries: X[i * rs + k * cs]
+// one operand of a product seen as rows of K entries: X[i * rs + k * cs]
 struct OzOp {
   const z* X;
   int64_t rows, rs, cs;
@@ -411,6 +449,18 @@ struct OzOp {
   int* e;        // per row: largest exponent field of the re and im parts
   uint8_t* out;  // slice tiles
 };
+// B enters as rows n with K along the row
+__device__ __forceinline__ OzOp oz_operand(const OzTask& g, uint8_t* buf, bool isb) {
+  OzOp o;
+  o.X = isb ? g.B : g.A;
+  o.rows = isb ? g.N : g.M;
+  o.rs = isb ? g.b_rs : g.a_rs;
+  o.cs = isb ? g.b_ks : g.a_ks;
+  o.conj = isb ? g.conj_b : g.conj_a;
+  o.e = (int*)(buf + g.offE) + (isb ? g.M : 0);
+  o.out = buf + (isb ? g.offB : g.offA);
+  return o;
+}
 
 // largest exponent field of every row.  Entries contiguous along K: one warp per row;
 // otherwise 32 rows by 64 of K per CTA, neighbouring lanes on neighbouring rows, combined
@@ -418,13 +468,16 @@ struct OzOp {
 __device__ __forceinline__ unsigned oz_exp(z v) {
   return max(((unsigned)__double2hiint(v.x) >> 20) & 0x7ffu, ((unsigned)__double2hiint(v.y) >> 20) & 0x7ffu);
 }
-__host__ __device__ inline int64_t oz_scale_blocks(const OzOp& o, int64_t K) {
-  return o.cs == 1 ? (o.rows + 7) / 8 : ((o.rows + 31) / 32) * ((K + 63) / 64);
+__host__ __device__ inline int64_t oz_scale_blocks(int64_t rows, int64_t ks, int64_t K) {
+  return ks == 1 ? (rows + 7) / 8 : ((rows + 31) / 32) * ((K + 63) / 64);
 }
-__global__ void __launch_bounds__(256) k_oz_scale(OzOp a, OzOp b, int64_t K, int64_t nba) {
-  const bool isb = blockIdx.x >= nba;
-  const OzOp o = isb ? b : a;
-  const int64_t blk = isb ? (int64_t)blockIdx.x - nba : (int64_t)blockIdx.x;
+template <int CAP>
+__global__ void __launch_bounds__(256) k_oz_scale(const __grid_constant__ OzTasks<CAP> T) {
+  const OzTask& g = T.t[oz_find(T, [](const OzTask& t) { return t.scale0; }, blockIdx.x)];
+  const int64_t K = g.K, nba = oz_scale_blocks(g.M, g.a_ks, K);
+  const bool isb = (int64_t)blockIdx.x - g.scale0 >= nba;
+  const OzOp o = oz_operand(g, T.buf, isb);
+  const int64_t blk = (int64_t)blockIdx.x - g.scale0 - (isb ? nba : 0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (o.cs == 1) {
     const int64_t i = blk * 8 + warp;
@@ -497,32 +550,18 @@ __device__ __forceinline__ void oz_slice_atom(const OzOp& o, int64_t K, int nkb,
     *(uint4*)(q + ROWS * 64) = make_uint4(wi[0], wi[1], wi[2], wi[3]);
   }
 }
-__global__ void __launch_bounds__(256) k_oz_slice(OzOp a, OzOp b, int64_t K, int nkb, int64_t na, int64_t nb) {
+template <int CAP>
+__global__ void __launch_bounds__(256) k_oz_slice(const __grid_constant__ OzTasks<CAP> T) {
   const int lane = threadIdx.x & 31;
-  for (int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); w < na + nb; w += (int64_t)gridDim.x * 8) {
-    if (w < na) oz_slice_atom<2>(a, K, nkb, w, lane);
-    else oz_slice_atom<3>(b, K, nkb, w - na, lane);
+  for (int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); w < T.atoms; w += (int64_t)gridDim.x * 8) {
+    const OzTask& g = T.t[oz_find(T, [](const OzTask& t) { return t.atom0; }, w)];
+    const int64_t a = w - g.atom0, na = (int64_t)g.ntm * (OZ_BM / 8) * g.nkb;
+    if (a < na) oz_slice_atom<2>(oz_operand(g, T.buf, false), g.K, g.nkb, a, lane);
+    else oz_slice_atom<3>(oz_operand(g, T.buf, true), g.K, g.nkb, a - na, lane);
   }
 }
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
-
-// sizes of the context-owned buffer of one product
-struct OzSize {
-  int64_t ntm, ntn, nkb;
-  size_t a, b, e, p;
-};
-OzSize oz_size(int64_t M, int64_t N, int64_t K, int ks) {
-  OzSize s;
-  s.ntm = cdiv(M, OZ_BM);
-  s.ntn = cdiv(N, OZ_BN);
-  s.nkb = cdiv(K, OZ_KB);
-  s.a = ws_round((size_t)(s.ntm * s.nkb) * OZ_S * OZ_TA);
-  s.b = ws_round((size_t)(s.ntn * s.nkb) * OZ_S * OZ_TB);
-  s.e = ws_round(sizeof(int) * (size_t)(M + N));
-  s.p = ws_round(sizeof(longlong2) * 2 * (size_t)ks * M * N);
-  return s;
-}
 
 // How a product of `tiles` output tiles and nkb K blocks is dealt to nsm SMs: K splits, and
 // whether an item takes both level groups (one CTA then loads the rings once) or one.  In
@@ -577,70 +616,162 @@ bool ozgemm_eligible(const Ctx* c, const ZGemm& g) {
   return (double)g.K * std::max(1.0, tiles / 152.0) >= 110.0;
 }
 
-// C = A B (FP64-accurate) through the integer-slice tensor-core kernel; slices and partial
-// sums live in the context's own buffer (grown between calls, never inside a capture)
-int ozgemm(Ctx* c, const ZGemm& g) {
-  const int64_t M = g.M, N = g.N, K = g.K;
-  static int sm = 0;
-  if (!sm) {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) v = 152;
-    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
-    sm = v;
+namespace {
+int oz_sm_count(Ctx* c, int* sm) {
+  static int v = 0;
+  if (!v) {
+    int n = 0;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || n < 1) n = 152;
+    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_oz_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
+    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_oz_gemm<OZ_MAXT>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
+    v = n;
   }
-  OzSize s = oz_size(M, N, K, 0);
-  OzDeal deal = oz_deal(s.ntm * s.ntn, s.nkb, sm);
-  while (deal.ks > 1 && 32.0 * deal.ks * (double)M * (double)N > 256e6) --deal.ks;
-  s = oz_size(M, N, K, deal.ks);
-  const size_t need = s.a + s.b + s.e + s.p;
-  if (need > c->oz_cap) {
+  *sm = v;
+  return TNT_OK;
+}
+
+// products tk[0..n) in one set of launches; slices and partial sums live in the context's own
+// buffer (grown between calls, never inside a capture)
+template <int CAP>
+int oz_launch(Ctx* c, const GemmTask* const* tk, int n, int sm) {
+  OzTasks<CAP> T;
+  T.n = n;
+  T.status = c->d_status;
+  size_t off = 0;
+  int64_t items = 0, scale = 0, fin = 0, rows = 0;
+  double work = 0, flop = 0, bytes = 0;
+  T.atoms = 0;
+  for (int i = 0; i < n; ++i) {
+    const ZGemm& g = tk[i]->g;
+    OzTask& o = T.t[i];
+    o.A = g.A; o.B = g.B; o.C = g.C;
+    o.a_rs = g.a_rs; o.a_ks = g.a_cs; o.b_rs = g.b_cs; o.b_ks = g.b_rs; o.c_rs = g.c_rs;
+    o.conj_a = g.conj_a; o.conj_b = g.conj_b;
+    o.herm = tk[i]->herm; o.sub = tk[i]->sub;
+    o.M = (int)g.M; o.N = (int)g.N; o.K = (int)g.K;
+    o.ntm = (int)cdiv(g.M, OZ_BM);
+    o.ntn = (int)cdiv(g.N, OZ_BN);
+    o.nkb = (int)cdiv(g.K, OZ_KB);
+    work += 36.0 * o.nkb * o.ntm * o.ntn;
+    flop += (o.herm ? 4.0 : 8.0) * (double)g.M * (double)g.N * (double)g.K;
+  }
+  for (int i = 0; i < n; ++i) {
+    OzTask& o = T.t[i];
+    const double mn = (double)o.M * (double)o.N;
+    OzDeal deal{1, 1};
+    if (n == 1) {
+      deal = oz_deal((int64_t)o.ntm * o.ntn, o.nkb, sm);
+    } else if (work < 4.0 * sm * 36.0 * o.nkb) {
+      // few items per SM: none longer than half of an SM's share, nor shorter than two blocks
+      const double share = std::max(work / sm * 0.5, 72.0);
+      deal.ks = (int)std::min<int64_t>(std::max(1, o.nkb / 2), (int64_t)std::ceil(36.0 * o.nkb / share));
+    }
+    while (deal.ks > 1 && 32.0 * deal.ks * mn > 256e6) --deal.ks;
+    o.ks = deal.ks;
+    o.both = deal.both;
+    o.offA = (int64_t)off;
+    off += ws_round((size_t)o.ntm * o.nkb * OZ_S * OZ_TA);
+    o.offB = (int64_t)off;
+    off += ws_round((size_t)o.ntn * o.nkb * OZ_S * OZ_TB);
+    o.offP = (int64_t)off;
+    off += ws_round(sizeof(longlong2) * 2 * (size_t)o.ks * (size_t)mn);
+    bytes += 16.0 * ((double)o.M + o.N) * o.K + (double)(o.offP - o.offA);
+    o.item0 = (int)items;
+    items += (int64_t)o.ntm * o.ntn * o.ks * (o.both ? 1 : 2);
+    o.scale0 = (int)scale;
+    scale += oz_scale_blocks(o.M, o.a_ks, o.K) + oz_scale_blocks(o.N, o.b_ks, o.K);
+    o.atom0 = T.atoms;
+    T.atoms += ((int64_t)o.ntm * (OZ_BM / 8) + (int64_t)o.ntn * (OZ_BN / 8)) * o.nkb;
+    o.fin0 = (int)fin;
+    fin += cdiv((int64_t)o.M * o.N, 256);
+  }
+  const size_t off_e = off;
+  for (int i = 0; i < n; ++i) {
+    T.t[i].offE = (int64_t)(off_e + sizeof(int) * (size_t)rows);
+    rows += T.t[i].M + T.t[i].N;
+  }
+  off += ws_round(sizeof(int) * (size_t)rows);
+  if (items > INT32_MAX || scale > INT32_MAX || fin > INT32_MAX)
+    return set_err(c, TNT_E_UNSUPPORTED, "FP64 products too large for one launch");
+  T.items = (int)items;
+  T.scale_blocks = (int)scale;
+  T.fin_blocks = (int)fin;
+  if (off > c->oz_cap) {
     TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     dev_free(c->dalloc, c->oz_buf);
     c->oz_buf = nullptr;
     c->oz_cap = 0;
-    if (dev_alloc(c->dalloc, &c->oz_buf, need) != 0)
-      return set_err(c, TNT_E_ALLOC, "device allocation of %zu bytes (FP64 product slices) failed", need);
-    c->oz_cap = need;
+    if (dev_alloc(c->dalloc, &c->oz_buf, off) != 0)
+      return set_err(c, TNT_E_ALLOC, "device allocation of %zu bytes (FP64 product slices) failed", off);
+    c->oz_cap = off;
   }
-  uint8_t* b = (uint8_t*)c->oz_buf;
-  OzOp oa{g.A, M, g.a_rs, g.a_cs, g.conj_a, (int*)(b + s.a + s.b), b};
-  // B enters as rows n with K along the row: B^T[n][k] = B[k * b_rs + n * b_cs]
-  OzOp ob{g.B, N, g.b_cs, g.b_rs, g.conj_b, oa.e + M, b + s.a};
+  T.buf = (uint8_t*)c->oz_buf;
   {
-    ProfScope ps(c, "oz_slice", 16.0 * (double)(M + N) * (double)K + (double)(s.a + s.b));
-    const int64_t nba = oz_scale_blocks(oa, K), nbb = oz_scale_blocks(ob, K);
-    TNT_CUDA_TRY(c, cudaMemsetAsync(oa.e, 0, sizeof(int) * (size_t)(M + N), c->stream));
-    k_oz_scale<<<(unsigned)(nba + nbb), 256, 0, c->stream>>>(oa, ob, K, nba);
-    const int64_t na = s.ntm * (OZ_BM / 8) * s.nkb, nb = s.ntn * (OZ_BN / 8) * s.nkb;
-    k_oz_slice<<<(unsigned)std::min<int64_t>(cdiv(na + nb, 8), 152 * 16), 256, 0, c->stream>>>(
-        oa, ob, K, (int)s.nkb, na, nb);
+    ProfScope ps(c, "oz_slice", bytes);
+    TNT_CUDA_TRY(c, cudaMemsetAsync(T.buf + off_e, 0, sizeof(int) * (size_t)rows, c->stream));
+    k_oz_scale<CAP><<<(unsigned)scale, 256, 0, c->stream>>>(T);
+    k_oz_slice<CAP><<<(unsigned)std::min<int64_t>(cdiv(T.atoms, 8), 152 * 16), 256, 0, c->stream>>>(T);
   }
-  c->launches += 2;
-  TNT_CHECK_LAUNCH(c);
-  OzArgs a;
-  a.M = M;
-  a.N = N;
-  a.ntm = (int)s.ntm;
-  a.ntn = (int)s.ntn;
-  a.nkb = (int)s.nkb;
-  a.ks = deal.ks;
-  a.both = deal.both;
-  a.A = oa.out;
-  a.B = ob.out;
-  a.P = (longlong2*)(b + s.a + s.b + s.e);
-  a.lower = g.lower_only;
-  a.status = c->d_status;
   {
-    ProfScope ps(c, "oz_gemm", (g.lower_only ? 4.0 : 8.0) * (double)M * (double)N * (double)K);
-    k_oz_gemm<<<(unsigned)std::min(oz_items(a), sm), OZ_THREADS, OZ_SMEM, c->stream>>>(a);
-    c->launches++;
-    k_oz_finish<<<(unsigned)std::min<int64_t>(cdiv(M * N, 256), 152 * 8), 256, 0, c->stream>>>(
-        a.P, a.ks, M, N, oa.e, ob.e, g.lower_only, g.C, g.c_rs);
-    c->launches++;
+    ProfScope ps(c, "oz_gemm", flop);
+    k_oz_gemm<CAP><<<(unsigned)std::min<int64_t>(items, sm), OZ_THREADS, OZ_SMEM, c->stream>>>(T);
+    k_oz_finish<CAP><<<(unsigned)std::min<int64_t>(fin, 152 * 8), 256, 0, c->stream>>>(T);
   }
+  c->launches += 4;
   TNT_CHECK_LAUNCH(c);
   return TNT_OK;
+}
+}  // namespace
+
+int ozgemm(Ctx* c, const ZGemm& g) {
+  int sm = 0;
+  TNT_TRY(oz_sm_count(c, &sm));
+  const GemmTask t{g, 0, 0};
+  const GemmTask* p = &t;
+  return oz_launch<1>(c, &p, 1, sm);
+}
+
+// The products of `tasks` (alpha = 1, beta = 0, batch = 1; independent of one another) with as
+// few launches as their number allows.  They go to the slice kernels together when their
+// FP64 tiles, dealt to the SMs, would take longer than the slice launches' 30 us (the rule of
+// ozgemm_eligible for the whole set); products with a side below 16 stay on FP64 units.
+int zgemm_tasks(Ctx* c, const std::vector<GemmTask>& tasks) {
+  int sm = 0;
+  TNT_TRY(oz_sm_count(c, &sm));
+  double rounds = 0, longest = 0;
+  for (const GemmTask& t : tasks) {
+    const double k = (double)t.g.K;
+    rounds += k * (double)cdiv(t.g.M, 16) * (double)cdiv(t.g.N, 16) * (t.herm ? 0.5 : 1.0) / sm;
+    longest = std::max(longest, k);
+  }
+  const bool slices = c->oz_mode != 0 && std::max(rounds, longest) >= 110.0;
+  std::vector<const GemmTask*> oz, fma;
+  for (const GemmTask& t : tasks) {
+    const ZGemm& g = t.g;
+    if (g.M <= 0 || g.N <= 0) continue;
+    if (c->oz_mode == 0 && cdiv(g.M, 64) * cdiv(g.N, 64) >= sm && (!t.herm || g.c_rs == g.M)) {
+      // FP64 units alone: a large product fills the GPU by itself with 64 x 64 tiles
+      ZGemm h = g;
+      h.lower_only = t.herm;
+      if (t.sub) {
+        h.alpha = zmk(-1, 0);
+        h.beta = zmk(1, 0);
+      }
+      TNT_TRY(zgemm(c, h));
+      if (t.herm) TNT_TRY(herm_mirror(c, g.C, g.M));
+      continue;
+    }
+    if (g.K <= 0 || g.batch != 1) return set_err(c, TNT_E_INVALID, "grouped FP64 product with K = %lld", (long long)g.K);
+    (slices && std::min(g.M, std::min(g.N, g.K)) >= 16 && std::max(g.M, g.N) < (1LL << 31) ? oz : fma).push_back(&t);
+  }
+  // longest items first
+  std::stable_sort(oz.begin(), oz.end(), [](const GemmTask* a, const GemmTask* b) { return a->g.K > b->g.K; });
+  for (size_t i = 0; i < oz.size(); i += OZ_MAXT) {
+    const int n = (int)std::min<size_t>(OZ_MAXT, oz.size() - i);
+    if (n == 1) TNT_TRY(oz_launch<1>(c, oz.data() + i, 1, sm));
+    else TNT_TRY(oz_launch<OZ_MAXT>(c, oz.data() + i, n, sm));
+  }
+  return fma.empty() ? TNT_OK : zgemm_fma_tasks(c, fma.data(), (int)fma.size());
 }
 
 }  // namespace tnt

@@ -11,8 +11,7 @@
 // keeps its absolute error at ~eps |M| instead of the sqrt(eps) relative floor of
 // sqrt(lambda).  All candidates are then ordered globally (sigma desc, charge asc, index
 // asc) and cut by the four rules in one kernel.  Every block is diagonalised by Householder
-// tridiagonalisation, bisection and inverse iteration (heig.cu): blocks up to 256 rows are
-// reduced together, one CTA each in one launch, larger ones across the whole GPU.
+// tridiagonalisation, bisection and inverse iteration, all blocks together (heig.cu).
 #include <algorithm>
 #include <cmath>
 #include <map>
@@ -100,14 +99,39 @@ __global__ void k_block_apply(z* __restrict__ Mp, const int64_t* __restrict__ bo
     Mp[off + i] = zscale(Mp[off + i], sc);
 }
 
-// dst[r * ldd + c] = src[r * lds + c], r < rows, c < cols
-__global__ void k_copy_strided(const z* __restrict__ src, int64_t rows, int64_t cols, int64_t lds,
-                               z* __restrict__ dst, int64_t ldd) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < rows * cols;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e / cols, cc = e % cols;
-    dst[r * ldd + cc] = src[r * lds + cc];
+// dst[r * ldd + c] = src[r * lds + c], r < rows, c < cols, for a set of matrices
+constexpr int COPY_MAX = 64;
+struct CopyTask {
+  const z* src;
+  z* dst;
+  int64_t lds, ldd;
+  int rows, cols;
+};
+struct CopyTasks {
+  int n;
+  CopyTask t[COPY_MAX];
+};
+__global__ void __launch_bounds__(256) k_copy_tasks(const __grid_constant__ CopyTasks T) {
+  const CopyTask& a = T.t[blockIdx.y];
+  const int64_t total = (int64_t)a.rows * a.cols;
+  for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < total; e += (int64_t)gridDim.x * 256) {
+    const int64_t r = e / a.cols, cc = e % a.cols;
+    a.dst[r * a.ldd + cc] = a.src[r * a.lds + cc];
   }
+}
+
+// the charge blocks of M, packed: block q (blockIdx.y) is rows x cols of M (leading dimension n)
+struct GatherBlk {
+  int64_t moff, roff, coff, mq, nq;
+};
+__global__ void __launch_bounds__(256) k_gather_blocks(const z* __restrict__ M, int64_t n,
+                                                       const GatherBlk* __restrict__ blks,
+                                                       const int64_t* __restrict__ rows,
+                                                       const int64_t* __restrict__ cols, z* __restrict__ Mp) {
+  const GatherBlk B = blks[blockIdx.y];
+  const int64_t total = B.mq * B.nq;
+  for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < total; e += (int64_t)gridDim.x * 256)
+    Mp[B.moff + e] = M[rows[B.roff + e / B.nq] * n + cols[B.coff + e % B.nq]];
 }
 
 // -------------------------------------------------------------- global selection
@@ -330,15 +354,13 @@ static size_t autoblock_bytes(int64_t m, int64_t n) {
 
 size_t svd_scratch_bound(int64_t m, int64_t n) {
   const size_t mx = (size_t)std::max(m, n), mn = (size_t)std::min(m, n);
-  // the eigen phase of the small blocks (Gram side <= 256, every eigenpair formed): per
-  // block n k <= 256 n of work, iterates, two eigenvector copies and k^2 coefficients
-  const size_t small_eig = (6 * 8 + 8 + 2 * 16 + 16) * 256 * mx + (size_t)(1 << 20);
-  // the tail pass: its Gram matrices and eigenvectors (sum t^2 <= mx mn each), one rotation
-  // buffer (<= mx mn), eigenvalues
-  const size_t tail = 3 * 16 * mx * mn + 8 * std::max<size_t>(mx * mn, 8192);
+  // the tail pass: its Gram matrices and eigenvectors (sum t^2 <= mx mn each), the blocks'
+  // rotation buffers (g t and rows x columns, each <= mx mx in all), eigenvalues
+  const size_t tail = 2 * 16 * mx * mn + 2 * 16 * mx * mx + 8 * std::max<size_t>(mx * mn, 8192);
   return autoblock_bytes(m, n) + 8 * (size_t)(m + n) + 2 * 16 * (size_t)m * n + 2 * 16 * mx * mx + 6 * 8 * mx +
          sizeof(KeptIdx) * mx + 12 * 8192 + tail +
-         std::max(heig_scratch_bound((int64_t)mx, (int64_t)mx), small_eig) + (size_t)(4 << 20);
+         std::max(heig_scratch_bound((int64_t)mx, (int64_t)mx), heig_blocks_scratch((int64_t)mx, (int64_t)mx)) +
+         (size_t)(4 << 20);
 }
 
 namespace {
@@ -359,55 +381,11 @@ struct Blk {
 // eps |M|; U_t <- U_t W (V_t <- V_t W) and X_t <- W^H X_t (Y_t <- Y_t W) rotate the
 // candidates within the tail subspace, keeping them orthonormal, and the projection norms
 // are taken again.
-// Blocks of up to 256 rows are reduced either together, one CTA (one SM) each, or one by
-// one by the cooperative kernel across the GPU.  On one SM a block costs about
-// 1.3e-9 n^3 s (its 4 n^3 FP64 FMAs at two per clock, plus per-column overhead); across
-// the GPU about 15 us per column, plus 6.4e-12 n^3 s of FP64 work and 0.5 ms for its own
-// eigenvalue, vector and back-transformation launches.  The batch takes as long as its
-// largest block, or its total over the SMs.  The largest blocks move to the cooperative
-// path while that shortens the estimate: a lone 256-row block (the tail of a truncated
-// SVD whose spectrum falls fast) takes about 4 ms there against about 20 ms on one SM.
-std::vector<char> route_coop(const std::vector<int64_t>& ns, int nsm) {
-  auto t_cta = [](double n) { return 1.3e-9 * n * n * n; };
-  auto t_coop = [](double n) { return 15e-6 * n + 6.4e-12 * n * n * n + 5e-4; };
-  std::vector<int> ord(ns.size());
-  for (size_t i = 0; i < ns.size(); ++i) ord[i] = (int)i;
-  std::sort(ord.begin(), ord.end(), [&](int a, int b) { return ns[(size_t)a] > ns[(size_t)b]; });
-  auto batch = [&](size_t from) {  // the one-CTA batch over ord[from..]
-    double mx = 0, sum = 0;
-    for (size_t i = from; i < ord.size(); ++i) {
-      const double t = t_cta((double)ns[(size_t)ord[i]]);
-      mx = std::max(mx, t);
-      sum += t;
-    }
-    return std::max(mx, sum / std::max(1, nsm));
-  };
-  double best = batch(0), acc = 0;
-  size_t moved = 0;
-  for (size_t i = 0; i < ord.size(); ++i) {
-    acc += t_coop((double)ns[(size_t)ord[i]]);
-    const double cand = acc + batch(i + 1);
-    if (cand < best) {
-      best = cand;
-      moved = i + 1;
-    }
-  }
-  std::vector<char> coop(ns.size(), 0);
-  for (size_t i = 0; i < moved; ++i) coop[(size_t)ord[i]] = 1;
-  return coop;
-}
-
-int sm_count(Ctx* c) {
-  int nsm = 0;
-  if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) nsm = 1;
-  return nsm;
-}
-
 constexpr double TAIL_REL = 1e-4;
 
 struct TailBlk {
   int b;
-  int64_t t0, t, toff;
+  int64_t t0, t, toff, poff;  // poff: the block's part of the rotation buffer
 };
 
 int refine_tails(Ctx* c, int side, const std::vector<Blk>& bl, z* Vp, z* Xp,
@@ -426,11 +404,11 @@ int refine_tails(Ctx* c, int side, const std::vector<Blk>& bl, z* Vp, z* Xp,
     while (t0 > 0 && !(hs[(size_t)(vbase + t0 - 1)] >= TAIL_REL * mx)) --t0;
     const int64_t t = B.k - t0;
     if (t >= 2 && mx > 0) {
-      tb.push_back(TailBlk{b, t0, t, gt});
+      tb.push_back(TailBlk{b, t0, t, gt, tmpmax});
       gt += t * t;
       const int64_t rows_x = (side == TNT_SVD_LEFT) ? t : B.mq;
       const int64_t cols_x = (side == TNT_SVD_LEFT) ? B.nq : t;
-      tmpmax = std::max(tmpmax, std::max(B.g * t, rows_x * cols_x));
+      tmpmax += std::max(B.g * t, rows_x * cols_x);
     }
     vbase += B.k;
   }
@@ -444,75 +422,80 @@ int refine_tails(Ctx* c, int side, const std::vector<Blk>& bl, z* Vp, z* Xp,
     c->ws.top = top;
     return set_err(c, TNT_E_ALLOC, "scratch exhausted (SVD tail pass)");
   }
+  auto product = [](int64_t M, int64_t N, int64_t K) {
+    GemmTask g{};
+    g.g.batch = 1;
+    g.g.alpha = zmk(1, 0);
+    g.g.M = M; g.g.N = N; g.g.K = K;
+    return g;
+  };
   // tail Gram matrices
+  std::vector<GemmTask> gs;
   for (const TailBlk& T : tb) {
     const Blk& B = bl[(size_t)T.b];
-    ZGemm g{};
-    g.batch = 1;
-    g.alpha = zmk(1, 0);
-    g.beta = zmk(0, 0);
-    g.M = T.t; g.N = T.t;
-    g.C = H + T.toff; g.c_rs = T.t;
+    GemmTask g = product(T.t, T.t, side == TNT_SVD_LEFT ? B.nq : B.mq);
+    g.herm = 1;
+    g.g.C = H + T.toff; g.g.c_rs = T.t;
     if (side == TNT_SVD_LEFT) {  // H = X_t X_t^H, X_t rows t0.. of X_q (ld n_q)
       const z* Xt = Xp + B.xoff + T.t0 * B.nq;
-      g.K = B.nq;
-      g.A = Xt; g.a_rs = B.nq; g.a_cs = 1;
-      g.B = Xt; g.b_rs = 1; g.b_cs = B.nq; g.conj_b = 1;
+      g.g.A = Xt; g.g.a_rs = B.nq; g.g.a_cs = 1;
+      g.g.B = Xt; g.g.b_rs = 1; g.g.b_cs = B.nq; g.g.conj_b = 1;
     } else {  // H = Y_t^H Y_t, Y_t columns t0.. of Y_q (ld k)
       const z* Yt = Xp + B.xoff + T.t0;
-      g.K = B.mq;
-      g.A = Yt; g.a_rs = 1; g.a_cs = B.k; g.conj_a = 1;
-      g.B = Yt; g.b_rs = B.k; g.b_cs = 1;
+      g.g.A = Yt; g.g.a_rs = 1; g.g.a_cs = B.k; g.g.conj_a = 1;
+      g.g.B = Yt; g.g.b_rs = B.k; g.g.b_cs = 1;
     }
-    TNT_TRY(zgemm(c, g));
+    gs.push_back(g);
   }
+  TNT_TRY(zgemm_tasks(c, gs));
   // eigenvectors of every tail Gram matrix (all of them, descending)
   {
-    std::vector<int64_t> ns;
-    for (const TailBlk& T : tb) ns.push_back(T.t <= 256 ? T.t : 0);
-    const std::vector<char> coop = route_coop(ns, sm_count(c));
-    std::vector<SmallEig> small;
-    for (size_t i = 0; i < tb.size(); ++i)
-      if (tb[i].t <= 256 && !coop[i]) small.push_back(SmallEig{tb[i].toff, tb[i].t, tb[i].t});
-    TNT_TRY(heig_small_blocks(c, H, small, W, ev));
-    for (size_t i = 0; i < tb.size(); ++i) {
-      const TailBlk& T = tb[i];
-      if (T.t > 256 || coop[i]) TNT_TRY(heig_top(c, H + T.toff, T.t, T.t, W + T.toff, T.t, ev));
-    }
+    std::vector<SmallEig> eig;
+    for (const TailBlk& T : tb) eig.push_back(SmallEig{T.toff, T.t, T.t});
+    TNT_TRY(heig_blocks(c, H, eig, W, ev));
   }
-  // rotate the tail candidates within their subspace
-  for (const TailBlk& T : tb) {
-    const Blk& B = bl[(size_t)T.b];
-    z* Wt = W + T.toff;
-    {  // eigenvectors: U_t (or V_t), g x t at column t0 of the block (ld g) <- U_t W
-      ZGemm g{};
-      g.batch = 1; g.alpha = zmk(1, 0); g.beta = zmk(0, 0);
-      g.M = B.g; g.N = T.t; g.K = T.t;
-      g.A = Vp + B.goff + T.t0; g.a_rs = B.g; g.a_cs = 1;
-      g.B = Wt; g.b_rs = T.t; g.b_cs = 1;
-      g.C = tmp; g.c_rs = T.t;
-      TNT_TRY(zgemm(c, g));
-      k_copy_strided<<<gridn(B.g * T.t), 256, 0, st>>>(tmp, B.g, T.t, T.t, Vp + B.goff + T.t0, B.g);
-      c->launches++;
+  // rotate the tail candidates within their subspace: first the eigenvectors, U_t (or V_t),
+  // g x t at column t0 of the block (ld g) <- U_t W; then X_t <- W^H X_t (rows), or
+  // Y_t <- Y_t W (columns)
+  for (int which = 0; which < 2; ++which) {
+    gs.clear();
+    for (const TailBlk& T : tb) {
+      const Blk& B = bl[(size_t)T.b];
+      z* Wt = W + T.toff;
+      GemmTask g{};
+      if (which == 0) {
+        g = product(B.g, T.t, T.t);
+        g.g.A = Vp + B.goff + T.t0; g.g.a_rs = B.g; g.g.a_cs = 1;
+        g.g.B = Wt; g.g.b_rs = T.t; g.g.b_cs = 1;
+        g.g.C = tmp + T.poff; g.g.c_rs = T.t;
+      } else if (side == TNT_SVD_LEFT) {
+        z* Xt = Xp + B.xoff + T.t0 * B.nq;
+        g = product(T.t, B.nq, T.t);
+        g.g.A = Wt; g.g.a_rs = 1; g.g.a_cs = T.t; g.g.conj_a = 1;
+        g.g.B = Xt; g.g.b_rs = B.nq; g.g.b_cs = 1;
+        g.g.C = tmp + T.poff; g.g.c_rs = B.nq;
+      } else {
+        z* Yt = Xp + B.xoff + T.t0;
+        g = product(B.mq, T.t, T.t);
+        g.g.A = Yt; g.g.a_rs = B.k; g.g.a_cs = 1;
+        g.g.B = Wt; g.g.b_rs = T.t; g.g.b_cs = 1;
+        g.g.C = tmp + T.poff; g.g.c_rs = T.t;
+      }
+      gs.push_back(g);
     }
-    ZGemm g{};
-    g.batch = 1; g.alpha = zmk(1, 0); g.beta = zmk(0, 0);
-    if (side == TNT_SVD_LEFT) {  // X_t <- W^H X_t  (t x n_q, contiguous rows)
-      z* Xt = Xp + B.xoff + T.t0 * B.nq;
-      g.M = T.t; g.N = B.nq; g.K = T.t;
-      g.A = Wt; g.a_rs = 1; g.a_cs = T.t; g.conj_a = 1;
-      g.B = Xt; g.b_rs = B.nq; g.b_cs = 1;
-      g.C = tmp; g.c_rs = B.nq;
-      TNT_TRY(zgemm(c, g));
-      TNT_CUDA_TRY(c, cudaMemcpyAsync(Xt, tmp, sizeof(z) * T.t * B.nq, cudaMemcpyDeviceToDevice, st));
-    } else {  // Y_t <- Y_t W  (m_q x t at column t0, ld k)
-      z* Yt = Xp + B.xoff + T.t0;
-      g.M = B.mq; g.N = T.t; g.K = T.t;
-      g.A = Yt; g.a_rs = B.k; g.a_cs = 1;
-      g.B = Wt; g.b_rs = T.t; g.b_cs = 1;
-      g.C = tmp; g.c_rs = T.t;
-      TNT_TRY(zgemm(c, g));
-      k_copy_strided<<<gridn(B.mq * T.t), 256, 0, st>>>(tmp, B.mq, T.t, T.t, Yt, B.k);
+    TNT_TRY(zgemm_tasks(c, gs));
+    for (size_t i0 = 0; i0 < tb.size(); i0 += COPY_MAX) {
+      CopyTasks ct;
+      ct.n = (int)std::min<size_t>(COPY_MAX, tb.size() - i0);
+      for (int i = 0; i < ct.n; ++i) {
+        const TailBlk& T = tb[i0 + (size_t)i];
+        const Blk& B = bl[(size_t)T.b];
+        if (which == 0) ct.t[i] = CopyTask{tmp + T.poff, Vp + B.goff + T.t0, T.t, B.g, (int)B.g, (int)T.t};
+        else if (side == TNT_SVD_LEFT)
+          ct.t[i] = CopyTask{tmp + T.poff, Xp + B.xoff + T.t0 * B.nq, B.nq, B.nq, (int)T.t, (int)B.nq};
+        else ct.t[i] = CopyTask{tmp + T.poff, Xp + B.xoff + T.t0, T.t, B.k, (int)B.mq, (int)T.t};
+      }
+      k_copy_tasks<<<dim3(64, (unsigned)ct.n), 256, 0, st>>>(ct);
       c->launches++;
     }
   }
@@ -616,36 +599,38 @@ int svd_trunc_impl(Ctx* c, const z* M, int64_t m, int64_t n, const int64_t* h_rq
   // ---- scratch
   int P2 = 1;
   while (P2 < ntot_vals) P2 <<= 1;
+  // host tables first, one after the other: they go up in one copy
+  const size_t tab_top = c->ws.top;
   int64_t* d_rows = (int64_t*)ws_alloc(c, ws_round(sizeof(int64_t) * rows_all.size()));
   int64_t* d_cols = (int64_t*)ws_alloc(c, ws_round(sizeof(int64_t) * cols_all.size()));
+  CandBlock* d_cb = (CandBlock*)ws_alloc(c, ws_round(sizeof(CandBlock) * nb));
+  GatherBlk* d_gb = (GatherBlk*)ws_alloc(c, ws_round(sizeof(GatherBlk) * nb));
+  int* d_blk = (int*)ws_alloc(c, ws_round(sizeof(double) * ntot_vals));
+  int* d_loc = (int*)ws_alloc(c, ws_round(sizeof(double) * ntot_vals));
+  int64_t* d_boff = (int64_t*)ws_alloc(c, ws_round(sizeof(int64_t) * 2 * nb));
+  const size_t tab_bytes = c->ws.top - tab_top;
+  char* const tab = (char*)d_rows;
   z* Mp = (z*)ws_alloc(c, ws_round(sizeof(z) * mtot));
   z* Gp = (z*)ws_alloc(c, ws_round(sizeof(z) * gtot));
   z* Vp = (z*)ws_alloc(c, ws_round(sizeof(z) * gtot));
   z* Xp = (z*)ws_alloc(c, ws_round(sizeof(z) * xtot));
   double* d_sig = (double*)ws_alloc(c, ws_round(sizeof(double) * ntot_vals));
-  int* d_blk = (int*)ws_alloc(c, ws_round(sizeof(double) * ntot_vals));
-  int* d_loc = (int*)ws_alloc(c, ws_round(sizeof(double) * ntot_vals));
   double* d_sig_s = (double*)ws_alloc(c, ws_round(sizeof(double) * ntot_vals));
   int* d_blk_s = (int*)ws_alloc(c, ws_round(sizeof(double) * ntot_vals));
   int* d_loc_s = (int*)ws_alloc(c, ws_round(sizeof(double) * ntot_vals));
   SelOut* d_sel = (SelOut*)ws_alloc(c, ws_round(sizeof(SelOut)));
-  CandBlock* d_cb = (CandBlock*)ws_alloc(c, ws_round(sizeof(CandBlock) * nb));
-  int64_t* d_goff = (int64_t*)ws_alloc(c, ws_round(sizeof(int64_t) * nb));
-  int* d_gdim = (int*)ws_alloc(c, ws_round(sizeof(int64_t) * nb));
   double* d_ev = (double*)ws_alloc(c, ws_round(sizeof(double) * 8192));
   double* d_tot = (double*)ws_alloc(c, ws_round(sizeof(double)));
   double* d_unscale = (double*)ws_alloc(c, ws_round(sizeof(double) * nb));
   unsigned* d_mexp = (unsigned*)ws_alloc(c, ws_round(sizeof(unsigned) * nb));
-  int64_t* d_boff = (int64_t*)ws_alloc(c, ws_round(sizeof(int64_t) * 2 * nb));
-  if (!d_unscale || !d_mexp || !d_boff) return set_err(c, TNT_E_ALLOC, "scratch exhausted (svd)");
+  if (!d_unscale || !d_mexp || !d_boff || !d_gb) return set_err(c, TNT_E_ALLOC, "scratch exhausted (svd)");
   if (!d_rows || !d_cols || !Mp || !Gp || !Vp || !Xp || !d_sig || !d_blk || !d_loc || !d_sig_s ||
-      !d_blk_s || !d_loc_s || !d_sel || !d_cb || !d_goff || !d_gdim || !d_ev || !d_tot)
+      !d_blk_s || !d_loc_s || !d_sel || !d_cb || !d_ev || !d_tot)
     return set_err(c, TNT_E_ALLOC, "scratch exhausted (svd)");
 
   // ---- host tables -> device (one synchronous upload of small integer tables)
   std::vector<CandBlock> hcb(nb);
-  std::vector<int64_t> hgoff(nb);
-  std::vector<int> hgdim(nb), hblk(ntot_vals), hloc(ntot_vals);
+  std::vector<int> hblk(ntot_vals), hloc(ntot_vals);
   std::vector<int64_t> hboff(2 * (size_t)nb);
   {
     int v = 0;
@@ -656,8 +641,6 @@ int svd_trunc_impl(Ctx* c, const z* M, int64_t m, int64_t n, const int64_t* h_rq
       hcb[b].r = (int)bl[b].k;
       hcb[b].vbase = v;
       hcb[b].by_row = (side == TNT_SVD_LEFT);
-      hgoff[b] = bl[b].goff;
-      hgdim[b] = (int)bl[b].g;
       hboff[b] = bl[b].moff;
       hboff[nb + b] = bl[b].mq * bl[b].nq;
       for (int k = 0; k < bl[b].k; ++k, ++v) {
@@ -667,19 +650,30 @@ int svd_trunc_impl(Ctx* c, const z* M, int64_t m, int64_t n, const int64_t* h_rq
     }
   }
   cudaStream_t st = c->stream;
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(d_rows, rows_all.data(), sizeof(int64_t) * rows_all.size(), cudaMemcpyHostToDevice, st));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(d_cols, cols_all.data(), sizeof(int64_t) * cols_all.size(), cudaMemcpyHostToDevice, st));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(d_cb, hcb.data(), sizeof(CandBlock) * nb, cudaMemcpyHostToDevice, st));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(d_goff, hgoff.data(), sizeof(int64_t) * nb, cudaMemcpyHostToDevice, st));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(d_gdim, hgdim.data(), sizeof(int) * nb, cudaMemcpyHostToDevice, st));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(d_blk, hblk.data(), sizeof(int) * ntot_vals, cudaMemcpyHostToDevice, st));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(d_loc, hloc.data(), sizeof(int) * ntot_vals, cudaMemcpyHostToDevice, st));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(d_boff, hboff.data(), sizeof(int64_t) * 2 * nb, cudaMemcpyHostToDevice, st));
+  std::vector<GatherBlk> hgb((size_t)nb);
+  for (int b = 0; b < nb; ++b) hgb[(size_t)b] = GatherBlk{bl[b].moff, bl[b].roff, bl[b].coff, bl[b].mq, bl[b].nq};
+  {
+    std::vector<char> host(tab_bytes, 0);
+    auto put = [&](const void* dev, const void* src, size_t bytes) {
+      memcpy(host.data() + ((const char*)dev - tab), src, bytes);
+    };
+    put(d_rows, rows_all.data(), sizeof(int64_t) * rows_all.size());
+    put(d_cols, cols_all.data(), sizeof(int64_t) * cols_all.size());
+    put(d_cb, hcb.data(), sizeof(CandBlock) * nb);
+    put(d_gb, hgb.data(), sizeof(GatherBlk) * nb);
+    put(d_blk, hblk.data(), sizeof(int) * ntot_vals);
+    put(d_loc, hloc.data(), sizeof(int) * ntot_vals);
+    put(d_boff, hboff.data(), sizeof(int64_t) * 2 * nb);
+    TNT_CUDA_TRY(c, cudaMemcpyAsync(tab, host.data(), tab_bytes, cudaMemcpyHostToDevice, st));
+  }
 
   // ---- gather blocks, |M|_F^2 (unscaled), scale each block, Gram matrices
-  for (int b = 0; b < nb; ++b) {
-    const Blk& B = bl[b];
-    TNT_TRY(gather2d(c, M, n, d_rows + B.roff, B.mq, d_cols + B.coff, B.nq, Mp + B.moff, B.nq, 0));
+  {
+    int64_t mxcnt = 1;
+    for (int b = 0; b < nb; ++b) mxcnt = std::max<int64_t>(mxcnt, bl[b].mq * bl[b].nq);
+    k_gather_blocks<<<dim3((unsigned)std::min<int64_t>((mxcnt + 255) / 256, 256), (unsigned)nb), 256, 0, st>>>(
+        M, n, d_gb, d_rows, d_cols, Mp);
+    c->launches++;
   }
   TNT_TRY(vec_norm2(c, Mp, mtot, d_tot));
   {
@@ -692,12 +686,14 @@ int svd_trunc_impl(Ctx* c, const z* M, int64_t m, int64_t n, const int64_t* h_rq
     c->launches += 2;
   }
   TNT_CHECK_LAUNCH(c);
+  std::vector<GemmTask> prods;
+  std::vector<SmallEig> eig;
   for (int b = 0; b < nb; ++b) {
     const Blk& B = bl[b];
-    ZGemm g{};
+    GemmTask t{};
+    ZGemm& g = t.g;
     g.batch = 1;
     g.alpha = zmk(1, 0);
-    g.beta = zmk(0, 0);
     g.C = Gp + B.goff;
     g.c_rs = B.g;
     if (side == TNT_SVD_LEFT) {  // G = M M^H
@@ -709,35 +705,22 @@ int svd_trunc_impl(Ctx* c, const z* M, int64_t m, int64_t n, const int64_t* h_rq
       g.A = Mp + B.moff; g.a_rs = 1; g.a_cs = B.nq; g.conj_a = 1;
       g.B = Mp + B.moff; g.b_rs = B.nq; g.b_cs = 1;
     }
-    g.lower_only = 1;  // G is Hermitian: form the lower tiles, mirror the rest
-    TNT_TRY(zgemm(c, g));
-    TNT_TRY(herm_mirror(c, Gp + B.goff, B.g));
+    t.herm = 1;
+    prods.push_back(t);
+    eig.push_back(SmallEig{B.goff, B.g, B.k});
+    if (B.g > 8192) return set_err(c, TNT_E_UNSUPPORTED, "SVD block of dim %lld > 8192", (long long)B.g);
   }
-  // ---- eigensolves: blocks up to 256 rows reduced together (one CTA each, one launch),
-  // larger ones, and small ones that would hold the batch back (route_coop), one by one
-  // across the whole GPU
-  {
-    std::vector<int64_t> ns;
-    for (int b = 0; b < nb; ++b) ns.push_back(bl[b].g <= 256 ? bl[b].g : 0);
-    const std::vector<char> coop = route_coop(ns, sm_count(c));
-    std::vector<SmallEig> small;
-    for (int b = 0; b < nb; ++b)
-      if (bl[b].g <= 256 && !coop[(size_t)b]) small.push_back(SmallEig{bl[b].goff, bl[b].g, bl[b].k});
-    TNT_TRY(heig_small_blocks(c, Gp, small, Vp, d_ev));
-    for (int b = 0; b < nb; ++b) {
-      if (bl[b].g <= 256 && !coop[(size_t)b]) continue;
-      const Blk& B = bl[b];
-      if (B.g > 8192) return set_err(c, TNT_E_UNSUPPORTED, "SVD block of dim %lld > 8192", (long long)B.g);
-      TNT_TRY(heig_top(c, Gp + B.goff, B.g, B.k, Vp + B.goff, B.g, d_ev));
-    }
-  }
+  TNT_TRY(zgemm_tasks(c, prods));
+  // ---- eigensolves of all blocks together
+  TNT_TRY(heig_blocks(c, Gp, eig, Vp, d_ev));
   // ---- candidate products and their norms
+  prods.clear();
   for (int b = 0; b < nb; ++b) {
     const Blk& B = bl[b];
-    ZGemm g{};
+    GemmTask t{};
+    ZGemm& g = t.g;
     g.batch = 1;
     g.alpha = zmk(1, 0);
-    g.beta = zmk(0, 0);
     if (side == TNT_SVD_LEFT) {  // X_q = U_q[:, :k]^H M_q  (k x n_q)
       g.M = B.k; g.N = B.nq; g.K = B.mq;
       g.A = Vp + B.goff; g.a_rs = 1; g.a_cs = B.g; g.conj_a = 1;
@@ -749,8 +732,9 @@ int svd_trunc_impl(Ctx* c, const z* M, int64_t m, int64_t n, const int64_t* h_rq
       g.B = Vp + B.goff; g.b_rs = B.g; g.b_cs = 1;
       g.C = Xp + B.xoff; g.c_rs = B.k;
     }
-    TNT_TRY(zgemm(c, g));
+    prods.push_back(t);
   }
+  TNT_TRY(zgemm_tasks(c, prods));
   {
     int64_t rmax = 1;
     for (int b = 0; b < nb; ++b) rmax = std::max<int64_t>(rmax, bl[b].k);
@@ -776,11 +760,17 @@ int svd_trunc_impl(Ctx* c, const z* M, int64_t m, int64_t n, const int64_t* h_rq
   SelOut sel;
   std::vector<double> hs(ntot_vals);
   std::vector<int> hb(ntot_vals), hl(ntot_vals);
+  int h_status = 0;
+  TNT_CUDA_TRY(c, cudaMemcpyAsync(&h_status, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
   TNT_CUDA_TRY(c, cudaMemcpyAsync(&sel, d_sel, sizeof(SelOut), cudaMemcpyDeviceToHost, st));
   TNT_CUDA_TRY(c, cudaMemcpyAsync(hs.data(), d_sig_s, sizeof(double) * ntot_vals, cudaMemcpyDeviceToHost, st));
   TNT_CUDA_TRY(c, cudaMemcpyAsync(hb.data(), d_blk_s, sizeof(int) * ntot_vals, cudaMemcpyDeviceToHost, st));
   TNT_CUDA_TRY(c, cudaMemcpyAsync(hl.data(), d_loc_s, sizeof(int) * ntot_vals, cudaMemcpyDeviceToHost, st));
   TNT_CUDA_TRY(c, cudaStreamSynchronize(st));
+  if (h_status & 2) {
+    cudaMemsetAsync(c->d_status, 0, sizeof(int), st);
+    return set_err(c, TNT_E_TIMEOUT, "tridiagonal reduction: a grid barrier wait expired");
+  }
   const int64_t chi = sel.chi;
   if (chi < 1 || chi > ntot_vals) return set_err(c, TNT_E_NAN, "SVD selection returned chi = %lld of %lld", (long long)chi, (long long)ntot_vals);
   for (int64_t k = 0; k < ntot_vals; ++k)  // report the block of a non-finite value first

@@ -158,6 +158,15 @@ int zgemm(Ctx* c, const ZGemm& g);
 // large products with alpha = 1, beta = 0, batch = 1 there when the context allows it
 bool ozgemm_eligible(const Ctx* c, const ZGemm& g);
 int ozgemm(Ctx* c, const ZGemm& g);
+// One of a set of independent products run in grouped launches: herm, the result is
+// Hermitian (its lower triangle is computed and mirrored); sub, C -= A B instead of C = A B
+struct GemmTask {
+  ZGemm g;
+  int herm, sub;
+};
+int zgemm_tasks(Ctx* c, const std::vector<GemmTask>& tasks);
+// the same on the FP64 units alone
+int zgemm_fma_tasks(Ctx* c, const GemmTask* const* tasks, int n);
 // FP64 FMA GEMMs only while the guard lives (paths that must not allocate)
 struct OzOff {
   Ctx* c;
@@ -240,17 +249,17 @@ int tridiag_lowest_batched(Ctx* c, const double* d_alpha, const double* d_beta, 
 // U: n x k with leading dimension ldu; ev: device, k values.
 size_t heig_scratch_bound(int64_t n, int64_t k);
 int heig_top(Ctx* c, z* G, int64_t n, int64_t k, z* U, int64_t ldu, double* ev);
-// Many small blocks (n <= 256) at once, one CTA per block for the reduction.  A block of
-// heig_small_blocks: offset of its n x n Gram block (and of its eigenvector columns,
-// leading dimension n), its size and the number of eigenvectors wanted
+// Many blocks at once, every stage one launch (or a few) over all of them: offset of a block's
+// n x n Gram matrix (and of its eigenvector columns, leading dimension n), its size and
+// the number of eigenvectors wanted
 struct SmallEig {
   int64_t goff, n, k;
 };
-int heig_small_blocks(Ctx* c, z* G, const std::vector<SmallEig>& blocks, z* U, double* ev);
+int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& blocks, z* U, double* ev);
+// scratch of heig_blocks for blocks whose sizes sum to n (and eigenvectors to k)
+size_t heig_blocks_scratch(int64_t n, int64_t k);
 
-// Helpers: gather / scatter / conversion
-int gather2d(Ctx* c, const z* src, int64_t src_ld, const int64_t* d_rows, int64_t nr,
-             const int64_t* d_cols, int64_t nc, z* dst, int64_t dst_ld, int conj_t);
+// Helpers: fill and scale
 int zfill(Ctx* c, z* p, int64_t n, z v);
 int zscale_inplace(Ctx* c, z* p, int64_t n, const double* d_scale, int mode);
 
