@@ -649,6 +649,36 @@ U1Plan::~U1Plan() {
   }
 }
 
+namespace {
+constexpr double U1_OZ_MIN_FLOPS = 1.2e8;
+
+// the FP64 products of stage 1 (T1 = L theta, B offsets from the input vector) or stage 4
+// (Y = T3 R^T), with the plan's buffers (null while the layout is being made)
+std::vector<GemmTask> oz_stage(const U1Plan& p, int stage) {
+  std::vector<GemmTask> out;
+  const std::vector<TaskDesc>& ts = stage == 1 ? p.s1 : p.s4;
+  for (size_t i = 0; i < ts.size(); ++i) {
+    const TaskDesc& t = ts[i];
+    GemmTask g{};
+    g.g.batch = 1;
+    g.g.alpha = zmk(1, 0);
+    g.g.M = t.M; g.g.N = t.N; g.g.K = t.K;
+    if (stage == 1) {
+      g.g.A = p.A1z + t.a_row0 * p.KA1; g.g.a_rs = p.KA1; g.g.a_cs = 1;
+      g.g.B = (const z*)nullptr + p.slabs[i].src; g.g.b_rs = t.N; g.g.b_cs = 1;
+      g.g.C = p.T1z + t.c_off;
+    } else {
+      g.g.A = p.A4z + t.a_row0 * p.KA4; g.g.a_rs = p.KA4; g.g.a_cs = 1;
+      g.g.B = p.B4z + t.b_row0 * p.KA4; g.g.b_rs = 1; g.g.b_cs = p.KA4;
+      g.g.C = p.Yz + t.c_off;
+    }
+    g.g.c_rs = t.ldc;
+    out.push_back(g);
+  }
+  return out;
+}
+}  // namespace
+
 int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
   p->nprob = (int)probs.size();
   p->n = 0;
@@ -889,6 +919,16 @@ int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
   b += ws_round(sizeof(int4) * (t1 + t4 + z1 + z4)) + ws_round(sizeof(GTask) * (p->s1.size() + p->s4.size())) +
        ws_round(sizeof(ZTask) * (p->s1.size() + p->s4.size()));
   p->bytes = b + (size_t)(1 << 20);
+  // FP64 stages as slice products: eight launches of about 50 us in all, against the FP64
+  // units' 1 TFLOP/s (32 chains at chi = 256, d = 5: 13 GFLOP, 28 ms)
+  int64_t k1 = 0;
+  for (const TaskDesc& t : p->s1) k1 = std::max(k1, t.K);
+  p->oz = c && c->oz_mode != 0 && p->flops >= U1_OZ_MIN_FLOPS && k1 <= 512;
+  if (p->oz) {
+    const size_t o1 = oz_plan_bytes(c, oz_stage(*p, 1)), o4 = oz_plan_bytes(c, oz_stage(*p, 4));
+    if (o1 && o4) p->bytes += o1 + o4 + (size_t)(1 << 16);
+    else p->oz = false;
+  }
   return TNT_OK;
 }
 
@@ -956,7 +996,7 @@ constexpr double TUNE_MIN_FLOPS = 2e9;  // below this a matvec is launch-bound: 
 
 int autotune(Ctx* c, U1Plan* p) {
   auto it = c->tune.find(p->sig);
-  if (it != c->tune.end()) return set_tiles(c, p, it->second[0], it->second[1], it->second[2]);
+  if (it != c->tune.end() && !it->second.empty()) return set_tiles(c, p, it->second[0], it->second[1], it->second[2]);
   if (p->flops < TUNE_MIN_FLOPS) {
     c->tune[p->sig] = std::vector<int>{128, 128, 1};
     return set_tiles(c, p, 128, 128, 1);
@@ -986,6 +1026,7 @@ int autotune(Ctx* c, U1Plan* p) {
 
 int u1_prepare(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
   (void)probs;
+  c->tune.emplace(p->sig, std::vector<int>());  // known; its tiles are chosen when first needed
   const size_t f = sizeof(float);
   auto fa = [&](size_t n) { return (float*)ws_alloc(c, ws_round(f * std::max<size_t>(n, 1))); };
   auto za = [&](size_t n) { return (z*)ws_alloc(c, ws_round(sizeof(z) * std::max<size_t>(n, 1))); };
@@ -1004,18 +1045,12 @@ int u1_prepare(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
       !p->A4z || !p->B4z || !p->Yz)
     return set_err(c, TNT_E_ALLOC, "scratch exhausted (grouped matvec buffers)");
   // zero padding (K columns beyond a task's K, and the T3 entries no pair writes)
-  TNT_CUDA_TRY(c, cudaMemsetAsync(p->A1p, 0, 4 * f * p->rowsA1 * p->KA1, c->stream));
-  TNT_CUDA_TRY(c, cudaMemsetAsync(p->B1p, 0, 4 * f * p->rowsB1 * p->KA1, c->stream));
-  TNT_CUDA_TRY(c, cudaMemsetAsync(p->A4p, 0, 4 * f * p->rowsA4 * p->KA4, c->stream));
-  TNT_CUDA_TRY(c, cudaMemsetAsync(p->B4p, 0, 4 * f * p->rowsB4 * p->KA4, c->stream));
-  TNT_CUDA_TRY(c, cudaMemsetAsync(p->Yf, 0, 8 * f * p->P4, c->stream));
   TNT_CUDA_TRY(c, cudaMemsetAsync(p->A1z, 0, sizeof(z) * p->rowsA1 * p->KA1, c->stream));
   TNT_CUDA_TRY(c, cudaMemsetAsync(p->A4z, 0, sizeof(z) * p->rowsA4 * p->KA4, c->stream));
   TNT_CUDA_TRY(c, cudaMemsetAsync(p->B4z, 0, sizeof(z) * p->rowsB4 * p->KA4, c->stream));
   // tables
-  PackSeg *dA1 = nullptr, *dB4 = nullptr;
-  TNT_TRY(upload(c, &dA1, p->segA1));
-  TNT_TRY(upload(c, &dB4, p->segB4));
+  TNT_TRY(upload(c, &p->d_segA1, p->segA1));
+  TNT_TRY(upload(c, &p->d_segB4, p->segB4));
   TNT_TRY(upload(c, &p->d_slabs, p->slabs));
   TNT_TRY(upload(c, &p->d_ttiles, p->ttiles));
   TNT_TRY(upload(c, &p->d_pairs, p->pairs));
@@ -1056,24 +1091,53 @@ int u1_prepare(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
   TNT_TRY(upload(c, &p->d_g4, none, p->s4.size()));
   TNT_TRY(upload(c, &p->d_g1tiles, none4, (size_t)p->cap_g1tiles));
   TNT_TRY(upload(c, &p->d_g4tiles, none4, (size_t)p->cap_g4tiles));
-  // constant operands: environments into split planes and FP64 packs
+  // constant operands: environments into FP64 packs (pageable tables are staged by the copies)
   const int nA = (int)p->segA1.size(), nB = (int)p->segB4.size();
-  const int64_t plA = p->rowsA1 * p->KA1, plB = p->rowsB4 * p->KA4;
-  k_pack_segs<true><<<cap_grid((nA + 7) / 8, 152 * 8), 256, 0, c->stream>>>(dA1, nA, p->A1p, plA, nullptr);
-  k_pack_segs<false><<<cap_grid((nA + 7) / 8, 152 * 8), 256, 0, c->stream>>>(dA1, nA, nullptr, 0, p->A1z);
-  k_pack_segs<true><<<cap_grid((nB + 7) / 8, 152 * 8), 256, 0, c->stream>>>(dB4, nB, p->B4p, plB, nullptr);
-  k_pack_segs<false><<<cap_grid((nB + 7) / 8, 152 * 8), 256, 0, c->stream>>>(dB4, nB, nullptr, 0, p->B4z);
-  c->launches += 4;
+  k_pack_segs<false><<<cap_grid((nA + 7) / 8, 152 * 8), 256, 0, c->stream>>>(p->d_segA1, nA, nullptr, 0, p->A1z);
+  k_pack_segs<false><<<cap_grid((nB + 7) / 8, 152 * 8), 256, 0, c->stream>>>(p->d_segB4, nB, nullptr, 0, p->B4z);
+  c->launches += 2;
   TNT_CHECK_LAUNCH(c);
-  TNT_TRY(tma_map_planes(c, &p->tmA1, p->A1p, p->rowsA1, p->KA1, 128));
-  TNT_TRY(tma_map_planes(c, &p->tmA4, p->A4p, p->rowsA4, p->KA4, 128));
-  TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  TNT_TRY(autotune(c, p));
+  if (p->oz) {
+    TNT_TRY(oz_plan_build(c, oz_stage(*p, 1), 1, &p->oz1));
+    TNT_TRY(oz_plan_build(c, oz_stage(*p, 4), 2, &p->oz4));
+  }
   // arguments of the nodes whose pointers change per matvec
   p->in_tp = TPArgs{nullptr, p->d_slabs, p->d_ttiles, p->n_ttiles, p->B1p, p->KA1, p->rowsB1 * p->KA1};
   p->in_zg = ZGArgs{p->d_z1, p->d_z1tiles, p->n_z1tiles, p->A1z, nullptr, p->T1z};
   p->out_g[0] = GthArgs{p->d_rows, p->n_rows, nullptr, 0, 0, 0, p->Yz, nullptr};
+  return TNT_OK;
+}
+
+// split-TF32 operands and tiles, at the first split-TF32 matvec of the plan
+static int u1_prepare_mixed(Ctx* c, U1Plan* p) {
+  const size_t f = sizeof(float);
+  TNT_CUDA_TRY(c, cudaMemsetAsync(p->A1p, 0, 4 * f * p->rowsA1 * p->KA1, c->stream));
+  TNT_CUDA_TRY(c, cudaMemsetAsync(p->B1p, 0, 4 * f * p->rowsB1 * p->KA1, c->stream));
+  TNT_CUDA_TRY(c, cudaMemsetAsync(p->A4p, 0, 4 * f * p->rowsA4 * p->KA4, c->stream));
+  TNT_CUDA_TRY(c, cudaMemsetAsync(p->B4p, 0, 4 * f * p->rowsB4 * p->KA4, c->stream));
+  TNT_CUDA_TRY(c, cudaMemsetAsync(p->Yf, 0, 8 * f * p->P4, c->stream));
+  const int nA = (int)p->segA1.size(), nB = (int)p->segB4.size();
+  const int64_t plA = p->rowsA1 * p->KA1, plB = p->rowsB4 * p->KA4;
+  k_pack_segs<true><<<cap_grid((nA + 7) / 8, 152 * 8), 256, 0, c->stream>>>(p->d_segA1, nA, p->A1p, plA, nullptr);
+  k_pack_segs<true><<<cap_grid((nB + 7) / 8, 152 * 8), 256, 0, c->stream>>>(p->d_segB4, nB, p->B4p, plB, nullptr);
+  c->launches += 2;
+  TNT_CHECK_LAUNCH(c);
+  TNT_TRY(tma_map_planes(c, &p->tmA1, p->A1p, p->rowsA1, p->KA1, 128));
+  TNT_TRY(tma_map_planes(c, &p->tmA4, p->A4p, p->rowsA4, p->KA4, 128));
+  TNT_TRY(autotune(c, p));
   p->out_g[1] = GthArgs{p->d_rows, p->n_rows, p->Yf, p->P4, 2 * p->P4, p->split4, nullptr, nullptr};
+  p->mixed_ready = true;
+  return TNT_OK;
+}
+
+int u1_tune(Ctx* c, const std::vector<U1Spec>& probs) {
+  Scope sc(c);
+  U1Plan p;
+  TNT_TRY(u1_layout(c, probs, &p));
+  TNT_TRY(ws_reserve(c, p.bytes));
+  TNT_TRY(u1_prepare(c, probs, &p));
+  TNT_TRY(u1_prepare_mixed(c, &p));
+  TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   return TNT_OK;
 }
 
@@ -1136,15 +1200,30 @@ int build_graph(Ctx* c, U1Plan& p, int mixed) {
     TNT_TRY(add(knp((void*)k_gather_u1<true>, gg, 256, 0, a4)));
     p.out_node[1] = node;
   } else {
-    ZGArgs z1 = p.in_zg;
-    void* a0[] = {&z1};
-    TNT_TRY(add(knp(zfn(p), cap_grid(p.n_z1tiles, zcap(p)), 256, 0, a0)));
-    p.in_node[0] = node;
+    ZGArgs z1 = p.in_zg, z4{p.d_z4, p.d_z4tiles, p.n_z4tiles, p.A4z, p.B4z, p.Yz};
+    alignas(16) unsigned char oa[sizeof(p.oz1.args)];
+    void* ao[] = {oa};
+    if (p.oz) {
+      oz_plan_args(p.oz1, nullptr, oa);
+      for (int i = 0; i < 4; ++i) {
+        const OzNode& q = p.oz1.node[i];
+        TNT_TRY(add(knp(q.fn, q.grid, q.block, q.smem, ao)));
+        if (i < 2) p.oz_node[i] = node;
+      }
+    } else {
+      void* a0[] = {&z1};
+      TNT_TRY(add(knp(zfn(p), cap_grid(p.n_z1tiles, zcap(p)), 256, 0, a0)));
+      p.in_node[0] = node;
+    }
     void* a1[] = {&wa};
     TNT_TRY(add(knp((void*)k_wop<false>, gw, 256, 0, a1)));
-    ZGArgs z4{p.d_z4, p.d_z4tiles, p.n_z4tiles, p.A4z, p.B4z, p.Yz};
-    void* a2[] = {&z4};
-    TNT_TRY(add(knp(zfn(p), cap_grid(p.n_z4tiles, zcap(p)), 256, 0, a2)));
+    if (p.oz) {
+      oz_plan_args(p.oz4, nullptr, oa);
+      for (const OzNode& q : p.oz4.node) TNT_TRY(add(knp(q.fn, q.grid, q.block, q.smem, ao)));
+    } else {
+      void* a2[] = {&z4};
+      TNT_TRY(add(knp(zfn(p), cap_grid(p.n_z4tiles, zcap(p)), 256, 0, a2)));
+    }
     GthArgs ga = p.out_g[0];
     void* a3[] = {&ga};
     TNT_TRY(add(knp((void*)k_gather_u1<false>, gg, 256, 0, a3)));
@@ -1158,8 +1237,6 @@ int run_direct(Ctx* c, U1Plan& p, const z* x, z* y, int mixed) {
   WArgs wa = wargs(p);
   const unsigned gw = cap_grid(p.n_wtiles, 152 * 8);
   const unsigned gg = cap_grid((p.n_rows + 7) / 8, 152 * 8);
-  const double wflops = 8.0 * 0;  // counted within the plan's total
-  (void)wflops;
   if (mixed) {
     TPArgs tp = p.in_tp;
     tp.x = x;
@@ -1200,23 +1277,31 @@ int run_direct(Ctx* c, U1Plan& p, const z* x, z* y, int mixed) {
     for (const TaskDesc& t : p.s4) f4 += 8.0 * t.M * t.N * t.K;
     ZGArgs z1 = p.in_zg;
     z1.B = x;
-    {
+    if (p.oz) {
+      ProfScope ps(c, "oz_gemm", f1);
+      TNT_TRY(oz_plan_run(c, p.oz1, x));
+    } else {
       ProfScope ps(c, "zgemm_grouped", f1);
       zlaunch(c, p, z1, p.n_z1tiles);
+      c->launches++;
     }
     {
       ProfScope ps(c, "u1_wop_f64", 16.0 * (double)p.P1 + 16.0 * (double)(p.rowsA4 * p.KA4));
       k_wop<false><<<gw, 256, 0, c->stream>>>(wa);
     }
     ZGArgs z4{p.d_z4, p.d_z4tiles, p.n_z4tiles, p.A4z, p.B4z, p.Yz};
-    {
+    if (p.oz) {
+      ProfScope ps(c, "oz_gemm", f4);
+      TNT_TRY(oz_plan_run(c, p.oz4, nullptr));
+    } else {
       ProfScope ps(c, "zgemm_grouped", f4);
       zlaunch(c, p, z4, p.n_z4tiles);
+      c->launches++;
     }
     GthArgs ga = p.out_g[0];
     ga.y = y;
     k_gather_u1<false><<<gg, 256, 0, c->stream>>>(ga);
-    c->launches += 4;
+    c->launches += 2;
     TNT_CHECK_LAUNCH(c);
   }
   return TNT_OK;
@@ -1225,7 +1310,9 @@ int run_direct(Ctx* c, U1Plan& p, const z* x, z* y, int mixed) {
 
 int u1_run(Ctx* c, U1Plan& p, const z* x, z* y, int precision) {
   const int mixed = (precision == TNT_PREC_MIXED) ? 1 : 0;
-  if (!c->use_graphs || !c->prof_cls.empty()) return run_direct(c, p, x, y, mixed);
+  if (mixed && !p.mixed_ready) TNT_TRY(u1_prepare_mixed(c, &p));
+  // a plan used once needs no graph (its instantiation costs more than the launches it saves)
+  if (!c->use_graphs || !c->prof_cls.empty() || p.runs[mixed]++ == 0) return run_direct(c, p, x, y, mixed);
   if (!p.exec[mixed]) TNT_TRY(build_graph(c, p, mixed));
   if (mixed) {
     TPArgs tp = p.in_tp;
@@ -1240,11 +1327,23 @@ int u1_run(Ctx* c, U1Plan& p, const z* x, z* y, int precision) {
     TNT_CUDA_TRY(c, cudaGraphExecKernelNodeSetParams(p.exec[1], p.out_node[1], &k2));
     c->launches += 5;
   } else {
-    ZGArgs z1 = p.in_zg;
-    z1.B = x;
-    void* a[] = {&z1};
-    cudaKernelNodeParams k = knp(zfn(p), cap_grid(p.n_z1tiles, zcap(p)), 256, 0, a);
-    TNT_CUDA_TRY(c, cudaGraphExecKernelNodeSetParams(p.exec[0], p.in_node[0], &k));
+    if (p.oz) {
+      alignas(16) unsigned char oa[sizeof(p.oz1.args)];
+      oz_plan_args(p.oz1, x, oa);
+      void* a[] = {oa};
+      for (int i = 0; i < 2; ++i) {
+        const OzNode& q = p.oz1.node[i];
+        cudaKernelNodeParams k = knp(q.fn, q.grid, q.block, q.smem, a);
+        TNT_CUDA_TRY(c, cudaGraphExecKernelNodeSetParams(p.exec[0], p.oz_node[i], &k));
+      }
+      c->launches += 6;
+    } else {
+      ZGArgs z1 = p.in_zg;
+      z1.B = x;
+      void* a[] = {&z1};
+      cudaKernelNodeParams k = knp(zfn(p), cap_grid(p.n_z1tiles, zcap(p)), 256, 0, a);
+      TNT_CUDA_TRY(c, cudaGraphExecKernelNodeSetParams(p.exec[0], p.in_node[0], &k));
+    }
     GthArgs ga = p.out_g[0];
     ga.y = y;
     void* b[] = {&ga};

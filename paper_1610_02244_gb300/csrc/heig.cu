@@ -19,6 +19,7 @@
 #include <cmath>
 
 #include "heff_plan.cuh"
+#include "f32conv.cuh"
 
 namespace tnt {
 
@@ -30,6 +31,8 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;
 }
+
+__device__ __forceinline__ int hi_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 
 // x -= a conj(b) as four FMAs (the FP64 pipe is the bottleneck of these kernels on GB300)
 __device__ __forceinline__ void zsub_mul_conj(z& x, z a, z b) {
@@ -366,28 +369,31 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tridiag_persistent(TriArgs a) {
 // one CTA needs none, and keeps p in shared memory.
 // Reflector j is v_j = (1, conj(x_c) s_j for c > j+1) with x row j of the updated matrix
 // and s_j its scale; p_j = tau_j T_j v_j is formed without v_j as
-// tau_j (T(g, j+1) + s_j sum_{c > j+1} T(g, c) conj(x_c)), so that the reflector's
-// scalars are computed by a warp of their own (TRI_WARPS, a square root and two divisions:
-// about 100 FP64 instructions in sequence, 3 us) while the others update the rows.
+// tau_j (T(g, j+1) + s_j sum_{c > j+1} T(g, c) conj(x_c)), so that the reflector's scalars are
+// computed by a warp of their own (TRI_WARPS) while the others update the rows.
+// K_j = v_j^H T_j v_j is real, and with it w_j = p_j + c_j v_j, c_j = -|tau_j|^2 K_j / 2, and the
+// next source row x'(c) = T_j(j+1, c) - conj(p_j(c)) - (p_j(j+1) + 2 c_j) conj(v_j(c)).
 // Entering column j every CTA holds x (in sx, the entry j+1 zeroed), tau_j and s_j, and p_j
-// with the per-CTA partial sums of p_j^H v_j is in global memory:
-//   the scalar warp: cf = -(tau_j / 2) p_j^H v_j; the others: v_j(c), and loads of p_j and
-//     row j+1;
-//   one pass over the columns c > j: w_j(c) = p_j(c) + cf v_j(c), and
-//     x'(c) = T_j(j+1, c) - conj(w_j(c)) - w_j(j+1) conj(v_j(c)), row j+1 after the
-//     update (v_j(j+1) = 1), into sx, with the sum of |x'(c)|^2 over c > j+2;
+// with the per-CTA parts of K_j is in global memory:
+//   the scalar warp: c_j from the parts; the others: v_j(c), and x'(c) but for its c_j term;
+//   x' (into sx) and w_j, with the sum of |x'(c)|^2 over c > j+2;
 //   the scalar warp: reflector j+1; the others, the CTA's rows g > j+1 of T_j, flattened over
 //     (row, column) and split evenly over the warps: T <- T - v_j w_j^H - w_j v_j^H and
 //     sum_c T(g, c) conj(x'(c)); the owner of row j+2 also stores it in global memory;
-//   warp 0: p_{j+1}(g) for the CTA's rows and its share of p_{j+1}^H v_{j+1};
+//   warp 0: p_{j+1}(g) for the CTA's rows and its part of K_{j+1};
 //   group barrier.
 // Reflector j replaces row j of the block in global memory (columns 0 .. n-j-2), the layout
 // the back-transformation reads: no CTA reads row j after its barrier j.
 // Vectors are indexed by row of the block.  Per column a CTA spends 16 FP64 operations per
-// trailing entry on the shared vectors and 12 per entry of its rows.
+// trailing entry on the shared vectors and 12 per entry of its rows: that work bounds large
+// blocks (two operations per SM and clock); small ones are bound by the sequence of about 60
+// dependent FP64 instructions at 100 to 200 clocks each, the barrier and the loads.  The
+// barrier is one release-add and an acquire-poll of a counter (an atomic with its old value, a
+// generation word and a timer read per poll took 9000 to 13000 clocks); square root and
+// reciprocal are Newton steps from FP32 seeds (library calls: 5000 clocks).
 // Before, blocks of up to 256 rows were reduced on one SM each (a 200-row block: 3.8 ms,
 // the FP64 pipe of one SM) and larger ones one after the other across the GPU (500 rows
-// 4.5 ms, 1024 rows 24.4 ms with the scalars between two barriers of the CTA).
+// 4.5 ms, 1024 rows 24.4 ms).
 static_assert(TRI_WARPS == 16, "the flattened row split divides by 16 with shifts");
 constexpr int TRI_VEC = 3;              // vector entries per thread
 constexpr int64_t TRI_ROWS_NMAX = 1216; // <= TRI_VEC * TRI_THREADS; (8 + 3) n entries fit
@@ -401,49 +407,72 @@ struct TriBlk {
   double* d;
   double* e;
   z* p;          // 2 x n: p of even / odd columns
-  z* part;       // 2 x nb partial sums of p^H v
+  double* part;  // 2 x nb parts of v^H T v
   int n, c0, nb; // CTAs [c0, c0 + nb)
 };
 struct TriGroup {
   int nblk;
-  unsigned* bar;   // 32 words per block: arrivals, generation
-  int* abort_flag;
+  unsigned* bar;   // 32 words per block: arrivals (zero before the launch)
   int* status;
   TriBlk b[TRI_MAXB];
 };
 
-// false: a wait expired here or elsewhere, the CTA must stop
-__device__ bool group_barrier(const TriGroup& t, int grp, int nb) {
+// Barrier j of a group of nb CTAs: each adds one to the group's counter (release: its threads'
+// stores before the CTA barrier are visible to whoever sees the sum) and waits until all
+// have.  false: the wait expired, the CTA must stop (and so will the others of its group).
+__device__ bool group_barrier(const TriGroup& t, int grp, int nb, int j) {
   __shared__ int s_ok;
   __syncthreads();
   if (nb == 1) return true;
   if (threadIdx.x == 0) {
     unsigned* bar = t.bar + 32 * grp;
-    volatile unsigned* gen = bar + 1;
-    const unsigned g = *gen;
-    __threadfence();
+    const unsigned want = (unsigned)nb * (unsigned)(j + 1);
+    unsigned seen;
     int ok = 1;
-    if (atomicAdd(bar, 1u) == (unsigned)nb - 1u) {
-      bar[0] = 0;
-      __threadfence();
-      atomicAdd(bar + 1, 1u);
-    } else {
-      const uint64_t t0 = gtime();
-      while (*gen == g) {
-        if (*(volatile int*)t.abort_flag) break;
-        if (gtime() - t0 > 2000000000ull) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(bar), "r"(1u) : "memory");
+    uint64_t t0 = 0;
+    for (unsigned polls = 0;; ++polls) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+      if (seen >= want) break;
+      if ((polls & 1023u) == 1023u) {
+        const uint64_t now = gtime();
+        if (!t0) t0 = now;
+        if (now - t0 > 2000000000ull) {
           atomicOr(t.status, 2);
-          atomicExch(t.abort_flag, 1);
+          ok = 0;
           break;
         }
       }
     }
-    __threadfence();
-    if (*(volatile int*)t.abort_flag) ok = 0;
     s_ok = ok;
   }
   __syncthreads();
   return s_ok != 0;
+}
+
+// 1 / sqrt(s) and 1 / d for normal positive s, d != 0: an FP32 seed (relative error e0 of about
+// 2^-22), one step of third order, y (1 + e/2 + 3/8 e^2) with e = 1 - s y^2, and
+// r (1 + e + e^2) with e = 1 - d r: the error left is of order e0^3, below FP64 rounding.
+// The arguments are scaled to [1, 4) and [1, 2) by exponent arithmetic.
+__device__ __forceinline__ double rsqrt_newton(double s) {
+  const int hi = __double2hiint(s), ex = (hi >> 20) - 1023, h = ex >> 1;
+  const double m = __hiloint2double((hi & 0xfffff) | ((1023 + (ex & 1)) << 20), __double2loint(s));
+  float y0;
+  asm("rsqrt.approx.f32 %0, %1;" : "=f"(y0) : "f"(f32_of(m)));
+  const double y = f64_of(y0);
+  const double e = fma(-m * y, y, 1.0);
+  const double r = fma(y, e * fma(e, 0.375, 0.5), y);
+  return __hiloint2double(__double2hiint(r) - (h << 20), __double2loint(r));
+}
+__device__ __forceinline__ double rcp_newton(double d) {
+  const int hi = __double2hiint(d), ex = ((hi >> 20) & 0x7ff) - 1023;
+  const double m = __hiloint2double((hi & 0x800fffff) | (1023 << 20), __double2loint(d));
+  float r0;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r0) : "f"(f32_of(m)));
+  const double r = f64_of(r0);
+  const double e = fma(-m, r, 1.0);
+  const double q = fma(r, fma(e, e, e), r);
+  return __hiloint2double(__double2hiint(q) - (ex << 20), __double2loint(q));
 }
 
 // (a, b) summed over the warp with five FP64 adds (the two sums share each step); every
@@ -457,40 +486,70 @@ __device__ __forceinline__ void warp_sum_pair(double& a, double& b) {
   b = __shfl_sync(0xffffffffu, v, 16);
 }
 
+// four values summed over the warp with seven FP64 adds: lane l returns the total of s[l & 3]
+__device__ __forceinline__ double warp_sum4(double* s) {
+  const int l = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 2; o >= 1; o >>= 1) {
+    const bool up = (l & o) != 0;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const double give = up ? s[i] : s[i + o], keep = up ? s[i + o] : s[i];
+      s[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  double r = s[0];
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  return r;
+}
+
+struct GroupRefl {
+  z tau, scale;
+  double beta, c;  // c = -|tau|^2 / 2
+};
 struct RowsShared {
-  double br[TRI_WARPS][2], bi[TRI_WARPS][2];  // few rows: per warp and row segment, sum T conj(x)
-  z q0[TRI_RMAX], q1[TRI_RMAX];               // many rows: per row, from its start / its second warp
-  double nrm[TRI_WARPS];                      // per warp: sum |x|^2
-  Refl rf[2];                                 // reflectors of even / odd columns
-  z cf, alpha, part;
+  double b4[TRI_WARPS][4];       // few rows: per warp, sum T conj(x) of its two row segments
+  z q0[TRI_RMAX], q1[TRI_RMAX];  // many rows: per row, from its start / its second warp
+  double nrm[TRI_WARPS];         // per warp: sum |x|^2
+  GroupRefl rf[2];               // reflectors of even / odd columns
+  z alpha;
+  double cf, part;
 };
 
-// Reflector parameters by one warp (refl_params with the two divisions side by side)
-__device__ Refl refl_warp(z alpha, double xn2, bool empty) {
-  Refl R;
-  if (empty || (xn2 == 0.0 && alpha.y == 0.0)) {
-    R.tau = zmk(0, 0);
-    R.beta = alpha.x;
-    R.scale = zmk(0, 0);
-    return R;
+// Reflector parameters (refl_params) by one warp
+__device__ GroupRefl refl_warp(z alpha, double xn2, bool empty) {
+  GroupRefl R;
+  R.tau = R.scale = zmk(0, 0);
+  R.beta = alpha.x;
+  R.c = 0;
+  if (empty || (xn2 == 0.0 && alpha.y == 0.0)) return R;
+  const double s = fma(alpha.x, alpha.x, fma(alpha.y, alpha.y, xn2));
+  double nrm, inv;
+  if (hi_exp(s) > 100 && hi_exp(s) < 1946) {  // squares well inside the normal range
+    inv = rsqrt_newton(s);
+    nrm = s * inv;
+  } else {
+    nrm = sqrt(s);
+    inv = 1.0 / nrm;
   }
-  const double nrm = sqrt(fma(alpha.x, alpha.x, fma(alpha.y, alpha.y, xn2)));
   R.beta = alpha.x >= 0 ? -nrm : nrm;
-  const z den = zmk(alpha.x - R.beta, alpha.y);  // scale = 1 / (alpha - beta)
+  const z den = zmk(alpha.x - R.beta, alpha.y);  // scale = 1 / (alpha - beta), |den| >= nrm
   const double dd = fma(den.x, den.x, den.y * den.y);
-  const double r = 1.0 / ((threadIdx.x & 1) ? dd : R.beta);
-  const double rb = __shfl_sync(0xffffffffu, r, 0), rd = __shfl_sync(0xffffffffu, r, 1);
-  R.tau = zmk(-den.x * rb, -alpha.y * rb);
+  const double rd = hi_exp(dd) > 100 && hi_exp(dd) < 1946 ? rcp_newton(dd) : 1.0 / dd;
+  const double rb = alpha.x >= 0 ? inv : -inv;  // -1 / beta
+  R.tau = zmk(den.x * rb, alpha.y * rb);
   R.scale = zmk(den.x * rd, -den.y * rd);
+  R.c = -0.5 * fma(R.tau.x, R.tau.x, R.tau.y * R.tau.y);
   return R;
 }
 
 // one segment of a row: T(g, c) -= v(g) conj(w(c)) + w(g) conj(v(c)) (with UPD; also to gout)
-// for c0 <= c < c1, and the sum of T(g, c) conj(x(c)); every lane returns it
+// for c0 <= c < c1, and the lane's sum of T(g, c) conj(x(c)) to sr, si
 template <bool UPD>
-__device__ __forceinline__ z row_segment(z* rw, int c0, int c1, z vr, z wr, const z* v, const z* w, const z* x,
-                                         z* gout) {
-  double sr = 0, si = 0;
+__device__ __forceinline__ void row_segment(z* rw, int c0, int c1, z vr, z wr, const z* v, const z* w, const z* x,
+                                            z* gout, double& sr, double& si) {
+  sr = si = 0;
 #pragma unroll 2
   for (int c = c0 + (threadIdx.x & 31); c < c1; c += 32) {
     z t = rw[c];
@@ -504,14 +563,17 @@ __device__ __forceinline__ z row_segment(z* rw, int c0, int c1, z vr, z wr, cons
     sr = fma(t.x, y.x, fma(t.y, y.y, sr));
     si = fma(t.y, y.x, fma(-t.x, y.y, si));
   }
-  warp_sum_pair(sr, si);
-  return zmk(sr, si);
 }
 
-// Rows g >= lo of this CTA (rows[i] = row b + nb i, R of them) over the 16 row warps: warp w
-// covers [f0, f1) of the flattened (row, column) range, f0 = ract L w / 16, and starts in row
-// floor(ract w / 16) (exact: floor(floor(x) / L) = floor(x / L)).  Fewer than 16 rows: a warp
-// meets at most two rows, a row several warps.  16 and more: a row meets at most two warps.
+// The row warps a column's work is split over, as a power of two: at least 64 entries each
+// (their sums are added one after the other afterwards, at 150 to 200 clocks an addition).
+__device__ __forceinline__ int row_warps_log2(unsigned total) {
+  return total >= 1024u ? 4 : total >= 512u ? 3 : total >= 256u ? 2 : total >= 128u ? 1 : 0;
+}
+// Rows g >= lo of this CTA (rows[i] = row b + nb i, R of them) over W = 2^s row warps: warp w
+// covers [f0, f1) of the flattened (row, column) range, f0 = ract L w / W, and starts in row
+// floor(ract w / W) (exact: floor(floor(x) / L) = floor(x / L)).  Fewer than W rows: a warp
+// meets at most two rows, a row several warps.  W and more: a row meets at most two warps.
 template <bool UPD>
 __device__ void rows_update(z* rows, int R, int b, int nb, int n, int lo, const z* v, const z* w, const z* x,
                             z* grow, RowsShared& S) {
@@ -519,24 +581,26 @@ __device__ void rows_update(z* rows, int R, int b, int nb, int n, int lo, const 
   const int i0 = (lo > b) ? (lo - b + nb - 1) / nb : 0;
   const int ract = R - i0 > 0 ? R - i0 : 0;
   const unsigned L = (unsigned)(n - lo), total = (unsigned)ract * L;
-  const unsigned f0 = (total * (unsigned)warp) >> 4, f1 = (total * (unsigned)(warp + 1)) >> 4;
-  const int r0 = (ract * warp) >> 4;
-  if (ract < 16) {
+  const int ws = row_warps_log2(total);
+  if (warp >> ws) return;
+  const unsigned f0 = (total * (unsigned)warp) >> ws, f1 = (total * (unsigned)(warp + 1)) >> ws;
+  const int r0 = (ract * warp) >> ws;
+  if (ract < (1 << ws)) {
+    double s4[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int seg = 0; seg < 2; ++seg) {
       const int ri = r0 + seg;  // row of this segment
       const int s0 = (seg == 0) ? (int)f0 - ri * (int)L : 0;
       const int s1 = min((int)L, (int)f1 - ri * (int)L);
-      z s = zmk(0, 0);
       if (ri < ract && s0 < s1) {
         const int i = i0 + ri, g = b + nb * i;
-        s = row_segment<UPD>(rows + (int64_t)i * n, lo + s0, lo + s1, UPD ? v[g] : zmk(0, 0), UPD ? w[g] : zmk(0, 0),
-                             v, w, x, (UPD && g == lo) ? grow : nullptr);
+        row_segment<UPD>(rows + (int64_t)i * n, lo + s0, lo + s1, UPD ? v[g] : zmk(0, 0), UPD ? w[g] : zmk(0, 0), v,
+                         w, x, (UPD && g == lo) ? grow : nullptr, s4[2 * seg], s4[2 * seg + 1]);
       }
-      if (lane == 0) {
-        S.br[warp][seg] = s.x;
-        S.bi[warp][seg] = s.y;
-      }
+    }
+    if (f0 < f1) {
+      const double s = warp_sum4(s4);
+      if (lane < 4) S.b4[warp][lane] = s;
     }
     return;
   }
@@ -544,60 +608,71 @@ __device__ void rows_update(z* rows, int R, int b, int nb, int n, int lo, const 
     const int s0 = max(0, (int)f0 - ri * (int)L), s1 = min((int)L, (int)f1 - ri * (int)L);
     if (s0 >= s1) continue;
     const int i = i0 + ri, g = b + nb * i;
-    const z s = row_segment<UPD>(rows + (int64_t)i * n, lo + s0, lo + s1, UPD ? v[g] : zmk(0, 0),
-                                 UPD ? w[g] : zmk(0, 0), v, w, x, (UPD && g == lo) ? grow : nullptr);
+    double sr, si;
+    row_segment<UPD>(rows + (int64_t)i * n, lo + s0, lo + s1, UPD ? v[g] : zmk(0, 0), UPD ? w[g] : zmk(0, 0), v, w, x,
+                     (UPD && g == lo) ? grow : nullptr, sr, si);
+    warp_sum_pair(sr, si);
     if (lane == 0) {
-      if (s0 == 0) S.q0[ri] = s;
-      else S.q1[ri] = s;
+      if (s0 == 0) S.q0[ri] = zmk(sr, si);
+      else S.q1[ri] = zmk(sr, si);
     }
   }
 }
 
 // Warp 0 after rows_update, with reflector rf of the column whose trailing block starts at lo:
-// p(g) = tau (T(g, lo) + s sum) for the CTA's rows g >= lo into pout, the CTA's sum of
-// conj(p(g)) v(g) into *partout (v(lo) = 1, v(c) = conj(x(c)) s).
-__device__ void rows_finish(const z* rows, int R, int b, int nb, int n, int lo, const z* x, const Refl& rf, z* pout,
-                            z* partout, RowsShared& S) {
+// q = T(g, lo) + s sum and p(g) = tau q for the CTA's rows g >= lo into pout, the CTA's part
+// of v^H T v, the sum of Re(conj(v(g)) q) (v(lo) = 1, v(c) = conj(x(c)) s), into *partout.
+__device__ void rows_finish(const z* rows, int R, int b, int nb, int n, int lo, const z* x, const GroupRefl& rf,
+                            z* pout, double* partout, RowsShared& S) {
   const int lane = threadIdx.x & 31;
   const int i0 = (lo > b) ? (lo - b + nb - 1) / nb : 0;
   const int ract = R - i0 > 0 ? R - i0 : 0;
   const unsigned L = (unsigned)(n - lo), total = (unsigned)ract * L;
-  double pr = 0, pi = 0;
+  const int ws = row_warps_log2(total);
+  double part = 0;
   for (int r = lane; r < ract; r += 32) {
+    const int g = b + nb * (i0 + r);
+    const z t0 = rows[(int64_t)(i0 + r) * n + lo];
+    const z vg = (g == lo) ? zmk(1, 0) : zmul(zconj(x[g]), rf.scale);
     double sr = 0, si = 0;
-    if (ract < 16) {
-      for (int w = 0; w < TRI_WARPS; ++w) {  // the warps whose range meets row r, in order
-        const unsigned f0 = (total * (unsigned)w) >> 4, f1 = (total * (unsigned)(w + 1)) >> 4;
-        const int r0 = (ract * w) >> 4;
+    if (ract < (1 << ws)) {
+      for (int w = 0; w < (1 << ws); ++w) {  // the warps whose range meets row r, in order
+        const unsigned f0 = (total * (unsigned)w) >> ws, f1 = (total * (unsigned)(w + 1)) >> ws;
+        const int r0 = (ract * w) >> ws;
         if (f0 < f1 && r0 == r) {
-          sr += S.br[w][0];
-          si += S.bi[w][0];
+          sr += S.b4[w][0];
+          si += S.b4[w][1];
         } else if (f0 < f1 && r0 + 1 == r && f1 > (unsigned)r * L) {
-          sr += S.br[w][1];
-          si += S.bi[w][1];
+          sr += S.b4[w][2];
+          si += S.b4[w][3];
         }
       }
     } else {
       sr = S.q0[r].x;
       si = S.q0[r].y;
       // the first warp boundary after the row's start, if it falls inside the row
-      const unsigned rl = (unsigned)r * L, w = (16u * (rl + 1u) + total - 1u) / total;
-      if (w < 16u && ((total * w) >> 4) < rl + L) {
+      const unsigned rl = (unsigned)r * L, w = (((rl + 1u) << ws) + total - 1u) / total;
+      if (w < (1u << ws) && ((total * w) >> ws) < rl + L) {
         sr += S.q1[r].x;
         si += S.q1[r].y;
       }
     }
-    const int g = b + nb * (i0 + r);
-    const z t0 = rows[(int64_t)(i0 + r) * n + lo];
-    const z q = zmk(t0.x + rf.scale.x * sr - rf.scale.y * si, t0.y + rf.scale.x * si + rf.scale.y * sr);
-    const z pv = zmul(rf.tau, q);
-    pout[g] = pv;
-    const z vg = (g == lo) ? zmk(1, 0) : zmul(zconj(x[g]), rf.scale);
-    pr = fma(pv.x, vg.x, fma(pv.y, vg.y, pr));
-    pi = fma(pv.x, vg.y, fma(-pv.y, vg.x, pi));
+    const z q = zmk(fma(rf.scale.x, sr, fma(-rf.scale.y, si, t0.x)), fma(rf.scale.x, si, fma(rf.scale.y, sr, t0.y)));
+    pout[g] = zmul(rf.tau, q);
+    part = fma(vg.x, q.x, fma(vg.y, q.y, part));
   }
-  warp_sum_pair(pr, pi);
-  if (lane == 0) *partout = zmk(pr, pi);
+  for (int o = ract > 16 ? 16 : ract > 8 ? 8 : ract > 4 ? 4 : ract > 2 ? 2 : ract > 1 ? 1 : 0; o > 0; o >>= 1)
+    part += __shfl_xor_sync(0xffffffffu, part, o);
+  if (lane == 0) *partout = part;
+}
+
+// the 16 row warps' sums of |x|^2, in every lane of the scalar warp
+__device__ __forceinline__ double nrm_total(const RowsShared& S) {
+  const int lane = threadIdx.x & 31;
+  double nr = S.nrm[lane & 15];
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
+  return nr;
 }
 
 __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_constant__ TriGroup T) {
@@ -639,11 +714,7 @@ __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_
     }
     __syncthreads();
     if (scalar) {
-      double nr = lane < TRI_WARPS ? S.nrm[lane] : 0.0;
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
-      nr = __shfl_sync(0xffffffffu, nr, 0);
-      const Refl rf = refl_warp(n > 1 ? S.alpha : zmk(0, 0), nr, n < 2);
+      const GroupRefl rf = refl_warp(n > 1 ? S.alpha : zmk(0, 0), nrm_total(S), n < 2);
       if (lane == 0) {
         S.rf[0] = rf;
         if (b == 0) {
@@ -659,66 +730,61 @@ __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_
     if (warp == 0) rows_finish(rows, R, b, nb, n, 1, sx, S.rf[0], one ? sp : a.p, one ? &S.part : a.part + b, S);
   }
   for (int j = 0; j + 1 < n; ++j) {
-    if (!group_barrier(T, grp, nb)) return;
-    const Refl rf = S.rf[j & 1];  // reflector j
+    if (!group_barrier(T, grp, nb, j)) return;
     const z* pj = one ? sp : a.p + (j & 1) * n;
     z* pn = one ? sp : a.p + ((j + 1) & 1) * n;
-    const z* partj = one ? &S.part : a.part + (j & 1) * nb;
-    z* partn = one ? &S.part : a.part + ((j + 1) & 1) * nb;
+    const double* partj = one ? &S.part : a.part + (j & 1) * nb;
+    double* partn = one ? &S.part : a.part + ((j + 1) & 1) * nb + b;
     const z* grow = one ? rows + (int64_t)(j + 1) * n : a.G + (int64_t)(j + 1) * n;
-    z pc[TRI_VEC], rc[TRI_VEC], vc[TRI_VEC];
-    z p1 = zmk(0, 0);
-    if (scalar) {  // the group's partial sums, by 32 lanes at once
-      double sa = 0, sb = 0;
-      for (int q = lane; q < nb; q += 32) {
-        const z pq = one ? partj[q] : __ldcg(partj + q);
-        sa += pq.x;
-        sb += pq.y;
+    z pc[TRI_VEC], tc[TRI_VEC], vc[TRI_VEC];
+    if (scalar) {  // c_j: the group's parts of K, by 32 lanes at once
+      double s[5], k = 0;
+#pragma unroll
+      for (int i = 0; i < 5; ++i) {
+        const int q = lane + 32 * i;
+        s[i] = q < nb ? (one ? partj[q] : __ldcg(partj + q)) : 0.0;
       }
-      warp_sum_pair(sa, sb);
-      if (lane == 0) {
-        const z ts = zmul(rf.tau, zmk(sa, sb));
-        S.cf = zmk(-0.5 * ts.x, -0.5 * ts.y);
-      }
+      k = ((s[0] + s[1]) + (s[2] + s[3])) + s[4];
+      for (int q = lane + 160; q < nb; q += 32) k += __ldcg(partj + q);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+      if (lane == 0) S.cf = S.rf[j & 1].c * k;
     } else {
+      const z scale = S.rf[j & 1].scale;
+      const z p1 = one ? pj[j + 1] : __ldcg(pj + j + 1);
 #pragma unroll
       for (int k = 0; k < TRI_VEC; ++k) {
         const int c = j + 1 + tid + k * TRI_THREADS;
-        pc[k] = rc[k] = zmk(0, 0);
         if (c < n) {
           pc[k] = one ? pj[c] : __ldcg(pj + c);
-          rc[k] = one ? grow[c] : __ldcg(grow + c);
+          tc[k] = one ? grow[c] : __ldcg(grow + c);
         }
       }
-      p1 = one ? pj[j + 1] : __ldcg(pj + j + 1);
 #pragma unroll
       for (int k = 0; k < TRI_VEC; ++k) {  // v_j, written out for the back-transformation
         const int c = j + 1 + tid + k * TRI_THREADS;
         if (c < n) {
-          vc[k] = (c == j + 1) ? zmk(1, 0) : zmul(zconj(sx[c]), rf.scale);
+          vc[k] = (c == j + 1) ? zmk(1, 0) : zmul(zconj(sx[c]), scale);
           sv[c] = vc[k];
           if (b == 0) a.G[(int64_t)j * n + (c - j - 1)] = vc[k];
+          tc[k].x -= pc[k].x;  // T(j+1, c) - conj(p(c)) - p(j+1) conj(v(c))
+          tc[k].y += pc[k].y;
+          zsub_mul_conj(tc[k], p1, vc[k]);
         }
       }
     }
     __syncthreads();
-    double d1 = 0;
     if (!scalar) {
-      const z cf = S.cf;
-      const z w1 = zmk(p1.x + cf.x, p1.y + cf.y);  // w_j(j+1), as v_j(j+1) = 1
+      const double cf = S.cf, cf2 = 2.0 * cf;
       double acc = 0;
 #pragma unroll
       for (int k = 0; k < TRI_VEC; ++k) {
         const int c = j + 1 + tid + k * TRI_THREADS;
         if (c < n) {
-          const z vv = vc[k];
-          const z wv = zmk(fma(cf.x, vv.x, fma(-cf.y, vv.y, pc[k].x)),
-                           fma(cf.x, vv.y, fma(cf.y, vv.x, pc[k].y)));
-          sw[c] = wv;
-          z xn = zmk(rc[k].x - wv.x, rc[k].y + wv.y);
-          zsub_mul_conj(xn, w1, vv);
+          const z xn = zmk(fma(-cf2, vc[k].x, tc[k].x), fma(cf2, vc[k].y, tc[k].y));
+          sw[c] = zmk(fma(cf, vc[k].x, pc[k].x), fma(cf, vc[k].y, pc[k].y));
           if (c == j + 1) {
-            d1 = xn.x;
+            if (b == 0) a.d[j + 1] = xn.x;
           } else if (c == j + 2) {
             S.alpha = zconj(xn);
             sx[c] = zmk(0, 0);
@@ -728,30 +794,25 @@ __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_
           }
         }
       }
-      acc = warp_sum_d(acc);
+      if (j + 1 + 32 * warp < n) acc = warp_sum_d(acc);
       if (lane == 0) S.nrm[warp] = acc;
-      if (b == 0 && tid == 0) a.d[j + 1] = d1;  // thread 0 holds column j+1
     }
     __syncthreads();
     const bool empty = n - j - 2 <= 0;  // length of reflector j+1
     if (scalar) {
-      double nr = lane < TRI_WARPS ? S.nrm[lane] : 0.0;
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
-      nr = __shfl_sync(0xffffffffu, nr, 0);
-      const Refl r2 = refl_warp(empty ? zmk(0, 0) : S.alpha, nr, empty);
+      const GroupRefl rf = refl_warp(empty ? zmk(0, 0) : S.alpha, nrm_total(S), empty);
       if (lane == 0) {
-        S.rf[(j + 1) & 1] = r2;
+        S.rf[(j + 1) & 1] = rf;
         if (b == 0) {
-          a.tau[j + 1] = r2.tau;
-          if (!empty) a.e[j + 1] = r2.beta;
+          a.tau[j + 1] = rf.tau;
+          if (!empty) a.e[j + 1] = rf.beta;
         }
       }
     } else {
       rows_update<true>(rows, R, b, nb, n, j + 2, sv, sw, sx, one ? nullptr : a.G + (int64_t)(j + 2) * n, S);
     }
     __syncthreads();
-    if (warp == 0) rows_finish(rows, R, b, nb, n, j + 2, sx, S.rf[(j + 1) & 1], pn, partn + (one ? 0 : b), S);
+    if (warp == 0) rows_finish(rows, R, b, nb, n, j + 2, sx, S.rf[(j + 1) & 1], pn, partn, S);
   }
 }
 
@@ -829,7 +890,6 @@ __global__ void __launch_bounds__(4 * WY_SUB) k_wy_t(const WySub* __restrict__ s
 // rescaled by an exact power of two when its exponent leaves [-400, 400]; signs and
 // exponents are read as integers.  A zero minor is replaced by 2^-60 |p_{i-1}| with the
 // sign opposite to its predecessor (the tiny negative pivot of the ratio form).
-__device__ __forceinline__ int hi_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 __device__ int sturm_lt(const double* d, const double* e, int64_t n, double x, double pivmin) {
   (void)pivmin;
   double pm2 = 1.0, pm1 = d[0] - x;
@@ -1434,14 +1494,14 @@ namespace {
 // smem bytes: the shortest common time by the model
 //   t(n, nb) = n t_col + (2 n^3 / nb + 4 n^2) / f,
 // 12 FP64 operations per trailing entry of a CTA's rows and 16 per entry of its vectors at two
-// per SM and clock, and a column's latency t_col (barrier, loads, scalars: 2.5 us in a group
-// of one CTA, 6 us with a barrier).  Returns how many of the blocks fit the launch.
+// per SM and clock, and a column's latency t_col (scalars, loads, barrier: 4 us in a group
+// of one CTA, 5 us and 0.01 us per CTA with a barrier).  Returns how many of the blocks fit the launch.
 int tri_deal(const std::vector<int64_t>& n, int nsm, size_t smem, std::vector<int>* nb) {
   auto fits = [&](int64_t m, int64_t q) {
     const int64_t rows = (m + q - 1) / q;
     return rows <= TRI_RMAX && (size_t)(rows + 3 + (q == 1)) * m * sizeof(z) <= smem;
   };
-  auto time = [](double m, double q) { return m * (q > 1 ? 6.0 : 2.5) + (2.0 * m * m * m / q + 4.0 * m * m) / 2070.0; };
+  auto time = [](double m, double q) { return m * (q > 1 ? 5.0 + 0.01 * q : 4.0) + (2.0 * m * m * m / q + 4.0 * m * m) / 2070.0; };
   std::vector<int> lo;
   int used = 0;
   for (int64_t m : n) {  // the least group that holds each block
@@ -1647,8 +1707,8 @@ int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& all, z* U, double* ev
   double* e = (double*)ws_alloc(c, ws_round(sizeof(double) * tot));
   z* tau = (z*)ws_alloc(c, ws_round(sizeof(z) * tot));
   z* p = (z*)ws_alloc(c, ws_round(sizeof(z) * 2 * tot));
-  z* part = (z*)ws_alloc(c, ws_round(sizeof(z) * 2 * (size_t)nsm));
-  unsigned* bar = (unsigned*)ws_alloc(c, ws_round(sizeof(unsigned) * 32 * (TRI_MAXB + 1)));
+  double* part = (double*)ws_alloc(c, ws_round(sizeof(double) * 2 * (size_t)nsm));
+  unsigned* bar = (unsigned*)ws_alloc(c, ws_round(sizeof(unsigned) * 32 * TRI_MAXB));
   double* tn = (double*)ws_alloc(c, ws_round(sizeof(double) * nb));
   int64_t* nr = (int64_t*)ws_alloc(c, ws_round(sizeof(int64_t) * nb));
   double* work = (double*)ws_alloc(c, ws_round(sizeof(double) * 6 * nk));
@@ -1709,7 +1769,6 @@ int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& all, z* U, double* ev
       TriGroup T;
       T.nblk = cnt;
       T.bar = bar;
-      T.abort_flag = (int*)(bar + 32 * TRI_MAXB);
       T.status = c->d_status;
       int ctas = 0;
       size_t smem = 0;
@@ -1722,7 +1781,7 @@ int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& all, z* U, double* ev
         ctas += q[(size_t)i];
         smem = std::max(smem, (size_t)(rows + 3 + (q[(size_t)i] == 1)) * b.n * sizeof(z));
       }
-      TNT_CUDA_TRY(c, cudaMemsetAsync(bar, 0, sizeof(unsigned) * 32 * (TRI_MAXB + 1), st));
+      TNT_CUDA_TRY(c, cudaMemsetAsync(bar, 0, sizeof(unsigned) * 32 * TRI_MAXB, st));
       void* args[] = {&T};
       TNT_CUDA_TRY(c, cudaLaunchCooperativeKernel((void*)k_tridiag_group, dim3((unsigned)ctas), dim3(TRI_GTHREADS),
                                                   args, smem, st));

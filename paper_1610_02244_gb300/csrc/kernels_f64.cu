@@ -943,7 +943,7 @@ int vec_normalize(Ctx* c, const z* x, z* y, int64_t n, const double* d_norm2) {
 // of all CTAs are added in CTA order by every CTA, so all hold the same c, and the result is
 // deterministic.
 // What bounds it: the FP64 pipe, 16 k n FMAs at two per SM and clock (27 us at n = 65536,
-// k = 16), and three grid barriers of about 1.5 us.  The separate launches it replaces took
+// k = 16), and three grid barriers.  The separate launches it replaces took
 // 160 us there (four dot-product launches of eight vectors at 27 to 30 us, whatever n: with
 // one element per thread each spent its time reducing 16 sums per thread), 115 us at
 // n = 5000.
@@ -965,40 +965,38 @@ struct GsArgs {
   double* beta;
   z* part;       // 2 x 64 x gridDim.x
   double* npart; // gridDim.x
-  unsigned* bar; // arrivals, generation, abort flag
+  unsigned* bar; // arrivals since the solve began
+  unsigned base; // its value before this launch
   int* status;
   int S;
   int keep;      // V slices in shared memory
 };
 
-// false: a wait expired here or elsewhere, the CTA must stop
-__device__ bool gs_barrier(const GsArgs& a) {
+// Every CTA adds one to the counter (release) and waits (acquire) until it has moved by
+// `want` since the solve began; the count wraps.  false: the wait expired, the CTA must stop
+// (and so will the others).
+__device__ bool gs_barrier(const GsArgs& a, unsigned want) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    volatile unsigned* gen = a.bar + 1;
-    const unsigned g = *gen;
-    __threadfence();
+    unsigned seen;
     int ok = 1;
-    if (atomicAdd(a.bar, 1u) == gridDim.x - 1) {
-      a.bar[0] = 0;
-      __threadfence();
-      atomicAdd(a.bar + 1, 1u);
-    } else {
-      uint64_t t0, t1;
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-      while (*gen == g) {
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
-        if (*(volatile unsigned*)(a.bar + 2)) break;
-        if (t1 - t0 > 2000000000ull) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(a.bar), "r"(1u) : "memory");
+    uint64_t t0 = 0;
+    for (unsigned polls = 0;; ++polls) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.bar) : "memory");
+      if ((int)(seen - want) >= 0) break;
+      if ((polls & 1023u) == 1023u) {
+        uint64_t now;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+        if (!t0) t0 = now;
+        if (now - t0 > 2000000000ull) {
           atomicOr(a.status, 2);
-          atomicExch(a.bar + 2, 1u);
+          ok = 0;
           break;
         }
       }
     }
-    __threadfence();
-    if (*(volatile unsigned*)(a.bar + 2)) ok = 0;
     s_ok = ok;
   }
   __syncthreads();
@@ -1132,21 +1130,21 @@ __global__ void __launch_bounds__(GS_THREADS, 1) k_gs_step(GsArgs a) {
   else gs_dots<false>(a, sw, sv, Vg, a.n, cnt, p1);
   const z* V = a.keep ? sv : Vg;
   const int64_t ld = a.keep ? a.S : a.n;
-  bool ok = gs_barrier(a);
+  bool ok = gs_barrier(a, a.base + 1u * gridDim.x);
   if (ok) {
     gs_total(a, p1, sc);
     if (blockIdx.x == 0 && tid == 0) a.alpha[a.k - 1] = sc[a.k - 1].x;
     gs_update(a, sw, V, ld, cnt, sc);
     __syncthreads();
     gs_dots<false>(a, sw, sv, V, ld, cnt, p2);
-    ok = gs_barrier(a);
+    ok = gs_barrier(a, a.base + 2u * gridDim.x);
   }
   if (ok) {
     gs_total(a, p2, sc);
     double acc = gs_update(a, sw, V, ld, cnt, sc);
     acc = block_sum(acc, sh);
     if (tid == 0) a.npart[blockIdx.x] = acc;
-    ok = gs_barrier(a);
+    ok = gs_barrier(a, a.base + 3u * gridDim.x);
   }
   if (!ok) {  // the host reads a NaN beta, and the status word names the wait
     if (blockIdx.x == 0 && tid == 0) a.beta[a.k - 1] = __longlong_as_double(0x7ff8000000000000ll);
@@ -1174,7 +1172,8 @@ __global__ void __launch_bounds__(GS_THREADS, 1) k_gs_step(GsArgs a) {
 bool vec_gs_eligible(int64_t n) { return n <= GS_MAX_N; }
 
 int vec_gs_reset(Ctx* c) {
-  TNT_CUDA_TRY(c, cudaMemsetAsync(c->d_count + 16, 0, 3 * sizeof(unsigned), c->stream));
+  TNT_CUDA_TRY(c, cudaMemsetAsync(c->d_count + 16, 0, sizeof(unsigned), c->stream));
+  c->gs_arrivals = 0;
   return TNT_OK;
 }
 
@@ -1197,9 +1196,11 @@ int vec_gs_step(Ctx* c, const z* V, int k, const z* w, int64_t n, z* vnext, doub
   a.alpha = d_alpha; a.beta = d_beta;
   a.part = part; a.npart = npart;
   a.bar = c->d_count + 16;
+  a.base = c->gs_arrivals;
   a.status = c->d_status;
   a.S = (int)std::max<int64_t>(64, (n + nsm - 1) / nsm);
   const int grid = (int)((n + a.S - 1) / a.S);
+  c->gs_arrivals += 3u * (unsigned)grid;
   const size_t sw = sizeof(z) * (size_t)a.S, all = sw * (size_t)(k + 1);
   a.keep = all <= (size_t)GS_SMEM;
   const size_t smem = a.keep ? all : sw;

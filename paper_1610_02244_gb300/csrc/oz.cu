@@ -67,39 +67,53 @@ static_assert(2LL * OZ_S * OZ_CHUNK * OZ_KB * 64 * 64 <= (1LL << 24),
               "a level sum over one K chunk must stay exact in FP32");
 static_assert(OZ_SMEM <= 227 * 1024, "rings fit the shared memory of an SM");
 
-// one product of a launch; offsets are bytes into the context's buffer
+// one product of a launch; offsets are bytes into the launch's buffer
 struct OzTask {
   const z *A, *B;
   z* C;
   int64_t a_rs, a_ks, b_rs, b_ks, c_rs;  // A(i, k) = A[i a_rs + k a_ks], B(k, j) = B[j b_rs + k b_ks]
   int64_t offA, offB, offE, offP;        // slice tiles, exponent fields (M then N), partial sums
-  int64_t atom0;                         // first slice atom of the task among all tasks'
+  int64_t atom0[2];                      // first slice atom among all tasks', per side
   int M, N, K;
   int ntm, ntn, nkb;                     // tiles along M and N, K blocks of 32
   int ks, both;                          // K splits; an item runs both level groups, or one
   int conj_a, conj_b;
   int herm;  // C = A B is Hermitian: tiles strictly above the diagonal are mirrored, not computed
   int sub;   // C -= A B
-  int item0, scale0, fin0;               // first item / scale block / finish block
+  int item0, scale0[2], fin0;            // first item / scale block (per side) / finish block
 };
-// The products of one launch travel as a kernel argument: no table upload.
+// The products of one launch travel as a kernel argument (no table upload), or, for a plan
+// whose products repeat, in device memory (CAP = 0).
 constexpr int OZ_MAXT = 40;
-template <int CAP>
-struct OzTasks {
-  int n, items, scale_blocks, fin_blocks;
-  int64_t atoms;
+struct OzHead {
+  int n, items, fin_blocks;
+  int scale_blocks[2];  // per side (A, B)
+  int64_t atoms[2];
+  int sides;            // the sides to scale and slice: bit 0 A, bit 1 B
+  int64_t add_b;        // bytes added to every task's B
   uint8_t* buf;
   int* status;
+};
+template <int CAP>
+struct OzTasks {
+  OzHead h;
   OzTask t[CAP];
+  __device__ __forceinline__ const OzTask& at(int i) const { return t[i]; }
+};
+template <>
+struct OzTasks<0> {
+  OzHead h;
+  const OzTask* t;
+  __device__ __forceinline__ const OzTask& at(int i) const { return t[i]; }
 };
 // the last task whose first index (by FIRST) is at most w
 template <int CAP, typename F>
 __device__ __forceinline__ int oz_find(const OzTasks<CAP>& T, F first, int64_t w) {
   if (CAP == 1) return 0;
-  int lo = 0, hi = T.n;
+  int lo = 0, hi = T.h.n;
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
-    if ((int64_t)first(T.t[mid]) <= w) lo = mid;
+    if ((int64_t)first(T.at(mid)) <= w) lo = mid;
     else hi = mid;
   }
   return lo;
@@ -112,7 +126,7 @@ struct OzItem {
 template <int CAP>
 __device__ __forceinline__ bool oz_item(const OzTasks<CAP>& T, int w, OzItem* it) {
   it->task = oz_find(T, [](const OzTask& t) { return t.item0; }, w);
-  const OzTask& g = T.t[it->task];
+  const OzTask& g = T.at(it->task);
   w -= g.item0;
   const int ntiles = g.ntm * g.ntn;
   const int t = w % ntiles, r = w / ntiles;
@@ -252,7 +266,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(const __grid_constant
   uint32_t* tmem_slot = (uint32_t*)(acce + 4);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nitems = T.items;
+  const int nitems = T.h.items;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < OZ_NA; ++s) {
@@ -288,7 +302,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(const __grid_constant
     auto load = [&](uint8_t* ring, uint64_t* full, uint64_t* empty, uint32_t& i, int n, uint32_t bytes,
                     const uint8_t* src) {
       const int s = (int)(i % (uint32_t)n);
-      if (i >= (uint32_t)n && !mbar_wait(&empty[s], ((i / n) & 1) ^ 1, T.status)) *abort_flag = 1;
+      if (i >= (uint32_t)n && !mbar_wait(&empty[s], ((i / n) & 1) ^ 1, T.h.status)) *abort_flag = 1;
       if (*abort_flag) {
         stop = true;
         return;
@@ -300,14 +314,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(const __grid_constant
     for (int w = blockIdx.x; w < nitems && !stop; w += gridDim.x) {
       OzItem it;
       if (!oz_item(T, w, &it)) continue;
-      const OzTask& g = T.t[it.task];
+      const OzTask& g = T.at(it.task);
       for (int grp = it.g0; grp <= it.g1 && !stop; ++grp) {
         int l0, l1;
         oz_levels(grp, &l0, &l1);
         const int pmax = min(OZ_S, l1 - 1);
         for (int kb = it.kb0; kb < it.kb1 && !stop; ++kb) {
-          const uint8_t* A = T.buf + g.offA + ((int64_t)it.mt * g.nkb + kb) * (OZ_S * OZ_TA);
-          const uint8_t* B = T.buf + g.offB + ((int64_t)it.nt * g.nkb + kb) * (OZ_S * OZ_TB);
+          const uint8_t* A = T.h.buf + g.offA + ((int64_t)it.mt * g.nkb + kb) * (OZ_S * OZ_TA);
+          const uint8_t* B = T.h.buf + g.offB + ((int64_t)it.nt * g.nkb + kb) * (OZ_S * OZ_TB);
           int qnext = min(OZ_S, l1 - 1);  // next slice of B to load (descending)
           for (int p = 1; p <= pmax && !stop; ++p) {
             const int qlo = max(1, l0 - p);
@@ -320,9 +334,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(const __grid_constant
     }
     // copies in flight land before the CTA may exit
     for (uint32_t i = (ia > (uint32_t)OZ_NA ? ia - OZ_NA : 0u); i < ia; ++i)
-      mbar_wait(&R.fa[i % OZ_NA], (i / OZ_NA) & 1, T.status);
+      mbar_wait(&R.fa[i % OZ_NA], (i / OZ_NA) & 1, T.h.status);
     for (uint32_t i = (ib > (uint32_t)OZ_NB ? ib - OZ_NB : 0u); i < ib; ++i)
-      mbar_wait(&R.fb[i % OZ_NB], (i / OZ_NB) & 1, T.status);
+      mbar_wait(&R.fb[i % OZ_NB], (i / OZ_NB) & 1, T.h.status);
   } else if (warp == 1 && lane == 0) {
     // ------------------------------------------------ MMA issue
     uint32_t sub = 0;
@@ -337,7 +351,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(const __grid_constant
           bool ok = *abort_flag == 0;
           r.acce = first && sub > 0 ? acce : nullptr;
           r.pacc = (sub - 1) & 1;
-          if (ok) ok = grp ? oz_issue_block<1>(r, tmem, first, T.status) : oz_issue_block<0>(r, tmem, first, T.status);
+          if (ok) ok = grp ? oz_issue_block<1>(r, tmem, first, T.h.status) : oz_issue_block<0>(r, tmem, first, T.h.status);
           if (!ok) {
             *abort_flag = 1;
             stop = true;
@@ -360,7 +374,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(const __grid_constant
     for (int w = blockIdx.x; w < nitems && !stop; w += gridDim.x) {
       OzItem it;
       if (!oz_item(T, w, &it)) continue;
-      const OzTask& g = T.t[it.task];
+      const OzTask& g = T.at(it.task);
       const int64_t gm = (int64_t)it.mt * OZ_BM + row;
       const int64_t gn0 = (int64_t)it.nt * OZ_BN + half * 32;
       for (int grp = it.g0; grp <= it.g1 && !stop; ++grp) {
@@ -368,7 +382,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(const __grid_constant
 #pragma unroll
         for (int j = 0; j < 32; ++j) re[j] = im[j] = 0;
         for (int kb = it.kb0; kb < it.kb1; kb += OZ_CHUNK) {
-          if (*abort_flag || !mbar_wait(accf, sub & 1, T.status)) {
+          if (*abort_flag || !mbar_wait(accf, sub & 1, T.h.status)) {
             *abort_flag = 1;
             stop = true;
             break;
@@ -398,7 +412,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(const __grid_constant
         if (stop || gm >= g.M) continue;
         const int nc = (int)min((int64_t)32, (int64_t)g.N - gn0);  // columns of this half tile
         if (nc <= 0) continue;
-        oz_put((longlong2*)(T.buf + g.offP) + ((int64_t)(2 * it.sp + grp) * g.M + gm) * g.N + gn0, nc, re, im);
+        oz_put((longlong2*)(T.h.buf + g.offP) + ((int64_t)(2 * it.sp + grp) * g.M + gm) * g.N + gn0, nc, re, im);
       }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -415,13 +429,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(const __grid_constant
 // triangle, mirrored.
 template <int CAP>
 __global__ void __launch_bounds__(256) k_oz_finish(const __grid_constant__ OzTasks<CAP> T) {
-  for (int fb = blockIdx.x; fb < T.fin_blocks; fb += gridDim.x) {
-    const OzTask& g = T.t[oz_find(T, [](const OzTask& t) { return t.fin0; }, fb)];
+  for (int fb = blockIdx.x; fb < T.h.fin_blocks; fb += gridDim.x) {
+    const OzTask& g = T.at(oz_find(T, [](const OzTask& t) { return t.fin0; }, fb));
     const int64_t total = (int64_t)g.M * g.N, e = (int64_t)(fb - g.fin0) * 256 + threadIdx.x;
     if (e >= total) continue;
     const int64_t i = e / g.N, j = e % g.N;
     if (g.herm && j > i) continue;
-    const longlong2* P = (const longlong2*)(T.buf + g.offP) + e;
+    const longlong2* P = (const longlong2*)(T.h.buf + g.offP) + e;
     longlong2 h = make_longlong2(0, 0), l = h;
     for (int s = 0; s < g.ks; ++s) {
       const longlong2 a = P[(int64_t)(2 * s) * total], b = P[(int64_t)(2 * s + 1) * total];
@@ -430,7 +444,7 @@ __global__ void __launch_bounds__(256) k_oz_finish(const __grid_constant__ OzTas
       l.x += b.x;
       l.y += b.y;
     }
-    const int* ex = (const int*)(T.buf + g.offE);
+    const int* ex = (const int*)(T.h.buf + g.offE);
     const int ea = ex[i], eb = ex[g.M + j];
     z v = zmk(oz_value(h.x, l.x, ea, eb), oz_value(h.y, l.y, ea, eb));
     z* o = g.C + i * g.c_rs + j;
@@ -450,9 +464,10 @@ struct OzOp {
   uint8_t* out;  // slice tiles
 };
 // B enters as rows n with K along the row
-__device__ __forceinline__ OzOp oz_operand(const OzTask& g, uint8_t* buf, bool isb) {
+__device__ __forceinline__ OzOp oz_operand(const OzTask& g, const OzHead& h, bool isb) {
+  uint8_t* buf = h.buf;
   OzOp o;
-  o.X = isb ? g.B : g.A;
+  o.X = isb ? (const z*)((const char*)g.B + h.add_b) : g.A;
   o.rows = isb ? g.N : g.M;
   o.rs = isb ? g.b_rs : g.a_rs;
   o.cs = isb ? g.b_ks : g.a_ks;
@@ -463,21 +478,24 @@ __device__ __forceinline__ OzOp oz_operand(const OzTask& g, uint8_t* buf, bool i
 }
 
 // largest exponent field of every row.  Entries contiguous along K: one warp per row;
-// otherwise 32 rows by 64 of K per CTA, neighbouring lanes on neighbouring rows, combined
-// with an atomic maximum (e zeroed before)
+// otherwise 32 rows by up to OZ_SCALE_K of K per CTA, neighbouring lanes on neighbouring rows
+// (a longer K combines its parts with an atomic maximum, e zeroed before)
+constexpr int OZ_SCALE_K = 512;
 __device__ __forceinline__ unsigned oz_exp(z v) {
   return max(((unsigned)__double2hiint(v.x) >> 20) & 0x7ffu, ((unsigned)__double2hiint(v.y) >> 20) & 0x7ffu);
 }
 __host__ __device__ inline int64_t oz_scale_blocks(int64_t rows, int64_t ks, int64_t K) {
-  return ks == 1 ? (rows + 7) / 8 : ((rows + 31) / 32) * ((K + 63) / 64);
+  return ks == 1 ? (rows + 7) / 8 : ((rows + 31) / 32) * ((K + OZ_SCALE_K - 1) / OZ_SCALE_K);
 }
 template <int CAP>
 __global__ void __launch_bounds__(256) k_oz_scale(const __grid_constant__ OzTasks<CAP> T) {
-  const OzTask& g = T.t[oz_find(T, [](const OzTask& t) { return t.scale0; }, blockIdx.x)];
-  const int64_t K = g.K, nba = oz_scale_blocks(g.M, g.a_ks, K);
-  const bool isb = (int64_t)blockIdx.x - g.scale0 >= nba;
-  const OzOp o = oz_operand(g, T.buf, isb);
-  const int64_t blk = (int64_t)blockIdx.x - g.scale0 - (isb ? nba : 0);
+  const int na = (T.h.sides & 1) ? T.h.scale_blocks[0] : 0;
+  const bool isb = (int)blockIdx.x >= na;
+  const int w = (int)blockIdx.x - (isb ? na : 0);
+  const OzTask& g = T.at(isb ? oz_find(T, [](const OzTask& t) { return t.scale0[1]; }, w)
+                             : oz_find(T, [](const OzTask& t) { return t.scale0[0]; }, w));
+  const int64_t K = g.K, blk = w - g.scale0[isb];
+  const OzOp o = oz_operand(g, T.h, isb);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (o.cs == 1) {
     const int64_t i = blk * 8 + warp;
@@ -493,14 +511,19 @@ __global__ void __launch_bounds__(256) k_oz_scale(const __grid_constant__ OzTask
   __shared__ unsigned s_mx[32];
   if (threadIdx.x < 32) s_mx[threadIdx.x] = 0;
   __syncthreads();
-  const int64_t nk = (K + 63) / 64, i = (blk / nk) * 32 + lane, k0 = (blk % nk) * 64;
+  const int64_t nk = (K + OZ_SCALE_K - 1) / OZ_SCALE_K, i = (blk / nk) * 32 + lane, k0 = (blk % nk) * OZ_SCALE_K;
   unsigned mx = 0;
-  if (i < o.rows)
-#pragma unroll
-    for (int64_t k = k0 + warp; k < min(K, k0 + 64); k += 8) mx = max(mx, oz_exp(o.X[i * o.rs + k * o.cs]));
+  if (i < o.rows) {
+    const int64_t k1 = min(K, k0 + OZ_SCALE_K);
+#pragma unroll 8
+    for (int64_t k = k0 + warp; k < k1; k += 8) mx = max(mx, oz_exp(o.X[i * o.rs + k * o.cs]));
+  }
   if (mx) atomicMax(&s_mx[lane], mx);
   __syncthreads();
-  if (warp == 0 && i < o.rows && s_mx[lane]) atomicMax((unsigned*)o.e + i, s_mx[lane]);
+  if (warp == 0 && i < o.rows) {
+    if (nk == 1) o.e[i] = (int)s_mx[lane];
+    else atomicMax((unsigned*)o.e + i, s_mx[lane]);
+  }
 }
 
 // slices of 8 rows by 32 of K per warp: lane = (row, 8 of K), so every plane's 512-byte
@@ -553,11 +576,15 @@ __device__ __forceinline__ void oz_slice_atom(const OzOp& o, int64_t K, int nkb,
 template <int CAP>
 __global__ void __launch_bounds__(256) k_oz_slice(const __grid_constant__ OzTasks<CAP> T) {
   const int lane = threadIdx.x & 31;
-  for (int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); w < T.atoms; w += (int64_t)gridDim.x * 8) {
-    const OzTask& g = T.t[oz_find(T, [](const OzTask& t) { return t.atom0; }, w)];
-    const int64_t a = w - g.atom0, na = (int64_t)g.ntm * (OZ_BM / 8) * g.nkb;
-    if (a < na) oz_slice_atom<2>(oz_operand(g, T.buf, false), g.K, g.nkb, a, lane);
-    else oz_slice_atom<3>(oz_operand(g, T.buf, true), g.K, g.nkb, a - na, lane);
+  const int64_t na = (T.h.sides & 1) ? T.h.atoms[0] : 0, all = na + ((T.h.sides & 2) ? T.h.atoms[1] : 0);
+  for (int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); w < all; w += (int64_t)gridDim.x * 8) {
+    if (w < na) {
+      const OzTask& g = T.at(oz_find(T, [](const OzTask& t) { return t.atom0[0]; }, w));
+      oz_slice_atom<2>(oz_operand(g, T.h, false), g.K, g.nkb, w - g.atom0[0], lane);
+    } else {
+      const OzTask& g = T.at(oz_find(T, [](const OzTask& t) { return t.atom0[1]; }, w - na));
+      oz_slice_atom<3>(oz_operand(g, T.h, true), g.K, g.nkb, w - na - g.atom0[1], lane);
+    }
   }
 }
 
@@ -624,26 +651,24 @@ int oz_sm_count(Ctx* c, int* sm) {
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || n < 1) n = 152;
     TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_oz_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
     TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_oz_gemm<OZ_MAXT>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
+    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_oz_gemm<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
     v = n;
   }
   *sm = v;
   return TNT_OK;
 }
 
-// products tk[0..n) in one set of launches; slices and partial sums live in the context's own
-// buffer (grown between calls, never inside a capture)
-template <int CAP>
-int oz_launch(Ctx* c, const GemmTask* const* tk, int n, int sm) {
-  OzTasks<CAP> T;
-  T.n = n;
-  T.status = c->d_status;
+// tables of the products tk[0..n): T's head and tasks, and the bytes of buffer they use
+size_t oz_layout(const GemmTask* const* tk, int n, int sm, OzHead* h, OzTask* t, double* flop, double* bytes) {
   size_t off = 0;
-  int64_t items = 0, scale = 0, fin = 0, rows = 0;
-  double work = 0, flop = 0, bytes = 0;
-  T.atoms = 0;
+  int64_t items = 0, scale[2] = {0, 0}, fin = 0, rows = 0;
+  double work = 0, wflop = 0, wbytes = 0;
+  *h = OzHead{};
+  h->n = n;
+  h->sides = 3;
   for (int i = 0; i < n; ++i) {
     const ZGemm& g = tk[i]->g;
-    OzTask& o = T.t[i];
+    OzTask& o = t[i];
     o.A = g.A; o.B = g.B; o.C = g.C;
     o.a_rs = g.a_rs; o.a_ks = g.a_cs; o.b_rs = g.b_cs; o.b_ks = g.b_rs; o.c_rs = g.c_rs;
     o.conj_a = g.conj_a; o.conj_b = g.conj_b;
@@ -653,10 +678,10 @@ int oz_launch(Ctx* c, const GemmTask* const* tk, int n, int sm) {
     o.ntn = (int)cdiv(g.N, OZ_BN);
     o.nkb = (int)cdiv(g.K, OZ_KB);
     work += 36.0 * o.nkb * o.ntm * o.ntn;
-    flop += (o.herm ? 4.0 : 8.0) * (double)g.M * (double)g.N * (double)g.K;
+    wflop += (o.herm ? 4.0 : 8.0) * (double)g.M * (double)g.N * (double)g.K;
   }
   for (int i = 0; i < n; ++i) {
-    OzTask& o = T.t[i];
+    OzTask& o = t[i];
     const double mn = (double)o.M * (double)o.N;
     OzDeal deal{1, 1};
     if (n == 1) {
@@ -675,53 +700,153 @@ int oz_launch(Ctx* c, const GemmTask* const* tk, int n, int sm) {
     off += ws_round((size_t)o.ntn * o.nkb * OZ_S * OZ_TB);
     o.offP = (int64_t)off;
     off += ws_round(sizeof(longlong2) * 2 * (size_t)o.ks * (size_t)mn);
-    bytes += 16.0 * ((double)o.M + o.N) * o.K + (double)(o.offP - o.offA);
+    wbytes += 16.0 * ((double)o.M + o.N) * o.K + (double)(o.offP - o.offA);
     o.item0 = (int)items;
     items += (int64_t)o.ntm * o.ntn * o.ks * (o.both ? 1 : 2);
-    o.scale0 = (int)scale;
-    scale += oz_scale_blocks(o.M, o.a_ks, o.K) + oz_scale_blocks(o.N, o.b_ks, o.K);
-    o.atom0 = T.atoms;
-    T.atoms += ((int64_t)o.ntm * (OZ_BM / 8) + (int64_t)o.ntn * (OZ_BN / 8)) * o.nkb;
+    o.scale0[0] = (int)scale[0];
+    o.scale0[1] = (int)scale[1];
+    scale[0] += oz_scale_blocks(o.M, o.a_ks, o.K);
+    scale[1] += oz_scale_blocks(o.N, o.b_ks, o.K);
+    o.atom0[0] = h->atoms[0];
+    o.atom0[1] = h->atoms[1];
+    h->atoms[0] += (int64_t)o.ntm * (OZ_BM / 8) * o.nkb;
+    h->atoms[1] += (int64_t)o.ntn * (OZ_BN / 8) * o.nkb;
     o.fin0 = (int)fin;
     fin += cdiv((int64_t)o.M * o.N, 256);
   }
-  const size_t off_e = off;
-  for (int i = 0; i < n; ++i) {
-    T.t[i].offE = (int64_t)(off_e + sizeof(int) * (size_t)rows);
-    rows += T.t[i].M + T.t[i].N;
+  for (int i = 0; i < n; ++i) {  // the exponent fields are the buffer's end
+    t[i].offE = (int64_t)(off + sizeof(int) * (size_t)rows);
+    rows += t[i].M + t[i].N;
   }
   off += ws_round(sizeof(int) * (size_t)rows);
-  if (items > INT32_MAX || scale > INT32_MAX || fin > INT32_MAX)
-    return set_err(c, TNT_E_UNSUPPORTED, "FP64 products too large for one launch");
-  T.items = (int)items;
-  T.scale_blocks = (int)scale;
-  T.fin_blocks = (int)fin;
-  if (off > c->oz_cap) {
+  if (items > INT32_MAX || scale[0] + scale[1] > INT32_MAX || fin > INT32_MAX) return 0;
+  h->items = (int)items;
+  h->scale_blocks[0] = (int)scale[0];
+  h->scale_blocks[1] = (int)scale[1];
+  h->fin_blocks = (int)fin;
+  *flop = wflop;
+  *bytes = wbytes;
+  return off;
+}
+template <int CAP>
+unsigned oz_scale_grid(const OzTasks<CAP>& T) {
+  return (unsigned)(((T.h.sides & 1) ? T.h.scale_blocks[0] : 0) + ((T.h.sides & 2) ? T.h.scale_blocks[1] : 0));
+}
+template <int CAP>
+unsigned oz_slice_grid(const OzTasks<CAP>& T) {
+  const int64_t a = ((T.h.sides & 1) ? T.h.atoms[0] : 0) + ((T.h.sides & 2) ? T.h.atoms[1] : 0);
+  return (unsigned)std::min<int64_t>(cdiv(a, 8), 152 * 16);
+}
+
+// products tk[0..n) in one set of launches; slices and partial sums live in the context's own
+// buffer (grown between calls, never inside a capture)
+template <int CAP>
+int oz_launch(Ctx* c, const GemmTask* const* tk, int n, int sm) {
+  OzTasks<CAP> T;
+  double flop = 0, bytes = 0;
+  const size_t need = oz_layout(tk, n, sm, &T.h, T.t, &flop, &bytes);
+  if (!need) return set_err(c, TNT_E_UNSUPPORTED, "FP64 products too large for one launch");
+  T.h.status = c->d_status;
+  if (need > c->oz_cap) {
     TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     dev_free(c->dalloc, c->oz_buf);
     c->oz_buf = nullptr;
     c->oz_cap = 0;
-    if (dev_alloc(c->dalloc, &c->oz_buf, off) != 0)
-      return set_err(c, TNT_E_ALLOC, "device allocation of %zu bytes (FP64 product slices) failed", off);
-    c->oz_cap = off;
+    if (dev_alloc(c->dalloc, &c->oz_buf, need) != 0)
+      return set_err(c, TNT_E_ALLOC, "device allocation of %zu bytes (FP64 product slices) failed", need);
+    c->oz_cap = need;
   }
-  T.buf = (uint8_t*)c->oz_buf;
+  T.h.buf = (uint8_t*)c->oz_buf;
   {
     ProfScope ps(c, "oz_slice", bytes);
-    TNT_CUDA_TRY(c, cudaMemsetAsync(T.buf + off_e, 0, sizeof(int) * (size_t)rows, c->stream));
-    k_oz_scale<CAP><<<(unsigned)scale, 256, 0, c->stream>>>(T);
-    k_oz_slice<CAP><<<(unsigned)std::min<int64_t>(cdiv(T.atoms, 8), 152 * 16), 256, 0, c->stream>>>(T);
+    for (int i = 0; i < n; ++i) {  // maxima combined from several CTAs start from zero
+      const OzTask& o = T.t[i];
+      if (o.K > OZ_SCALE_K && (o.a_ks != 1 || o.b_ks != 1))
+        TNT_CUDA_TRY(c, cudaMemsetAsync(T.h.buf + o.offE, 0, sizeof(int) * (size_t)(o.M + o.N), c->stream));
+    }
+    k_oz_scale<CAP><<<oz_scale_grid(T), 256, 0, c->stream>>>(T);
+    k_oz_slice<CAP><<<oz_slice_grid(T), 256, 0, c->stream>>>(T);
   }
   {
     ProfScope ps(c, "oz_gemm", flop);
-    k_oz_gemm<CAP><<<(unsigned)std::min<int64_t>(items, sm), OZ_THREADS, OZ_SMEM, c->stream>>>(T);
-    k_oz_finish<CAP><<<(unsigned)std::min<int64_t>(fin, 152 * 8), 256, 0, c->stream>>>(T);
+    k_oz_gemm<CAP><<<(unsigned)std::min(T.h.items, sm), OZ_THREADS, OZ_SMEM, c->stream>>>(T);
+    k_oz_finish<CAP><<<(unsigned)std::min(T.h.fin_blocks, 152 * 8), 256, 0, c->stream>>>(T);
   }
   c->launches += 4;
   TNT_CHECK_LAUNCH(c);
   return TNT_OK;
 }
 }  // namespace
+
+// ---------------------------------------------------------------- repeated products
+size_t oz_plan_bytes(Ctx* c, const std::vector<GemmTask>& tasks) {
+  int sm = 0;
+  if (tasks.empty() || oz_sm_count(c, &sm) != TNT_OK) return 0;
+  std::vector<const GemmTask*> tk;
+  for (const GemmTask& t : tasks) tk.push_back(&t);
+  std::vector<OzTask> t(tasks.size());
+  OzHead h;
+  double f, b;
+  const size_t need = oz_layout(tk.data(), (int)tk.size(), sm, &h, t.data(), &f, &b);
+  return need ? need + ws_round(sizeof(OzTask) * t.size()) : 0;
+}
+
+int oz_plan_build(Ctx* c, const std::vector<GemmTask>& tasks, int fixed_sides, OzPlan* p) {
+  int sm = 0;
+  TNT_TRY(oz_sm_count(c, &sm));
+  std::vector<const GemmTask*> tk;
+  for (const GemmTask& t : tasks) {
+    tk.push_back(&t);
+    if (t.g.K > OZ_SCALE_K && (t.g.a_cs != 1 || t.g.b_rs != 1))
+      return set_err(c, TNT_E_UNSUPPORTED, "planned FP64 product with a strided K of %lld", (long long)t.g.K);
+  }
+  std::vector<OzTask> t(tasks.size());
+  static_assert(sizeof(OzTasks<0>) <= sizeof(p->args), "the plan's argument block holds the kernels' argument");
+  OzTasks<0> T;
+  double f, b;
+  const size_t need = oz_layout(tk.data(), (int)tk.size(), sm, &T.h, t.data(), &f, &b);
+  uint8_t* buf = (uint8_t*)ws_alloc(c, need);
+  OzTask* dt = (OzTask*)ws_alloc(c, ws_round(sizeof(OzTask) * t.size()));
+  if (!need || !buf || !dt) return set_err(c, TNT_E_ALLOC, "scratch exhausted (planned FP64 products)");
+  TNT_CUDA_TRY(c, cudaMemcpyAsync(dt, t.data(), sizeof(OzTask) * t.size(), cudaMemcpyHostToDevice, c->stream));
+  T.h.buf = buf;
+  T.h.status = c->d_status;
+  T.t = dt;
+  if (fixed_sides) {
+    T.h.sides = fixed_sides;
+    k_oz_scale<0><<<oz_scale_grid(T), 256, 0, c->stream>>>(T);
+    k_oz_slice<0><<<oz_slice_grid(T), 256, 0, c->stream>>>(T);
+    c->launches += 2;
+    TNT_CHECK_LAUNCH(c);
+  }
+  T.h.sides = 3 & ~fixed_sides;
+  memcpy(p->args, &T, sizeof(T));
+  p->flop = f;
+  p->node[0] = OzNode{(void*)k_oz_scale<0>, oz_scale_grid(T), 256, 0};
+  p->node[1] = OzNode{(void*)k_oz_slice<0>, oz_slice_grid(T), 256, 0};
+  p->node[2] = OzNode{(void*)k_oz_gemm<0>, (unsigned)std::min(T.h.items, sm), OZ_THREADS, OZ_SMEM};
+  p->node[3] = OzNode{(void*)k_oz_finish<0>, (unsigned)std::min(T.h.fin_blocks, 152 * 8), 256, 0};
+  return TNT_OK;
+}
+
+void oz_plan_args(const OzPlan& p, const z* add_b, void* out) {
+  OzTasks<0> T;
+  memcpy(&T, p.args, sizeof(T));
+  T.h.add_b = (int64_t)(intptr_t)add_b;
+  memcpy(out, &T, sizeof(T));
+}
+
+int oz_plan_run(Ctx* c, const OzPlan& p, const z* add_b) {
+  alignas(16) unsigned char a[sizeof(p.args)];
+  oz_plan_args(p, add_b, a);
+  void* args[] = {a};
+  for (const OzNode& n : p.node) {
+    TNT_CUDA_TRY(c, cudaLaunchKernel(n.fn, dim3(n.grid), dim3(n.block), args, n.smem, c->stream));
+    c->launches++;
+  }
+  TNT_CHECK_LAUNCH(c);
+  return TNT_OK;
+}
 
 int ozgemm(Ctx* c, const ZGemm& g) {
   int sm = 0;

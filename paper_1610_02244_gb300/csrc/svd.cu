@@ -141,6 +141,38 @@ struct SelOut {
   int tie;
 };
 
+// suffix sums over the block: thread t's values v[0..m) are elements t m .. t m + m - 1; on
+// return v[i] is the sum of element t m + i and all after it (threads in order, every step the
+// same tree: deterministic)
+__device__ void block_suffix(double* v, int m, double* sh) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  for (int i = m - 2; i >= 0; --i) v[i] += v[i + 1];
+  double s = v[0];  // inclusive suffix over the warp's lanes
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double u = __shfl_down_sync(0xffffffffu, s, o);
+    if (lane + o < 32) s += u;
+  }
+  __syncthreads();
+  if (lane == 0) sh[warp] = s;
+  __syncthreads();
+  double w = lane < nw ? sh[lane] : 0.0;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double u = __shfl_down_sync(0xffffffffu, w, o);
+    if (lane + o < 32) w += u;
+  }
+  const double later = warp + 1 < 32 ? __shfl_sync(0xffffffffu, w, (warp + 1) & 31) : 0.0;
+  double after = __shfl_down_sync(0xffffffffu, s, 1);
+  if (lane == 31) after = 0.0;
+  after += later;
+  for (int i = 0; i < m; ++i) v[i] += after;
+}
+
+// All candidates in order (sigma descending, block ascending, index ascending), then the four
+// rules.  Keys compare as their bit patterns (non-negative doubles order as integers; the
+// padding is negative), and the rules take searches and block-wide sums: one thread's serial
+// loops over the candidates, with an FP64 division each, took 1.7 ms for 2600 of them.
 __global__ void __launch_bounds__(1024) k_select(const double* __restrict__ sig_in,
                                                  const int* __restrict__ blk_in,
                                                  const int* __restrict__ loc_in, int n, int P,
@@ -153,18 +185,22 @@ __global__ void __launch_bounds__(1024) k_select(const double* __restrict__ sig_
                                                  int* __restrict__ loc_out,
                                                  SelOut* __restrict__ res) {
   extern __shared__ double sm_sel[];
-  double* key = sm_sel;
+  __shared__ double sh[32];
+  __shared__ double s_nrm2, s_unseen;
+  __shared__ int s_chi4;
+  long long* key = (long long*)sm_sel;
   int* bk = (int*)(key + P);
   int* lc = bk + P;
-  for (int i = threadIdx.x; i < P; i += blockDim.x) {
-    key[i] = (i < n) ? sig_in[i] : -1.0;
+  const int tid = threadIdx.x;
+  for (int i = tid; i < P; i += blockDim.x) {
+    key[i] = (i < n) ? __double_as_longlong(sig_in[i]) : __double_as_longlong(-1.0);
     bk[i] = (i < n) ? blk_in[i] : 0x7fffffff;
     lc[i] = (i < n) ? loc_in[i] : 0x7fffffff;
   }
   __syncthreads();
   for (int k = 2; k <= P; k <<= 1) {
     for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < P; i += blockDim.x) {
+      for (int i = tid; i < P; i += blockDim.x) {
         int l = i ^ j;
         if (l > i) {
           bool desc_block = ((i & k) == 0);
@@ -172,7 +208,7 @@ __global__ void __launch_bounds__(1024) k_select(const double* __restrict__ sig_
                           (key[i] == key[l] && (bk[i] < bk[l] || (bk[i] == bk[l] && lc[i] < lc[l])));
           bool swap = desc_block ? !i_before : i_before;
           if (swap) {
-            double tk = key[i]; key[i] = key[l]; key[l] = tk;
+            long long tk = key[i]; key[i] = key[l]; key[l] = tk;
             int tb = bk[i]; bk[i] = bk[l]; bk[l] = tb;
             int tl = lc[i]; lc[i] = lc[l]; lc[l] = tl;
           }
@@ -181,61 +217,83 @@ __global__ void __launch_bounds__(1024) k_select(const double* __restrict__ sig_
       __syncthreads();
     }
   }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    sig_out[i] = key[i];
+  auto val = [&](int i) { return __longlong_as_double(key[i]); };
+  for (int i = tid; i < n; i += blockDim.x) {
+    sig_out[i] = val(i);
     blk_out[i] = bk[i];
     loc_out[i] = lc[i];
   }
-  if (threadIdx.x == 0) {
-    const double s0 = n > 0 ? key[0] : 0.0;
-    int64_t chi1 = n < chi_max ? n : chi_max;
-    int64_t chi2 = n;
-    if (a > 0) {
-      chi2 = 0;
-      while (chi2 < n && key[chi2] >= a) ++chi2;
+  constexpr int MAXV = 8;  // 8192 candidates
+  const int m = (n + (int)blockDim.x - 1) / (int)blockDim.x;
+  double v[MAXV];
+  // the candidates are each block's leading min(rank, chi_max) values; when that cuts a
+  // block short, the weight of the values never formed is |M|_F^2 minus the candidates'
+#pragma unroll
+  for (int i = 0; i < MAXV; ++i) {
+    const int q = tid * m + i;
+    v[i] = i < m && q < n ? val(q) * val(q) : 0.0;
+  }
+  block_suffix(v, m, sh);
+  if (tid == 0) {
+    const double sumc = v[0];
+    s_nrm2 = complete ? sumc : fmax(total_norm2[0], sumc);
+    s_unseen = complete ? 0.0 : fmax(0.0, total_norm2[0] - sumc);
+    s_chi4 = n;
+  }
+  __syncthreads();
+  const double nrm2 = s_nrm2, unseen = s_unseen;
+  const double nrm = sqrt(nrm2);
+  const double inv = nrm > 0 ? 1.0 / nrm : 1.0;
+  auto errf = [&](double acc) { return etype == TNT_TRUNC_2NORM ? sqrt(acc) : acc; };
+  const double acc0 = unseen * inv * inv;  // never formed values, in normalised units
+  double u[MAXV];  // truncation error terms of an element and all after it
+#pragma unroll
+  for (int i = 0; i < MAXV; ++i) {
+    const int q = tid * m + i;
+    const double s = i < m && q < n ? val(q) * inv : 0.0;
+    u[i] = etype == TNT_TRUNC_1NORM ? fabs(s) : s * s;
+  }
+  block_suffix(u, m, sh);
+  // rule 4: the smallest keep whose discards stay below the tolerance (they grow towards 0)
+  if (errf(acc0) < etol)
+    for (int i = 0; i < m; ++i) {
+      const int q = tid * m + i;
+      if (q < n && errf(acc0 + u[i]) < etol) {
+        atomicMin(&s_chi4, q);
+        break;
+      }
     }
-    int64_t chi3 = n;
-    if (s0 > 0) {
-      chi3 = 0;
-      while (chi3 < n && key[chi3] / s0 >= rtol) ++chi3;
-    }
-    // the candidates are each block's leading min(rank, chi_max) values; when that cuts a
-    // block short, the weight of the values never formed is |M|_F^2 minus the candidates'
-    double sumc = 0;
-    for (int i = n - 1; i >= 0; --i) sumc += key[i] * key[i];
-    const double nrm2 = complete ? sumc : fmax(total_norm2[0], sumc);
-    const double unseen = complete ? 0.0 : fmax(0.0, total_norm2[0] - sumc);
-    const double nrm = sqrt(nrm2);
-    const double inv = nrm > 0 ? 1.0 / nrm : 1.0;
-    auto term = [&](double s) {
-      double t = s * inv;
-      return etype == TNT_TRUNC_1NORM ? fabs(t) : t * t;
+  __syncthreads();
+  if (tid == 0) {
+    const double s0 = n > 0 ? val(0) : 0.0;
+    // first index whose value fails a bound that holds on a prefix
+    auto prefix = [&](auto holds) {
+      int lo = 0, hi = n;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (holds(val(mid))) lo = mid + 1;
+        else hi = mid;
+      }
+      return (int64_t)lo;
     };
-    auto errf = [&](double acc) { return etype == TNT_TRUNC_2NORM ? sqrt(acc) : acc; };
-    const double acc0 = unseen * inv * inv;  // never formed values, in normalised units
-    int64_t chi4 = n;
-    double acc = acc0;
-    if (!(errf(acc) < etol)) chi4 = n;
-    for (int keep = n - 1; keep >= 0 && errf(acc) < etol; --keep) {
-      acc += term(key[keep]);
-      if (errf(acc) < etol) chi4 = keep; else break;
-    }
-    int64_t chi = chi1;
-    if (chi2 < chi) chi = chi2;
-    if (chi3 < chi) chi = chi3;
-    if (chi4 < chi) chi = chi4;
+    int64_t chi = n < chi_max ? n : chi_max;
+    if (a > 0) chi = min(chi, prefix([&](double s) { return s >= a; }));
+    if (s0 > 0) chi = min(chi, prefix([&](double s) { return s / s0 >= rtol; }));
+    chi = min(chi, (int64_t)s_chi4);
     if (chi < 1) chi = 1;
     if (chi > n) chi = n;
-    double e = acc0, dsc = unseen;
-    for (int i = n - 1; i >= chi; --i) {
-      e += term(key[i]);
-      dsc += key[i] * key[i];
-    }
     res->chi = chi;
-    res->err = errf(e);
-    res->disc = dsc;
+    res->err = errf(acc0);
+    res->disc = unseen;
     res->norm2 = nrm2;
-    res->tie = (chi < n) && (key[chi - 1] - key[chi] < 1e-10 * s0);
+    res->tie = (chi < n) && (val((int)chi - 1) - val((int)chi) < 1e-10 * s0);
+    s_chi4 = (int)chi;
+  }
+  __syncthreads();
+  const int chi = s_chi4;
+  if (chi < n && tid == chi / m) {  // this thread holds the first discarded value
+    res->err = errf(acc0 + u[chi % m]);
+    res->disc = unseen + v[chi % m];
   }
 }
 

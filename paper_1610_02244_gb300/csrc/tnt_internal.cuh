@@ -67,6 +67,7 @@ struct Ctx {
   // arrival counters of the kernels that finish their reduction in the last CTA to arrive
   // (zero between launches: that CTA resets its counter)
   unsigned* d_count = nullptr;
+  unsigned gs_arrivals = 0;  // arrivals so far at the Gram-Schmidt step's grid barrier
   // counters (diagnostics, not hot-path state)
   int64_t launches = 0;
   // optional CUDA-event timing of one kernel class (tnt_profile_select)
@@ -167,6 +168,24 @@ struct GemmTask {
 int zgemm_tasks(Ctx* c, const std::vector<GemmTask>& tasks);
 // the same on the FP64 units alone
 int zgemm_fma_tasks(Ctx* c, const GemmTask* const* tasks, int n);
+// Products that repeat with the same shapes (oz.cu): tables and buffers from the scratch arena,
+// laid out once; the sides of fixed_sides (bit 0 A, bit 1 B) hold operands that do not change
+// and are sliced when the plan is built.  A task's B may be an offset from the vector given
+// at each run (add_b; null for absolute pointers).  The four kernels take one argument, for
+// graph nodes: oz_plan_args writes it.
+struct OzNode {
+  void* fn;
+  unsigned grid, block, smem;
+};
+struct OzPlan {
+  alignas(16) unsigned char args[128];
+  OzNode node[4];
+  double flop = 0;
+};
+size_t oz_plan_bytes(Ctx* c, const std::vector<GemmTask>& tasks);
+int oz_plan_build(Ctx* c, const std::vector<GemmTask>& tasks, int fixed_sides, OzPlan* p);
+void oz_plan_args(const OzPlan& p, const z* add_b, void* out);
+int oz_plan_run(Ctx* c, const OzPlan& p, const z* add_b);
 // FP64 FMA GEMMs only while the guard lives (paths that must not allocate)
 struct OzOff {
   Ctx* c;
@@ -223,7 +242,7 @@ int vec_dot(Ctx* c, const z* x, const z* y, int64_t n, z* d_dot);
 // vec_gs_eligible): w against V[0..k) (leading dimension n) twice, alpha[k-1] = Re <V_{k-1}|w>
 // of the first pass, beta[k-1] = |w| after the second, vnext = w / |w| (none if null); w
 // itself is left as it was.  vec_gs_reset before the first step of a solve: the grid barrier's
-// words (a barrier whose wait expired leaves them set).
+// count (a barrier whose wait expired leaves it behind).
 bool vec_gs_eligible(int64_t n);
 int vec_gs_reset(Ctx* c);
 int vec_gs_step(Ctx* c, const z* V, int k, const z* w, int64_t n, z* vnext, double* d_alpha,

@@ -173,6 +173,12 @@ struct U1Plan {
   GTask* d_g1 = nullptr; int4* d_g1tiles = nullptr; int n_g1tiles = 0;
   GTask* d_g4 = nullptr; int4* d_g4tiles = nullptr; int n_g4tiles = 0;
   int cap_g1tiles = 0, cap_g4tiles = 0;
+  PackSeg *d_segA1 = nullptr, *d_segB4 = nullptr;
+  // FP64 stages as planned slice products (oz.cu) where their work pays for the launches
+  bool oz = false;
+  OzPlan oz1, oz4;
+  bool mixed_ready = false;  // split-TF32 operands packed and tiles chosen (on first use)
+  int runs[2] = {0, 0};      // matvecs so far per precision: the graph is built at the second
   // tile choice (autotuned): N tile of stage 1 and stage 4, split-K of stage 4
   int bn1 = 128, bn4 = 128, split4 = 1;
   int ztile = 64;                   // FP64 grouped tiles: 64 x 64, or 16 x 16 for small structures
@@ -181,6 +187,7 @@ struct U1Plan {
   cudaGraph_t graph[2] = {nullptr, nullptr};
   cudaGraphExec_t exec[2] = {nullptr, nullptr};
   cudaGraphNode_t in_node[2] = {nullptr, nullptr}, out_node[2] = {nullptr, nullptr};
+  cudaGraphNode_t oz_node[2] = {nullptr, nullptr};  // the two kernels that read the input
   TPArgs in_tp{};
   ZGArgs in_zg{};
   GthArgs out_g[2]{};
@@ -192,9 +199,11 @@ struct U1Plan {
 
 // host layout of the grouped matvec (no device work); sets p->bytes
 int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p);
-// device buffers from the scratch arena (p->bytes must fit), packed constant operands,
-// tables, and the autotuned tile choice
+// device buffers from the scratch arena (p->bytes must fit), tables and packed FP64 operands;
+// the split-TF32 operands and the autotuned tile choice follow at the first such matvec
 int u1_prepare(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p);
+// chooses the split-TF32 tiles of these problems' block structure
+int u1_tune(Ctx* c, const std::vector<U1Spec>& probs);
 int u1_run(Ctx* c, U1Plan& p, const z* x, z* y, int precision);
 // compact length of one problem, and dense <-> compact conversion of theta
 int64_t u1_compact_size(const U1Spec& s);

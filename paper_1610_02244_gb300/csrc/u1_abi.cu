@@ -187,6 +187,10 @@ int tnt_u1_tiles(tnt_ctx* ctx, int nprob, const tnt_u1_problem* probs, int* h_ti
   TNT_TRY(u1_layout(c, specs, &p));
   auto it = c->tune.find(p.sig);
   if (it == c->tune.end()) return set_err(c, TNT_E_INVALID, "block structure not tuned yet");
+  if (it->second.empty()) {  // only FP64 matvecs so far
+    TNT_TRY(u1_tune(c, specs));
+    it = c->tune.find(p.sig);
+  }
   for (int i = 0; i < 3; ++i) h_tiles[i] = it->second[(size_t)i];
   return TNT_OK;
 }
