@@ -538,16 +538,7 @@ OZ_TENSOR_PER_USEFUL = 36.0  # slice pairs per complex product: 36 x 4 real MMAs
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
 # capture per kernel class, valid while the class's source file is unchanged: class ->
 # (bytes per launch, source file under csrc/, sha256 prefix of that file, capture).
-TRAFFIC = {
-    # both launches of one matvec (T1 = L theta: 22.78 + 1.90 MB; y = T3 R^T: 71.63 + 3.22 MB),
-    # averaged: profiles/cgemm_tf32x3_heff_cfg2.md (the key follows the file; since the
-    # capture only the gather kernel in it changed)
-    "cgemm_tf32x3": (49.76e6, "tc_mixed.cu", "8430c4ff3cf17339", "ncu, bench.py update step"),
-    # two launches per update: the 1024-row Gram block (16.93 MB, ncu; the matrix read once)
-    # and the ~231-row tail block (its entries x the same 16.1 B per entry: 0.86 MB), averaged:
-    # profiles/tridiag_rows_gram1024.md
-    "heig_tridiag": (8.9e6, "heig.cu", "6808812dfa05a999", "ncu, svd_large_block_cfg2_shape"),
-}
+TRAFFIC = {}
 
 
 def traffic_for(cls):

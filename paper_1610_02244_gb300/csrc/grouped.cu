@@ -136,32 +136,7 @@ __global__ void __launch_bounds__(192, 1) k_cgemm_grouped(const __grid_constant_
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t base = su32(smem + s * Cf::STAGE);
-        for (int ks = 0; ks < 2; ++ks) {  // K = 8 per tf32 MMA: 32 bytes along the row
-          const uint32_t off = ks * 32;
-          const uint64_t a_rh = desc_sw64(base + 0 * Cf::TILE_A + off);
-          const uint64_t a_rl = desc_sw64(base + 1 * Cf::TILE_A + off);
-          const uint64_t a_ih = desc_sw64(base + 2 * Cf::TILE_A + off);
-          const uint64_t a_il = desc_sw64(base + 3 * Cf::TILE_A + off);
-          const uint32_t bb = base + 4 * Cf::TILE_A;
-          const uint64_t b_rh = desc_sw64(bb + 0 * Cf::TILE_B + off);
-          const uint64_t b_rl = desc_sw64(bb + 1 * Cf::TILE_B + off);
-          const uint64_t b_ih = desc_sw64(bb + 2 * Cf::TILE_B + off);
-          const uint64_t b_il = desc_sw64(bb + 3 * Cf::TILE_B + off);
-          const uint32_t first = (kb == kb0 && ks == 0) ? 0u : 1u;
-          mma_tf32(t_re, a_rh, b_rh, id, first);
-          mma_tf32(t_re, a_rh, b_rl, id, 1);
-          mma_tf32(t_re, a_rl, b_rh, id, 1);
-          mma_tf32(t_rn, a_ih, b_ih, id, first);
-          mma_tf32(t_rn, a_ih, b_il, id, 1);
-          mma_tf32(t_rn, a_il, b_ih, id, 1);
-          mma_tf32(t_im, a_rh, b_ih, id, first);
-          mma_tf32(t_im, a_rh, b_il, id, 1);
-          mma_tf32(t_im, a_rl, b_ih, id, 1);
-          mma_tf32(t_im, a_ih, b_rh, id, 1);
-          mma_tf32(t_im, a_ih, b_rl, id, 1);
-          mma_tf32(t_im, a_il, b_rh, id, 1);
-        }
+        mma_cplx_tf32x3<Cf::TILE_A, Cf::TILE_B>(su32(smem + s * Cf::STAGE), t_re, t_im, t_rn, id, kb == kb0);
         mma_commit(&empty[s]);
         ++it;
       }
@@ -192,14 +167,12 @@ __global__ void __launch_bounds__(192, 1) k_cgemm_grouped(const __grid_constant_
         tmem_ld32(tmem + lane_addr + BN + c0, s);
         tmem_ld32(tmem + lane_addr + 2 * BN + c0, u);
         if (gm < tk.M) {
-          float* pr = Cre + gm * tk.ldc + tl.z + c0;
-          float* pi = Cim + gm * tk.ldc + tl.z + c0;
+          const int nc = min(32, tk.N - tl.z - c0);
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (tl.z + c0 + j < tk.N) {
-              pr[j] = __uint_as_float(r[j]) - __uint_as_float(u[j]);
-              pi[j] = __uint_as_float(s[j]);
-            }
+          for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) - __uint_as_float(u[j]));
+          if (nc > 0) {
+            store_row32(Cre + gm * tk.ldc + tl.z + c0, r, nc);
+            store_row32(Cim + gm * tk.ldc + tl.z + c0, s, nc);
           }
         }
       }
@@ -305,8 +278,7 @@ __global__ void __launch_bounds__(256) k_zgemm_grouped16(ZGArgs g) {
         Bs[ty][tx] = (gj < tk.N && gk < tk.K) ? B[gk * tk.b_rs + gj * tk.b_cs] : zmk(0, 0);
       }
       __syncthreads();
-#pragma unroll
-      for (int kk = 0; kk < 16; ++kk) zfma(acc, As[ty][kk], Bs[kk][tx]);
+      tile16_fma(acc, As, Bs, (int)min((int64_t)16, tk.M - tl.y), (int)min((int64_t)16, tk.K - k0));
       __syncthreads();
     }
     const int64_t gi = tl.y + ty, gj = tl.z + tx;
@@ -373,6 +345,9 @@ __global__ void __launch_bounds__(256) k_pack_theta_t(TPArgs a) {
 
 // ---------------------------------------------------------------- W contraction
 constexpr int W_MAX_OUT = 256, W_MAX_IN = 1024, W_TILE = 256;
+// A tile is up to W_TILE elements of one block pair; its (output, element) combinations are
+// dealt to the threads of gridDim.y CTAs, elements fastest, so that a pair of small
+// sectors (a few elements, dozens of outputs) still fills its warps.
 template <bool MIXED>
 __global__ void __launch_bounds__(256) k_wop(WArgs a) {
   __shared__ int64_t s_obase[W_MAX_OUT];
@@ -383,52 +358,70 @@ __global__ void __launch_bounds__(256) k_wop(WArgs a) {
   for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
     const int2 tl = a.tiles[t];
     const WPair pr = a.pairs[tl.x];
-    const int r_first = a.outs[pr.out0].r0;
-    const int r_last = a.outs[pr.out0 + pr.nout - 1].r1;
-    for (int i = threadIdx.x; i < pr.nout; i += blockDim.x) {
-      const WOut o = a.outs[pr.out0 + i];
+    // this CTA's outputs of the pair
+    const int per = (pr.nout + (int)gridDim.y - 1) / (int)gridDim.y, o0 = (int)blockIdx.y * per;
+    const int no = min(per, pr.nout - o0);
+    if (no <= 0) continue;
+    const int r_first = a.outs[pr.out0 + o0].r0;
+    const int r_last = a.outs[pr.out0 + o0 + no - 1].r1;
+    for (int i = threadIdx.x; i < no; i += blockDim.x) {
+      const WOut o = a.outs[pr.out0 + o0 + i];
       s_obase[i] = o.base;
       s_r0[i] = o.r0 - r_first;
       s_r1[i] = o.r1 - r_first;
     }
+    int cplx = 0;
     for (int i = threadIdx.x; i < r_last - r_first; i += blockDim.x) {
       const WIn w = a.ins[r_first + i];
       s_ibase[i] = w.base;
       s_irs[i] = w.rs;
       s_val[i] = w.val;
+      cplx |= w.val.y != 0.0;
     }
-    __syncthreads();
-    const int64_t e = (int64_t)tl.y + threadIdx.x;
-    if (e < pr.n_a * pr.n_b) {
+    cplx = __syncthreads_or(cplx);  // real entries (the models' MPOs): half the FP64 work
+    const int ne = (int)min((int64_t)W_TILE, pr.n_a * pr.n_b - tl.y);
+    for (int q = threadIdx.x; q < ne * no; q += blockDim.x) {
+      const int64_t e = (int64_t)tl.y + q % ne;
+      const int o = q / ne;
       const int64_t ia = e / pr.n_b, jb = e % pr.n_b;
-      for (int o = 0; o < pr.nout; ++o) {
-        const int64_t dst = s_obase[o] + ia * a.out_rs + jb;
-        if (MIXED) {
-          float xr = 0.f, xi = 0.f;
-          for (int r = s_r0[o]; r < s_r1[o]; ++r) {
-            const int64_t src = s_ibase[r] + ia * s_irs[r] + jb;
-            const float vr = a.t1f[src], vi = a.t1f[a.p1 + src];
-            const float wr = (float)s_val[r].x, wi = (float)s_val[r].y;
-            xr = fmaf(wr, vr, fmaf(-wi, vi, xr));
-            xi = fmaf(wr, vi, fmaf(wi, vr, xi));
-          }
-          float h, l;
-          split_tf32(xr, &h, &l);
-          a.a4f[dst] = h;
-          a.a4f[a.p4 + dst] = l;
-          split_tf32(xi, &h, &l);
-          a.a4f[2 * a.p4 + dst] = h;
-          a.a4f[3 * a.p4 + dst] = l;
-        } else {
-          z acc = zmk(0, 0);
-          for (int r = s_r0[o]; r < s_r1[o]; ++r)
-            zfma(acc, s_val[r], a.t1z[s_ibase[r] + ia * s_irs[r] + jb]);
-          a.a4z[dst] = acc;
+      const int64_t dst = s_obase[o] + ia * a.out_rs + jb;
+      if (MIXED) {
+        float xr = 0.f, xi = 0.f;
+        for (int r = s_r0[o]; r < s_r1[o]; ++r) {
+          const int64_t src = s_ibase[r] + ia * s_irs[r] + jb;
+          const float vr = a.t1f[src], vi = a.t1f[a.p1 + src];
+          const float wr = (float)s_val[r].x, wi = (float)s_val[r].y;
+          xr = fmaf(wr, vr, fmaf(-wi, vi, xr));
+          xi = fmaf(wr, vi, fmaf(wi, vr, xi));
         }
+        float h, l;
+        split_tf32(xr, &h, &l);
+        a.a4f[dst] = h;
+        a.a4f[a.p4 + dst] = l;
+        split_tf32(xi, &h, &l);
+        a.a4f[2 * a.p4 + dst] = h;
+        a.a4f[3 * a.p4 + dst] = l;
+      } else {
+        z acc = zmk(0, 0);
+        if (cplx) {
+          for (int r = s_r0[o]; r < s_r1[o]; ++r) zfma(acc, s_val[r], a.t1z[s_ibase[r] + ia * s_irs[r] + jb]);
+        } else {
+          for (int r = s_r0[o]; r < s_r1[o]; ++r) {
+            const z v = a.t1z[s_ibase[r] + ia * s_irs[r] + jb];
+            acc.x = fma(s_val[r].x, v.x, acc.x);
+            acc.y = fma(s_val[r].x, v.y, acc.y);
+          }
+        }
+        a.a4z[dst] = acc;
       }
     }
     __syncthreads();
   }
+}
+// output groups (gridDim.y) per tile: about four CTAs per SM
+inline dim3 wop_grid(int ntiles) {
+  const int gx = std::max(1, std::min(ntiles, 152 * 8));
+  return dim3((unsigned)gx, (unsigned)std::max(1, std::min(16, 152 * 4 / gx)));
 }
 
 // ---------------------------------------------------------------- gather
@@ -704,7 +697,8 @@ int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
   // pass 1: task shapes (KA1, KA4 need every task's K)
   struct P1Info { std::vector<std::vector<int64_t>> rowoff1; std::vector<int> task1; };
   std::vector<P1Info> info1(probs.size());
-  struct P4Info { std::vector<std::map<int64_t, int64_t>> rowoff4; std::vector<std::vector<int64_t>> koff4; std::vector<int> task4; };
+  // rowoff4: per right sector, indexed by (left sector, s1, s2): -1 if absent
+  struct P4Info { std::vector<std::vector<int64_t>> rowoff4; std::vector<std::vector<int64_t>> koff4; std::vector<int> task4; };
   std::vector<P4Info> info4(probs.size());
   for (size_t pi = 0; pi < probs.size(); ++pi) {
     const U1Spec& s = probs[pi];
@@ -737,13 +731,13 @@ int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
     P4Info& i4 = info4[pi];
     for (size_t jQ = 0; jQ < l.Rs.size(); ++jQ) {
       const Sector& sQ = l.Rs[jQ];
-      std::map<int64_t, int64_t> ro;
+      std::vector<int64_t> ro(l.Ls.size() * (size_t)(d * d), -1);
       int64_t M = 0;
       for (size_t iL = 0; iL < l.Ls.size(); ++iL)
         for (int64_t s1 = 0; s1 < d; ++s1)
           for (int64_t s2 = 0; s2 < d; ++s2)
             if (l.Ls[iL].q + s1 + s2 == sQ.q) {
-              ro[((int64_t)iL * d + s1) * d + s2] = M;
+              ro[(size_t)(((int64_t)iL * d + s1) * d + s2)] = M;
               M += l.Ls[iL].size;
             }
       std::vector<int64_t> ko((size_t)D, -1);
@@ -771,6 +765,41 @@ int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
   if (p->s1.empty() || p->s4.empty()) return set_err(c, TNT_E_INVALID, "U(1) problem has no allowed blocks");
   if (p->rowsA1 + 256 > INT32_MAX || p->rowsA4 + 256 > INT32_MAX || p->rowsB1 + 256 > INT32_MAX)
     return set_err(c, TNT_E_INVALID, "grouped matvec too large for 32-bit tile coordinates");
+  // device copies of W without a host copy, all in one read-back
+  std::vector<std::vector<z>> hW(2 * probs.size());
+  {
+    size_t need = 0;
+    for (const U1Spec& s : probs) need += (size_t)(2 * s.D * s.D * s.d * s.d) * sizeof(z) * ((s.hW1 && s.hW2) ? 0 : 1);
+    if (need) {
+      TNT_TRY(pinned_reserve(c, need));
+      char* h = (char*)c->h_pinned;
+      for (int pass = 0; pass < 2; ++pass) {
+        size_t off = 0;
+        for (size_t pi = 0; pi < probs.size(); ++pi) {
+          const U1Spec& s = probs[pi];
+          if (s.hW1 && s.hW2) continue;
+          const size_t n = (size_t)(s.D * s.D * s.d * s.d);
+          for (int k = 0; k < 2; ++k, off += n * sizeof(z)) {
+            if (pass == 0)
+              TNT_CUDA_TRY(c, cudaMemcpyAsync(h + off, k ? s.W2 : s.W1, n * sizeof(z), cudaMemcpyDeviceToHost, c->stream));
+            else
+              hW[2 * pi + (size_t)k].assign((const z*)(h + off), (const z*)(h + off) + n);
+          }
+        }
+        if (pass == 0) TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+      }
+    }
+  }
+  std::vector<z> W12;
+  std::vector<std::vector<int>> nz2, cols;
+  {
+    size_t nr = 0, ns = 0;
+    for (const TaskDesc& t : p->s4) nr += (size_t)t.M;
+    for (const U1Spec& s : probs) ns += (size_t)(s.chl + s.chr) * (size_t)s.D;
+    p->rows.reserve(nr);
+    p->segA1.reserve(ns);
+    p->segB4.reserve(ns);
+  }
   // pass 2: pack segments, theta slabs, W pairs, output rows
   for (size_t pi = 0; pi < probs.size(); ++pi) {
     const U1Spec& s = probs[pi];
@@ -778,28 +807,42 @@ int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
     const int64_t d = s.d, D = s.D;
     const P1Info& i1 = info1[pi];
     const P4Info& i4 = info4[pi];
-    // W12[(s1' s2' w2), (w s1 s2)] = sum_w1 W1[w,w1,s1',s1] W2[w1,w2,s2',s2]  (host, FP64)
-    std::vector<z> W1((size_t)(D * D * d * d)), W2((size_t)(D * D * d * d));
-    if (s.hW1) std::copy(s.hW1, s.hW1 + W1.size(), W1.begin());
-    else TNT_TRY(read_small(c, s.W1, W1.data(), W1.size() * sizeof(z)));
-    if (s.hW2) std::copy(s.hW2, s.hW2 + W2.size(), W2.begin());
-    else TNT_TRY(read_small(c, s.W2, W2.data(), W2.size() * sizeof(z)));
-    auto at = [&](const std::vector<z>& W, int64_t w, int64_t wp, int64_t so, int64_t si) {
-      return W[(size_t)(((w * D + wp) * d + so) * d + si)];
-    };
+    // W12[(s1' s2' w2), (w s1 s2)] = sum_w1 W1[w,w1,s1',s1] W2[w1,w2,s2',s2]  (host, FP64),
+    // from the non-zero entries of the two tensors; per row its non-zero columns in order
+    const z* W1 = s.hW1 ? s.hW1 : hW[2 * pi].data();
+    const z* W2 = s.hW2 ? s.hW2 : hW[2 * pi + 1].data();
     const int64_t nI = d * d * D, nJ = D * d * d;
-    std::vector<z> W12((size_t)(nI * nJ), zmk(0, 0));
-    for (int64_t s1o = 0; s1o < d; ++s1o)
-      for (int64_t s2o = 0; s2o < d; ++s2o)
-        for (int64_t w2 = 0; w2 < D; ++w2)
-          for (int64_t w = 0; w < D; ++w)
-            for (int64_t s1 = 0; s1 < d; ++s1)
-              for (int64_t s2 = 0; s2 < d; ++s2) {
-                z acc = zmk(0, 0);
-                for (int64_t w1 = 0; w1 < D; ++w1)
-                  zfma(acc, at(W1, w, w1, s1o, s1), at(W2, w1, w2, s2o, s2));
-                W12[(size_t)((((s1o * d + s2o) * D + w2) * nJ) + (w * d + s1) * d + s2)] = acc;
-              }
+    W12.assign((size_t)(nI * nJ), zmk(0, 0));
+    nz2.assign((size_t)D, {});
+    for (int64_t w1 = 0; w1 < D; ++w1)
+      for (int64_t e = 0; e < D * d * d; ++e) {  // e = (w2, s2', s2)
+        const z v = W2[w1 * D * d * d + e];
+        if (v.x != 0.0 || v.y != 0.0) nz2[(size_t)w1].push_back((int)e);
+      }
+    for (int64_t w1 = 0; w1 < D; ++w1)
+      for (int64_t w = 0; w < D; ++w)
+        for (int64_t s1o = 0; s1o < d; ++s1o)
+          for (int64_t s1 = 0; s1 < d; ++s1) {
+            const z u = W1[((w * D + w1) * d + s1o) * d + s1];
+            if (u.x == 0.0 && u.y == 0.0) continue;
+            for (int e : nz2[(size_t)w1]) {
+              const int64_t w2 = e / (d * d), s2o = (e / d) % d, s2 = e % d;
+              zfma(W12[(size_t)(((s1o * d + s2o) * D + w2) * nJ + (w * d + s1) * d + s2)], u, W2[w1 * D * d * d + e]);
+            }
+          }
+    cols.assign((size_t)nI, {});
+    for (int64_t i = 0; i < nI; ++i)
+      for (int64_t j = 0; j < nJ; ++j) {
+        const z v = W12[(size_t)(i * nJ + j)];
+        if (v.x != 0.0 || v.y != 0.0) cols[(size_t)i].push_back((int)j);
+      }
+    // sector index of a charge, as left sector shifted by -wq[w] and as right sector
+    std::vector<int> lsh(l.Ls.size() * (size_t)D, -1);
+    for (size_t i = 0; i < l.Ls.size(); ++i)
+      for (int64_t w = 0; w < D; ++w) {
+        auto it = l.Li.find(l.Ls[i].q - s.wq[(size_t)w]);
+        if (it != l.Li.end()) lsh[i * (size_t)D + (size_t)w] = it->second;
+      }
     // stage 1 operands
     for (size_t iL = 0; iL < l.Ls.size(); ++iL) {
       const int ti = i1.task1[iL];
@@ -833,8 +876,9 @@ int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
           p->segB4.push_back(PackSeg{s.R + ((sQ.start + b) * D + w2) * s.chr + sb.start,
                                      (t.b_row0 + b) * p->KA4 + ko, sb.size});
         }
-      for (const auto& kv : i4.rowoff4[jQ]) {
-        const int64_t key = kv.first, ro = kv.second;
+      for (int64_t key = 0; key < (int64_t)i4.rowoff4[jQ].size(); ++key) {
+        const int64_t ro = i4.rowoff4[jQ][(size_t)key];
+        if (ro < 0) continue;
         const int64_t iL = key / (d * d), s12 = key % (d * d);
         const Sector& sa = l.Ls[(size_t)iL];
         for (int64_t a = 0; a < sa.size; ++a)
@@ -860,27 +904,21 @@ int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
               const int jQ = itQ->second;
               const int t4 = i4.task4[(size_t)jQ];
               const TaskDesc& T4 = p->s4[(size_t)t4];
-              const int64_t ro = i4.rowoff4[(size_t)jQ].at(((int64_t)iLp * d + s1o) * d + s2o);
+              const int64_t ro = i4.rowoff4[(size_t)jQ][(size_t)(((int64_t)iLp * d + s1o) * d + s2o)];
               const int64_t ko = i4.koff4[(size_t)jQ][(size_t)w2];
               WOut o{(T4.a_row0 + ro) * p->KA4 + ko, (int)p->ins.size(), 0};
-              const int64_t irow = ((s1o * d + s2o) * D + w2) * nJ;
-              for (int64_t w = 0; w < D; ++w) {
-                auto itq = l.Li.find(sa.q - s.wq[(size_t)w]);
-                if (itq == l.Li.end()) continue;
-                const int iL = itq->second;
+              const int64_t i = (s1o * d + s2o) * D + w2;
+              for (int j : cols[(size_t)i]) {
+                const int64_t w = j / (d * d), s1 = (j / d) % d, s2 = j % d;
+                const int iL = lsh[iLp * (size_t)D + (size_t)w];
+                if (iL < 0 || l.Ls[(size_t)iL].q + s1 + s2 != sb.q) continue;
                 const int t1 = i1.task1[(size_t)iL];
                 if (t1 < 0) continue;
                 const TaskDesc& T1 = p->s1[(size_t)t1];
                 const int64_t ro1 = i1.rowoff1[(size_t)iL][(size_t)w];
-                for (int64_t s1 = 0; s1 < d; ++s1)
-                  for (int64_t s2 = 0; s2 < d; ++s2) {
-                    if (l.Ls[(size_t)iL].q + s1 + s2 != sb.q) continue;
-                    const z v = W12[(size_t)(irow + (w * d + s1) * d + s2)];
-                    if (v.x == 0.0 && v.y == 0.0) continue;
-                    const int64_t co = l.coff[(size_t)iL][(size_t)(s1 * d + s2)];
-                    p->ins.push_back(WIn{T1.c_off + ro1 * T1.ldc + co, T1.ldc, v});
-                    p->flops += 8.0 * (double)sa.size * (double)sb.size;
-                  }
+                const int64_t co = l.coff[(size_t)iL][(size_t)(s1 * d + s2)];
+                p->ins.push_back(WIn{T1.c_off + ro1 * T1.ldc + co, T1.ldc, W12[(size_t)(i * nJ + j)]});
+                p->flops += 8.0 * (double)sa.size * (double)sb.size;
               }
               o.r1 = (int)p->ins.size();
               if (o.r1 - o.r0 > W_MAX_IN) return set_err(c, TNT_E_INVALID, "W contraction: too many terms for one output");
@@ -1152,10 +1190,10 @@ void zlaunch(Ctx* c, const U1Plan& p, const ZGArgs& a, int ntiles) {
 }
 
 // kernel-node parameters for a graph; args points at the single struct argument
-cudaKernelNodeParams knp(void* fn, unsigned grid, unsigned block, unsigned smem, void** args) {
+cudaKernelNodeParams knp(void* fn, dim3 grid, unsigned block, unsigned smem, void** args) {
   cudaKernelNodeParams k{};
   k.func = fn;
-  k.gridDim = dim3(grid);
+  k.gridDim = grid;
   k.blockDim = dim3(block);
   k.sharedMemBytes = smem;
   k.kernelParams = args;
@@ -1174,7 +1212,7 @@ int build_graph(Ctx* c, U1Plan& p, int mixed) {
     return TNT_OK;
   };
   WArgs wa = wargs(p);
-  const unsigned gw = cap_grid(p.n_wtiles, 152 * 8);
+  const dim3 gw = wop_grid(p.n_wtiles);
   const unsigned gg = cap_grid((p.n_rows + 7) / 8, 152 * 8);
   if (mixed) {
     TPArgs tp = p.in_tp;
@@ -1235,7 +1273,7 @@ int build_graph(Ctx* c, U1Plan& p, int mixed) {
 
 int run_direct(Ctx* c, U1Plan& p, const z* x, z* y, int mixed) {
   WArgs wa = wargs(p);
-  const unsigned gw = cap_grid(p.n_wtiles, 152 * 8);
+  const dim3 gw = wop_grid(p.n_wtiles);
   const unsigned gg = cap_grid((p.n_rows + 7) / 8, 152 * 8);
   if (mixed) {
     TPArgs tp = p.in_tp;

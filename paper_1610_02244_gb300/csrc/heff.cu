@@ -9,8 +9,18 @@
 namespace tnt {
 
 int read_small(Ctx* c, const void* dsrc, void* hdst, size_t bytes) {
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(hdst, dsrc, bytes, cudaMemcpyDeviceToHost, c->stream));
+  return read_small2(c, dsrc, hdst, bytes, nullptr, nullptr, 0);
+}
+
+// two small device arrays to the host with one wait, through the pinned buffer
+int read_small2(Ctx* c, const void* d1, void* h1, size_t b1, const void* d2, void* h2, size_t b2) {
+  TNT_TRY(pinned_reserve(c, b1 + b2));
+  char* h = (char*)c->h_pinned;
+  TNT_CUDA_TRY(c, cudaMemcpyAsync(h, d1, b1, cudaMemcpyDeviceToHost, c->stream));
+  if (b2) TNT_CUDA_TRY(c, cudaMemcpyAsync(h + b1, d2, b2, cudaMemcpyDeviceToHost, c->stream));
   TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  memcpy(h1, h, b1);
+  if (b2) memcpy(h2, h + b1, b2);
   return TNT_OK;
 }
 
@@ -21,30 +31,29 @@ size_t heff_scratch_bound(int64_t chl, int64_t d, int64_t D, int64_t chr, int pr
   return b;
 }
 
-// W12[(s1',s2',w2),(w,s1,s2)] = sum_w1 W1[w,w1,s1',s1] W2[w1,w2,s2',s2]  (host, tiny)
+// W12[(s1',s2',w2),(w,s1,s2)] = sum_w1 W1[w,w1,s1',s1] W2[w1,w2,s2',s2]  (host, tiny; from the
+// non-zero entries of the two tensors, w1 ascending)
 static void build_w12(const std::vector<z>& W1, const std::vector<z>& W2, int64_t d, int64_t D,
                       std::vector<z>* W12) {
-  const int64_t nI = d * d * D, nJ = D * d * d;
+  const int64_t nI = d * d * D, nJ = D * d * d, slab = D * d * d;
   W12->assign((size_t)(nI * nJ), zmk(0, 0));
-  auto at1 = [&](int64_t w, int64_t v, int64_t so, int64_t si) {
-    return W1[(size_t)(((w * D + v) * d + so) * d + si)];
-  };
-  auto at2 = [&](int64_t w, int64_t v, int64_t so, int64_t si) {
-    return W2[(size_t)(((w * D + v) * d + so) * d + si)];
-  };
-  for (int64_t s1o = 0; s1o < d; ++s1o)
-    for (int64_t s2o = 0; s2o < d; ++s2o)
-      for (int64_t w2 = 0; w2 < D; ++w2) {
-        const int64_t i = (s1o * d + s2o) * D + w2;
-        for (int64_t w = 0; w < D; ++w)
-          for (int64_t s1 = 0; s1 < d; ++s1)
-            for (int64_t s2 = 0; s2 < d; ++s2) {
-              const int64_t j = (w * d + s1) * d + s2;
-              z acc = zmk(0, 0);
-              for (int64_t w1 = 0; w1 < D; ++w1) zfma(acc, at1(w, w1, s1o, s1), at2(w1, w2, s2o, s2));
-              (*W12)[(size_t)(i * nJ + j)] = acc;
-            }
-      }
+  std::vector<int> nz;
+  for (int64_t w1 = 0; w1 < D; ++w1) {
+    const z* v2 = W2.data() + w1 * slab;  // (w2, s2', s2)
+    nz.clear();
+    for (int64_t e = 0; e < slab; ++e)
+      if (v2[e].x != 0.0 || v2[e].y != 0.0) nz.push_back((int)e);
+    for (int64_t w = 0; w < D; ++w)
+      for (int64_t s1o = 0; s1o < d; ++s1o)
+        for (int64_t s1 = 0; s1 < d; ++s1) {
+          const z u = W1[(size_t)(((w * D + w1) * d + s1o) * d + s1)];
+          if (u.x == 0.0 && u.y == 0.0) continue;
+          for (int e : nz) {
+            const int64_t w2 = e / (d * d), s2o = (e / d) % d, s2 = e % d;
+            zfma((*W12)[(size_t)(((s1o * d + s2o) * D + w2) * nJ + (w * d + s1) * d + s2)], u, v2[e]);
+          }
+        }
+  }
 }
 
 int heff_prepare(Ctx* c, const z* L, const z* W1, const z* W2, const z* R, int64_t chl,
@@ -59,10 +68,12 @@ int heff_prepare(Ctx* c, const z* L, const z* W1, const z* W2, const z* R, int64
   p->precision = precision;
   const size_t nW = (size_t)(D * D * d * d);
   std::vector<z> h1(nW), h2(nW), w12;
-  if (hW1) std::copy(hW1, hW1 + nW, h1.begin());
-  else TNT_TRY(read_small(c, W1, h1.data(), nW * sizeof(z)));
-  if (hW2) std::copy(hW2, hW2 + nW, h2.begin());
-  else TNT_TRY(read_small(c, W2, h2.data(), nW * sizeof(z)));
+  if (hW1 && hW2) {
+    std::copy(hW1, hW1 + nW, h1.begin());
+    std::copy(hW2, hW2 + nW, h2.begin());
+  } else {
+    TNT_TRY(read_small2(c, W1, h1.data(), nW * sizeof(z), W2, h2.data(), nW * sizeof(z)));
+  }
   build_w12(h1, h2, d, D, &w12);
   const int nI = (int)(d * d * D), nJ = (int)(D * d * d);
   std::vector<int64_t> in_off(nJ), out_off(nI);

@@ -25,6 +25,7 @@ namespace tnt {
 
 namespace {
 constexpr double EPS = 2.220446049250313e-16;
+constexpr double SPLIT_TOL = 1e3 * EPS;  // negligible against |T| (k_split)
 
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
@@ -157,13 +158,19 @@ __device__ double block_sum0(double v, double* sh) {
 // v = (1, conj(x_r) scale, ...) maps conj(x) to beta e_1, beta real.  Computed by one thread:
 // a full-block FP64 square root and three divisions cost more FP64-pipe issue slots on
 // GB300 than the vector work of a short column.
+// A row whose squares sum to less than 2^-900 counts as zero (no reflection): the blocks are
+// scaled to a largest entry of about one, and a matrix of low rank leaves trailing blocks of
+// 1e-16, 1e-32, 1e-48, ... whose squares would underflow after a few columns.
 struct Refl {
   z tau, scale;
   double beta;
 };
+__device__ __forceinline__ bool refl_none(z alpha, double xn2) {
+  return hi_exp(fma(alpha.x, alpha.x, fma(alpha.y, alpha.y, xn2))) < 1023 - 900 || (xn2 == 0.0 && alpha.y == 0.0);
+}
 __device__ Refl refl_params(z alpha, double xn2, bool empty) {
   Refl R;
-  if (empty || (xn2 == 0.0 && alpha.y == 0.0)) {
+  if (empty || refl_none(alpha, xn2)) {
     R.tau = zmk(0, 0);
     R.beta = alpha.x;
     R.scale = zmk(0, 0);
@@ -384,6 +391,12 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tridiag_persistent(TriArgs a) {
 //   group barrier.
 // Reflector j replaces row j of the block in global memory (columns 0 .. n-j-2), the layout
 // the back-transformation reads: no CTA reads row j after its barrier j.
+// A Gram matrix is positive semidefinite, so its trailing block is bounded by the block's
+// trace, which is what the diagonal entries found so far leave of the whole trace.  Once an
+// entry and what is left are both at most SPLIT_TOL / 4 times the largest entry, so is the
+// coupling (the square root of their product), and the reduction stops: the rest is the
+// negligible range that k_split takes off (d = e = 0, no reflectors).  A 5 : 1 block of a
+// centre move has a fifth of its columns left to do, theta of a truncated state about half.
 // Vectors are indexed by row of the block.  Per column a CTA spends 16 FP64 operations per
 // trailing entry on the shared vectors and 12 per entry of its rows: that work bounds large
 // blocks (two operations per SM and clock); small ones are bound by the sequence of about 60
@@ -450,31 +463,6 @@ __device__ bool group_barrier(const TriGroup& t, int grp, int nb, int j) {
   return s_ok != 0;
 }
 
-// 1 / sqrt(s) and 1 / d for normal positive s, d != 0: an FP32 seed (relative error e0 of about
-// 2^-22), one step of third order, y (1 + e/2 + 3/8 e^2) with e = 1 - s y^2, and
-// r (1 + e + e^2) with e = 1 - d r: the error left is of order e0^3, below FP64 rounding.
-// The arguments are scaled to [1, 4) and [1, 2) by exponent arithmetic.
-__device__ __forceinline__ double rsqrt_newton(double s) {
-  const int hi = __double2hiint(s), ex = (hi >> 20) - 1023, h = ex >> 1;
-  const double m = __hiloint2double((hi & 0xfffff) | ((1023 + (ex & 1)) << 20), __double2loint(s));
-  float y0;
-  asm("rsqrt.approx.f32 %0, %1;" : "=f"(y0) : "f"(f32_of(m)));
-  const double y = f64_of(y0);
-  const double e = fma(-m * y, y, 1.0);
-  const double r = fma(y, e * fma(e, 0.375, 0.5), y);
-  return __hiloint2double(__double2hiint(r) - (h << 20), __double2loint(r));
-}
-__device__ __forceinline__ double rcp_newton(double d) {
-  const int hi = __double2hiint(d), ex = ((hi >> 20) & 0x7ff) - 1023;
-  const double m = __hiloint2double((hi & 0x800fffff) | (1023 << 20), __double2loint(d));
-  float r0;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r0) : "f"(f32_of(m)));
-  const double r = f64_of(r0);
-  const double e = fma(-m, r, 1.0);
-  const double q = fma(r, fma(e, e, e), r);
-  return __hiloint2double(__double2hiint(q) - (ex << 20), __double2loint(q));
-}
-
 // (a, b) summed over the warp with five FP64 adds (the two sums share each step); every
 // lane returns both
 __device__ __forceinline__ void warp_sum_pair(double& a, double& b) {
@@ -515,6 +503,8 @@ struct RowsShared {
   GroupRefl rf[2];               // reflectors of even / odd columns
   z alpha;
   double cf, part;
+  double trace, dmax;            // of the trailing block; largest diagonal entry so far
+  int done;                      // the rest of the block is negligible
 };
 
 // Reflector parameters (refl_params) by one warp
@@ -523,10 +513,10 @@ __device__ GroupRefl refl_warp(z alpha, double xn2, bool empty) {
   R.tau = R.scale = zmk(0, 0);
   R.beta = alpha.x;
   R.c = 0;
-  if (empty || (xn2 == 0.0 && alpha.y == 0.0)) return R;
+  if (empty || refl_none(alpha, xn2)) return R;
   const double s = fma(alpha.x, alpha.x, fma(alpha.y, alpha.y, xn2));
   double nrm, inv;
-  if (hi_exp(s) > 100 && hi_exp(s) < 1946) {  // squares well inside the normal range
+  if (hi_exp(s) < 1946) {  // not below 2^-900
     inv = rsqrt_newton(s);
     nrm = s * inv;
   } else {
@@ -536,7 +526,7 @@ __device__ GroupRefl refl_warp(z alpha, double xn2, bool empty) {
   R.beta = alpha.x >= 0 ? -nrm : nrm;
   const z den = zmk(alpha.x - R.beta, alpha.y);  // scale = 1 / (alpha - beta), |den| >= nrm
   const double dd = fma(den.x, den.x, den.y * den.y);
-  const double rd = hi_exp(dd) > 100 && hi_exp(dd) < 1946 ? rcp_newton(dd) : 1.0 / dd;
+  const double rd = hi_exp(dd) < 1946 ? rcp_newton(dd) : 1.0 / dd;  // dd >= s
   const double rb = alpha.x >= 0 ? inv : -inv;  // -1 / beta
   R.tau = zmk(den.x * rb, alpha.y * rb);
   R.scale = zmk(den.x * rd, -den.y * rd);
@@ -692,6 +682,18 @@ __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_
   z* sx = sw + n;                    // x of the next reflector (its first entry zeroed)
   z* sp = sx + n;                    // p, in a group of one CTA
   const bool one = nb == 1;
+  if (scalar) {  // the trace, in the same order in every CTA
+    double s = 0;
+    for (int i = lane; i < n; i += 32) s += __ldcg(a.G + (int64_t)i * n + i).x;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+      const double d0 = __ldcg(a.G).x;
+      S.trace = s - d0;
+      S.dmax = d0;
+      S.done = 0;
+    }
+  }
   for (int i = 0; i < R; ++i) {
     const z* src = a.G + (b + (int64_t)nb * i) * n;
     for (int c = tid; c < n; c += TRI_GTHREADS) rows[(int64_t)i * n + c] = __ldcg(src + c);
@@ -783,8 +785,12 @@ __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_
         if (c < n) {
           const z xn = zmk(fma(-cf2, vc[k].x, tc[k].x), fma(cf2, vc[k].y, tc[k].y));
           sw[c] = zmk(fma(cf, vc[k].x, pc[k].x), fma(cf, vc[k].y, pc[k].y));
-          if (c == j + 1) {
+          if (c == j + 1) {  // thread 0
             if (b == 0) a.d[j + 1] = xn.x;
+            const double left = S.trace - xn.x, top = fmax(S.dmax, xn.x), tol = 0.25 * SPLIT_TOL * top;
+            S.trace = left;
+            S.dmax = top;
+            S.done = xn.x <= tol && left <= tol;
           } else if (c == j + 2) {
             S.alpha = zconj(xn);
             sx[c] = zmk(0, 0);
@@ -798,6 +804,15 @@ __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_
       if (lane == 0) S.nrm[warp] = acc;
     }
     __syncthreads();
+    if (S.done) {  // the same decision in every CTA of the group
+      if (b == 0)
+        for (int i = j + 1 + tid; i < n; i += TRI_GTHREADS) {
+          a.tau[i] = zmk(0, 0);
+          a.e[i] = 0.0;
+          if (i > j + 1) a.d[i] = 0.0;
+        }
+      return;
+    }
     const bool empty = n - j - 2 <= 0;  // length of reflector j+1
     if (scalar) {
       const GroupRefl rf = refl_warp(empty ? zmk(0, 0) : S.alpha, nrm_total(S), empty);
@@ -887,11 +902,10 @@ __global__ void __launch_bounds__(4 * WY_SUB) k_wy_t(const WySub* __restrict__ s
 // a step perturbs only d_i and e_{i-1} by O(eps) relative, so the count is that of a
 // matrix within O(eps |T|).  Division-free: a full-warp FP64 division costs several times
 // the FP64-pipe issue slots of these three operations.  The pair (p_{i-1}, p_i) is
-// rescaled by an exact power of two when its exponent leaves [-400, 400]; signs and
+// rescaled by an exact power of two when its exponent leaves [-400, 400]; e2 = e^2; signs and
 // exponents are read as integers.  A zero minor is replaced by 2^-60 |p_{i-1}| with the
 // sign opposite to its predecessor (the tiny negative pivot of the ratio form).
-__device__ int sturm_lt(const double* d, const double* e, int64_t n, double x, double pivmin) {
-  (void)pivmin;
+__device__ int sturm_lt(const double* d, const double* e2, int64_t n, double x) {
   double pm2 = 1.0, pm1 = d[0] - x;
   int neg_prev = 0;  // sign of p_0 = 1
   int cnt = 0;
@@ -900,8 +914,7 @@ __device__ int sturm_lt(const double* d, const double* e, int64_t n, double x, d
   cnt += neg != neg_prev;
   neg_prev = neg;
   for (int64_t i = 1; i < n; ++i) {
-    const double ei = e[i - 1];
-    double p = fma(d[i] - x, pm1, -(ei * ei) * pm2);
+    double p = fma(d[i] - x, pm1, -e2[i - 1] * pm2);
     if (p == 0.0) p = neg_prev ? 0x1p-60 * fabs(pm1) : -0x1p-60 * fabs(pm1);
     neg = __double2hiint(p) < 0;
     cnt += neg != neg_prev;
@@ -910,7 +923,32 @@ __device__ int sturm_lt(const double* d, const double* e, int64_t n, double x, d
     pm1 = p;
     const int ex = hi_exp(p);
     if (ex > 1023 + 400 || ex < 1023 - 400) {  // keep the pair in range: exact scaling
-      const double f = ldexp(1.0, 1023 - ex);
+      const double f = __hiloint2double((2046 - ex) << 20, 0);
+      pm1 *= f;
+      pm2 *= f;
+    }
+  }
+  return cnt;
+}
+// the same in FP32, for T scaled to entries of at most about one
+__device__ int sturm_lt32(const float* d, const float* e2, int64_t n, float x) {
+  float pm2 = 1.f, pm1 = d[0] - x;
+  int neg_prev = 0, cnt = 0;
+  if (pm1 == 0.f) pm1 = -0x1p-30f;
+  int neg = __float_as_int(pm1) < 0;
+  cnt += neg != neg_prev;
+  neg_prev = neg;
+  for (int64_t i = 1; i < n; ++i) {
+    float p = fmaf(d[i] - x, pm1, -e2[i - 1] * pm2);
+    if (p == 0.f) p = neg_prev ? 0x1p-30f * fabsf(pm1) : -0x1p-30f * fabsf(pm1);
+    neg = __float_as_int(p) < 0;
+    cnt += neg != neg_prev;
+    neg_prev = neg;
+    pm2 = pm1;
+    pm1 = p;
+    const int ex = (__float_as_int(p) >> 23) & 0xff;
+    if (ex > 127 + 40 || ex < 127 - 40) {
+      const float f = __int_as_float((254 - ex) << 23);
       pm1 *= f;
       pm2 *= f;
     }
@@ -941,7 +979,6 @@ struct EBlk {
 // eigenbasis to that accuracy: the canonical vectors e_s, ..., e_{n-1} are taken, exactly
 // orthonormal to each other and (zero beyond s) to the iterates of T[0, s), with no
 // inverse iteration.  One warp per problem: |T| (Gershgorin) to tnorm, s to nr.
-constexpr double SPLIT_TOL = 1e3 * 2.220446049250313e-16;
 __global__ void k_split(const double* __restrict__ dAll, const double* __restrict__ eAll,
                         const EBlk* __restrict__ blks, double* __restrict__ tnorm,
                         int64_t* __restrict__ nr) {
@@ -971,10 +1008,14 @@ __global__ void k_split(const double* __restrict__ dAll, const double* __restric
 // FP64 units favour short dependent chains over many of them.  Warp g works on eigenvalue
 // eig[g].y of problem eig[g].x, on the leading block T[0, s) of the split; indices from s
 // on belong to the negligible block and take its diagonal entry.
-__global__ void k_bisect(const double* __restrict__ dAll, const double* __restrict__ eAll,
+// The first four steps, down to 8e-7 of the Gershgorin interval, run on FP32 counts of T
+// scaled to that interval: such a count is exact for a matrix within a few FP32 roundings of
+// T, so the bracket is widened by 2e-6 of the interval and holds the eigenvalue (FP64 steps
+// cost a full FP64-pipe pass over T each, 3 instructions of 64 clocks per row).
+__global__ void __launch_bounds__(32) k_bisect(const double* __restrict__ dAll, const double* __restrict__ eAll,
                          const EBlk* __restrict__ blks, const int2* __restrict__ eig,
-                         const int64_t* __restrict__ nrAll, const double* __restrict__ tnorm,
-                         double* __restrict__ evAll) {
+                         const int64_t* __restrict__ nrAll, double* __restrict__ evAll) {
+  extern __shared__ double sm_bis[];  // e^2 (n), then the FP32 copies (2 n floats)
   const int lane = threadIdx.x & 31;
   const int2 gi = eig[blockIdx.x];
   const EBlk B = blks[gi.x];
@@ -985,31 +1026,51 @@ __global__ void k_bisect(const double* __restrict__ dAll, const double* __restri
     if (lane == 0) evAll[B.evo + i] = d[i];
     return;
   }
-  double lo = INFINITY, hi = -INFINITY, emax2 = 0;
+  double lo = INFINITY, hi = -INFINITY;
   for (int64_t r = lane; r < n; r += 32) {
-    const double rad = (r > 0 ? fabs(e[r - 1]) : 0.0) + (r < n - 1 ? fabs(e[r]) : 0.0);
+    const double er = r < n - 1 ? e[r] : 0.0;
+    const double rad = (r > 0 ? fabs(e[r - 1]) : 0.0) + fabs(er);
     lo = fmin(lo, d[r] - rad);
     hi = fmax(hi, d[r] + rad);
-    if (r < n - 1) emax2 = fmax(emax2, e[r] * e[r]);
+    sm_bis[r] = er * er;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
     hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    emax2 = fmax(emax2, __shfl_xor_sync(0xffffffffu, emax2, o));
   }
-  const double tn = tnorm[gi.x];
-  const double pivmin = fmax(1e-300, EPS * EPS * fmax(emax2, 1e-300)) + 1e-300;
   const int64_t idx = n - 1 - i;
-  const double pad = 2 * EPS * tn + 1e-300;
+  const double pad = 2 * EPS * fmax(fabs(lo), fabs(hi)) + 1e-300;
   lo -= pad;
   hi += pad;
+  const double w0 = hi - lo;
+  if (n > 1 && w0 > 1e-200 && w0 < 1e200) {
+    float* fd = (float*)(sm_bis + n);
+    float* fe = fd + n;
+    const double inv = 1.0 / w0;
+    for (int64_t r = lane; r < n; r += 32) {
+      fd[r] = (float)((d[r] - lo) * inv);
+      fe[r] = (float)(sm_bis[r] * inv * inv);
+    }
+    __syncwarp();
+    float fl = 0.f, fw = 1.f;
+    for (int it = 0; it < 4; ++it) {
+      const float x = fl + fw * (float)(lane + 1) * (1.f / 33.f);
+      const int p = __popc(__ballot_sync(0xffffffffu, sturm_lt32(fd, fe, n, x) <= (int)idx));
+      fl += fw * (float)p * (1.f / 33.f);
+      fw *= 1.f / 33.f;
+    }
+    const double l2 = lo + w0 * ((double)fl - 2e-6), h2 = lo + w0 * ((double)fl + (double)fw + 2e-6);
+    lo = fmax(lo, l2);
+    hi = fmin(hi, h2);
+  }
+  __syncwarp();
   const double tol = 1e-300;  // full precision: the shifts must resolve close eigenvalues
   for (int it = 0; it < 64; ++it) {
     const double width = hi - lo;
     if (width <= fmax(tol, 4 * EPS * fmax(fabs(lo), fabs(hi)))) break;
     const double x = lo + width * (double)(lane + 1) / 33.0;
-    const unsigned below = __ballot_sync(0xffffffffu, sturm_lt(d, e, n, x, pivmin) <= idx);
+    const unsigned below = __ballot_sync(0xffffffffu, sturm_lt(d, sm_bis, n, x) <= idx);
     const int p = __popc(below);  // points left of eigenvalue idx (counts are monotone)
     const double nlo = p > 0 ? lo + width * (double)p / 33.0 : lo;
     const double nhi = p < 32 ? lo + width * (double)(p + 1) / 33.0 : hi;
@@ -1209,8 +1270,9 @@ __global__ void __launch_bounds__(256) k_backtransform(const double* __restrict_
                                                        z* __restrict__ U0All) {
   extern __shared__ double sm_bt[];
   z* y = (z*)sm_bt;  // cols x n (cols = BT_COLS, or 1 when two vectors do not fit)
-  __shared__ double shr[8][BT_COLS], shi[8][BT_COLS];
+  __shared__ double shw[8][4];
   __shared__ z s_ts[BT_COLS];
+  static_assert(BT_COLS == 2, "four sums per reflector");
   const int2 gb = bt[blockIdx.x];
   const EBlk B = blks[gb.x];
   const int64_t n = B.n, k = B.k, i0 = gb.y;
@@ -1229,36 +1291,28 @@ __global__ void __launch_bounds__(256) k_backtransform(const double* __restrict_
     if (t.x == 0.0 && t.y == 0.0) continue;
     const int64_t m = n - j - 1;
     const z* v = Hv + j * n;
-    double sr[BT_COLS], si[BT_COLS];  // s = v^H y[j+1:] per column
-#pragma unroll
-    for (int q = 0; q < BT_COLS; ++q) sr[q] = si[q] = 0;
+    double s4[2 * BT_COLS] = {0, 0, 0, 0};  // s = v^H y[j+1:] per column, (re, im) pairs
     for (int64_t r = threadIdx.x; r < m; r += blockDim.x) {
       const z a = v[r];
 #pragma unroll
       for (int q = 0; q < BT_COLS; ++q) {
         if (q >= cols) break;
         const z b = y[q * n + j + 1 + r];
-        sr[q] = fma(a.x, b.x, fma(a.y, b.y, sr[q]));
-        si[q] = fma(a.x, b.y, fma(-a.y, b.x, si[q]));
+        s4[2 * q] = fma(a.x, b.x, fma(a.y, b.y, s4[2 * q]));
+        s4[2 * q + 1] = fma(a.x, b.y, fma(-a.y, b.x, s4[2 * q + 1]));
       }
     }
-#pragma unroll
-    for (int q = 0; q < BT_COLS; ++q) {
-      sr[q] = warp_sum_d(sr[q]);
-      si[q] = warp_sum_d(si[q]);
-      if (lane == 0) {
-        shr[warp][q] = sr[q];
-        shi[warp][q] = si[q];
-      }
+    {  // the four sums: seven adds per warp, then a butterfly over the warps' sums
+      const double s = warp_sum4(s4);
+      if (lane < 4) shw[warp][lane] = s;
     }
     __syncthreads();
-    if (threadIdx.x < cols) {
-      double a = 0, b = 0;
-      for (int w = 0; w < 8; ++w) {
-        a += shr[w][threadIdx.x];
-        b += shi[w][threadIdx.x];
-      }
-      s_ts[threadIdx.x] = zmul(t, zmk(a, b));
+    if (warp == 0) {  // lane = (warp's sum, value): lane l holds value l & 3 of warp l >> 2
+      double s = shw[lane >> 2][lane & 3];
+#pragma unroll
+      for (int o = 16; o >= 4; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      const double im = __shfl_down_sync(0xffffffffu, s, 1);
+      if (lane < 4 && (lane & 1) == 0) s_ts[lane >> 1] = zmul(t, zmk(s, im));
     }
     __syncthreads();
     for (int64_t r = threadIdx.x; r < m; r += blockDim.x) {
@@ -1348,6 +1402,15 @@ size_t heig_scratch_bound(int64_t n, int64_t k) {
          (size_t)(1 << 20);
 }
 
+// one warp per eigenvalue, the largest problem of n rows
+static int launch_bisect(Ctx* c, int64_t n, int64_t kt, const double* d, const double* e, const EBlk* dblk,
+                         const int2* deig, const int64_t* nr, double* ev) {
+  const size_t smem = sizeof(double) * 2 * (size_t)n;
+  TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_bisect, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_bisect<<<(unsigned)kt, 32, smem, c->stream>>>(d, e, dblk, deig, nr, ev);
+  return TNT_OK;
+}
+
 // Second half of the eigensolve: from the tridiagonal form (d, e) and its reflectors
 // (Hv, row j = v_j, row stride n; tau) to the eigenvectors of the k largest eigenvalues
 // in U (n x k, leading dimension ldu), descending; ev (device, k).
@@ -1381,7 +1444,7 @@ int heig_finish(Ctx* c, int64_t n, int64_t k, const z* Hv, const z* tau, const d
   {
     ProfScope ps(c, "heig_tridiag_eig");
     k_split<<<1, 32, 0, st>>>(d, e, dblk, tn, nr);
-    k_bisect<<<(unsigned)k, 32, 0, st>>>(d, e, dblk, deig, nr, tn, ev);
+    TNT_TRY(launch_bisect(c, n, k, d, e, dblk, deig, nr, ev));
     k_inviter<<<(unsigned)k, IV_THREADS, 0, st>>>(d, e, dblk, deig, nr, ev, tn, work, Y);
     c->launches += 2;
     TNT_CHECK_LAUNCH(c);
@@ -1792,7 +1855,7 @@ int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& all, z* U, double* ev
   {
     ProfScope ps(c, "heig_tridiag_eig");
     k_split<<<(unsigned)nb, 32, 0, st>>>(d, e, dblk, tn, nr);
-    k_bisect<<<(unsigned)kt, 32, 0, st>>>(d, e, dblk, deig, nr, tn, ev);
+    TNT_TRY(launch_bisect(c, blocks[0].n, kt, d, e, dblk, deig, nr, ev));
     k_inviter<<<(unsigned)kt, IV_THREADS, 0, st>>>(d, e, dblk, deig, nr, ev, tn, work, Y);
     c->launches += 3;
     TNT_CHECK_LAUNCH(c);

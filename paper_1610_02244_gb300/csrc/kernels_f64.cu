@@ -129,8 +129,7 @@ __global__ void __launch_bounds__(256) k_zgemm16(ZGemm g) {
       Bs[ty][tx] = v;
     }
     __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) zfma(acc, As[ty][kk], Bs[kk][tx]);
+    tile16_fma(acc, As, Bs, (int)min((int64_t)16, g.M - m0), (int)min((int64_t)16, g.K - k0));
     __syncthreads();
   }
   const int64_t gi = m0 + ty, gj = n0 + tx;
@@ -222,8 +221,7 @@ __global__ void __launch_bounds__(256) k_zgemm16_tasks(const __grid_constant__ F
         Bs[ty][tx] = v;
       }
       __syncthreads();
-#pragma unroll
-      for (int kk = 0; kk < 16; ++kk) zfma(acc, As[ty][kk], Bs[kk][tx]);
+      tile16_fma(acc, As, Bs, (int)min((int64_t)16, g.M - m0), (int)min((int64_t)16, g.K - k0));
       __syncthreads();
     }
     const int64_t gi = m0 + ty, gj = n0 + tx;
@@ -388,9 +386,8 @@ int op_upload(Ctx* c, const std::vector<z>& dense, int nI, int nJ,
   memcpy(host.data() + b_row + b_col, val.data(), sizeof(z) * val.size());
   memcpy(host.data() + b_row + b_col + b_val, in_off.data(), sizeof(int64_t) * nJ);
   memcpy(host.data() + b_row + b_col + b_val + b_in, out_off.data(), sizeof(int64_t) * nI);
-  // synchronous: the host vector dies at return (tables are a few KB)
+  // (a pageable copy is staged before the call returns: the host vector may go)
   TNT_CUDA_TRY(c, cudaMemcpyAsync(dev, host.data(), total, cudaMemcpyHostToDevice, c->stream));
-  TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   a->nI = nI;
   a->nJ = nJ;
   a->nnz = row[nI];
@@ -935,7 +932,9 @@ int vec_normalize(Ctx* c, const z* x, z* y, int64_t n, const double* d_norm2) {
 // Gram-Schmidt passes of w against V[0..k), the norm, and the next basis vector.
 //   phase 1: c = V^H w           | grid barrier
 //   phase 2: w -= V c, c' = V^H w | grid barrier
-//   phase 3: w -= V c', |w|^2     | grid barrier;  v_k = w / |w|
+//   phase 3: w -= V c', v_k = w / |w|
+// |w|^2 after phase 3 is |w|^2 before it (summed with c') minus |c'|^2, V being orthonormal;
+// where c' takes more than a quarter of it, the sum is taken directly behind a third barrier.
 // CTA b keeps elements [b S, (b + 1) S) of w in shared memory, and of the basis too where
 // they fit (k S 16 bytes), so that V is read from L2 once.  Each warp takes whole vectors
 // (v = warp, warp + 8, ...) of its CTA's slice: the lanes' sums are combined by a transposed
@@ -949,13 +948,13 @@ int vec_normalize(Ctx* c, const z* x, z* y, int64_t n, const double* d_norm2) {
 // n = 5000.
 namespace {
 constexpr int GS_THREADS = 256, GS_WARPS = GS_THREADS / 32;
-constexpr int GS_SMEM = 208 * 1024;
+constexpr int GS_SMEM = 204 * 1024;
 // Above this the slice of w alone nears the shared memory of an SM, and both forms are bound
 // by the FP64 pipe.  FP64 solves of this size, fused / separate launches: n = 2^12 9.7 / 27
 // ms, 2^16 28 / 50, 2^18 60 / 80, 2^20 232 / 239.
 constexpr int64_t GS_MAX_N = 1 << 20;
 
-struct GsArgs {
+struct GsArgs {  // part: 64 vectors' sums, npart: the norm's
   const z* V;
   int64_t n;
   int k;
@@ -964,7 +963,7 @@ struct GsArgs {
   double* alpha;  // alpha[k - 1] and beta[k - 1] of the step
   double* beta;
   z* part;       // 2 x 64 x gridDim.x
-  double* npart; // gridDim.x
+  double* npart; // 2 x gridDim.x
   unsigned* bar; // arrivals since the solve began
   unsigned base; // its value before this launch
   int* status;
@@ -1083,9 +1082,33 @@ __device__ void gs_total(const GsArgs& a, const z* part, z* sc) {
   __syncthreads();
 }
 
-// w -= V c over the CTA's slice; returns the thread's share of |w|^2
-__device__ double gs_update(const GsArgs& a, z* sw, const z* V0, int64_t ld, int cnt, const z* sc) {
+// w -= V c over the CTA's slice; returns the thread's share of |w|^2.  A slice of at most 64
+// elements would leave most threads idle behind chains of 2 k dependent FMAs: there four
+// threads share an element, each a quarter of the vectors, and their sums meet in sacc.
+__device__ double gs_update(const GsArgs& a, z* sw, const z* V0, int64_t ld, int cnt, const z* sc, z* sacc) {
   double acc = 0;
+  if (cnt <= 64) {
+    const int e = threadIdx.x & 63, q = threadIdx.x >> 6;
+    z s0 = zmk(0, 0), s1 = s0;
+    if (e < cnt) {
+      int v = q;
+      for (; v + 4 < a.k; v += 8) {
+        const z u0 = V0[(int64_t)v * ld + e], u1 = V0[(int64_t)(v + 4) * ld + e];
+        zfma(s0, sc[v], u0);
+        zfma(s1, sc[v + 4], u1);
+      }
+      if (v < a.k) zfma(s0, sc[v], V0[(int64_t)v * ld + e]);
+      sacc[threadIdx.x] = zadd(s0, s1);
+    }
+    __syncthreads();
+    if (threadIdx.x < cnt) {
+      const z p = zadd(zadd(sacc[e], sacc[64 + e]), zadd(sacc[128 + e], sacc[192 + e]));
+      const z x = zsub(sw[e], p);
+      sw[e] = x;
+      acc = fma(x.x, x.x, x.y * x.y);
+    }
+    return acc;
+  }
   for (int e = threadIdx.x; e < cnt; e += GS_THREADS) {
     z x = sw[e];
     int v = 0;
@@ -1114,8 +1137,10 @@ __device__ double gs_update(const GsArgs& a, z* sw, const z* V0, int64_t ld, int
 __global__ void __launch_bounds__(GS_THREADS, 1) k_gs_step(GsArgs a) {
   extern __shared__ z sm_gs[];
   __shared__ z sc[64];
+  __shared__ z sacc[GS_THREADS];
   __shared__ double sh[32];
   __shared__ double s_rn;
+  __shared__ int s_direct;
   z* sw = sm_gs;
   z* sv = sm_gs + a.S;
   const int64_t lo = (int64_t)blockIdx.x * a.S;
@@ -1134,31 +1159,64 @@ __global__ void __launch_bounds__(GS_THREADS, 1) k_gs_step(GsArgs a) {
   if (ok) {
     gs_total(a, p1, sc);
     if (blockIdx.x == 0 && tid == 0) a.alpha[a.k - 1] = sc[a.k - 1].x;
-    gs_update(a, sw, V, ld, cnt, sc);
+    double acc = gs_update(a, sw, V, ld, cnt, sc, sacc);
     __syncthreads();
     gs_dots<false>(a, sw, sv, V, ld, cnt, p2);
+    acc = block_sum(acc, sh);
+    if (tid == 0) a.npart[blockIdx.x] = acc;
     ok = gs_barrier(a, a.base + 2u * gridDim.x);
   }
   if (ok) {
     gs_total(a, p2, sc);
-    double acc = gs_update(a, sw, V, ld, cnt, sc);
-    acc = block_sum(acc, sh);
-    if (tid == 0) a.npart[blockIdx.x] = acc;
-    ok = gs_barrier(a, a.base + 3u * gridDim.x);
+    if (tid < 32) {  // |w|^2 before the second update, and what c' takes of it
+      double r = 0, q = 0;
+      for (int b = tid; b < (int)gridDim.x; b += 32) r += __ldcg(a.npart + b);
+      for (int v = tid; v < a.k; v += 32) q = fma(sc[v].x, sc[v].x, fma(sc[v].y, sc[v].y, q));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        r += __shfl_xor_sync(0xffffffffu, r, o);
+        q += __shfl_xor_sync(0xffffffffu, q, o);
+      }
+      if (tid == 0) {
+        sh[0] = r - q;
+        s_direct = !(q <= 0.25 * r);
+      }
+    }
+    const double acc0 = gs_update(a, sw, V, ld, cnt, sc, sacc);
+    __syncthreads();
+    if (s_direct) {  // the same decision in every CTA
+      __shared__ double sh2[32];
+      const double acc = block_sum(acc0, sh2);
+      if (tid == 0) a.npart[gridDim.x + blockIdx.x] = acc;
+      ok = gs_barrier(a, a.base + 3u * gridDim.x);
+      if (ok && tid < 32) {
+        double r = 0;
+        for (int b = tid; b < (int)gridDim.x; b += 32) r += __ldcg(a.npart + gridDim.x + b);
+        r = warp_sum(r);
+        if (tid == 0) sh[0] = r;
+      }
+    } else if (blockIdx.x == 0 && tid == 0) {
+      // the launch counts three arrivals per CTA
+      asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(a.bar), "r"(gridDim.x) : "memory");
+    }
   }
   if (!ok) {  // the host reads a NaN beta, and the status word names the wait
     if (blockIdx.x == 0 && tid == 0) a.beta[a.k - 1] = __longlong_as_double(0x7ff8000000000000ll);
     return;
   }
-  if (tid < 32) {
-    double r = 0;
-    for (int b = tid; b < (int)gridDim.x; b += 32) r += __ldcg(a.npart + b);
-    r = warp_sum(r);
-    if (tid == 0) {
-      const double nr = sqrt(r);
-      s_rn = 1.0 / nr;
-      if (blockIdx.x == 0) a.beta[a.k - 1] = nr;
+  if (tid == 0) {
+    const double r = sh[0];
+    const int ex = (__double2hiint(r) >> 20) & 0x7ff;
+    double nr, rn;
+    if (r > 0 && ex > 0 && ex < 2047) {
+      rn = rsqrt_newton(r);
+      nr = r * rn;
+    } else {
+      nr = sqrt(r);
+      rn = 1.0 / nr;
     }
+    s_rn = rn;
+    if (blockIdx.x == 0) a.beta[a.k - 1] = nr;
   }
   __syncthreads();
   const double rn = s_rn;
@@ -1188,7 +1246,7 @@ int vec_gs_step(Ctx* c, const z* V, int k, const z* w, int64_t n, z* vnext, doub
   }
   const size_t top = c->ws.top;
   z* part = (z*)ws_alloc(c, ws_round(sizeof(z) * 2 * 64 * (size_t)nsm));
-  double* npart = (double*)ws_alloc(c, ws_round(sizeof(double) * (size_t)nsm));
+  double* npart = (double*)ws_alloc(c, ws_round(sizeof(double) * 2 * (size_t)nsm));
   c->ws.top = top;  // used by this launch only (stream order serialises its reuse)
   if (!part || !npart) return set_err(c, TNT_E_ALLOC, "scratch exhausted (Gram-Schmidt step)");
   GsArgs a;

@@ -17,7 +17,7 @@
 //     are exact over all of K; C = (2^28 H + L) 2^(a_i + b_j - 61), rounded once, by a
 //     second kernel (in the MMA kernel's eight epilogue warps that conversion took 25 to
 //     60 us a tile, more than the tile's MMAs).
-// The pairs left out (p + q > 9) and the digits' rounding are below K 2^-53 2^(a_i + b_j) in
+// The pairs left out (p + q > 9) and the digits' rounding are below 3 K 2^-53 2^(a_i + b_j) in
 // the worst case and of random sign; the result does not depend on tiling or K splits.
 // No FP64-pipe instruction runs in these kernels: an SM retires two FP64 operations per
 // clock, and combining the level sums in FP64 (with TF32 operands, six-bit digits and 45
@@ -158,8 +158,6 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 }
 // instruction descriptor: D = F32, A = B = F16, both K-major, M = 128, N = 128
 constexpr uint32_t OZ_IDESC = (1u << 4) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-// high word of a shared-memory descriptor (as tc::desc_sw64); the low word is the address / 16
-constexpr uint32_t OZ_DESC_HI = (512u >> 4) | (1u << 14) | (4u << 29);
 __device__ __forceinline__ void mma_f16(uint32_t tmem, uint32_t alo, uint32_t blo, uint32_t acc) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
@@ -167,7 +165,7 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem, uint32_t alo, uint32_t bl
       "mov.b64 a, {%1, %5};\n\t"
       "mov.b64 b, {%2, %5};\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}\n" ::"r"(tmem),
-      "r"(alo), "r"(blo), "r"(OZ_IDESC), "r"(acc), "r"(OZ_DESC_HI)
+      "r"(alo), "r"(blo), "r"(OZ_IDESC), "r"(acc), "r"(DESC_SW64_HI)
       : "memory");
 }
 
@@ -177,7 +175,7 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem, uint32_t alo, uint32_t bl
 // 1024 x 1024 x 1024 product that is 142 us of MMAs).  sa / sb: ring slots of the block's
 // first A and B slice, with the phases of their barriers in pa / pb.
 struct OzIssue {
-  uint32_t a0, b0;  // shared-memory addresses / 16 of the rings
+  uint32_t a0, b0;  // descriptor low words of the rings
   uint64_t *fa, *ea, *fb, *eb;
   uint64_t* acce;  // set: a level's first MMA waits until its last sums have been read
   uint32_t pacc;
@@ -341,7 +339,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(const __grid_constant
     // ------------------------------------------------ MMA issue
     uint32_t sub = 0;
     bool stop = false;
-    OzIssue r{su32(R.a) >> 4, su32(R.b) >> 4, R.fa, R.ea, R.fb, R.eb, nullptr, 0, 0, 0, 0, 0};
+    OzIssue r{desc_lo(su32(R.a)), desc_lo(su32(R.b)), R.fa, R.ea, R.fb, R.eb, nullptr, 0, 0, 0, 0, 0};
     for (int w = blockIdx.x; w < nitems && !stop; w += gridDim.x) {
       OzItem it;
       if (!oz_item(T, w, &it)) continue;

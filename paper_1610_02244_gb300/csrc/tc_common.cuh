@@ -61,28 +61,66 @@ __device__ __forceinline__ void tma_load3(void* dst, const CUtensorMap* tm, uint
       "l"((uint64_t)tm), "r"(su32(bar)), "r"(c0), "r"(c1), "r"(c2)
       : "memory");
 }
-// K-major operand tile, 64-byte rows, 64-byte swizzle: 8-row atoms of 512 bytes
-__device__ __forceinline__ uint64_t desc_sw64(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)1 << 16;                        // leading byte offset (unused here)
-  d |= (uint64_t)((512u >> 4) & 0x3FFFu) << 32;  // stride byte offset: next 8-row atom
-  d |= (uint64_t)1 << 46;                        // descriptor version
-  d |= (uint64_t)4 << 61;                        // swizzle: 64 B
-  return d;
-}
+// K-major operand tile, 64-byte rows, 64-byte swizzle: 8-row atoms of 512 bytes.  The low word of
+// the descriptor is the shared-memory address / 16 with the (here unused) leading byte offset
+// 1 above it, the high word constant: the stride byte offset to the next 8-row atom, the
+// descriptor version and the 64-byte swizzle.  The issuing thread adds to low words only: with
+// 64-bit descriptors built per MMA it took longer than the MMAs.
+constexpr uint32_t DESC_SW64_HI = (512u >> 4) | (1u << 14) | (4u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return (saddr >> 4) | (1u << 16); }
 // instruction descriptor: D = F32, A = B = TF32, both K-major, M = 128, N = n
 __host__ __device__ constexpr uint32_t idesc_tf32_n(int n) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
-__device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t id,
+__device__ __forceinline__ void mma_tf32(uint32_t tmem, uint32_t alo, uint32_t blo, uint32_t id,
                                          uint32_t acc) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
-      "l"(ad), "l"(bd), "r"(id), "r"(acc)
+      "mov.b64 a, {%1, %5};\n\t"
+      "mov.b64 b, {%2, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::tf32 [%0], a, b, %3, p;\n\t}\n" ::"r"(tmem),
+      "r"(alo), "r"(blo), "r"(id), "r"(acc), "r"(DESC_SW64_HI)
       : "memory");
+}
+// The split-TF32 complex products of one stage (16 of K: two MMA steps) at shared address
+// `base`: A planes re_hi, re_lo, im_hi, im_lo of TA bytes each, then B's of TB bytes.  re-re
+// products into t_re, im-im into t_rn (subtracted by the epilogue), the cross terms into
+// t_im; first: the accumulators start here.
+template <int TA, int TB>
+__device__ __forceinline__ void mma_cplx_tf32x3(uint32_t base, uint32_t t_re, uint32_t t_im, uint32_t t_rn,
+                                                uint32_t id, bool first) {
+  const uint32_t a0 = desc_lo(base), b0 = a0 + (4 * TA >> 4);
+#pragma unroll
+  for (int ks = 0; ks < 2; ++ks) {  // K = 8 per tf32 MMA: 32 bytes along the row
+    const uint32_t a_rh = a0 + 2 * ks, a_rl = a_rh + (TA >> 4), a_ih = a_rl + (TA >> 4), a_il = a_ih + (TA >> 4);
+    const uint32_t b_rh = b0 + 2 * ks, b_rl = b_rh + (TB >> 4), b_ih = b_rl + (TB >> 4), b_il = b_ih + (TB >> 4);
+    const uint32_t acc = (ks == 0 && first) ? 0u : 1u;
+    mma_tf32(t_re, a_rh, b_rh, id, acc);
+    mma_tf32(t_re, a_rh, b_rl, id, 1);
+    mma_tf32(t_re, a_rl, b_rh, id, 1);
+    mma_tf32(t_rn, a_ih, b_ih, id, acc);
+    mma_tf32(t_rn, a_ih, b_il, id, 1);
+    mma_tf32(t_rn, a_il, b_ih, id, 1);
+    mma_tf32(t_im, a_rh, b_ih, id, acc);
+    mma_tf32(t_im, a_rh, b_il, id, 1);
+    mma_tf32(t_im, a_rl, b_ih, id, 1);
+    mma_tf32(t_im, a_ih, b_rh, id, 1);
+    mma_tf32(t_im, a_ih, b_rl, id, 1);
+    mma_tf32(t_im, a_il, b_rh, id, 1);
+  }
+}
+// 32 values of one row to memory (nc of them exist): 16 bytes per store where p allows it (one
+// float per store put each of a warp's 32 rows into its own sector, 32 times over)
+__device__ __forceinline__ void store_row32(float* p, const uint32_t* v, int nc) {
+  if (nc >= 32 && ((uintptr_t)p & 15) == 0) {
+#pragma unroll
+    for (int j = 0; j < 32; j += 4) *(uint4*)(p + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    if (j < nc) p[j] = __uint_as_float(v[j]);
 }
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile(

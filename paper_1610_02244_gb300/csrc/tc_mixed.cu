@@ -107,46 +107,16 @@ __global__ void __launch_bounds__(192, 1) k_cgemm_tf32x3(const __grid_constant__
     // ------------------------------------------------ MMA issuer
     const uint32_t id = idesc_tf32_n(BN);
     const uint32_t t_re = tmem, t_im = tmem + BN, t_rn = tmem + 2 * BN;
-    bool ok = true;
     for (int i = 0; i < nkb; ++i) {
       const int s = i % STAGES;
       if (!mbar_wait(&full[s], (i / STAGES) & 1, g.status)) {
         *abort_flag = 1;
-        ok = false;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t base = su32(smem + s * STAGE_BYTES);
-      for (int ks = 0; ks < BK / 8; ++ks) {  // K = 8 per tf32 MMA: 32 bytes along the row
-        const uint32_t off = ks * 32;
-        const uint64_t a_rh = desc_sw64(base + 0 * TILE_A + off);
-        const uint64_t a_rl = desc_sw64(base + 1 * TILE_A + off);
-        const uint64_t a_ih = desc_sw64(base + 2 * TILE_A + off);
-        const uint64_t a_il = desc_sw64(base + 3 * TILE_A + off);
-        const uint32_t bb = base + 4 * TILE_A;
-        const uint64_t b_rh = desc_sw64(bb + 0 * TILE_B + off);
-        const uint64_t b_rl = desc_sw64(bb + 1 * TILE_B + off);
-        const uint64_t b_ih = desc_sw64(bb + 2 * TILE_B + off);
-        const uint64_t b_il = desc_sw64(bb + 3 * TILE_B + off);
-        const uint32_t first = (i == 0 && ks == 0) ? 0u : 1u;
-        // real part: re_re products (+) and im_im products (accumulated apart, subtracted)
-        mma_tf32(t_re, a_rh, b_rh, id, first);
-        mma_tf32(t_re, a_rh, b_rl, id, 1);
-        mma_tf32(t_re, a_rl, b_rh, id, 1);
-        mma_tf32(t_rn, a_ih, b_ih, id, first);
-        mma_tf32(t_rn, a_ih, b_il, id, 1);
-        mma_tf32(t_rn, a_il, b_ih, id, 1);
-        // imaginary part
-        mma_tf32(t_im, a_rh, b_ih, id, first);
-        mma_tf32(t_im, a_rh, b_il, id, 1);
-        mma_tf32(t_im, a_rl, b_ih, id, 1);
-        mma_tf32(t_im, a_ih, b_rh, id, 1);
-        mma_tf32(t_im, a_ih, b_rl, id, 1);
-        mma_tf32(t_im, a_il, b_rh, id, 1);
-      }
+      mma_cplx_tf32x3<TILE_A, TILE_B>(su32(smem + s * STAGE_BYTES), t_re, t_im, t_rn, id, i == 0);
       mma_commit(&empty[s]);  // stage s is free once these MMAs have read it
     }
-    (void)ok;
     mma_commit(accb);  // accumulators complete (arrives after all MMAs issued above)
   } else if (warp >= 2) {
     // ------------------------------------------------ epilogue: TMEM -> global (FP32)
@@ -165,14 +135,12 @@ __global__ void __launch_bounds__(192, 1) k_cgemm_tf32x3(const __grid_constant__
         tmem_ld32(tmem + lane_addr + BN + c0, s);
         tmem_ld32(tmem + lane_addr + 2 * BN + c0, u);
         if (gm < g.M) {
-          float* pr = Cre + gm * g.ldc + n0 + c0;
-          float* pi = Cim + gm * g.ldc + n0 + c0;
+          const int nc = (int)min((int64_t)32, g.N - n0 - c0);
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (n0 + c0 + j < g.N) {
-              pr[j] = __uint_as_float(r[j]) - __uint_as_float(u[j]);
-              pi[j] = __uint_as_float(s[j]);
-            }
+          for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) - __uint_as_float(u[j]));
+          if (nc > 0) {
+            store_row32(Cre + gm * g.ldc + n0 + c0, r, nc);
+            store_row32(Cim + gm * g.ldc + n0 + c0, s, nc);
           }
         }
       }
@@ -238,23 +206,14 @@ __global__ void k_split_transpose(const z* __restrict__ src, int64_t K, int64_t 
 
 // T3 planes = W12 (x) T1 (FP32 re/im planes in, split TF32 planes out).  FP32 arithmetic:
 // T1 itself carries the split-TF32 products' ~2^-22 relative error and W12 has a handful of
-// O(1) entries per output, so FP64 here would buy nothing (and ran on the FP64 pipe).
-__global__ void __launch_bounds__(256) k_op_mixed(OpApply a, const float* __restrict__ t1,
-                                                  int64_t t1_plane, float* __restrict__ t3,
-                                                  int64_t t3_plane) {
-  __shared__ int s_row[257];
-  __shared__ int s_col[2048];
-  __shared__ float2 s_val[2048];
-  __shared__ int64_t s_in[256];
-  __shared__ int64_t s_out[256];
-  for (int t = threadIdx.x; t <= a.nI; t += blockDim.x) s_row[t] = a.row_ptr[t];
-  for (int t = threadIdx.x; t < a.nnz; t += blockDim.x) {
-    s_col[t] = a.col[t];
-    s_val[t] = make_float2((float)a.val[t].x, (float)a.val[t].y);
-  }
-  for (int t = threadIdx.x; t < a.nJ; t += blockDim.x) s_in[t] = a.in_off[t];
-  for (int t = threadIdx.x; t < a.nI; t += blockDim.x) s_out[t] = a.out_off[t];
-  __syncthreads();
+// O(1) entries per output, so FP64 here would buy nothing (and ran on the FP64 pipe).  One
+// thread per (a', b) and group of `rows` output indices (blockIdx.y); real entries (the models'
+// MPOs) skip the imaginary products, which add exact zeros.
+template <bool REAL>
+__device__ __forceinline__ void op_mixed_rows(const OpApply& a, int i0, int i1, const int* s_row, const int* s_col,
+                                              const float2* s_val, const int64_t* s_in, const int64_t* s_out,
+                                              const float* __restrict__ t1, int64_t t1_plane, float* __restrict__ t3,
+                                              int64_t t3_plane) {
   const int64_t total = a.B0 * a.B2;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -262,14 +221,19 @@ __global__ void __launch_bounds__(256) k_op_mixed(OpApply a, const float* __rest
     const float* ire = t1 + b0 * a.is0 + b2 * a.is2;
     const float* iim = ire + t1_plane;
     float* o = t3 + b0 * a.os0 + b2 * a.os2;
-    for (int i = 0; i < a.nI; ++i) {
+    for (int i = i0; i < i1; ++i) {
       float xr = 0.f, xi = 0.f;
       for (int t = s_row[i]; t < s_row[i + 1]; ++t) {
         const float2 w = s_val[t];
         const int64_t off = s_in[s_col[t]];
         const float vr = ire[off], vi = iim[off];
-        xr = fmaf(w.x, vr, fmaf(-w.y, vi, xr));
-        xi = fmaf(w.x, vi, fmaf(w.y, vr, xi));
+        if (REAL) {
+          xr = fmaf(w.x, vr, xr);
+          xi = fmaf(w.x, vi, xi);
+        } else {
+          xr = fmaf(w.x, vr, fmaf(-w.y, vi, xr));
+          xi = fmaf(w.x, vi, fmaf(w.y, vr, xi));
+        }
       }
       float h, l;
       const int64_t off = s_out[i];
@@ -281,6 +245,30 @@ __global__ void __launch_bounds__(256) k_op_mixed(OpApply a, const float* __rest
       o[3 * t3_plane + off] = l;
     }
   }
+}
+__global__ void __launch_bounds__(256) k_op_mixed(OpApply a, int rows, const float* __restrict__ t1,
+                                                  int64_t t1_plane, float* __restrict__ t3,
+                                                  int64_t t3_plane) {
+  __shared__ int s_row[257];
+  __shared__ int s_col[2048];
+  __shared__ float2 s_val[2048];
+  __shared__ int64_t s_in[256];
+  __shared__ int64_t s_out[256];
+  const int i0 = blockIdx.y * rows, i1 = min(a.nI, i0 + rows);
+  for (int t = threadIdx.x; t <= a.nI; t += blockDim.x) s_row[t] = a.row_ptr[t];
+  for (int t = threadIdx.x; t < a.nJ; t += blockDim.x) s_in[t] = a.in_off[t];
+  for (int t = threadIdx.x; t < a.nI; t += blockDim.x) s_out[t] = a.out_off[t];
+  __syncthreads();
+  int cplx = 0;
+  for (int t = s_row[i0] + threadIdx.x; t < s_row[i1]; t += blockDim.x) {
+    s_col[t] = a.col[t];
+    const z v = a.val[t];
+    s_val[t] = make_float2((float)v.x, (float)v.y);
+    cplx |= v.y != 0.0;
+  }
+  cplx = __syncthreads_or(cplx);
+  if (cplx) op_mixed_rows<false>(a, i0, i1, s_row, s_col, s_val, s_in, s_out, t1, t1_plane, t3, t3_plane);
+  else op_mixed_rows<true>(a, i0, i1, s_row, s_col, s_val, s_in, s_out, t1, t1_plane, t3, t3_plane);
 }
 
 // y (FP64 interleaved, M x N) = sum over splits of the FP32 (re, im) planes, fixed order
@@ -429,7 +417,8 @@ int heff_mixed_prepare(Ctx* c, HeffPlan* p) {
   k_split_rows<<<grid1(m.Mp1 * m.Kp1), 256, 0, c->stream>>>(p->L, m.M1, m.K1, chl, m.Mp1, m.Kp1, m.Lp);
   k_split_rows<<<grid1(m.Np4 * m.Kp4), 256, 0, c->stream>>>(p->R, m.N4, m.K4, D * chr, m.Np4, m.Kp4, m.Rp);
   c->launches += 2;
-  TNT_CUDA_TRY(c, cudaMemsetAsync(m.T3p, 0, 4 * sizeof(float) * m.Mp4 * m.Kp4, c->stream));
+  if (m.Mp4 != m.M4 || m.Kp4 != m.K4)  // padding rows and columns
+    TNT_CUDA_TRY(c, cudaMemsetAsync(m.T3p, 0, 4 * sizeof(float) * m.Mp4 * m.Kp4, c->stream));
   TNT_CHECK_LAUNCH(c);
   TNT_TRY(make_map(c, &m.tmL, m.Lp, m.Mp1, m.Kp1, BM));
   TNT_TRY(make_map(c, &m.tmTh, m.Thp, m.Np1, m.Kp1, BN));
@@ -445,8 +434,8 @@ int heff_mixed_prepare(Ctx* c, HeffPlan* p) {
         out_off[(size_t)((s1 * d + s2) * D + w2)] = (s1 * d + s2) * m.Kp4 + w2 * chr;
   int64_t* d_out = (int64_t*)ws_alloc(c, ws_round(sizeof(int64_t) * nI));
   if (!d_out) return set_err(c, TNT_E_ALLOC, "scratch exhausted (mixed op table)");
+  // (a pageable copy is staged before the call returns)
   TNT_CUDA_TRY(c, cudaMemcpyAsync(d_out, out_off.data(), sizeof(int64_t) * nI, cudaMemcpyHostToDevice, c->stream));
-  TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   m.op.out_off = d_out;
   m.op.B0 = chl;
   m.op.B1 = 1;
@@ -472,8 +461,12 @@ int heff_run_mixed(Ctx* c, const HeffPlan& p, const z* theta, z* y) {
   int64_t blocks = std::min<int64_t>((total + 255) / 256, 152 * 16);
   {
     ProfScope ps(c, "op_mixed", 8.0 * (double)m.M1 * (double)m.N1 + 16.0 * (double)m.M4 * (double)m.K4);
-    k_op_mixed<<<(unsigned)std::max<int64_t>(blocks, 1), 256, 0, c->stream>>>(
-        m.op, m.T1, m.M1 * m.N1, m.T3p, m.Mp4 * m.Kp4);
+    // at least eight blocks per SM where the output indices allow it
+    blocks = std::max<int64_t>(blocks, 1);
+    const int64_t want = std::min<int64_t>(m.op.nI, (152 * 8 + blocks - 1) / blocks);
+    const int rows = (int)((m.op.nI + want - 1) / want);
+    k_op_mixed<<<dim3((unsigned)blocks, (unsigned)((m.op.nI + rows - 1) / rows)), 256, 0, c->stream>>>(
+        m.op, rows, m.T1, m.M1 * m.N1, m.T3p, m.Mp4 * m.Kp4);
   }
   c->launches++;
   TNT_CHECK_LAUNCH(c);

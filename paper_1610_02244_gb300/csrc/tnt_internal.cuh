@@ -33,6 +33,26 @@ __host__ __device__ __forceinline__ void zfma(z& acc, z a, z b) {
   acc.y = fma(a.y, b.x, acc.y);
 }
 
+#ifdef __CUDACC__
+// acc += As[ty][0..k) Bs[0..k)[tx] for a 16 x 16 tile of 256 threads: only the k entries that
+// exist, and not at all for a warp whose two rows lie beyond `rows` (a small charge block
+// fills a fraction of its tile, and every FMA issued holds the FP64 pipe for 64 clocks); two
+// accumulators, so that consecutive terms do not wait for one another
+__device__ __forceinline__ void tile16_fma(z& acc, const z (*As)[17], const z (*Bs)[17], int rows, int k) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  if ((ty & ~1) >= rows) return;
+  z a1 = zmk(0, 0);
+  int kk = 0;
+#pragma unroll 4
+  for (; kk + 2 <= k; kk += 2) {
+    zfma(acc, As[ty][kk], Bs[kk][tx]);
+    zfma(a1, As[ty][kk + 1], Bs[kk + 1][tx]);
+  }
+  if (kk < k) zfma(acc, As[ty][kk], Bs[kk][tx]);
+  acc = zadd(acc, a1);
+}
+#endif
+
 // ---------------------------------------------------------------- context
 struct Arena {
   // A bump allocator over one device block; grown (reallocated) only between calls.
@@ -296,6 +316,7 @@ int heff_mixed(Ctx* c, const z* L, const z* W1, const z* W2, const z* R, const z
 
 // host copies of MPO tensors are needed to build the CSR ops: read back W (tiny)
 int read_small(Ctx* c, const void* dsrc, void* hdst, size_t bytes);
+int read_small2(Ctx* c, const void* d1, void* h1, size_t b1, const void* d2, void* h2, size_t b2);
 
 int bh_mpo_site_host(int n_max, double J, double U, double mu, double V, double j, double jc,
                      z* W);

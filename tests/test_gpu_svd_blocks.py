@@ -1,0 +1,71 @@
+"""The truncated SVD's block-parallel eigen path (`csrc/heig.cu`) where it can go wrong: blocks
+around the sizes at which a CTA group, a panel of reflectors or a route changes, many
+uneven blocks in one call, and exactly low-rank blocks, whose reduction leaves trailing
+matrices that shrink by sixteen decades per column.
+
+Tolerances: the Gram matrix and its reduction resolve singular values to about
+n eps sigma_max in absolute terms (1e-13 with room for n up to 600), U (or V) is orthonormal to
+the Newton-Schulz steps' 1e-13.  The factors multiply back to M up to what the kept vectors
+miss of its range: a Gram matrix larger than the rank mixes the smallest kept direction with
+its null space by an angle of n eps (sigma_max / sigma_k)^2, which moves M by that times
+sigma_k."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1610_02244_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1610_02244_gb300 import build as b
+    b.build()
+    from paper_1610_02244_gb300 import tnt
+    return tnt.Context(0)
+
+
+def check(ctx, M, rq=None, cq=None, side=0):
+    U, X, S, bq, info = ctx.svd_trunc(torch.from_numpy(np.ascontiguousarray(M)).to("cuda:0"), rq, cq, side=side)
+    U, X = U.cpu().numpy(), X.cpu().numpy()
+    assert np.all(np.isfinite(U)) and np.all(np.isfinite(X)) and np.all(np.isfinite(S))
+    sref = np.linalg.svd(M, compute_uv=False)
+    k = len(S)
+    assert np.abs(np.sort(S)[::-1] - sref[:k]).max() <= 1e-13 * sref[0]
+    assert np.linalg.norm(sref[k:]) <= 2e-8 * sref[0]  # the default truncation error
+    Q = U if side == 0 else X.conj().T
+    assert np.abs(Q.conj().T @ Q - np.eye(k)).max() <= 1e-13
+    null = len(sref) * 2.0 ** -52 * sref[0] ** 2 / S.min()
+    assert np.linalg.norm(U @ X - M) <= np.linalg.norm(sref[k:]) + 1e-13 * len(sref) * sref[0] + null
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 31, 32, 33, 64, 65, 127, 129, 192, 193, 257, 320, 600])
+@pytest.mark.parametrize("side", [0, 1])
+def test_single_block(ctx, n, side):
+    g = synth.rng(n)
+    check(ctx, synth.complex_gaussian(g, (n, n + 5)) @ np.diag(np.logspace(0, -3, n + 5)), side=side)
+
+
+@pytest.mark.parametrize("m,n,rank", [(20, 1, 1), (20, 2, 2), (64, 3, 2), (200, 40, 1), (250, 250, 5)])
+@pytest.mark.parametrize("side", [0, 1])
+def test_exactly_low_rank(ctx, m, n, rank, side):
+    for seed in range(12):
+        g = synth.rng(1000 * rank + seed)
+        if seed % 2:  # small integers: exact cancellations
+            M = (g.integers(-3, 4, (m, rank)) + 1j * g.integers(-3, 4, (m, rank))) @ g.integers(-3, 4, (rank, n))
+            M[0, 0] += 1
+        else:
+            M = synth.complex_gaussian(g, (m, rank)) @ synth.complex_gaussian(g, (rank, n))
+        check(ctx, M.astype(np.complex128), side=side)
+
+
+@pytest.mark.parametrize("sizes", [(500, 400, 300, 200, 100, 50, 20, 5, 1), (7,) * 60, (260, 255, 1, 193, 192)])
+@pytest.mark.parametrize("side", [0, 1])
+def test_many_uneven_blocks(ctx, sizes, side):
+    g = synth.rng(sum(sizes))
+    rq = np.concatenate([np.full(s, i) for i, s in enumerate(sizes)])
+    cq = np.concatenate([np.full(max(1, s - i % 3), i) for i, s in enumerate(sizes)])
+    M = synth.complex_gaussian(g, (len(rq), len(cq))) * (rq[:, None] == cq[None, :])
+    M *= np.logspace(0, -2, len(cq))[None, :]
+    check(ctx, M, rq, cq, side=side)
