@@ -256,33 +256,21 @@ __global__ void __launch_bounds__(256) k_zgemm_grouped(ZGArgs g) {
   }
 }
 
-// the same over 16 x 16 tiles, one output per thread: for block structures whose 64 x 64
-// tiles would leave most SMs without FP64 work
+// the same over R x 16 tiles: for block structures whose 64 x 64 tiles would leave most SMs
+// without FP64 work
+template <int R>
 __global__ void __launch_bounds__(256) k_zgemm_grouped16(ZGArgs g) {
-  __shared__ z As[16][17];
+  __shared__ z As[R][17];
   __shared__ z Bs[16][17];
+  __shared__ z part[R < 16 ? 256 : 1];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   for (int t = blockIdx.x; t < g.ntiles; t += gridDim.x) {
     const int4 tl = g.tiles[t];
     const ZTask tk = g.tasks[tl.x];
-    const z* A = g.A + tk.a_off;
-    const z* B = g.B + tk.b_off;
-    z acc = zmk(0, 0);
-    for (int64_t k0 = 0; k0 < tk.K; k0 += 16) {
-      {
-        const int64_t gi = tl.y + ty, gk = k0 + tx;
-        As[ty][tx] = (gi < tk.M && gk < tk.K) ? A[gi * tk.a_rs + gk * tk.a_cs] : zmk(0, 0);
-      }
-      {
-        const int64_t gk = k0 + ty, gj = tl.z + tx;
-        Bs[ty][tx] = (gj < tk.N && gk < tk.K) ? B[gk * tk.b_rs + gj * tk.b_cs] : zmk(0, 0);
-      }
-      __syncthreads();
-      tile16_fma(acc, As, Bs, (int)min((int64_t)16, tk.M - tl.y), (int)min((int64_t)16, tk.K - k0));
-      __syncthreads();
-    }
+    const z acc = tile_product<R>(g.A + tk.a_off, tk.a_rs, tk.a_cs, 0, g.B + tk.b_off, tk.b_rs, tk.b_cs, 0, tl.y, tl.z,
+                                  tk.M, tk.N, tk.K, As, Bs, part);
     const int64_t gi = tl.y + ty, gj = tl.z + tx;
-    if (gi < tk.M && gj < tk.N) g.C[tk.c_off + gi * tk.c_rs + gj] = acc;
+    if (ty < R && gi < tk.M && gj < tk.N) g.C[tk.c_off + gi * tk.c_rs + gj] = acc;
   }
 }
 
@@ -545,10 +533,11 @@ void make_tiles(const std::vector<TaskDesc>& ts, int bn, int split, std::vector<
 }
 
 void make_ztiles(const std::vector<ZTask>& ts, int tile, std::vector<int4>* tiles) {
+  const int tn = std::max(tile, 16);
   tiles->clear();
   for (size_t i = 0; i < ts.size(); ++i)
     for (int64_t m0 = 0; m0 < ts[i].M; m0 += tile)
-      for (int64_t n0 = 0; n0 < ts[i].N; n0 += tile) tiles->push_back(make_int4((int)i, (int)m0, (int)n0, 0));
+      for (int64_t n0 = 0; n0 < ts[i].N; n0 += tn) tiles->push_back(make_int4((int)i, (int)m0, (int)n0, 0));
 }
 
 template <typename T>
@@ -949,9 +938,11 @@ int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
        ws_round(sizeof(int2) * p->wtiles.size()) + ws_round(sizeof(GRow) * p->rows.size());
   // tiles: worst case N tile 64 and split 4
   int64_t t1 = 0, t4 = 0, z1 = 0, z4 = 0;
-  // FP64 tiles counted at the smaller (16 x 16) size, the larger of the two lists
+  // FP64 tiles counted at 16 x 16; lower ones are taken up to 304 of these (tile_rows), and
+  // there are at most four times as many of them
   for (const TaskDesc& t : p->s1) { t1 += ((t.M + 127) / 128) * ((t.N + 63) / 64); z1 += ((t.M + 15) / 16) * ((t.N + 15) / 16); }
   for (const TaskDesc& t : p->s4) { t4 += 4 * ((t.M + 127) / 128) * ((t.N + 63) / 64); z4 += ((t.M + 15) / 16) * ((t.N + 15) / 16); }
+  if (std::max(z1, z4) <= 2 * sm_count()) z1 *= 4, z4 *= 4;
   p->cap_g1tiles = (int)t1;
   p->cap_g4tiles = (int)t4;
   b += ws_round(sizeof(int4) * (t1 + t4 + z1 + z4)) + ws_round(sizeof(GTask) * (p->s1.size() + p->s4.size())) +
@@ -1116,6 +1107,11 @@ int u1_prepare(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
   if (p->ztile == 16) {
     make_ztiles(z1, 16, &zt1);
     make_ztiles(z4, 16, &zt4);
+    p->ztile = tile_rows((int64_t)std::max(zt1.size(), zt4.size()), sm_count());
+    if (p->ztile < 16) {
+      make_ztiles(z1, p->ztile, &zt1);
+      make_ztiles(z4, p->ztile, &zt4);
+    }
   }
   TNT_TRY(upload(c, &p->d_z1, z1));
   TNT_TRY(upload(c, &p->d_z4, z4));
@@ -1180,13 +1176,19 @@ int u1_tune(Ctx* c, const std::vector<U1Spec>& probs) {
 }
 
 namespace {
-void* zfn(const U1Plan& p) { return p.ztile == 16 ? (void*)k_zgemm_grouped16 : (void*)k_zgemm_grouped; }
-int64_t zcap(const U1Plan& p) { return p.ztile == 16 ? 152 * 8 : 152 * 2; }
-void zlaunch(Ctx* c, const U1Plan& p, const ZGArgs& a, int ntiles) {
-  if (p.ztile == 16)
-    k_zgemm_grouped16<<<cap_grid(ntiles, zcap(p)), 256, 0, c->stream>>>(a);
-  else
-    k_zgemm_grouped<<<cap_grid(ntiles, zcap(p)), 256, 0, c->stream>>>(a);
+void* zfn(const U1Plan& p) {
+  return p.ztile == 16 ? (void*)k_zgemm_grouped16<16>
+         : p.ztile == 8 ? (void*)k_zgemm_grouped16<8>
+         : p.ztile == 4 ? (void*)k_zgemm_grouped16<4>
+                        : (void*)k_zgemm_grouped;
+}
+int64_t zcap(const U1Plan& p) { return p.ztile <= 16 ? 152 * 8 : 152 * 2; }
+int zlaunch(Ctx* c, const U1Plan& p, const ZGArgs& a, int ntiles) {
+  ZGArgs arg = a;
+  void* args[] = {&arg};
+  TNT_CUDA_TRY(c, cudaLaunchKernel(zfn(p), dim3(cap_grid(ntiles, zcap(p))), dim3(256), args, 0, c->stream));
+  c->launches++;
+  return TNT_OK;
 }
 
 // kernel-node parameters for a graph; args points at the single struct argument
@@ -1320,8 +1322,7 @@ int run_direct(Ctx* c, U1Plan& p, const z* x, z* y, int mixed) {
       TNT_TRY(oz_plan_run(c, p.oz1, x));
     } else {
       ProfScope ps(c, "zgemm_grouped", f1);
-      zlaunch(c, p, z1, p.n_z1tiles);
-      c->launches++;
+      TNT_TRY(zlaunch(c, p, z1, p.n_z1tiles));
     }
     {
       ProfScope ps(c, "u1_wop_f64", 16.0 * (double)p.P1 + 16.0 * (double)(p.rowsA4 * p.KA4));
@@ -1333,8 +1334,7 @@ int run_direct(Ctx* c, U1Plan& p, const z* x, z* y, int mixed) {
       TNT_TRY(oz_plan_run(c, p.oz4, nullptr));
     } else {
       ProfScope ps(c, "zgemm_grouped", f4);
-      zlaunch(c, p, z4, p.n_z4tiles);
-      c->launches++;
+      TNT_TRY(zlaunch(c, p, z4, p.n_z4tiles));
     }
     GthArgs ga = p.out_g[0];
     ga.y = y;

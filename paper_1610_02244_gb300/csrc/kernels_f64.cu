@@ -95,45 +95,26 @@ __global__ void __launch_bounds__(256) k_zgemm(ZGemm g) {
 }  // namespace
 
 namespace {
-// 16 x 16 output tiles, one element per thread: for products too small to give every SM
-// a 64 x 64 tile (GB300's FP64 units are ~2 FMA per clock per SM, so the FP64 work of a
-// small product must be spread thin)
+// R x 16 output tiles of 256 threads (R = 16, 8, 4), 16 / R threads per output, each taking
+// every (16 / R)-th term: for products too small to give every SM a 64 x 64 tile (GB300's
+// FP64 units are ~2 FMA per clock per SM, so the FP64 work of a small product must be spread
+// thin: a 16 x 16 tile of K = 128 takes 32 us on its SM)
+template <int R>
 __global__ void __launch_bounds__(256) k_zgemm16(ZGemm g) {
-  __shared__ z As[16][17];
+  __shared__ z As[R][17];
   __shared__ z Bs[16][17];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int64_t m0 = (int64_t)blockIdx.y * 16, n0 = (int64_t)blockIdx.x * 16;
-  if (g.lower_only && m0 + 16 <= n0) return;
+  __shared__ z part[R < 16 ? 256 : 1];
+  const int64_t m0 = (int64_t)blockIdx.y * R, n0 = (int64_t)blockIdx.x * 16;
+  if (g.lower_only && m0 + R <= n0) return;
   const int64_t bt = blockIdx.z;
   const z* A = g.A + bt * g.a_bs;
   const z* B = g.B + bt * g.b_bs;
   z* C = g.C + bt * g.c_bs;
-  z acc = zmk(0, 0);
-  for (int64_t k0 = 0; k0 < g.K; k0 += 16) {
-    {
-      const int64_t gi = m0 + ty, gk = k0 + tx;
-      z v = zmk(0, 0);
-      if (gi < g.M && gk < g.K) {
-        v = A[gi * g.a_rs + gk * g.a_cs];
-        if (g.conj_a) v.y = -v.y;
-      }
-      As[ty][tx] = v;
-    }
-    {
-      const int64_t gk = k0 + ty, gj = n0 + tx;
-      z v = zmk(0, 0);
-      if (gj < g.N && gk < g.K) {
-        v = B[gk * g.b_rs + gj * g.b_cs];
-        if (g.conj_b) v.y = -v.y;
-      }
-      Bs[ty][tx] = v;
-    }
-    __syncthreads();
-    tile16_fma(acc, As, Bs, (int)min((int64_t)16, g.M - m0), (int)min((int64_t)16, g.K - k0));
-    __syncthreads();
-  }
+  const z acc = tile_product<R>(A, g.a_rs, g.a_cs, g.conj_a, B, g.b_rs, g.b_cs, g.conj_b, m0, n0, g.M, g.N, g.K, As,
+                                Bs, part);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int64_t gi = m0 + ty, gj = n0 + tx;
-  if (gi < g.M && gj < g.N) {
+  if (ty < R && gi < g.M && gj < g.N) {
     z v = zmul(g.alpha, acc);
     z* p = C + gi * g.c_rs + gj;
     if (g.beta.x != 0.0 || g.beta.y != 0.0) v = zadd(v, zmul(g.beta, *p));
@@ -141,6 +122,15 @@ __global__ void __launch_bounds__(256) k_zgemm16(ZGemm g) {
   }
 }
 }  // namespace
+
+// the tile height for `tiles` 16 x 16 tiles: the one whose rounds over the SMs take least;
+// beyond two rounds the last one is no longer worth re-reading B more often
+int tile_rows(int64_t tiles, int nsm) {
+  if (tiles > 2 * nsm) return 16;
+  const int64_t r16 = 4 * ((tiles + nsm - 1) / nsm), r8 = 2 * ((2 * tiles + nsm - 1) / nsm),
+                r4 = (4 * tiles + nsm - 1) / nsm;
+  return r16 <= r8 && r16 <= r4 ? 16 : r8 <= r4 ? 8 : 4;
+}
 
 int zgemm(Ctx* c, const ZGemm& g) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return TNT_OK;
@@ -155,10 +145,14 @@ int zgemm(Ctx* c, const ZGemm& g) {
       nsm = 152;
     const int64_t tiles64 = ((g.M + GM - 1) / GM) * ((g.N + GN - 1) / GN) * g.batch;
     if (tiles64 < nsm && (g.M + 15) / 16 <= 65535 && g.batch <= 65535) {
-      dim3 grid((unsigned)((g.N + 15) / 16), (unsigned)((g.M + 15) / 16), (unsigned)g.batch);
+      const int64_t tiles16 = ((g.M + 15) / 16) * ((g.N + 15) / 16) * g.batch;
+      const int R = (g.M + 3) / 4 <= 65535 ? tile_rows(tiles16, nsm) : 16;
+      dim3 grid((unsigned)((g.N + 15) / 16), (unsigned)((g.M + R - 1) / R), (unsigned)g.batch);
       ProfScope ps(c, "zgemm_f64", (g.lower_only ? 4.0 : 8.0) * (double)g.M * (double)g.N *
                                        (double)g.K * (double)g.batch);
-      k_zgemm16<<<grid, 256, 0, c->stream>>>(g);
+      if (R == 16) k_zgemm16<16><<<grid, 256, 0, c->stream>>>(g);
+      else if (R == 8) k_zgemm16<8><<<grid, 256, 0, c->stream>>>(g);
+      else k_zgemm16<4><<<grid, 256, 0, c->stream>>>(g);
       c->launches++;
       TNT_CHECK_LAUNCH(c);
       return TNT_OK;
@@ -191,9 +185,11 @@ struct FmaTasks {
   int n, tiles;
   FmaTask t[FT_MAX];
 };
+template <int R>
 __global__ void __launch_bounds__(256) k_zgemm16_tasks(const __grid_constant__ FmaTasks T) {
-  __shared__ z As[16][17];
+  __shared__ z As[R][17];
   __shared__ z Bs[16][17];
+  __shared__ z part[R < 16 ? 256 : 1];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   for (int w = blockIdx.x; w < T.tiles; w += gridDim.x) {
     int lo = 0, hi = T.n;
@@ -204,28 +200,12 @@ __global__ void __launch_bounds__(256) k_zgemm16_tasks(const __grid_constant__ F
     }
     const FmaTask& g = T.t[lo];
     const int ntn = (g.N + 15) / 16, tile = w - g.tile0;
-    const int64_t m0 = (int64_t)(tile / ntn) * 16, n0 = (int64_t)(tile % ntn) * 16;
-    if (g.herm && n0 > m0) continue;
-    z acc = zmk(0, 0);
-    for (int64_t k0 = 0; k0 < g.K; k0 += 16) {
-      {
-        const int64_t gi = m0 + ty, gk = k0 + tx;
-        z v = (gi < g.M && gk < g.K) ? g.A[gi * g.a_rs + gk * g.a_cs] : zmk(0, 0);
-        if (g.conj_a) v.y = -v.y;
-        As[ty][tx] = v;
-      }
-      {
-        const int64_t gk = k0 + ty, gj = n0 + tx;
-        z v = (gj < g.N && gk < g.K) ? g.B[gk * g.b_rs + gj * g.b_cs] : zmk(0, 0);
-        if (g.conj_b) v.y = -v.y;
-        Bs[ty][tx] = v;
-      }
-      __syncthreads();
-      tile16_fma(acc, As, Bs, (int)min((int64_t)16, g.M - m0), (int)min((int64_t)16, g.K - k0));
-      __syncthreads();
-    }
+    const int64_t m0 = (int64_t)(tile / ntn) * R, n0 = (int64_t)(tile % ntn) * 16;
+    if (g.herm && n0 >= m0 + R) continue;
+    z acc = tile_product<R>(g.A, g.a_rs, g.a_cs, g.conj_a, g.B, g.b_rs, g.b_cs, g.conj_b, m0, n0, g.M, g.N, g.K, As, Bs,
+                            part);
     const int64_t gi = m0 + ty, gj = n0 + tx;
-    if (gi < g.M && gj < g.N && !(g.herm && gj > gi)) {
+    if (ty < R && gi < g.M && gj < g.N && !(g.herm && gj > gi)) {
       z* p = g.C + gi * g.c_rs + gj;
       if (g.sub) acc = zsub(*p, acc);
       *p = acc;
@@ -236,6 +216,10 @@ __global__ void __launch_bounds__(256) k_zgemm16_tasks(const __grid_constant__ F
 }  // namespace
 
 int zgemm_fma_tasks(Ctx* c, const GemmTask* const* tasks, int n) {
+  int64_t t16 = 0;
+  for (int i = 0; i < n; ++i)
+    t16 += ((tasks[i]->g.M + 15) / 16) * ((tasks[i]->g.N + 15) / 16) / (tasks[i]->herm ? 2 : 1);
+  const int R = tile_rows(t16, 152);
   for (int i0 = 0; i0 < n; i0 += FT_MAX) {
     FmaTasks T;
     T.n = std::min(FT_MAX, n - i0);
@@ -250,13 +234,16 @@ int zgemm_fma_tasks(Ctx* c, const GemmTask* const* tasks, int n) {
       o.conj_a = g.conj_a; o.conj_b = g.conj_b;
       o.herm = tasks[i0 + i]->herm; o.sub = tasks[i0 + i]->sub;
       o.tile0 = (int)tiles;
-      tiles += ((g.M + 15) / 16) * ((g.N + 15) / 16);
+      tiles += ((g.M + R - 1) / R) * ((g.N + 15) / 16);
       flop += (o.herm ? 4.0 : 8.0) * (double)g.M * (double)g.N * (double)g.K;
     }
     if (tiles > INT32_MAX) return set_err(c, TNT_E_UNSUPPORTED, "grouped FP64 products: too many tiles");
     T.tiles = (int)tiles;
     ProfScope ps(c, "zgemm_f64", flop);
-    k_zgemm16_tasks<<<(unsigned)std::min<int64_t>(tiles, 152 * 8), 256, 0, c->stream>>>(T);
+    const unsigned grid = (unsigned)std::min<int64_t>(tiles, 152 * 8);
+    if (R == 16) k_zgemm16_tasks<16><<<grid, 256, 0, c->stream>>>(T);
+    else if (R == 8) k_zgemm16_tasks<8><<<grid, 256, 0, c->stream>>>(T);
+    else k_zgemm16_tasks<4><<<grid, 256, 0, c->stream>>>(T);
     c->launches++;
   }
   TNT_CHECK_LAUNCH(c);
@@ -1625,11 +1612,12 @@ __device__ bool tridiag_twisted(TwistShared& S, int k, double lo, double hi, dou
 }
 
 // one block per problem: problem p's alpha, beta, y at p * 64, out at p * 2 (skipped
-// where skip[p] is set)
+// where skip[p] is set); a single problem's E, |y_{k-1}| and beta_{k-1} also to pinned host
+// memory (no copy on the stream behind the kernel)
 __global__ void __launch_bounds__(32) k_tridiag_lowest(const double* __restrict__ alpha,
                                                        const double* __restrict__ beta, int k,
-                                                       double* __restrict__ out, double* __restrict__ y,
-                                                       const int* __restrict__ skip) {
+                                                       double* out, double* __restrict__ y,
+                                                       const int* __restrict__ skip, double* host) {
   const int pb = blockIdx.x;
   if (skip && skip[pb]) return;
   alpha += 64 * pb;
@@ -1654,22 +1642,18 @@ __global__ void __launch_bounds__(32) k_tridiag_lowest(const double* __restrict_
     hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
   }
   if (!tridiag_twisted(S, k, lo, hi, out, y)) tridiag_bisect(S.a, S.b, k, lo, hi, out, y);
+  if (host) {
+    __syncwarp();
+    if (l < 2) host[l] = out[l];
+    if (l == 2) host[2] = beta[k - 1];
+  }
 }
 }  // namespace
 
-int tridiag_lowest(Ctx* c, const double* d_alpha, const double* d_beta, int k, double* d_out,
-                   double* d_y) {
-  if (k < 1 || k > 64) return set_err(c, TNT_E_UNSUPPORTED, "tridiagonal size %d", k);
-  k_tridiag_lowest<<<1, 32, 0, c->stream>>>(d_alpha, d_beta, k, d_out, d_y, nullptr);
-  c->launches++;
-  TNT_CHECK_LAUNCH(c);
-  return TNT_OK;
-}
-
 int tridiag_lowest_on(Ctx* c, cudaStream_t st, const double* d_alpha, const double* d_beta, int k,
-                      double* d_out, double* d_y) {
+                      double* d_out, double* d_y, double* h_out) {
   if (k < 1 || k > 64) return set_err(c, TNT_E_UNSUPPORTED, "tridiagonal size %d", k);
-  k_tridiag_lowest<<<1, 32, 0, st>>>(d_alpha, d_beta, k, d_out, d_y, nullptr);
+  k_tridiag_lowest<<<1, 32, 0, st>>>(d_alpha, d_beta, k, d_out, d_y, nullptr, h_out);
   c->launches++;
   TNT_CHECK_LAUNCH(c);
   return TNT_OK;
@@ -1688,7 +1672,7 @@ int side_stream(Ctx* c) {
 int tridiag_lowest_batched(Ctx* c, const double* d_alpha, const double* d_beta, int k,
                            double* d_out, double* d_y, int nprob, const int* d_skip) {
   if (k < 1 || k > 64) return set_err(c, TNT_E_UNSUPPORTED, "tridiagonal size %d", k);
-  k_tridiag_lowest<<<nprob, 32, 0, c->stream>>>(d_alpha, d_beta, k, d_out, d_y, d_skip);
+  k_tridiag_lowest<<<nprob, 32, 0, c->stream>>>(d_alpha, d_beta, k, d_out, d_y, d_skip, nullptr);
   c->launches++;
   TNT_CHECK_LAUNCH(c);
   return TNT_OK;

@@ -95,7 +95,7 @@ static int lanczos_cycle_loop(Ctx* c, const MatVec& A, z* theta, int precision,
   bool have_prev = false;
   double E_prev = 0;
   // T_k's lowest eigenpair runs on the side stream one Krylov step behind the vector work:
-  // step k's scalars are handed over by an event, its result comes back into pinned slot
+  // step k's scalars are handed over by an event, its kernel writes its result into pinned slot
   // k & 1, and the host checks step k - 1 while step k runs.  A solve that converges at
   // k - 1 has computed one step more than it uses (not counted in n_matvec); the Ritz
   // vector is that of step k - 1, from V[0..k-1] and y of slot (k-1) & 1.
@@ -105,9 +105,7 @@ static int lanczos_cycle_loop(Ctx* c, const MatVec& A, z* theta, int precision,
     double* tk = tri2 + 2 * (k & 1);
     TNT_CUDA_TRY(c, cudaEventRecord(c->ev_main[k & 1], c->stream));
     TNT_CUDA_TRY(c, cudaStreamWaitEvent(c->side, c->ev_main[k & 1], 0));
-    TNT_TRY(tridiag_lowest_on(c, c->side, alpha, beta, k + 1, tk, y2 + 64 * (k & 1)));
-    TNT_CUDA_TRY(c, cudaMemcpyAsync(hp + 4 * (k & 1), tk, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->side));
-    TNT_CUDA_TRY(c, cudaMemcpyAsync(hp + 4 * (k & 1) + 2, beta + k, sizeof(double), cudaMemcpyDeviceToHost, c->side));
+    TNT_TRY(tridiag_lowest_on(c, c->side, alpha, beta, k + 1, tk, y2 + 64 * (k & 1), hp + 4 * (k & 1)));
     TNT_CUDA_TRY(c, cudaEventRecord(c->ev_side[k & 1], c->side));
     last_side = k & 1;
     return TNT_OK;

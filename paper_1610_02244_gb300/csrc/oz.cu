@@ -629,16 +629,18 @@ OzDeal oz_deal(int64_t tiles, int64_t nkb, int nsm) {
 }  // namespace
 
 // Where the slice product is the faster one.  The FP64 kernel's 16 x 16 tiles take 0.27 us per
-// K entry and round of one tile per SM (512 FMAs of 256 threads at two per clock); the five
-// launches here take about 30 us however small the product.  Measured on both sides of the
-// line (FP64 / slices, us): 128 x 512 x 32 35 / 30, 64 x 512 x 64 18 / 27, 128 x 64 x 128
-// 36 / 29, 256 x 256 x 64 36 / 30, 256 x 1024 x 64 125 / 32, 64 x 64 x 1024 280 / 39.
+// K entry and round of one tile per SM (512 FMAs of 256 threads at two per clock), down to a
+// quarter of that for tiles four rows high when there are few; the launches here take about
+// 30 us however small the product.  Measured with 16 x 16 tiles (FP64 / slices, us):
+// 128 x 512 x 32 35 / 30, 64 x 512 x 64 18 / 27, 256 x 256 x 64 36 / 30,
+// 256 x 1024 x 64 125 / 32, 64 x 64 x 1024 280 / 39.
+static double fma_rounds(double k, double tiles) { return k * std::max(0.3, tiles / 152.0); }
 bool ozgemm_eligible(const Ctx* c, const ZGemm& g) {
   if (c->oz_mode == 0 || g.batch != 1 || g.alpha.x != 1.0 || g.alpha.y != 0.0 || g.beta.x != 0.0 ||
       g.beta.y != 0.0 || g.M < 16 || g.N < 16 || g.K < 16 || g.M >= (1LL << 31) || g.N >= (1LL << 31))
     return false;
   const double tiles = (double)cdiv(g.M, 16) * (double)cdiv(g.N, 16) * (g.lower_only ? 0.5 : 1.0);
-  return (double)g.K * std::max(1.0, tiles / 152.0) >= 110.0;
+  return fma_rounds((double)g.K, tiles) >= 110.0;
 }
 
 namespace {
@@ -865,7 +867,7 @@ int zgemm_tasks(Ctx* c, const std::vector<GemmTask>& tasks) {
   for (const GemmTask& t : tasks) {
     const double k = (double)t.g.K;
     rounds += k * (double)cdiv(t.g.M, 16) * (double)cdiv(t.g.N, 16) * (t.herm ? 0.5 : 1.0) / sm;
-    longest = std::max(longest, k);
+    longest = std::max(longest, fma_rounds(k, 0.0));
   }
   const bool slices = c->oz_mode != 0 && std::max(rounds, longest) >= 110.0;
   std::vector<const GemmTask*> oz, fma;

@@ -34,22 +34,54 @@ __host__ __device__ __forceinline__ void zfma(z& acc, z a, z b) {
 }
 
 #ifdef __CUDACC__
-// acc += As[ty][0..k) Bs[0..k)[tx] for a 16 x 16 tile of 256 threads: only the k entries that
-// exist, and not at all for a warp whose two rows lie beyond `rows` (a small charge block
-// fills a fraction of its tile, and every FMA issued holds the FP64 pipe for 64 clocks); two
-// accumulators, so that consecutive terms do not wait for one another
-__device__ __forceinline__ void tile16_fma(z& acc, const z (*As)[17], const z (*Bs)[17], int rows, int k) {
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  if ((ty & ~1) >= rows) return;
-  z a1 = zmk(0, 0);
-  int kk = 0;
+// One R x 16 tile at (m0, n0) of op(A) B over all of K by 256 threads, 16 / R of them per output,
+// each taking every (16 / R)-th term; returned to threads 0 .. 16 R - 1 (row threadIdx.x / 16).
+// Only the K entries that exist are multiplied, and none by a warp whose rows lie beyond M (a
+// small charge block fills a fraction of its tile, and every FMA issued holds the FP64 pipe
+// for 64 clocks); two accumulators, so that consecutive terms do not wait for one another.
+template <int R>
+__device__ __forceinline__ z tile_product(const z* __restrict__ A, int64_t a_rs, int64_t a_cs, int conj_a,
+                                          const z* __restrict__ B, int64_t b_rs, int64_t b_cs, int conj_b, int64_t m0,
+                                          int64_t n0, int64_t M, int64_t N, int64_t K, z (*As)[17], z (*Bs)[17],
+                                          z* part) {
+  constexpr int G = 16 / R;  // threads per output
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4, row = ty % R, grp = ty / R;
+  z acc = zmk(0, 0), a1 = zmk(0, 0);
+  // the operands of the next 16 terms are loaded while these are multiplied
+  const bool ina = ty < R && m0 + ty < M, inb = n0 + tx < N;
+  const z* pa = A + (m0 + ty) * a_rs;
+  const z* pb = B + (n0 + tx) * b_cs;
+  z va = ina && tx < K ? pa[tx * a_cs] : zmk(0, 0);
+  z vb = inb && ty < K ? pb[ty * b_rs] : zmk(0, 0);
+  for (int64_t k0 = 0; k0 < K; k0 += 16) {
+    if (ty < R) As[ty][tx] = zmk(va.x, conj_a ? -va.y : va.y);
+    Bs[ty][tx] = zmk(vb.x, conj_b ? -vb.y : vb.y);
+    __syncthreads();
+    const int64_t k1 = k0 + 16;
+    va = ina && k1 + tx < K ? pa[(k1 + tx) * a_cs] : zmk(0, 0);
+    vb = inb && k1 + ty < K ? pb[(k1 + ty) * b_rs] : zmk(0, 0);
+    if (m0 + (row & ~1) < M) {
+      const int k = (int)(K - k0 < 16 ? K - k0 : 16);
+      int kk = grp;
 #pragma unroll 4
-  for (; kk + 2 <= k; kk += 2) {
-    zfma(acc, As[ty][kk], Bs[kk][tx]);
-    zfma(a1, As[ty][kk + 1], Bs[kk + 1][tx]);
+      for (; kk + G < k; kk += 2 * G) {
+        zfma(acc, As[row][kk], Bs[kk][tx]);
+        zfma(a1, As[row][kk + G], Bs[kk + G][tx]);
+      }
+      if (kk < k) zfma(acc, As[row][kk], Bs[kk][tx]);
+    }
+    __syncthreads();
   }
-  if (kk < k) zfma(acc, As[ty][kk], Bs[kk][tx]);
   acc = zadd(acc, a1);
+  if (G > 1) {
+    part[threadIdx.x] = acc;
+    __syncthreads();
+    if (grp == 0)
+#pragma unroll
+      for (int q = 1; q < G; ++q) acc = zadd(acc, part[q * R * 16 + threadIdx.x]);
+    __syncthreads();
+  }
+  return acc;
 }
 #endif
 
@@ -175,6 +207,8 @@ struct ZGemm {
   int lower_only;  // Hermitian result: skip 64x64 tiles strictly above the diagonal
 };
 int zgemm(Ctx* c, const ZGemm& g);
+// height (16, 8 or 4) of the tiles of a small FP64 product of `tiles` 16 x 16 tiles
+int tile_rows(int64_t tiles, int nsm);
 // FP64-accurate C = A B on the tensor cores by exact integer slicing (oz.cu); zgemm routes
 // large products with alpha = 1, beta = 0, batch = 1 there when the context allows it
 bool ozgemm_eligible(const Ctx* c, const ZGemm& g);
@@ -268,13 +302,11 @@ int vec_gs_reset(Ctx* c);
 int vec_gs_step(Ctx* c, const z* V, int k, const z* w, int64_t n, z* vnext, double* d_alpha,
                 double* d_beta);
 
-// Lanczos tridiagonal: lowest eigenpair of T (k x k) given alpha[0..k-1], beta[0..k-2];
-// writes out[0] = E, out[1] = |y_{k-1}|, and y[0..k-1].
-int tridiag_lowest(Ctx* c, const double* d_alpha, const double* d_beta, int k, double* d_out,
-                   double* d_y);
-// The same on stream st (the Lanczos runs it on the context's side stream)
+// Lanczos tridiagonal: lowest eigenpair of T (k x k) given alpha[0..k-1], beta[0..k-2], on
+// stream st (the Lanczos runs it on the context's side stream); writes out[0] = E,
+// out[1] = |y_{k-1}|, y[0..k-1], and E, |y_{k-1}|, beta[k-1] to the pinned host array h_out.
 int tridiag_lowest_on(Ctx* c, cudaStream_t st, const double* d_alpha, const double* d_beta, int k,
-                      double* d_out, double* d_y);
+                      double* d_out, double* d_y, double* h_out);
 // Creates the context's side stream and its events on first use
 int side_stream(Ctx* c);
 // the same for nprob problems at once: problem p's alpha, beta, y at p * 64, out at p * 2;

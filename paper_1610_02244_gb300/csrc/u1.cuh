@@ -181,7 +181,7 @@ struct U1Plan {
   int runs[2] = {0, 0};      // matvecs so far per precision: the graph is built at the second
   // tile choice (autotuned): N tile of stage 1 and stage 4, split-K of stage 4
   int bn1 = 128, bn4 = 128, split4 = 1;
-  int ztile = 64;                   // FP64 grouped tiles: 64 x 64, or 16 x 16 for small structures
+  int ztile = 64;                   // FP64 grouped tiles: 64 x 64, or 16, 8 or 4 x 16 for small structures
   CUtensorMap tmA1, tmB1, tmA4, tmB4;  // B maps are rebuilt for the chosen N tile
   // CUDA graphs of one matvec per precision (input / output pointers patched per replay)
   cudaGraph_t graph[2] = {nullptr, nullptr};

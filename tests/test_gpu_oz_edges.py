@@ -29,7 +29,8 @@ def dev(x):
 
 
 @pytest.mark.parametrize("M,N,K", [(16, 16, 16 * 110), (17, 4100, 130), (127, 63, 257), (128, 64, 256), (129, 65, 258),
-                                   (130, 1, 400), (255, 193, 31), (700, 130, 33), (64, 64, 8192)])
+                                   (130, 1, 400), (255, 193, 31), (700, 130, 33), (64, 64, 8192), (127, 63, 513), (128, 64, 512),
+                                   (129, 65, 514)])
 @pytest.mark.parametrize("conj,order", [(False, "rr"), (True, "cc")])
 def test_ragged_products(ctx, M, N, K, conj, order):
     g = synth.rng(M + 3 * N + 7 * K)
