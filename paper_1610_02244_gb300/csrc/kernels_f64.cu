@@ -915,24 +915,29 @@ int vec_normalize(Ctx* c, const z* x, z* y, int64_t n, const double* d_norm2) {
 }
 
 // ============================================================ one Gram-Schmidt step
-// The vector work of one FP64 Krylov step in one cooperative launch: two classical
-// Gram-Schmidt passes of w against V[0..k), the norm, and the next basis vector.
-//   phase 1: c = V^H w           | grid barrier
-//   phase 2: w -= V c, c' = V^H w | grid barrier
+// The vector work of one FP64 Krylov step in one cooperative launch: w orthogonalised against
+// V[0..k), the norm, and the next basis vector.  A is Hermitian, so that w = A v_{k-1} has
+// components above the rounding level along v_{k-1} and v_{k-2} only: those two are taken out
+// first, then one classical Gram-Schmidt pass over all of V.
+//   phase 1: c = (v_{k-2}, v_{k-1})^H w    | grid barrier
+//   phase 2: w -= (v_{k-2}, v_{k-1}) c, c' = V^H w | grid barrier
 //   phase 3: w -= V c', v_k = w / |w|
-// |w|^2 after phase 3 is |w|^2 before it (summed with c') minus |c'|^2, V being orthonormal;
-// where c' takes more than a quarter of it, the sum is taken directly behind a third barrier.
+// |w|^2 after phase 3 is |w|^2 before it (summed with c') minus |c'|^2, V being orthonormal.
+// Where c' takes more than a quarter of it (w nearly in the span of V), one pass is not
+// enough: a second one over all of V follows, and the sum is taken directly (two more
+// barriers).
 // CTA b keeps elements [b S, (b + 1) S) of w in shared memory, and of the basis too where
-// they fit (k S 16 bytes), so that V is read from L2 once.  Each warp takes whole vectors
+// they fit (k S 16 bytes), copied there while phase 1 runs.  Each warp takes whole vectors
 // (v = warp, warp + 8, ...) of its CTA's slice: the lanes' sums are combined by a transposed
 // butterfly over four vectors' eight sums (nine FP64 adds instead of 40).  The partial sums
 // of all CTAs are added in CTA order by every CTA, so all hold the same c, and the result is
 // deterministic.
-// What bounds it: the FP64 pipe, 16 k n FMAs at two per SM and clock (27 us at n = 65536,
-// k = 16), and three grid barriers.  The separate launches it replaces took
-// 160 us there (four dot-product launches of eight vectors at 27 to 30 us, whatever n: with
-// one element per thread each spent its time reducing 16 sums per thread), 115 us at
-// n = 5000.
+// What bounds it: the FP64 pipe, 8 (k + 2) n FMAs at two per SM and clock (15 us at n = 65536,
+// k = 16), and two grid barriers.  Measured over a solve at n = 65536, k up to 32: 35 us a
+// step on average, 55 us with both passes over all of V; at n of about 2000 16 and 24 us.  The separate
+// launches it replaces took 160 us there (four dot-product launches of eight vectors at 27 to
+// 30 us, whatever n: with one element per thread each spent its time reducing 16 sums per
+// thread), 115 us at n = 5000.
 namespace {
 constexpr int GS_THREADS = 256, GS_WARPS = GS_THREADS / 32;
 constexpr int GS_SMEM = 204 * 1024;
@@ -1007,9 +1012,26 @@ __device__ __forceinline__ double sum8(double* s) {
   return r;
 }
 
+// four sums over the warp: lane l returns the total of s[l & 3]
+__device__ __forceinline__ double sum4(double* s) {
+  const int l = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 2; o >= 1; o >>= 1) {
+    const bool up = (l & o) != 0;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const double give = up ? s[i] : s[i + o], keep = up ? s[i + o] : s[i];
+      s[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  double r = s[0];
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  return r;
+}
+
 // the CTA's share of V^H w to part[v][blockIdx.x]
-template <bool STORE>
-__device__ void gs_dots(const GsArgs& a, const z* sw, z* sv, const z* V0, int64_t ld, int cnt, z* part) {
+__device__ void gs_dots(const GsArgs& a, const z* sw, const z* V0, int64_t ld, int cnt, z* part) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int v0 = warp; v0 < a.k; v0 += 4 * GS_WARPS) {
     double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -1025,7 +1047,6 @@ __device__ void gs_dots(const GsArgs& a, const z* sw, z* sv, const z* V0, int64_
         for (int q = 0; q < 4; ++q) u[q] = p0[q * st + e];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          if (STORE) sv[(int64_t)(v0 + q * GS_WARPS) * a.S + e] = u[q];
           s[2 * q] = fma(u[q].x, x.x, fma(u[q].y, x.y, s[2 * q]));
           s[2 * q + 1] = fma(u[q].x, x.y, fma(-u[q].y, x.x, s[2 * q + 1]));
         }
@@ -1037,7 +1058,6 @@ __device__ void gs_dots(const GsArgs& a, const z* sw, z* sv, const z* V0, int64_
 #pragma unroll 4
         for (int e = lane; e < cnt; e += 32) {
           const z x = sw[e], u = p0[q * st + e];
-          if (STORE) sv[(int64_t)(v0 + q * GS_WARPS) * a.S + e] = u;
           s[2 * q] = fma(u.x, x.x, fma(u.y, x.y, s[2 * q]));
           s[2 * q + 1] = fma(u.x, x.y, fma(-u.y, x.x, s[2 * q + 1]));
         }
@@ -1128,27 +1148,77 @@ __global__ void __launch_bounds__(GS_THREADS, 1) k_gs_step(GsArgs a) {
   __shared__ double sh[32];
   __shared__ double s_rn;
   __shared__ int s_direct;
+  __shared__ double s4[GS_WARPS][4];
   z* sw = sm_gs;
   z* sv = sm_gs + a.S;
   const int64_t lo = (int64_t)blockIdx.x * a.S;
   const int cnt = (int)max((int64_t)0, min((int64_t)a.S, a.n - lo));
-  const int tid = threadIdx.x;
-  for (int e = tid; e < cnt; e += GS_THREADS) sw[e] = a.w[lo + e];
-  __syncthreads();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   z* p1 = a.part;
   z* p2 = a.part + (int64_t)64 * gridDim.x;
   const z* Vg = a.V + lo;
-  if (a.keep) gs_dots<true>(a, sw, sv, Vg, a.n, cnt, p1);
-  else gs_dots<false>(a, sw, sv, Vg, a.n, cnt, p1);
+  const z* Va = Vg + (int64_t)(a.k - 1) * a.n;                 // v_{k-1}
+  const z* Vb = Vg + (int64_t)(a.k > 1 ? a.k - 2 : 0) * a.n;   // v_{k-2}; k = 1: taken with c = 0
+  double d4[4] = {0, 0, 0, 0};
+  for (int e = tid; e < cnt; e += GS_THREADS) {
+    const z x = a.w[lo + e], u = Va[e], u1 = Vb[e];
+    sw[e] = x;
+    d4[0] = fma(u.x, x.x, fma(u.y, x.y, d4[0]));
+    d4[1] = fma(u.x, x.y, fma(-u.y, x.x, d4[1]));
+    d4[2] = fma(u1.x, x.x, fma(u1.y, x.y, d4[2]));
+    d4[3] = fma(u1.x, x.y, fma(-u1.y, x.x, d4[3]));
+  }
+  if (a.keep) {
+    for (int v = warp; v < a.k; v += GS_WARPS)
+      for (int e = lane; e < cnt; e += 32)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(sv + (int64_t)v * a.S + e)),
+                     "l"(Vg + (int64_t)v * a.n + e)
+                     : "memory");
+  }
+  const int nw = min(GS_WARPS, (cnt + 31) >> 5);  // warps that have elements
+  if (warp < nw) {
+    const double r = sum4(d4);
+    if (lane < 4) s4[warp][lane] = r;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    double r = (lane >> 2) < nw ? s4[lane >> 2][lane & 3] : 0.0;
+    for (int o = 4; o < 4 * nw; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if (lane < 4) ((double*)(p1 + (int64_t)(lane >> 1) * gridDim.x + blockIdx.x))[lane & 1] = r;
+  }
   const z* V = a.keep ? sv : Vg;
   const int64_t ld = a.keep ? a.S : a.n;
   bool ok = gs_barrier(a, a.base + 1u * gridDim.x);
+  asm volatile("cp.async.wait_all;" ::: "memory");
   if (ok) {
-    gs_total(a, p1, sc);
-    if (blockIdx.x == 0 && tid == 0) a.alpha[a.k - 1] = sc[a.k - 1].x;
-    double acc = gs_update(a, sw, V, ld, cnt, sc, sacc);
+    if (warp < 2) {
+      double re = 0, im = 0;
+      for (int b = lane; b < (int)gridDim.x; b += 32) {
+        const z p = __ldcg(p1 + (int64_t)warp * gridDim.x + b);
+        re += p.x;
+        im += p.y;
+      }
+      re = warp_sum(re);
+      im = warp_sum(im);
+      if (lane == 0) sc[warp] = warp == 1 && a.k == 1 ? zmk(0, 0) : zmk(re, im);
+    }
     __syncthreads();
-    gs_dots<false>(a, sw, sv, V, ld, cnt, p2);
+    const z c0 = sc[0], c1 = sc[1];
+    if (blockIdx.x == 0 && tid == 0) a.alpha[a.k - 1] = c0.x;
+    double acc = 0;
+    for (int e = tid; e < cnt; e += GS_THREADS) {
+      const z u = V[(int64_t)(a.k - 1) * ld + e], u1 = V[(int64_t)(a.k > 1 ? a.k - 2 : 0) * ld + e];
+      z x = sw[e];
+      x.x = fma(-c0.x, u.x, fma(c0.y, u.y, x.x));
+      x.y = fma(-c0.x, u.y, fma(-c0.y, u.x, x.y));
+      x.x = fma(-c1.x, u1.x, fma(c1.y, u1.y, x.x));
+      x.y = fma(-c1.x, u1.y, fma(-c1.y, u1.x, x.y));
+      sw[e] = x;
+      acc = fma(x.x, x.x, fma(x.y, x.y, acc));
+    }
+    __syncthreads();
+    gs_dots(a, sw, V, ld, cnt, p2);
     acc = block_sum(acc, sh);
     if (tid == 0) a.npart[blockIdx.x] = acc;
     ok = gs_barrier(a, a.base + 2u * gridDim.x);
@@ -1169,13 +1239,18 @@ __global__ void __launch_bounds__(GS_THREADS, 1) k_gs_step(GsArgs a) {
         s_direct = !(q <= 0.25 * r);
       }
     }
-    const double acc0 = gs_update(a, sw, V, ld, cnt, sc, sacc);
+    gs_update(a, sw, V, ld, cnt, sc, sacc);
     __syncthreads();
     if (s_direct) {  // the same decision in every CTA
       __shared__ double sh2[32];
-      const double acc = block_sum(acc0, sh2);
-      if (tid == 0) a.npart[gridDim.x + blockIdx.x] = acc;
+      gs_dots(a, sw, V, ld, cnt, p1);
       ok = gs_barrier(a, a.base + 3u * gridDim.x);
+      if (ok) {
+        gs_total(a, p1, sc);
+        const double acc = block_sum(gs_update(a, sw, V, ld, cnt, sc, sacc), sh2);
+        if (tid == 0) a.npart[gridDim.x + blockIdx.x] = acc;
+        ok = gs_barrier(a, a.base + 4u * gridDim.x);
+      }
       if (ok && tid < 32) {
         double r = 0;
         for (int b = tid; b < (int)gridDim.x; b += 32) r += __ldcg(a.npart + gridDim.x + b);
@@ -1183,8 +1258,8 @@ __global__ void __launch_bounds__(GS_THREADS, 1) k_gs_step(GsArgs a) {
         if (tid == 0) sh[0] = r;
       }
     } else if (blockIdx.x == 0 && tid == 0) {
-      // the launch counts three arrivals per CTA
-      asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(a.bar), "r"(gridDim.x) : "memory");
+      // the launch counts four arrivals per CTA
+      asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(a.bar), "r"(2u * gridDim.x) : "memory");
     }
   }
   if (!ok) {  // the host reads a NaN beta, and the status word names the wait
@@ -1245,14 +1320,14 @@ int vec_gs_step(Ctx* c, const z* V, int k, const z* w, int64_t n, z* vnext, doub
   a.status = c->d_status;
   a.S = (int)std::max<int64_t>(64, (n + nsm - 1) / nsm);
   const int grid = (int)((n + a.S - 1) / a.S);
-  c->gs_arrivals += 3u * (unsigned)grid;
+  c->gs_arrivals += 4u * (unsigned)grid;
   const size_t sw = sizeof(z) * (size_t)a.S, all = sw * (size_t)(k + 1);
   a.keep = all <= (size_t)GS_SMEM;
   const size_t smem = a.keep ? all : sw;
   if (smem > (size_t)GS_SMEM) return set_err(c, TNT_E_UNSUPPORTED, "Gram-Schmidt step with n = %lld", (long long)n);
   void* args[] = {&a};
   {
-    ProfScope ps(c, "gs_step", (32.0 * (double)k + 6.0) * (double)n);  // FP64 FLOPs
+    ProfScope ps(c, "gs_step", (16.0 * (double)k + 38.0) * (double)n);  // FP64 FLOPs
     TNT_CUDA_TRY(c, cudaLaunchCooperativeKernel((void*)k_gs_step, dim3((unsigned)grid), dim3(GS_THREADS), args,
                                                 smem, c->stream));
   }
