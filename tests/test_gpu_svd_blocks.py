@@ -69,3 +69,17 @@ def test_many_uneven_blocks(ctx, sizes, side):
     M = synth.complex_gaussian(g, (len(rq), len(cq))) * (rq[:, None] == cq[None, :])
     M *= np.logspace(0, -2, len(cq))[None, :]
     check(ctx, M, rq, cq, side=side)
+
+
+@pytest.mark.parametrize("n", [3, 33, 130, 400])
+@pytest.mark.parametrize("spectrum", ["graded", "equal", "exact_pairs", "near_pairs", "two_levels"])
+def test_spacings_of_the_eigenvalues(ctx, n, spectrum):
+    """Brackets that hold one eigenvalue, several or a whole cluster: the determinants at their
+    ends guide the bisection in the first case only."""
+    h = np.linspace(1.0, 0.3, (n + 1) // 2)
+    s = {"graded": np.logspace(0, -4, n), "equal": np.ones(n), "exact_pairs": np.repeat(h, 2)[:n],
+         "near_pairs": (np.repeat(h, 2) * np.tile([1.0, 1.0 - 1e-9], h.size))[:n],
+         "two_levels": np.where(np.arange(n) < n // 2, 1.0, 1e-3)}[spectrum]
+    g = synth.rng(n)
+    U, V = (np.linalg.qr(synth.complex_gaussian(g, (n, n)))[0] for _ in range(2))
+    check(ctx, (U * s) @ V)
