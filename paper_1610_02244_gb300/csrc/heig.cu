@@ -746,7 +746,9 @@ __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_
         const int q = lane + 32 * i;
         s[i] = q < nb ? (one ? partj[q] : __ldcg(partj + q)) : 0.0;
       }
-      k = ((s[0] + s[1]) + (s[2] + s[3])) + s[4];
+      k = s[0];
+      if (nb > 64) k = (s[0] + s[1]) + ((s[2] + s[3]) + s[4]);
+      else if (nb > 32) k = s[0] + s[1];
       for (int q = lane + 160; q < nb; q += 32) k += __ldcg(partj + q);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
@@ -997,10 +999,12 @@ __global__ void k_split(const double* __restrict__ dAll, const double* __restric
     tn = fmax(tn, fabs(d[r]) + (r > 0 ? fabs(e[r - 1]) : 0.0) + (r < n - 1 ? fabs(e[r]) : 0.0));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, o));
+  const double tol = SPLIT_TOL * tn;
+  int64_t s = 0;  // one past the last row that is not negligible
+  for (int64_t r = lane; r < n; r += 32)
+    if (!(fabs(d[r]) <= tol && (r == 0 || fabs(e[r - 1]) <= tol))) s = r + 1;
+  s = __reduce_max_sync(0xffffffffu, (int)s);
   if (lane == 0) {
-    const double tol = SPLIT_TOL * tn;
-    int64_t s = n;
-    while (s > 0 && fabs(d[s - 1]) <= tol && (s - 1 == 0 || fabs(e[s - 2]) <= tol)) --s;
     tnorm[blockIdx.x] = tn;
     nr[blockIdx.x] = s;
   }
@@ -1078,7 +1082,9 @@ __global__ void __launch_bounds__(32) k_bisect(const double* __restrict__ dAll, 
     hi = fmin(hi, h2);
   }
   __syncwarp();
-  const double tol = 1e-300;  // full precision: the shifts must resolve close eigenvalues
+  // full precision, the shifts must resolve close eigenvalues: 4 eps |lambda|, but no more than
+  // the last bit of the largest ones, which T itself does not hold
+  const double tol = fmax(1e-300, 0.5 * EPS * w0);
   double guess = 0;
   bool guided = false;
   for (int it = 0; it < 64; ++it) {
@@ -1335,6 +1341,7 @@ __global__ void __launch_bounds__(256) k_backtransform(const double* __restrict_
     const z t = tau[j];
     if (t.x == 0.0 && t.y == 0.0) continue;
     const int64_t m = n - j - 1;
+    const int nw = (int)(m < 256 ? (m + 31) >> 5 : 8);  // warps that have entries
     const z* v = Hv + j * n;
     double s4[2 * BT_COLS] = {0, 0, 0, 0};  // s = v^H y[j+1:] per column, (re, im) pairs
     for (int64_t r = threadIdx.x; r < m; r += blockDim.x) {
@@ -1347,15 +1354,14 @@ __global__ void __launch_bounds__(256) k_backtransform(const double* __restrict_
         s4[2 * q + 1] = fma(a.x, b.y, fma(-a.y, b.x, s4[2 * q + 1]));
       }
     }
-    {  // the four sums: seven adds per warp, then a butterfly over the warps' sums
+    if (warp < nw) {  // the four sums: seven adds per warp, then a butterfly over the warps' sums
       const double s = warp_sum4(s4);
       if (lane < 4) shw[warp][lane] = s;
     }
     __syncthreads();
     if (warp == 0) {  // lane = (warp's sum, value): lane l holds value l & 3 of warp l >> 2
-      double s = shw[lane >> 2][lane & 3];
-#pragma unroll
-      for (int o = 16; o >= 4; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      double s = (lane >> 2) < nw ? shw[lane >> 2][lane & 3] : 0.0;
+      for (int o = 4; o < 4 * nw; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
       const double im = __shfl_down_sync(0xffffffffu, s, 1);
       if (lane < 4 && (lane & 1) == 0) s_ts[lane >> 1] = zmul(t, zmk(s, im));
     }

@@ -16,6 +16,7 @@
 #include <cmath>
 #include <map>
 
+#include "f32conv.cuh"
 #include "tnt_internal.cuh"
 
 namespace tnt {
@@ -144,8 +145,10 @@ struct SelOut {
 // suffix sums over the block: thread t's values v[0..m) are elements t m .. t m + m - 1; on
 // return v[i] is the sum of element t m + i and all after it (threads in order, every step the
 // same tree: deterministic)
-__device__ void block_suffix(double* v, int m, double* sh) {
+template <int m>
+__device__ void block_suffix(double* v, double* sh) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+#pragma unroll
   for (int i = m - 2; i >= 0; --i) v[i] += v[i + 1];
   double s = v[0];  // inclusive suffix over the warp's lanes
 #pragma unroll
@@ -166,13 +169,19 @@ __device__ void block_suffix(double* v, int m, double* sh) {
   double after = __shfl_down_sync(0xffffffffu, s, 1);
   if (lane == 31) after = 0.0;
   after += later;
+#pragma unroll
   for (int i = 0; i < m; ++i) v[i] += after;
 }
 
 // All candidates in order (sigma descending, block ascending, index ascending), then the four
 // rules.  Keys compare as their bit patterns (non-negative doubles order as integers; the
 // padding is negative), and the rules take searches and block-wide sums: one thread's serial
-// loops over the candidates, with an FP64 division each, took 1.7 ms for 2600 of them.
+// loops over the candidates, with an FP64 division each, took 1.7 ms for 2600 of them.  m
+// candidates a thread, and no more threads than they need: every warp's FP64 sums hold the
+// pipes of the one SM.  Square roots and divisions are taken only where a comparison of
+// squares or products is too close to decide (a chain of some twenty FP64 instructions each);
+// the searches try 32 places at once.
+template <int m>
 __global__ void __launch_bounds__(1024) k_select(const double* __restrict__ sig_in,
                                                  const int* __restrict__ blk_in,
                                                  const int* __restrict__ loc_in, int n, int P,
@@ -223,17 +232,15 @@ __global__ void __launch_bounds__(1024) k_select(const double* __restrict__ sig_
     blk_out[i] = bk[i];
     loc_out[i] = lc[i];
   }
-  constexpr int MAXV = 8;  // 8192 candidates
-  const int m = (n + (int)blockDim.x - 1) / (int)blockDim.x;
-  double v[MAXV];
+  double v[m];
   // the candidates are each block's leading min(rank, chi_max) values; when that cuts a
   // block short, the weight of the values never formed is |M|_F^2 minus the candidates'
 #pragma unroll
-  for (int i = 0; i < MAXV; ++i) {
+  for (int i = 0; i < m; ++i) {
     const int q = tid * m + i;
-    v[i] = i < m && q < n ? val(q) * val(q) : 0.0;
+    v[i] = q < n ? val(q) * val(q) : 0.0;
   }
-  block_suffix(v, m, sh);
+  block_suffix<m>(v, sh);
   if (tid == 0) {
     const double sumc = v[0];
     s_nrm2 = complete ? sumc : fmax(total_norm2[0], sumc);
@@ -242,58 +249,83 @@ __global__ void __launch_bounds__(1024) k_select(const double* __restrict__ sig_
   }
   __syncthreads();
   const double nrm2 = s_nrm2, unseen = s_unseen;
-  const double nrm = sqrt(nrm2);
-  const double inv = nrm > 0 ? 1.0 / nrm : 1.0;
+  const int nex = (__double2hiint(nrm2) >> 20) & 0x7ff;
+  const double inv = nex > 100 && nex < 1946 ? rsqrt_newton(nrm2) : nrm2 > 0 ? 1.0 / sqrt(nrm2) : 1.0;
   auto errf = [&](double acc) { return etype == TNT_TRUNC_2NORM ? sqrt(acc) : acc; };
+  // errf(acc) < etol; a square root only where the squares leave it open
+  const double et2 = etol * etol;
+  const bool clear = etype == TNT_TRUNC_2NORM && et2 > 1e-200 && et2 < 1e200;
+  auto small = [&](double acc) {
+    if (clear && acc < et2 * (1.0 - 1e-12)) return true;
+    if (clear && acc > et2 * (1.0 + 1e-12)) return false;
+    return errf(acc) < etol;
+  };
   const double acc0 = unseen * inv * inv;  // never formed values, in normalised units
-  double u[MAXV];  // truncation error terms of an element and all after it
+  double u[m];  // truncation error terms of an element and all after it
 #pragma unroll
-  for (int i = 0; i < MAXV; ++i) {
+  for (int i = 0; i < m; ++i) {
     const int q = tid * m + i;
-    const double s = i < m && q < n ? val(q) * inv : 0.0;
+    const double s = q < n ? val(q) * inv : 0.0;
     u[i] = etype == TNT_TRUNC_1NORM ? fabs(s) : s * s;
   }
-  block_suffix(u, m, sh);
+  block_suffix<m>(u, sh);
   // rule 4: the smallest keep whose discards stay below the tolerance (they grow towards 0)
-  if (errf(acc0) < etol)
-    for (int i = 0; i < m; ++i) {
+  if (small(acc0))
+#pragma unroll
+    for (int i = m - 1; i >= 0; --i) {
       const int q = tid * m + i;
-      if (q < n && errf(acc0 + u[i]) < etol) {
-        atomicMin(&s_chi4, q);
-        break;
-      }
+      if (q < n && small(acc0 + u[i])) atomicMin(&s_chi4, q);
     }
   __syncthreads();
-  if (tid == 0) {
+  if (tid < 32) {
     const double s0 = n > 0 ? val(0) : 0.0;
     // first index whose value fails a bound that holds on a prefix
     auto prefix = [&](auto holds) {
       int lo = 0, hi = n;
       while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (holds(val(mid))) lo = mid + 1;
-        else hi = mid;
+        const int w = (hi - lo + 31) / 32, q = lo + tid * w;
+        const int ok = __popc(__ballot_sync(0xffffffffu, q < hi && holds(val(q < hi ? q : lo))));
+        if (ok == 0) hi = lo;
+        else {
+          hi = min(hi, lo + ok * w);  // place ok fails, or is past the end
+          lo += (ok - 1) * w + 1;
+        }
       }
       return (int64_t)lo;
     };
     int64_t chi = n < chi_max ? n : chi_max;
     if (a > 0) chi = min(chi, prefix([&](double s) { return s >= a; }));
-    if (s0 > 0) chi = min(chi, prefix([&](double s) { return s / s0 >= rtol; }));
+    if (s0 > 0) {
+      const double b = rtol * s0;  // a division only where the product leaves it open
+      const bool sure = b > 1e-280 && b < 1e280;
+      chi = min(chi, prefix([&](double s) {
+                  if (sure && s > b * (1.0 + 1e-12)) return true;
+                  if (sure && s < b * (1.0 - 1e-12)) return false;
+                  return s / s0 >= rtol;
+                }));
+    }
     chi = min(chi, (int64_t)s_chi4);
     if (chi < 1) chi = 1;
     if (chi > n) chi = n;
-    res->chi = chi;
-    res->err = errf(acc0);
-    res->disc = unseen;
-    res->norm2 = nrm2;
-    res->tie = (chi < n) && (val((int)chi - 1) - val((int)chi) < 1e-10 * s0);
-    s_chi4 = (int)chi;
+    __syncwarp();
+    if (tid == 0) {
+      res->chi = chi;
+      res->err = errf(acc0);
+      res->disc = unseen;
+      res->norm2 = nrm2;
+      res->tie = (chi < n) && (val((int)chi - 1) - val((int)chi) < 1e-10 * s0);
+      s_chi4 = (int)chi;
+    }
   }
   __syncthreads();
   const int chi = s_chi4;
   if (chi < n && tid == chi / m) {  // this thread holds the first discarded value
-    res->err = errf(acc0 + u[chi % m]);
-    res->disc = unseen + v[chi % m];
+#pragma unroll
+    for (int i = 0; i < m; ++i)
+      if (i == chi % m) {
+        res->err = errf(acc0 + u[i]);
+        res->disc = unseen + v[i];
+      }
   }
 }
 
@@ -803,12 +835,15 @@ int svd_trunc_impl(Ctx* c, const z* M, int64_t m, int64_t n, const int64_t* h_rq
   // ---- global order and the four rules
   {
     size_t smem = (size_t)P2 * (sizeof(double) + 2 * sizeof(int));
-    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    auto select = ntot_vals <= 4096 ? k_select<4> : k_select<8>;  // 8192 candidates at most
+    unsigned threads = 64;
+    while (threads < 1024 && 4 * (int64_t)threads < ntot_vals) threads *= 2;
+    TNT_CUDA_TRY(c, cudaFuncSetAttribute(select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // never more than the blocks' rank bounds (at most min(m, n), the callers' capacity),
     // whatever the number of candidates formed
     int64_t rank_total = 0;
     for (const Blk& B : bl) rank_total += B.r;
-    k_select<<<1, 1024, smem, st>>>(d_sig, d_blk, d_loc, (int)ntot_vals, P2,
+    select<<<1, threads, smem, st>>>(d_sig, d_blk, d_loc, (int)ntot_vals, P2,
                                     std::min<int64_t>(P.chi_max, rank_total), P.trunc_abs,
                                     P.trunc_rel, P.trunc_err, P.trunc_type, d_tot, complete ? 1 : 0,
                                     d_sig_s, d_blk_s, d_loc_s, d_sel);
