@@ -426,15 +426,26 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(const __grid_constant
 // element per thread, a block's 256 elements in one task.  Hermitian results: the lower
 // triangle, mirrored.
 template <int CAP>
-__global__ void __launch_bounds__(256) k_oz_finish(const __grid_constant__ OzTasks<CAP> T) {
+__global__ void __launch_bounds__(256, 5) k_oz_finish(const __grid_constant__ OzTasks<CAP> T) {
   for (int fb = blockIdx.x; fb < T.h.fin_blocks; fb += gridDim.x) {
     const OzTask& g = T.at(oz_find(T, [](const OzTask& t) { return t.fin0; }, fb));
-    const int64_t total = (int64_t)g.M * g.N, e = (int64_t)(fb - g.fin0) * 256 + threadIdx.x;
+    const int64_t total = (int64_t)g.M * g.N, e0 = (int64_t)(fb - g.fin0) * 256, e = e0 + threadIdx.x;
     if (e >= total) continue;
-    const int64_t i = e / g.N, j = e % g.N;
+    // row and column from the block's first element, in 32 bits (a 64-bit division a thread
+    // cost as much as both conversions)
+    const unsigned N = (unsigned)g.N;
+    int64_t i = e < (1ll << 32) ? (unsigned)e0 / N : e0 / N;
+    unsigned j = (unsigned)(e0 - i * N) + threadIdx.x;
+    if (N > 256) {
+      if (j >= N) j -= N, ++i;
+    } else {
+      i += j / N;
+      j %= N;
+    }
     if (g.herm && j > i) continue;
     const longlong2* P = (const longlong2*)(T.h.buf + g.offP) + e;
     longlong2 h = make_longlong2(0, 0), l = h;
+#pragma unroll 2
     for (int s = 0; s < g.ks; ++s) {
       const longlong2 a = P[(int64_t)(2 * s) * total], b = P[(int64_t)(2 * s + 1) * total];
       h.x += a.x;
@@ -476,14 +487,16 @@ __device__ __forceinline__ OzOp oz_operand(const OzTask& g, const OzHead& h, boo
 }
 
 // largest exponent field of every row.  Entries contiguous along K: one warp per row;
-// otherwise 32 rows by up to OZ_SCALE_K of K per CTA, neighbouring lanes on neighbouring rows
-// (a longer K combines its parts with an atomic maximum, e zeroed before)
+// otherwise 8 rows by up to OZ_SCALE_K of K per CTA, eight neighbouring lanes on neighbouring
+// rows, one 128-byte line (a longer K combines its parts with an atomic maximum, e zeroed
+// before).  Latency-bound: with 32 rows a CTA there were 64 of them for 2048 rows, and each
+// thread had 64 loads to make.
 constexpr int OZ_SCALE_K = 512;
 __device__ __forceinline__ unsigned oz_exp(z v) {
   return max(((unsigned)__double2hiint(v.x) >> 20) & 0x7ffu, ((unsigned)__double2hiint(v.y) >> 20) & 0x7ffu);
 }
 __host__ __device__ inline int64_t oz_scale_blocks(int64_t rows, int64_t ks, int64_t K) {
-  return ks == 1 ? (rows + 7) / 8 : ((rows + 31) / 32) * ((K + OZ_SCALE_K - 1) / OZ_SCALE_K);
+  return ((rows + 7) / 8) * (ks == 1 ? 1 : (K + OZ_SCALE_K - 1) / OZ_SCALE_K);
 }
 template <int CAP>
 __global__ void __launch_bounds__(256) k_oz_scale(const __grid_constant__ OzTasks<CAP> T) {
@@ -506,19 +519,22 @@ __global__ void __launch_bounds__(256) k_oz_scale(const __grid_constant__ OzTask
     if (lane == 0) o.e[i] = (int)mx;
     return;
   }
-  __shared__ unsigned s_mx[32];
-  if (threadIdx.x < 32) s_mx[threadIdx.x] = 0;
+  __shared__ unsigned s_mx[8];
+  if (threadIdx.x < 8) s_mx[threadIdx.x] = 0;
   __syncthreads();
-  const int64_t nk = (K + OZ_SCALE_K - 1) / OZ_SCALE_K, i = (blk / nk) * 32 + lane, k0 = (blk % nk) * OZ_SCALE_K;
+  const int64_t nk = (K + OZ_SCALE_K - 1) / OZ_SCALE_K, k0 = (blk % nk) * OZ_SCALE_K, i = (blk / nk) * 8 + (lane & 7);
   unsigned mx = 0;
   if (i < o.rows) {
     const int64_t k1 = min(K, k0 + OZ_SCALE_K);
+    const z* x = o.X + i * o.rs;
 #pragma unroll 8
-    for (int64_t k = k0 + warp; k < k1; k += 8) mx = max(mx, oz_exp(o.X[i * o.rs + k * o.cs]));
+    for (int64_t k = k0 + (threadIdx.x >> 3); k < k1; k += 32) mx = max(mx, oz_exp(x[k * o.cs]));
   }
-  if (mx) atomicMax(&s_mx[lane], mx);
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+  if (mx && lane < 8) atomicMax(&s_mx[lane], mx);
   __syncthreads();
-  if (warp == 0 && i < o.rows) {
+  if (threadIdx.x < 8 && i < o.rows) {
     if (nk == 1) o.e[i] = (int)s_mx[lane];
     else atomicMax((unsigned*)o.e + i, s_mx[lane]);
   }
