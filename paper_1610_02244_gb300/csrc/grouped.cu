@@ -1245,10 +1245,10 @@ int build_graph(Ctx* c, U1Plan& p, int mixed) {
     void* ao[] = {oa};
     if (p.oz) {
       oz_plan_args(p.oz1, nullptr, oa);
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < p.oz1.nodes; ++i) {
         const OzNode& q = p.oz1.node[i];
         TNT_TRY(add(knp(q.fn, q.grid, q.block, q.smem, ao)));
-        if (i < 2) p.oz_node[i] = node;
+        if (i < p.oz1.inputs) p.oz_node[i] = node;
       }
     } else {
       void* a0[] = {&z1};
@@ -1259,7 +1259,10 @@ int build_graph(Ctx* c, U1Plan& p, int mixed) {
     TNT_TRY(add(knp((void*)k_wop<false>, gw, 256, 0, a1)));
     if (p.oz) {
       oz_plan_args(p.oz4, nullptr, oa);
-      for (const OzNode& q : p.oz4.node) TNT_TRY(add(knp(q.fn, q.grid, q.block, q.smem, ao)));
+      for (int i = 0; i < p.oz4.nodes; ++i) {
+        const OzNode& q = p.oz4.node[i];
+        TNT_TRY(add(knp(q.fn, q.grid, q.block, q.smem, ao)));
+      }
     } else {
       void* a2[] = {&z4};
       TNT_TRY(add(knp(zfn(p), cap_grid(p.n_z4tiles, zcap(p)), 256, 0, a2)));
@@ -1369,12 +1372,12 @@ int u1_run(Ctx* c, U1Plan& p, const z* x, z* y, int precision) {
       alignas(16) unsigned char oa[sizeof(p.oz1.args)];
       oz_plan_args(p.oz1, x, oa);
       void* a[] = {oa};
-      for (int i = 0; i < 2; ++i) {
+      for (int i = 0; i < p.oz1.inputs; ++i) {
         const OzNode& q = p.oz1.node[i];
         cudaKernelNodeParams k = knp(q.fn, q.grid, q.block, q.smem, a);
         TNT_CUDA_TRY(c, cudaGraphExecKernelNodeSetParams(p.exec[0], p.oz_node[i], &k));
       }
-      c->launches += 6;
+      c->launches += p.oz1.nodes + p.oz4.nodes - 2;
     } else {
       ZGArgs z1 = p.in_zg;
       z1.B = x;

@@ -81,6 +81,7 @@ struct OzTask {
   int herm;  // C = A B is Hermitian: tiles strictly above the diagonal are mirrored, not computed
   int sub;   // C -= A B
   int item0, scale0[2], fin0;            // first item / scale block (per side) / finish block
+  int grp0[2];                           // first group of eight rows, per side
 };
 // The products of one launch travel as a kernel argument (no table upload), or, for a plan
 // whose products repeat, in device memory (CAP = 0).
@@ -88,6 +89,7 @@ constexpr int OZ_MAXT = 40;
 struct OzHead {
   int n, items, fin_blocks;
   int scale_blocks[2];  // per side (A, B)
+  int groups[2];        // of eight rows, padding to whole tiles included
   int64_t atoms[2];
   int sides;            // the sides to scale and slice: bit 0 A, bit 1 B
   int64_t add_b;        // bytes added to every task's B
@@ -543,15 +545,12 @@ __global__ void __launch_bounds__(256) k_oz_scale(const __grid_constant__ OzTask
 // slices of 8 rows by 32 of K per warp: lane = (row, 8 of K), so every plane's 512-byte
 // swizzle atom is written whole.  Rows and K beyond the operand are zero.
 template <int PLANES>
-__device__ __forceinline__ void oz_slice_atom(const OzOp& o, int64_t K, int nkb, int64_t atom, int lane) {
+__device__ __forceinline__ void oz_slice_atom(const OzOp& o, int64_t K, int nkb, int64_t i8, int kb, int lane, int e) {
   constexpr int ROWS = PLANES == 2 ? OZ_BM : OZ_BN, TILE = PLANES == 2 ? OZ_TA : OZ_TB;
-  const int kb = (int)(atom % nkb);
-  const int64_t i8 = atom / nkb;  // group of 8 rows
   const int r = lane >> 2, c8 = lane & 3;
   const int64_t i = i8 * 8 + r, k0 = (int64_t)kb * OZ_KB + c8 * 8;
   uint64_t fr[8], fi[8];
   uint32_t sr[4], si[4];  // signs of the eight entries, as bits 15 and 31 of a word per pair
-  const int e = i < o.rows ? o.e[i] : 0;
   const z* x = o.X + i * o.rs + k0 * o.cs;
   z v[8];
 #pragma unroll
@@ -587,6 +586,11 @@ __device__ __forceinline__ void oz_slice_atom(const OzOp& o, int64_t K, int nkb,
     *(uint4*)(q + ROWS * 64) = make_uint4(wi[0], wi[1], wi[2], wi[3]);
   }
 }
+template <int PLANES>
+__device__ __forceinline__ void oz_slice_at(const OzOp& o, int64_t K, int nkb, int64_t atom, int lane) {
+  const int64_t i8 = atom / nkb, i = i8 * 8 + (lane >> 2);
+  oz_slice_atom<PLANES>(o, K, nkb, i8, (int)(atom % nkb), lane, i < o.rows ? o.e[i] : 0);
+}
 template <int CAP>
 __global__ void __launch_bounds__(256) k_oz_slice(const __grid_constant__ OzTasks<CAP> T) {
   const int lane = threadIdx.x & 31;
@@ -594,11 +598,58 @@ __global__ void __launch_bounds__(256) k_oz_slice(const __grid_constant__ OzTask
   for (int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); w < all; w += (int64_t)gridDim.x * 8) {
     if (w < na) {
       const OzTask& g = T.at(oz_find(T, [](const OzTask& t) { return t.atom0[0]; }, w));
-      oz_slice_atom<2>(oz_operand(g, T.h, false), g.K, g.nkb, w - g.atom0[0], lane);
+      oz_slice_at<2>(oz_operand(g, T.h, false), g.K, g.nkb, w - g.atom0[0], lane);
     } else {
       const OzTask& g = T.at(oz_find(T, [](const OzTask& t) { return t.atom0[1]; }, w - na));
-      oz_slice_atom<3>(oz_operand(g, T.h, true), g.K, g.nkb, w - na - g.atom0[1], lane);
+      oz_slice_at<3>(oz_operand(g, T.h, true), g.K, g.nkb, w - na - g.atom0[1], lane);
     }
+  }
+}
+
+// Scales and slices of K up to OZ_SCALE_K in one launch: a CTA takes eight rows, their
+// maxima first, then their slices (the second read hits L1 or L2).  Small products are bound by
+// the launches (scale and slice 5 to 7 us each); oz_one_prep says where.
+template <int CAP>
+__global__ void __launch_bounds__(256) k_oz_prep(const __grid_constant__ OzTasks<CAP> T) {
+  __shared__ unsigned s_mx[8];
+  const int na = (T.h.sides & 1) ? T.h.groups[0] : 0;
+  const bool isb = (int)blockIdx.x >= na;
+  const int w = (int)blockIdx.x - (isb ? na : 0);
+  const OzTask& g = T.at(isb ? oz_find(T, [](const OzTask& t) { return t.grp0[1]; }, w)
+                             : oz_find(T, [](const OzTask& t) { return t.grp0[0]; }, w));
+  const OzOp o = oz_operand(g, T.h, isb);
+  const int K = g.K, nkb = g.nkb, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t i8 = w - g.grp0[isb];
+  if (o.cs == 1) {
+    const int64_t i = i8 * 8 + warp;
+    unsigned mx = 0;
+    if (i < o.rows) {
+      const z* x = o.X + i * o.rs;
+#pragma unroll 8
+      for (int k = lane; k < K; k += 32) mx = max(mx, oz_exp(x[k]));
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) s_mx[warp] = mx;
+  } else {
+    if (threadIdx.x < 8) s_mx[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t i = i8 * 8 + (lane & 7);
+    unsigned mx = 0;
+    if (i < o.rows) {
+      const z* x = o.X + i * o.rs;
+#pragma unroll 8
+      for (int k = threadIdx.x >> 3; k < K; k += 32) mx = max(mx, oz_exp(x[k * o.cs]));
+    }
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+    if (mx && lane < 8) atomicMax(&s_mx[lane], mx);
+  }
+  __syncthreads();
+  if (threadIdx.x < 8 && i8 * 8 + threadIdx.x < o.rows) o.e[i8 * 8 + threadIdx.x] = (int)s_mx[threadIdx.x];
+  const int e = (int)s_mx[lane >> 2];
+  for (int kb = warp; kb < nkb; kb += 8) {
+    if (isb) oz_slice_atom<3>(o, K, nkb, i8, kb, lane, e);
+    else oz_slice_atom<2>(o, K, nkb, i8, kb, lane, e);
   }
 }
 
@@ -677,7 +728,7 @@ int oz_sm_count(Ctx* c, int* sm) {
 // tables of the products tk[0..n): T's head and tasks, and the bytes of buffer they use
 size_t oz_layout(const GemmTask* const* tk, int n, int sm, OzHead* h, OzTask* t, double* flop, double* bytes) {
   size_t off = 0;
-  int64_t items = 0, scale[2] = {0, 0}, fin = 0, rows = 0;
+  int64_t items = 0, scale[2] = {0, 0}, groups[2] = {0, 0}, fin = 0, rows = 0;
   double work = 0, wflop = 0, wbytes = 0;
   *h = OzHead{};
   h->n = n;
@@ -725,6 +776,12 @@ size_t oz_layout(const GemmTask* const* tk, int n, int sm, OzHead* h, OzTask* t,
     scale[1] += oz_scale_blocks(o.N, o.b_ks, o.K);
     o.atom0[0] = h->atoms[0];
     o.atom0[1] = h->atoms[1];
+    o.grp0[0] = h->groups[0];
+    o.grp0[1] = h->groups[1];
+    groups[0] += (int64_t)o.ntm * (OZ_BM / 8);
+    groups[1] += (int64_t)o.ntn * (OZ_BN / 8);
+    h->groups[0] = (int)groups[0];
+    h->groups[1] = (int)groups[1];
     h->atoms[0] += (int64_t)o.ntm * (OZ_BM / 8) * o.nkb;
     h->atoms[1] += (int64_t)o.ntn * (OZ_BN / 8) * o.nkb;
     o.fin0 = (int)fin;
@@ -735,7 +792,7 @@ size_t oz_layout(const GemmTask* const* tk, int n, int sm, OzHead* h, OzTask* t,
     rows += t[i].M + t[i].N;
   }
   off += ws_round(sizeof(int) * (size_t)rows);
-  if (items > INT32_MAX || scale[0] + scale[1] > INT32_MAX || fin > INT32_MAX) return 0;
+  if (items > INT32_MAX || scale[0] + scale[1] > INT32_MAX || groups[0] + groups[1] > INT32_MAX || fin > INT32_MAX) return 0;
   h->items = (int)items;
   h->scale_blocks[0] = (int)scale[0];
   h->scale_blocks[1] = (int)scale[1];
@@ -752,6 +809,22 @@ template <int CAP>
 unsigned oz_slice_grid(const OzTasks<CAP>& T) {
   const int64_t a = ((T.h.sides & 1) ? T.h.atoms[0] : 0) + ((T.h.sides & 2) ? T.h.atoms[1] : 0);
   return (unsigned)std::min<int64_t>(cdiv(a, 8), 152 * 16);
+}
+template <int CAP>
+unsigned oz_prep_grid(const OzTasks<CAP>& T) {
+  return (unsigned)(((T.h.sides & 1) ? T.h.groups[0] : 0) + ((T.h.sides & 2) ? T.h.groups[1] : 0));
+}
+// Whether the scales and slices of t[0..n) take one launch (k_oz_prep): rows of one CTA's
+// share of K, and no more row groups than about two CTAs for every SM; more of them are
+// bound by throughput, and the separate slice kernel keeps more loads in flight.  Whole
+// products, separate / one launch, us: 256 x 256 x 128 63.5 / 58.6, 1024 x 1024 x 64 86.7 / 81.8,
+// 1024 x 1024 x 512 189.7 / 186.1 (256 groups), 1024 x 4096 x 256 333.6 / 333.8 (640),
+// 2048 x 2048 x 512 536.7 / 539.1 (512), 256 x 8192 x 512 356.5 / 364.2 (1056).
+bool oz_one_prep(const OzHead& h, const OzTask* t, int n) {
+  if (h.groups[0] + h.groups[1] > 2 * 152) return false;
+  for (int i = 0; i < n; ++i)
+    if (t[i].K > OZ_SCALE_K) return false;
+  return true;
 }
 
 // products tk[0..n) in one set of launches; slices and partial sums live in the context's own
@@ -775,20 +848,26 @@ int oz_launch(Ctx* c, const GemmTask* const* tk, int n, int sm) {
   T.h.buf = (uint8_t*)c->oz_buf;
   {
     ProfScope ps(c, "oz_slice", bytes);
-    for (int i = 0; i < n; ++i) {  // maxima combined from several CTAs start from zero
-      const OzTask& o = T.t[i];
-      if (o.K > OZ_SCALE_K && (o.a_ks != 1 || o.b_ks != 1))
-        TNT_CUDA_TRY(c, cudaMemsetAsync(T.h.buf + o.offE, 0, sizeof(int) * (size_t)(o.M + o.N), c->stream));
+    if (oz_one_prep(T.h, T.t, n)) {
+      k_oz_prep<CAP><<<oz_prep_grid(T), 256, 0, c->stream>>>(T);
+      c->launches++;
+    } else {
+      for (int i = 0; i < n; ++i) {  // maxima combined from several CTAs start from zero
+        const OzTask& o = T.t[i];
+        if (o.K > OZ_SCALE_K && (o.a_ks != 1 || o.b_ks != 1))
+          TNT_CUDA_TRY(c, cudaMemsetAsync(T.h.buf + o.offE, 0, sizeof(int) * (size_t)(o.M + o.N), c->stream));
+      }
+      k_oz_scale<CAP><<<oz_scale_grid(T), 256, 0, c->stream>>>(T);
+      k_oz_slice<CAP><<<oz_slice_grid(T), 256, 0, c->stream>>>(T);
+      c->launches += 2;
     }
-    k_oz_scale<CAP><<<oz_scale_grid(T), 256, 0, c->stream>>>(T);
-    k_oz_slice<CAP><<<oz_slice_grid(T), 256, 0, c->stream>>>(T);
   }
   {
     ProfScope ps(c, "oz_gemm", flop);
     k_oz_gemm<CAP><<<(unsigned)std::min(T.h.items, sm), OZ_THREADS, OZ_SMEM, c->stream>>>(T);
     k_oz_finish<CAP><<<(unsigned)std::min(T.h.fin_blocks, 152 * 8), 256, 0, c->stream>>>(T);
   }
-  c->launches += 4;
+  c->launches += 2;
   TNT_CHECK_LAUNCH(c);
   return TNT_OK;
 }
@@ -828,20 +907,33 @@ int oz_plan_build(Ctx* c, const std::vector<GemmTask>& tasks, int fixed_sides, O
   T.h.buf = buf;
   T.h.status = c->d_status;
   T.t = dt;
+  const bool one = oz_one_prep(T.h, t.data(), (int)t.size());
+  auto inputs = [&](OzNode* node) {  // the launches that read the operands of T.h.sides
+    if (one) {
+      node[0] = OzNode{(void*)k_oz_prep<0>, oz_prep_grid(T), 256, 0};
+      return 1;
+    }
+    node[0] = OzNode{(void*)k_oz_scale<0>, oz_scale_grid(T), 256, 0};
+    node[1] = OzNode{(void*)k_oz_slice<0>, oz_slice_grid(T), 256, 0};
+    return 2;
+  };
   if (fixed_sides) {
     T.h.sides = fixed_sides;
-    k_oz_scale<0><<<oz_scale_grid(T), 256, 0, c->stream>>>(T);
-    k_oz_slice<0><<<oz_slice_grid(T), 256, 0, c->stream>>>(T);
-    c->launches += 2;
-    TNT_CHECK_LAUNCH(c);
+    OzNode node[2];
+    const int n = inputs(node);
+    void* args[] = {&T};
+    for (int i = 0; i < n; ++i) {
+      TNT_CUDA_TRY(c, cudaLaunchKernel(node[i].fn, dim3(node[i].grid), dim3(node[i].block), args, 0, c->stream));
+      c->launches++;
+    }
   }
   T.h.sides = 3 & ~fixed_sides;
   memcpy(p->args, &T, sizeof(T));
   p->flop = f;
-  p->node[0] = OzNode{(void*)k_oz_scale<0>, oz_scale_grid(T), 256, 0};
-  p->node[1] = OzNode{(void*)k_oz_slice<0>, oz_slice_grid(T), 256, 0};
-  p->node[2] = OzNode{(void*)k_oz_gemm<0>, (unsigned)std::min(T.h.items, sm), OZ_THREADS, OZ_SMEM};
-  p->node[3] = OzNode{(void*)k_oz_finish<0>, (unsigned)std::min(T.h.fin_blocks, 152 * 8), 256, 0};
+  p->inputs = inputs(p->node);
+  p->node[p->inputs] = OzNode{(void*)k_oz_gemm<0>, (unsigned)std::min(T.h.items, sm), OZ_THREADS, OZ_SMEM};
+  p->node[p->inputs + 1] = OzNode{(void*)k_oz_finish<0>, (unsigned)std::min(T.h.fin_blocks, 152 * 8), 256, 0};
+  p->nodes = p->inputs + 2;
   return TNT_OK;
 }
 
@@ -856,7 +948,8 @@ int oz_plan_run(Ctx* c, const OzPlan& p, const z* add_b) {
   alignas(16) unsigned char a[sizeof(p.args)];
   oz_plan_args(p, add_b, a);
   void* args[] = {a};
-  for (const OzNode& n : p.node) {
+  for (int i = 0; i < p.nodes; ++i) {
+    const OzNode& n = p.node[i];
     TNT_CUDA_TRY(c, cudaLaunchKernel(n.fn, dim3(n.grid), dim3(n.block), args, n.smem, c->stream));
     c->launches++;
   }

@@ -225,8 +225,8 @@ int zgemm_fma_tasks(Ctx* c, const GemmTask* const* tasks, int n);
 // Products that repeat with the same shapes (oz.cu): tables and buffers from the scratch arena,
 // laid out once; the sides of fixed_sides (bit 0 A, bit 1 B) hold operands that do not change
 // and are sliced when the plan is built.  A task's B may be an offset from the vector given
-// at each run (add_b; null for absolute pointers).  The four kernels take one argument, for
-// graph nodes: oz_plan_args writes it.
+// at each run (add_b; null for absolute pointers).  The kernels (the first `inputs` of them read
+// the operands) take one argument, for graph nodes: oz_plan_args writes it.
 struct OzNode {
   void* fn;
   unsigned grid, block, smem;
@@ -234,6 +234,7 @@ struct OzNode {
 struct OzPlan {
   alignas(16) unsigned char args[128];
   OzNode node[4];
+  int nodes = 0, inputs = 0;
   double flop = 0;
 };
 size_t oz_plan_bytes(Ctx* c, const std::vector<GemmTask>& tasks);

@@ -187,7 +187,7 @@ struct U1Plan {
   cudaGraph_t graph[2] = {nullptr, nullptr};
   cudaGraphExec_t exec[2] = {nullptr, nullptr};
   cudaGraphNode_t in_node[2] = {nullptr, nullptr}, out_node[2] = {nullptr, nullptr};
-  cudaGraphNode_t oz_node[2] = {nullptr, nullptr};  // the two kernels that read the input
+  cudaGraphNode_t oz_node[2] = {nullptr, nullptr};  // the kernels that read the input (one or two)
   TPArgs in_tp{};
   ZGArgs in_zg{};
   GthArgs out_g[2]{};
