@@ -171,7 +171,7 @@ int64_t tnt_launch_count(const tnt_ctx* ctx);
  * context's stream, and sum its algorithmic work.  Classes and their work unit:
  *   "cgemm_tf32x3" (useful FLOPs 8 M N K of the complex product), "zgemm_f64" (8 M N K),
  *   "op_apply" (FLOPs), "op_mixed", "split_theta" (bytes read plus written), "multidot",
- *   "multiaxpy" (FP64 FLOPs), "heig_tridiag" (FLOPs), "heig_tridiag_eig" (none),
+ *   "multiaxpy", "gs_step" (FP64 FLOPs), "heig_tridiag" (FLOPs), "heig_tridiag_eig" (none),
  *   "heig_backtransform" (FLOPs), "cgemm_grouped", "zgemm_grouped", "oz_gemm" (useful
  *   FLOPs), "u1_wop", "u1_pack_theta", "u1_gather", "oz_slice" (bytes).
  * NULL or "" switches timing off.  At most 16384 launches are recorded between reads. */

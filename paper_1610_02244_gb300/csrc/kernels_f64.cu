@@ -934,16 +934,16 @@ int vec_normalize(Ctx* c, const z* x, z* y, int64_t n, const double* d_norm2) {
 // deterministic.
 // What bounds it: the FP64 pipe, 8 (k + 2) n FMAs at two per SM and clock (15 us at n = 65536,
 // k = 16), and two grid barriers.  Measured over a solve at n = 65536, k up to 32: 35 us a
-// step on average, 55 us with both passes over all of V; at n of about 2000 16 and 24 us.  The separate
-// launches it replaces took 160 us there (four dot-product launches of eight vectors at 27 to
-// 30 us, whatever n: with one element per thread each spent its time reducing 16 sums per
-// thread), 115 us at n = 5000.
+// step on average, 55 us with both passes over all of V; at n of about 2000 16 and 24 us.
+// The separate launches it replaces took 160 us there (four dot-product launches of eight
+// vectors at 27 to 30 us, whatever n: with one element per thread each spent its time
+// reducing 16 sums per thread), 115 us at n = 5000.
 namespace {
 constexpr int GS_THREADS = 256, GS_WARPS = GS_THREADS / 32;
 constexpr int GS_SMEM = 204 * 1024;
 // Above this the slice of w alone nears the shared memory of an SM, and both forms are bound
-// by the FP64 pipe.  FP64 solves of this size, fused / separate launches: n = 2^12 9.7 / 27
-// ms, 2^16 28 / 50, 2^18 60 / 80, 2^20 232 / 239.
+// by the FP64 pipe.  FP64 solves of this size, fused (then with two passes over all of V) /
+// separate launches: n = 2^12 9.7 / 27 ms, 2^16 28 / 50, 2^18 60 / 80, 2^20 232 / 239.
 constexpr int64_t GS_MAX_N = 1 << 20;
 
 struct GsArgs {  // part: 64 vectors' sums, npart: the norm's

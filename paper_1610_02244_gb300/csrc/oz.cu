@@ -22,8 +22,8 @@
 // No FP64-pipe instruction runs in these kernels: an SM retires two FP64 operations per
 // clock, and combining the level sums in FP64 (with TF32 operands, six-bit digits and 45
 // pairs) took longer than the MMAs.  Measured: H_eff.theta at chi = 256, d = 4 (two products
-// of 1.07 G complex multiply-adds) 5.71 -> 0.72 ms; theta at chi = 512, d = 5 7.0 -> 0.76 ms
-// (34 TFLOP/s of the complex product's own operations).  What bounds it: operand reads from
+// of 1.07 G complex multiply-adds) 5.71 -> 0.67 ms; theta and its gate at chi = 512, d = 4 7.3 ->
+// 0.94 ms.  What bounds it: operand reads from
 // shared memory (an N = 128 MMA takes about 90 of the 64 clocks its arithmetic needs).
 //
 // Kernel: persistent, one CTA per SM over items (output tile 128 x 64, level group, K
