@@ -83,3 +83,29 @@ def test_spacings_of_the_eigenvalues(ctx, n, spectrum):
     g = synth.rng(n)
     U, V = (np.linalg.qr(synth.complex_gaussian(g, (n, n)))[0] for _ in range(2))
     check(ctx, (U * s) @ V)
+
+
+@pytest.mark.parametrize("total", [1, 255, 256, 257, 513, 4096, 4099])
+def test_selection_at_its_thread_counts(ctx, total):
+    """The global order and the truncation error over as many candidates as one, a thread's four,
+    or all of its eight hold.  Blocks of eight neighbouring values (1 to 1e-9 over all): the
+    Gram matrix of a block resolves them to 8 eps (largest / smallest)^2 < 1e-13 relative, and sums
+    of their squares over all to 1e-10 with room."""
+    s = np.logspace(0, -9, total)
+    g = synth.rng(total)
+    lab = np.arange(total) // 8
+    M = np.zeros((total, total), dtype=np.complex128)
+    for q in range(lab[-1] + 1):
+        i = np.flatnonzero(lab == q)
+        U, V = (np.linalg.qr(synth.complex_gaussian(g, (i.size, i.size)))[0] for _ in range(2))
+        M[np.ix_(i, i)] = (U * s[i]) @ V
+    perm = g.permutation(lab[-1] + 1)  # charges in another order than the values
+    order = np.argsort(perm[lab], kind="stable")
+    M, q = M[np.ix_(order, order)], perm[lab][order]
+    U, X, S, bq, info = ctx.svd_trunc(torch.from_numpy(M).to("cuda:0"), q, q)
+    tail = np.append(np.cumsum((s ** 2)[::-1])[::-1], 0.0) / (s ** 2).sum()  # discards from index i on
+    chi = max(1, int(np.argmax(np.sqrt(tail) < 1e-8)))  # the default 2-norm error
+    assert info["chi"] == chi == len(S)
+    assert np.abs(np.sort(S)[::-1] / s[:chi] - 1.0).max() <= 1e-12
+    assert abs(info["err"] - np.sqrt(tail[chi])) <= 1e-10 * np.sqrt(tail[chi])
+    assert np.array_equal(np.sort(bq), np.sort(perm[lab[:chi]]))
