@@ -545,7 +545,7 @@ TRAFFIC = {
     # two launches per update: the 1024-row Gram block (16.86 MB, ncu; the matrix read once)
     # and the ~231-row tail block (its entries x the same 16.1 B per entry: 0.86 MB), averaged:
     # profiles/tridiag_rows_gram1024.md
-    "heig_tridiag": (8.86e6, "heig.cu", "29a35a33c5ce4d71", "ncu, svd_large_block_cfg2_shape"),
+    "heig_tridiag": (8.86e6, "heig.cu", "8c47764a047592e0", "ncu, svd_large_block_cfg2_shape"),
 }
 
 

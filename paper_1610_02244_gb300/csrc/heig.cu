@@ -1214,7 +1214,7 @@ __device__ void iv_solve(double* __restrict__ y, int64_t n, const double* __rest
     y[r] = v;
     y2 = y1;
     y1 = v;
-    if (hi_exp(v) >= 1023 + 500) {
+    if (hi_exp(v) >= 1023 + 500 && hi_exp(v) < 2047) {  // (nothing to save in an infinity or NaN)
       for (int64_t q = 0; q < n; ++q) y[q] *= 0x1p-500;
       y1 *= 0x1p-500;
       y2 *= 0x1p-500;
