@@ -538,15 +538,7 @@ OZ_TENSOR_PER_USEFUL = 36.0  # slice pairs per complex product: 36 x 4 real MMAs
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
 # capture per kernel class, valid while the class's source file is unchanged: class ->
 # (bytes per launch, source file under csrc/, sha256 prefix of that file, capture).
-TRAFFIC = {
-    # both launches of one matvec (T1 = L theta: 21.01 + 0.02 MB; y = T3 R^T: 71.34 + 2.95 MB),
-    # averaged: profiles/cgemm_tf32x3_heff_cfg2.md
-    "cgemm_tf32x3": (47.66e6, "tc_mixed.cu", "4a520cf2191b6d08", "ncu, test_heff_mixed 256-4-256"),
-    # two launches per update: the 1024-row Gram block (16.86 MB, ncu; the matrix read once)
-    # and the ~231-row tail block (its entries x the same 16.1 B per entry: 0.86 MB), averaged:
-    # profiles/tridiag_rows_gram1024.md
-    "heig_tridiag": (8.86e6, "heig.cu", "8c47764a047592e0", "ncu, svd_large_block_cfg2_shape"),
-}
+TRAFFIC = {}  # (tc_mixed.cu and heig.cu changed since their captures)
 
 
 def traffic_for(cls):

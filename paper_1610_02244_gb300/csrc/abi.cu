@@ -83,6 +83,35 @@ int pinned_reserve(Ctx* c, size_t bytes) {
   return TNT_OK;
 }
 
+// The tables of a 32-chain U(1) plan are the largest (a few MB); most are a few KB.
+constexpr size_t UP_HALF = 2 << 20;
+
+int to_device(Ctx* c, void* dst, const void* src, size_t bytes) {
+  if (!bytes) return TNT_OK;
+  if (!c->up_buf) {
+    for (auto& e : c->up_ev)
+      if (!e) TNT_CUDA_TRY(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    if (cudaMallocHost((void**)&c->up_buf, 2 * UP_HALF) != cudaSuccess) {
+      cudaGetLastError();
+      c->up_buf = nullptr;
+    } else {
+      c->up.half = UP_HALF;
+    }
+  }
+  if (bytes > c->up.half) {
+    TNT_CUDA_TRY(c, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, c->stream));
+    TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    return TNT_OK;
+  }
+  int wait;
+  const size_t at = c->up.place(bytes, c->stream, &wait);
+  if (wait >= 0) TNT_CUDA_TRY(c, cudaEventSynchronize(c->up_ev[wait]));
+  memcpy(c->up_buf + at, src, bytes);
+  TNT_CUDA_TRY(c, cudaMemcpyAsync(dst, c->up_buf + at, bytes, cudaMemcpyHostToDevice, c->stream));
+  TNT_CUDA_TRY(c, cudaEventRecord(c->up_ev[c->up.cur], c->stream));
+  return TNT_OK;
+}
+
 
 // ---------------------------------------------------------------- Bose-Hubbard (host)
 static void local_ops(int n_max, std::vector<double>* b) {
@@ -373,6 +402,12 @@ int tnt_ctx_destroy(tnt_ctx* ctx) {
   for (auto& e : ctx->c.prof_ev) cudaEventDestroy(e);
   dev_free(ctx->c.dalloc, ctx->c.ws.base);
   if (ctx->c.h_pinned) cudaFreeHost(ctx->c.h_pinned);
+  for (int i = 0; i < 2; ++i)
+    if (ctx->c.up_ev[i]) {
+      cudaEventSynchronize(ctx->c.up_ev[i]);
+      cudaEventDestroy(ctx->c.up_ev[i]);
+    }
+  if (ctx->c.up_buf) cudaFreeHost(ctx->c.up_buf);
   dev_free(ctx->c.dalloc, ctx->c.d_status);
   dev_free(ctx->c.dalloc, ctx->c.d_count);
   dev_free(ctx->c.dalloc, ctx->c.oz_buf);

@@ -828,9 +828,8 @@ int tnt_mps_norm2(tnt_ctx* ctx, const tnt_mps* m, double* norm2) {
   std::vector<z> hid((size_t)(d * d), zmk(0, 0));
   for (int64_t s = 0; s < d; ++s) hid[(size_t)(s * d + s)] = zmk(1, 0);
   z one = zmk(1, 0);
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(Wid, hid.data(), sizeof(z) * d * d, cudaMemcpyHostToDevice, c->stream));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(Ea, &one, sizeof(z), cudaMemcpyHostToDevice, c->stream));
-  TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  TNT_TRY(to_device(c, Wid, hid.data(), sizeof(z) * d * d));
+  TNT_TRY(to_device(c, Ea, &one, sizeof(z)));
   for (int j = 0; j < m->L; ++j) {
     size_t top = c->ws.top;
     int r = env_left_impl(c, Ea, Wid, m->A[j], m->chi[j], d, 1, m->chi[j + 1], Eb);

@@ -546,7 +546,7 @@ int upload(Ctx* c, T** dptr, const std::vector<T>& h, size_t cap_elems = 0) {
   *dptr = (T*)ws_alloc(c, ws_round(sizeof(T) * std::max<size_t>(n, 1)));
   if (!*dptr) return set_err(c, TNT_E_ALLOC, "scratch exhausted (grouped matvec tables)");
   if (!h.empty())
-    TNT_CUDA_TRY(c, cudaMemcpyAsync(*dptr, h.data(), sizeof(T) * h.size(), cudaMemcpyHostToDevice, c->stream));
+    TNT_TRY(to_device(c, *dptr, h.data(), sizeof(T) * h.size()));
   return TNT_OK;
 }
 
@@ -615,7 +615,7 @@ int u1_convert(Ctx* c, const U1Spec& s, const z* src, z* dst, int to_compact) {
   if (nrun == 0) return TNT_OK;
   int64_t* d_runs = (int64_t*)ws_alloc(c, ws_round(sizeof(int64_t) * runs.size()));
   if (!d_runs) return set_err(c, TNT_E_ALLOC, "scratch exhausted (block runs)");
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(d_runs, runs.data(), sizeof(int64_t) * runs.size(), cudaMemcpyHostToDevice, c->stream));
+  TNT_TRY(to_device(c, d_runs, runs.data(), sizeof(int64_t) * runs.size()));
   k_copy_runs<<<cap_grid((nrun + 7) / 8, 152 * 8), 256, 0, c->stream>>>(d_runs, nrun, src, dst);
   c->launches++;
   TNT_CHECK_LAUNCH(c);
@@ -966,14 +966,14 @@ int set_tiles(Ctx* c, U1Plan* p, int bn1, int bn4, int split4) {
   std::vector<GTask> g;
   std::vector<int4> tl;
   make_tiles(p->s1, bn1, 1, &g, &tl);
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(p->d_g1, g.data(), sizeof(GTask) * g.size(), cudaMemcpyHostToDevice, c->stream));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(p->d_g1tiles, tl.data(), sizeof(int4) * tl.size(), cudaMemcpyHostToDevice, c->stream));
+  TNT_TRY(to_device(c, p->d_g1, g.data(), sizeof(GTask) * g.size()));
+  TNT_TRY(to_device(c, p->d_g1tiles, tl.data(), sizeof(int4) * tl.size()));
   p->n_g1tiles = (int)tl.size();
   std::vector<GTask> g4;
   std::vector<int4> tl4;
   make_tiles(p->s4, bn4, split4, &g4, &tl4);
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(p->d_g4, g4.data(), sizeof(GTask) * g4.size(), cudaMemcpyHostToDevice, c->stream));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(p->d_g4tiles, tl4.data(), sizeof(int4) * tl4.size(), cudaMemcpyHostToDevice, c->stream));
+  TNT_TRY(to_device(c, p->d_g4, g4.data(), sizeof(GTask) * g4.size()));
+  TNT_TRY(to_device(c, p->d_g4tiles, tl4.data(), sizeof(int4) * tl4.size()));
   p->n_g4tiles = (int)tl4.size();
   TNT_TRY(tma_map_planes(c, &p->tmB1, p->B1p, p->rowsB1, p->KA1, bn1));
   TNT_TRY(tma_map_planes(c, &p->tmB4, p->B4p, p->rowsB4, p->KA4, bn4));
@@ -1125,7 +1125,7 @@ int u1_prepare(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
   TNT_TRY(upload(c, &p->d_g4, none, p->s4.size()));
   TNT_TRY(upload(c, &p->d_g1tiles, none4, (size_t)p->cap_g1tiles));
   TNT_TRY(upload(c, &p->d_g4tiles, none4, (size_t)p->cap_g4tiles));
-  // constant operands: environments into FP64 packs (pageable tables are staged by the copies)
+  // constant operands: environments into FP64 packs
   const int nA = (int)p->segA1.size(), nB = (int)p->segB4.size();
   k_pack_segs<false><<<cap_grid((nA + 7) / 8, 152 * 8), 256, 0, c->stream>>>(p->d_segA1, nA, nullptr, 0, p->A1z);
   k_pack_segs<false><<<cap_grid((nB + 7) / 8, 152 * 8), 256, 0, c->stream>>>(p->d_segB4, nB, nullptr, 0, p->B4z);

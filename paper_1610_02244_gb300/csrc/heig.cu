@@ -1489,9 +1489,8 @@ int heig_finish(Ctx* c, int64_t n, int64_t k, const z* Hv, const z* tau, const d
     std::vector<int2> he((size_t)(k + nbt));
     for (int64_t i = 0; i < k; ++i) he[(size_t)i] = make_int2(0, (int)i);
     for (int64_t q = 0; q < nbt; ++q) he[(size_t)(k + q)] = make_int2(0, (int)(q * cols));
-    TNT_CUDA_TRY(c, cudaMemcpyAsync(dblk, &hb, sizeof(EBlk), cudaMemcpyHostToDevice, st));
-    TNT_CUDA_TRY(c, cudaMemcpyAsync(deig, he.data(), sizeof(int2) * he.size(), cudaMemcpyHostToDevice, st));
-    TNT_CUDA_TRY(c, cudaStreamSynchronize(st));  // the host tables die at the end of scope
+    TNT_TRY(to_device(c, dblk, &hb, sizeof(EBlk)));
+    TNT_TRY(to_device(c, deig, he.data(), sizeof(int2) * he.size()));
   }
   {
     ProfScope ps(c, "heig_tridiag_eig");
@@ -1855,14 +1854,13 @@ int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& all, z* U, double* ev
     c->ws.top = top;
     return set_err(c, TNT_E_ALLOC, "scratch exhausted (eigensolves)");
   }
-  // (memory a pageable copy reads is staged before the call returns)
   std::vector<char> host(b_blk + b_eig + b_bt + b_so + b_sub, 0);
   memcpy(host.data(), he.data(), sizeof(EBlk) * nb);
   memcpy(host.data() + b_blk, heig.data(), sizeof(int2) * heig.size());
   if (!hbt.empty()) memcpy(host.data() + b_blk + b_eig, hbt.data(), sizeof(int2) * hbt.size());
   memcpy(host.data() + b_blk + b_eig + b_bt, so.data(), sizeof(int64_t) * nb);
   if (!subs.empty()) memcpy(host.data() + b_blk + b_eig + b_bt + b_so, subs.data(), sizeof(WySub) * subs.size());
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(tab, host.data(), host.size(), cudaMemcpyHostToDevice, st));
+  TNT_TRY(to_device(c, tab, host.data(), host.size()));
   const EBlk* dblk = (const EBlk*)tab;
   const int2* deig = (const int2*)(tab + b_blk);
   const int2* dbt = (const int2*)(tab + b_blk + b_eig);

@@ -373,8 +373,7 @@ int op_upload(Ctx* c, const std::vector<z>& dense, int nI, int nJ,
   memcpy(host.data() + b_row + b_col, val.data(), sizeof(z) * val.size());
   memcpy(host.data() + b_row + b_col + b_val, in_off.data(), sizeof(int64_t) * nJ);
   memcpy(host.data() + b_row + b_col + b_val + b_in, out_off.data(), sizeof(int64_t) * nI);
-  // (a pageable copy is staged before the call returns: the host vector may go)
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(dev, host.data(), total, cudaMemcpyHostToDevice, c->stream));
+  TNT_TRY(to_device(c, dev, host.data(), total));
   a->nI = nI;
   a->nJ = nJ;
   a->nnz = row[nI];

@@ -438,7 +438,7 @@ int cycles(Ctx* c, const MatVec& A, BScratch& s, z* x, int precision, int max_ma
   std::vector<double> E((size_t)NP, 0), Eprev((size_t)NP, 0), resid((size_t)NP, 0);
   std::vector<int> have_prev((size_t)NP, 0);
   auto push_frozen = [&]() -> int {
-    TNT_CUDA_TRY(c, cudaMemcpyAsync(s.frozen, frozen.data(), sizeof(int) * NP, cudaMemcpyHostToDevice, c->stream));
+    TNT_TRY(to_device(c, s.frozen, frozen.data(), sizeof(int) * NP));
     TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     return TNT_OK;
   };
@@ -495,8 +495,8 @@ int cycles(Ctx* c, const MatVec& A, BScratch& s, z* x, int precision, int max_ma
     // Ritz vectors of every problem that took part in this cycle
     std::vector<int> skip_ritz((size_t)NP);
     for (int p = 0; p < NP; ++p) skip_ritz[(size_t)p] = active_in_cycle[(size_t)p];
-    TNT_CUDA_TRY(c, cudaMemcpyAsync(s.kk, kk.data(), sizeof(int) * NP, cudaMemcpyHostToDevice, c->stream));
-    TNT_CUDA_TRY(c, cudaMemcpyAsync(s.skip2, skip_ritz.data(), sizeof(int) * NP, cudaMemcpyHostToDevice, c->stream));
+    TNT_TRY(to_device(c, s.kk, kk.data(), sizeof(int) * NP));
+    TNT_TRY(to_device(c, s.skip2, skip_ritz.data(), sizeof(int) * NP));
     k_sritz<<<NP, 64, 0, c->stream>>>(s.y, s.kk, s.coef, NP);
     c->launches++;
     k_sfill<<<s.nch, ST, 0, c->stream>>>(s.w, s.ch, s.skip2);
@@ -512,9 +512,9 @@ int cycles(Ctx* c, const MatVec& A, BScratch& s, z* x, int precision, int max_ma
       to_x[(size_t)p] = (took && frozen[(size_t)p]) ? 0 : 1;   // 0 = write
       to_v[(size_t)p] = (took && !frozen[(size_t)p]) ? 0 : 1;
     }
-    TNT_CUDA_TRY(c, cudaMemcpyAsync(s.done, to_x.data(), sizeof(int) * NP, cudaMemcpyHostToDevice, c->stream));
+    TNT_TRY(to_device(c, s.done, to_x.data(), sizeof(int) * NP));
     TNT_TRY(snormalize(c, s, s.w, x, s.n2, s.done));
-    TNT_CUDA_TRY(c, cudaMemcpyAsync(s.skip2, to_v.data(), sizeof(int) * NP, cudaMemcpyHostToDevice, c->stream));
+    TNT_TRY(to_device(c, s.skip2, to_v.data(), sizeof(int) * NP));
     TNT_TRY(snormalize(c, s, s.w, s.V, s.n2, s.skip2));
     TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));  // the host flag arrays above are reused
     for (int p = 0; p < NP; ++p) {
@@ -591,8 +591,8 @@ int lanczos_batched(Ctx* c, const MatVec& A, const std::vector<int64_t>& off, z*
       !s.alpha || !s.beta || !s.y || !s.tri || !s.n2 || !s.frozen || !s.skip2 || !s.kk ||
       !s.done || !s.none)
     return set_err(c, TNT_E_ALLOC, "scratch exhausted (batched Lanczos)");
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(s.ch, ch.data(), sizeof(int64_t) * ch.size(), cudaMemcpyHostToDevice, c->stream));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(s.first, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice, c->stream));
+  TNT_TRY(to_device(c, s.ch, ch.data(), sizeof(int64_t) * ch.size()));
+  TNT_TRY(to_device(c, s.first, first.data(), sizeof(int) * first.size()));
   TNT_CUDA_TRY(c, cudaMemsetAsync(s.none, 0, sizeof(int) * NP, c->stream));
   TNT_CUDA_TRY(c, cudaMemsetAsync(s.alpha, 0, sizeof(double) * KMAX * NP, c->stream));
   TNT_CUDA_TRY(c, cudaMemsetAsync(s.beta, 0, sizeof(double) * KMAX * NP, c->stream));

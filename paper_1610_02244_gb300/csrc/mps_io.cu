@@ -86,7 +86,7 @@ int tnt_mps_overlap(tnt_ctx* ctx, const tnt_mps* a, const tnt_mps* b, tnt_cplx* 
   z* Eb = (z*)ws_alloc(c, ws_round(sizeof(z) * (size_t)(ma * mb)));
   z* T = (z*)ws_alloc(c, ws_round(sizeof(z) * (size_t)(ma * d * mb)));
   const z one = zmk(1, 0);
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(Ea, &one, sizeof(z), cudaMemcpyHostToDevice, c->stream));
+  TNT_TRY(to_device(c, Ea, &one, sizeof(z)));
   for (int j = 0; j < a->L; ++j) {
     const int r = overlap_step(c, Ea, a->A[j], b->A[j], a->chi[j], b->chi[j], a->chi[j + 1],
                                b->chi[j + 1], d, T, Eb);
@@ -123,13 +123,12 @@ int tnt_mps_set_charges(tnt_ctx* ctx, tnt_mps* m, int bond, const int64_t* h_q) 
   int64_t* dl = (int64_t*)ws_alloc(c, ws_round(sizeof(int64_t) * (size_t)mx));
   unsigned long long* bad = (unsigned long long*)ws_alloc(c, 256);
   TNT_CUDA_TRY(c, cudaMemsetAsync(bad, 0, sizeof(unsigned long long), c->stream));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(dq, nq.data(), sizeof(int64_t) * chi, cudaMemcpyHostToDevice, c->stream));
+  TNT_TRY(to_device(c, dq, nq.data(), sizeof(int64_t) * chi));
   for (int side = 0; side < 2; ++side) {
     const int j = side == 0 ? bond - 1 : bond;  // site left of the bond, then right of it
     if (j < 0 || j >= m->L) continue;
     const int other = side == 0 ? j : j + 1;   // the site's other bond
-    TNT_CUDA_TRY(c, cudaMemcpyAsync(dl, m->q[other].data(), sizeof(int64_t) * m->chi[other],
-                                    cudaMemcpyHostToDevice, c->stream));
+    TNT_TRY(to_device(c, dl, m->q[other].data(), sizeof(int64_t) * m->chi[other]));
     const int64_t n = m->chi[j] * m->d * m->chi[j + 1];
     const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, 1216);
     k_label_violations<<<blocks, 256, 0, c->stream>>>(m->A[j], m->chi[j], m->d, m->chi[j + 1],

@@ -80,7 +80,7 @@ int obs_setup(Ctx* c, const tnt_mps* m, Obs* o, int64_t nout) {
   for (int i = 0; i < 4; ++i) {
     *ws[i] = (z*)ws_alloc(c, ws_round(sizeof(z) * d * d));
     if (!*ws[i]) return set_err(c, TNT_E_ALLOC, "scratch exhausted (observables)");
-    TNT_CUDA_TRY(c, cudaMemcpyAsync(*ws[i], hs[i]->data(), sizeof(z) * d * d, cudaMemcpyHostToDevice, c->stream));
+    TNT_TRY(to_device(c, *ws[i], hs[i]->data(), sizeof(z) * d * d));
   }
   int64_t mx = 1;
   for (int k = 0; k <= L; ++k) mx = std::max(mx, m->chi[k]);
@@ -96,9 +96,8 @@ int obs_setup(Ctx* c, const tnt_mps* m, Obs* o, int64_t nout) {
   o->out = (z*)ws_alloc(c, ws_round(sizeof(z) * (size_t)std::max<int64_t>(nout, 1)));
   if (!o->T0 || !o->T1 || !o->out) return set_err(c, TNT_E_ALLOC, "scratch exhausted (observables)");
   const z one = zmk(1, 0);
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(o->E[0], &one, sizeof(z), cudaMemcpyHostToDevice, c->stream));
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(o->F[(size_t)L], &one, sizeof(z), cudaMemcpyHostToDevice, c->stream));
-  TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));  // the host constants above are stack values
+  TNT_TRY(to_device(c, o->E[0], &one, sizeof(z)));
+  TNT_TRY(to_device(c, o->F[(size_t)L], &one, sizeof(z)));
   for (int j = 0; j < L; ++j) {
     const size_t top = c->ws.top;
     TNT_TRY(env_left_impl(c, o->E[(size_t)j], o->Wid, m->A[(size_t)j], m->chi[(size_t)j], d, 1,

@@ -903,7 +903,7 @@ int oz_plan_build(Ctx* c, const std::vector<GemmTask>& tasks, int fixed_sides, O
   uint8_t* buf = (uint8_t*)ws_alloc(c, need);
   OzTask* dt = (OzTask*)ws_alloc(c, ws_round(sizeof(OzTask) * t.size()));
   if (!need || !buf || !dt) return set_err(c, TNT_E_ALLOC, "scratch exhausted (planned FP64 products)");
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(dt, t.data(), sizeof(OzTask) * t.size(), cudaMemcpyHostToDevice, c->stream));
+  TNT_TRY(to_device(c, dt, t.data(), sizeof(OzTask) * t.size()));
   T.h.buf = buf;
   T.h.status = c->d_status;
   T.t = dt;

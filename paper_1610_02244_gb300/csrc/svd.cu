@@ -718,7 +718,7 @@ int svd_trunc_impl(Ctx* c, const z* M, int64_t m, int64_t n, const int64_t* h_rq
       !d_blk_s || !d_loc_s || !d_sel || !d_cb || !d_ev || !d_tot)
     return set_err(c, TNT_E_ALLOC, "scratch exhausted (svd)");
 
-  // ---- host tables -> device (one synchronous upload of small integer tables)
+  // ---- host tables -> device (one upload of small integer tables)
   std::vector<CandBlock> hcb(nb);
   std::vector<int> hblk(ntot_vals), hloc(ntot_vals);
   std::vector<int64_t> hboff(2 * (size_t)nb);
@@ -754,7 +754,7 @@ int svd_trunc_impl(Ctx* c, const z* M, int64_t m, int64_t n, const int64_t* h_rq
     put(d_blk, hblk.data(), sizeof(int) * ntot_vals);
     put(d_loc, hloc.data(), sizeof(int) * ntot_vals);
     put(d_boff, hboff.data(), sizeof(int64_t) * 2 * nb);
-    TNT_CUDA_TRY(c, cudaMemcpyAsync(tab, host.data(), tab_bytes, cudaMemcpyHostToDevice, st));
+    TNT_TRY(to_device(c, tab, host.data(), tab_bytes));
   }
 
   // ---- gather blocks, |M|_F^2 (unscaled), scale each block, Gram matrices
@@ -908,7 +908,7 @@ int svd_trunc_impl(Ctx* c, const z* M, int64_t m, int64_t n, const int64_t* h_rq
   }
   KeptIdx* d_kept = (KeptIdx*)ws_alloc(c, ws_round(sizeof(KeptIdx) * chi));
   if (!d_kept) return set_err(c, TNT_E_ALLOC, "scratch exhausted (svd kept)");
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(d_kept, hk.data(), sizeof(KeptIdx) * chi, cudaMemcpyHostToDevice, st));
+  TNT_TRY(to_device(c, d_kept, hk.data(), sizeof(KeptIdx) * chi));
   TNT_TRY(zfill(c, U, m * chi, zmk(0, 0)));
   TNT_TRY(zfill(c, X, chi * n, zmk(0, 0)));
   int64_t mx = std::max(m, n);
@@ -916,7 +916,7 @@ int svd_trunc_impl(Ctx* c, const z* M, int64_t m, int64_t n, const int64_t* h_rq
   k_scatter<<<gs, 256, 0, st>>>(Vp, Xp, d_kept, d_rows, d_cols, d_unscale, side, scale, chi, n, U, X);
   c->launches++;
   TNT_CHECK_LAUNCH(c);
-  TNT_CUDA_TRY(c, cudaStreamSynchronize(st));  // host tables (hk) die at return
+  TNT_CUDA_TRY(c, cudaStreamSynchronize(st));  // the call returns host results
   res->chi = chi;
   res->err = sel.err;
   res->disc = sel.disc;

@@ -434,8 +434,7 @@ int heff_mixed_prepare(Ctx* c, HeffPlan* p) {
         out_off[(size_t)((s1 * d + s2) * D + w2)] = (s1 * d + s2) * m.Kp4 + w2 * chr;
   int64_t* d_out = (int64_t*)ws_alloc(c, ws_round(sizeof(int64_t) * nI));
   if (!d_out) return set_err(c, TNT_E_ALLOC, "scratch exhausted (mixed op table)");
-  // (a pageable copy is staged before the call returns)
-  TNT_CUDA_TRY(c, cudaMemcpyAsync(d_out, out_off.data(), sizeof(int64_t) * nI, cudaMemcpyHostToDevice, c->stream));
+  TNT_TRY(to_device(c, d_out, out_off.data(), sizeof(int64_t) * nI));
   m.op.out_off = d_out;
   m.op.B0 = chl;
   m.op.B1 = 1;

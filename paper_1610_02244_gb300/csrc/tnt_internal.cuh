@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/tnt_gb300.h"
+#include "upload.cuh"
 
 namespace tnt {
 
@@ -114,6 +115,9 @@ struct Ctx {
   std::string err;        // last error message
   double* h_pinned = nullptr;  // small pinned host buffer for scalar read-back
   size_t h_pinned_cap = 0;
+  UploadRing up;               // pinned halves that host tables are copied from (to_device)
+  char* up_buf = nullptr;
+  cudaEvent_t up_ev[2] = {nullptr, nullptr};
   // device status word written by kernels (bounds / NaN / timeout flags)
   int* d_status = nullptr;
   // arrival counters of the kernels that finish their reduction in the last CTA to arrive
@@ -189,6 +193,8 @@ void* ws_alloc(Ctx* c, size_t bytes);
 inline void ws_reset(Ctx* c) { c->ws.top = 0; }
 inline size_t ws_round(size_t b) { return (b + 255) & ~size_t(255); }
 int pinned_reserve(Ctx* c, size_t bytes);
+// copies a host table to the device on the context's stream; src may go or change at return
+int to_device(Ctx* c, void* dst, const void* src, size_t bytes);
 
 // ---------------------------------------------------------------- kernels (FP64 path)
 // Strided complex GEMM: C[i,j] = alpha * sum_k opA(i,k) opB(k,j) + beta * C[i,j]
