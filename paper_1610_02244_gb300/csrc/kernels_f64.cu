@@ -1261,7 +1261,7 @@ __global__ void __launch_bounds__(GS_THREADS, 1) k_gs_step(GsArgs a) {
       asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(a.bar), "r"(2u * gridDim.x) : "memory");
     }
   }
-  if (!ok) {  // the host reads a NaN beta, and the status word names the wait
+  if (!ok) {  // the host reads the status word with the step's numbers
     if (blockIdx.x == 0 && tid == 0) a.beta[a.k - 1] = __longlong_as_double(0x7ff8000000000000ll);
     return;
   }
@@ -1686,12 +1686,13 @@ __device__ bool tridiag_twisted(TwistShared& S, int k, double lo, double hi, dou
 }
 
 // one block per problem: problem p's alpha, beta, y at p * 64, out at p * 2 (skipped
-// where skip[p] is set); a single problem's E, |y_{k-1}| and beta_{k-1} also to pinned host
-// memory (no copy on the stream behind the kernel)
+// where skip[p] is set); a single problem's E, |y_{k-1}|, beta_{k-1} and the status word also to
+// pinned host memory (no copy on the stream behind the kernel)
 __global__ void __launch_bounds__(32) k_tridiag_lowest(const double* __restrict__ alpha,
                                                        const double* __restrict__ beta, int k,
                                                        double* out, double* __restrict__ y,
-                                                       const int* __restrict__ skip, double* host) {
+                                                       const int* __restrict__ skip, const int* status,
+                                                       KrylovSlot* host) {
   const int pb = blockIdx.x;
   if (skip && skip[pb]) return;
   alpha += 64 * pb;
@@ -1718,16 +1719,18 @@ __global__ void __launch_bounds__(32) k_tridiag_lowest(const double* __restrict_
   if (!tridiag_twisted(S, k, lo, hi, out, y)) tridiag_bisect(S.a, S.b, k, lo, hi, out, y);
   if (host) {
     __syncwarp();
-    if (l < 2) host[l] = out[l];
-    if (l == 2) host[2] = beta[k - 1];
+    if (l == 0) host->E = out[0];
+    if (l == 1) host->ylast = out[1];
+    if (l == 2) host->beta = beta[k - 1];
+    if (l == 3) host->status = (double)*status;
   }
 }
 }  // namespace
 
 int tridiag_lowest_on(Ctx* c, cudaStream_t st, const double* d_alpha, const double* d_beta, int k,
-                      double* d_out, double* d_y, double* h_out) {
+                      double* d_out, double* d_y, KrylovSlot* h_out) {
   if (k < 1 || k > 64) return set_err(c, TNT_E_UNSUPPORTED, "tridiagonal size %d", k);
-  k_tridiag_lowest<<<1, 32, 0, st>>>(d_alpha, d_beta, k, d_out, d_y, nullptr, h_out);
+  k_tridiag_lowest<<<1, 32, 0, st>>>(d_alpha, d_beta, k, d_out, d_y, nullptr, c->d_status, h_out);
   c->launches++;
   TNT_CHECK_LAUNCH(c);
   return TNT_OK;
@@ -1746,7 +1749,7 @@ int side_stream(Ctx* c) {
 int tridiag_lowest_batched(Ctx* c, const double* d_alpha, const double* d_beta, int k,
                            double* d_out, double* d_y, int nprob, const int* d_skip) {
   if (k < 1 || k > 64) return set_err(c, TNT_E_UNSUPPORTED, "tridiagonal size %d", k);
-  k_tridiag_lowest<<<nprob, 32, 0, c->stream>>>(d_alpha, d_beta, k, d_out, d_y, d_skip, nullptr);
+  k_tridiag_lowest<<<nprob, 32, 0, c->stream>>>(d_alpha, d_beta, k, d_out, d_y, d_skip, nullptr, nullptr);
   c->launches++;
   TNT_CHECK_LAUNCH(c);
   return TNT_OK;

@@ -101,11 +101,12 @@ static int lanczos_cycle_loop(Ctx* c, const MatVec& A, z* theta, int precision,
   // vector is that of step k - 1, from V[0..k-1] and y of slot (k-1) & 1.
   TNT_TRY(side_stream(c));
   int last_side = -1;  // slot of the last side-stream launch
+  KrylovSlot* const slots = (KrylovSlot*)hp;
   auto launch_tk = [&](int k) -> int {
     double* tk = tri2 + 2 * (k & 1);
     TNT_CUDA_TRY(c, cudaEventRecord(c->ev_main[k & 1], c->stream));
     TNT_CUDA_TRY(c, cudaStreamWaitEvent(c->side, c->ev_main[k & 1], 0));
-    TNT_TRY(tridiag_lowest_on(c, c->side, alpha, beta, k + 1, tk, y2 + 64 * (k & 1), hp + 4 * (k & 1)));
+    TNT_TRY(tridiag_lowest_on(c, c->side, alpha, beta, k + 1, tk, y2 + 64 * (k & 1), slots + (k & 1)));
     TNT_CUDA_TRY(c, cudaEventRecord(c->ev_side[k & 1], c->side));
     last_side = k & 1;
     return TNT_OK;
@@ -115,24 +116,20 @@ static int lanczos_cycle_loop(Ctx* c, const MatVec& A, z* theta, int precision,
   // step j's result: E_j, the residual estimate, and whether the solve may stop there
   auto check_step = [&](int j, bool* cv) -> int {
     TNT_CUDA_TRY(c, cudaEventSynchronize(c->ev_side[j & 1]));
-    const double* h = hp + 4 * (j & 1);
-    E = h[0];
-    const double bk = h[2];
-    resid = bk * h[1];
+    const KrylovSlot& h = slots[j & 1];
+    E = h.E;
+    const double bk = h.beta;
+    resid = bk * h.ylast;
     kk = j + 1;
     *cv = (resid_only || (have_prev && std::fabs(E - E_prev) <= tol * std::fabs(E))) &&
           resid <= rtol * std::fabs(E);
     if (bk <= rtol * std::fabs(E) * 1e-3 || bk == 0.0) *cv = true;
-    if (fused_gs && !std::isfinite(bk)) {  // a grid barrier's expired wait, or the numbers?
-      int st = 0;
-      TNT_CUDA_TRY(c, cudaMemcpyAsync(&st, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-      TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-      if (st & 2) {
-        cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
-        return set_err(c, TNT_E_TIMEOUT, "Gram-Schmidt step: a grid barrier wait expired");
-      }
+    const SlotState state = slot_state(h);
+    if (state == SLOT_TIMEOUT) {
+      cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);  // behind the step in flight
+      return set_err(c, TNT_E_TIMEOUT, "Lanczos step %d: a device-side wait expired (status %d)", total, (int)h.status);
     }
-    if (!std::isfinite(E) || !std::isfinite(bk))
+    if (state == SLOT_NAN)
       return set_err(c, TNT_E_NAN, "Lanczos produced a non-finite value at step %d (E = %g, beta = %g, %s matvec)",
                      total, E, bk, precision == TNT_PREC_MIXED ? "split-TF32" : "FP64");
     have_prev = true;

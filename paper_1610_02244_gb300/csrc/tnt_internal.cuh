@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/tnt_gb300.h"
+#include "krylov_slot.cuh"
 #include "upload.cuh"
 
 namespace tnt {
@@ -311,9 +312,9 @@ int vec_gs_step(Ctx* c, const z* V, int k, const z* w, int64_t n, z* vnext, doub
 
 // Lanczos tridiagonal: lowest eigenpair of T (k x k) given alpha[0..k-1], beta[0..k-2], on
 // stream st (the Lanczos runs it on the context's side stream); writes out[0] = E,
-// out[1] = |y_{k-1}|, y[0..k-1], and E, |y_{k-1}|, beta[k-1] to the pinned host array h_out.
+// out[1] = |y_{k-1}|, y[0..k-1], and the step's slot in pinned host memory, h_out.
 int tridiag_lowest_on(Ctx* c, cudaStream_t st, const double* d_alpha, const double* d_beta, int k,
-                      double* d_out, double* d_y, double* h_out);
+                      double* d_out, double* d_y, KrylovSlot* h_out);
 // Creates the context's side stream and its events on first use
 int side_stream(Ctx* c);
 // the same for nprob problems at once: problem p's alpha, beta, y at p * 64, out at p * 2;
