@@ -100,6 +100,15 @@ static int lanczos_cycle_loop(Ctx* c, const MatVec& A, z* theta, int precision,
   // k - 1 has computed one step more than it uses (not counted in n_matvec); the Ritz
   // vector is that of step k - 1, from V[0..k-1] and y of slot (k-1) & 1.
   TNT_TRY(side_stream(c));
+  // An error return may leave step k's eigenpair in flight on the side stream, which later calls
+  // on the main stream do not wait for: it would write into their scratch and pinned buffer.
+  struct SideDrain {
+    Ctx* c;
+    bool armed = true;
+    ~SideDrain() {
+      if (armed) cudaStreamSynchronize(c->side);
+    }
+  } drain{c};
   int last_side = -1;  // slot of the last side-stream launch
   KrylovSlot* const slots = (KrylovSlot*)hp;
   auto launch_tk = [&](int k) -> int {
@@ -204,6 +213,7 @@ static int lanczos_cycle_loop(Ctx* c, const MatVec& A, z* theta, int precision,
       res->resid = resid;
       res->n_matvec += total;
       res->converged = conv ? 1 : 0;
+      drain.armed = false;  // (the main stream waits for it)
       return TNT_OK;
     }
     TNT_TRY(vec_normalize(c, w, V, n, norm2));  // restart
