@@ -83,6 +83,14 @@ int pinned_reserve(Ctx* c, size_t bytes) {
   return TNT_OK;
 }
 
+int func_smem(Ctx* c, const void* fn, size_t bytes) {
+  size_t& have = c->smem_of[fn];
+  if (have >= bytes) return TNT_OK;
+  TNT_CUDA_TRY(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  have = bytes;
+  return TNT_OK;
+}
+
 // The tables of a 32-chain U(1) plan are the largest (a few MB); most are a few KB.
 constexpr size_t UP_HALF = 2 << 20;
 
@@ -344,6 +352,7 @@ static int ctx_create(int device, void* stream, const DevAlloc& a, tnt_ctx** out
   if (cudaSetDevice(device) != cudaSuccess) return TNT_E_CUDA;
   tnt_ctx* t = new tnt_ctx();
   t->c.device = device;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) == cudaSuccess && n > 0) t->c.nsm = n;
   t->c.stream = (cudaStream_t)stream;
   t->c.dalloc = a;
   tnt_params_default(&t->c.params);

@@ -444,16 +444,7 @@ __global__ void k_copy_runs(const int64_t* runs, int nrun, const z* src, z* dst)
   }
 }
 
-int sm_count() {
-  static int n = 0;
-  if (!n) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-      n = 152;
-  }
-  return n;
-}
+int sm_count(const Ctx* c) { return c ? c->nsm : 152; }  // (no context: the host check of the layout)
 unsigned cap_grid(int64_t work, int64_t cap) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(work, cap));
 }
@@ -558,13 +549,9 @@ struct ZHost {
 template <int BN>
 int launch_grouped(Ctx* c, const CUtensorMap& tA, const CUtensorMap& tB, const GArgs& g, int ntiles) {
   using Cf = GCfg<BN>;
-  static bool attr = false;
-  if (!attr) {
-    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_cgemm_grouped<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::SMEM));
-    attr = true;
-  }
+  TNT_TRY(func_smem(c, (const void*)k_cgemm_grouped<BN>, Cf::SMEM));
   if (ntiles <= 0) return TNT_OK;
-  k_cgemm_grouped<BN><<<cap_grid(ntiles, sm_count()), 192, Cf::SMEM, c->stream>>>(tA, tB, g);
+  k_cgemm_grouped<BN><<<cap_grid(ntiles, sm_count(c)), 192, Cf::SMEM, c->stream>>>(tA, tB, g);
   c->launches++;
   TNT_CHECK_LAUNCH(c);
   return TNT_OK;
@@ -942,7 +929,7 @@ int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
   // there are at most four times as many of them
   for (const TaskDesc& t : p->s1) { t1 += ((t.M + 127) / 128) * ((t.N + 63) / 64); z1 += ((t.M + 15) / 16) * ((t.N + 15) / 16); }
   for (const TaskDesc& t : p->s4) { t4 += 4 * ((t.M + 127) / 128) * ((t.N + 63) / 64); z4 += ((t.M + 15) / 16) * ((t.N + 15) / 16); }
-  if (std::max(z1, z4) <= 2 * sm_count()) z1 *= 4, z4 *= 4;
+  if (std::max(z1, z4) <= 2 * sm_count(c)) z1 *= 4, z4 *= 4;
   p->cap_g1tiles = (int)t1;
   p->cap_g4tiles = (int)t4;
   b += ws_round(sizeof(int4) * (t1 + t4 + z1 + z4)) + ws_round(sizeof(GTask) * (p->s1.size() + p->s4.size())) +
@@ -1103,11 +1090,11 @@ int u1_prepare(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
   make_ztiles(z1, ZM, &zt1);
   make_ztiles(z4, ZM, &zt4);
   // 16 x 16 tiles when the 64 x 64 ones would not give every SM FP64 work
-  p->ztile = ((int64_t)zt1.size() < sm_count() || (int64_t)zt4.size() < sm_count()) ? 16 : ZM;
+  p->ztile = ((int64_t)zt1.size() < sm_count(c) || (int64_t)zt4.size() < sm_count(c)) ? 16 : ZM;
   if (p->ztile == 16) {
     make_ztiles(z1, 16, &zt1);
     make_ztiles(z4, 16, &zt4);
-    p->ztile = tile_rows((int64_t)std::max(zt1.size(), zt4.size()), sm_count());
+    p->ztile = tile_rows((int64_t)std::max(zt1.size(), zt4.size()), sm_count(c));
     if (p->ztile < 16) {
       make_ztiles(z1, p->ztile, &zt1);
       make_ztiles(z4, p->ztile, &zt4);
@@ -1227,14 +1214,14 @@ int build_graph(Ctx* c, U1Plan& p, int mixed) {
     void* f1 = p.bn1 == 64 ? (void*)k_cgemm_grouped<64> : (void*)k_cgemm_grouped<128>;
     const int s1 = p.bn1 == 64 ? GCfg<64>::SMEM : GCfg<128>::SMEM;
     TNT_TRY(launch_grouped_bn(c, p.bn1, p.tmA1, p.tmB1, g1, 0));  // sets the smem attribute
-    TNT_TRY(add(knp(f1, cap_grid(p.n_g1tiles, sm_count()), 192, (unsigned)s1, a1)));
+    TNT_TRY(add(knp(f1, cap_grid(p.n_g1tiles, sm_count(c)), 192, (unsigned)s1, a1)));
     void* a2[] = {&wa};
     TNT_TRY(add(knp((void*)k_wop<true>, gw, 256, 0, a2)));
     void* a3[] = {&m4a, &m4b, &g4};
     void* f4 = p.bn4 == 64 ? (void*)k_cgemm_grouped<64> : (void*)k_cgemm_grouped<128>;
     const int s4 = p.bn4 == 64 ? GCfg<64>::SMEM : GCfg<128>::SMEM;
     TNT_TRY(launch_grouped_bn(c, p.bn4, p.tmA4, p.tmB4, g4, 0));
-    TNT_TRY(add(knp(f4, cap_grid(p.n_g4tiles, sm_count()), 192, (unsigned)s4, a3)));
+    TNT_TRY(add(knp(f4, cap_grid(p.n_g4tiles, sm_count(c)), 192, (unsigned)s4, a3)));
     GthArgs ga = p.out_g[1];
     void* a4[] = {&ga};
     TNT_TRY(add(knp((void*)k_gather_u1<true>, gg, 256, 0, a4)));

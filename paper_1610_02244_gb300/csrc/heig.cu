@@ -1454,11 +1454,14 @@ size_t heig_scratch_bound(int64_t n, int64_t k) {
          (size_t)(1 << 20);
 }
 
+constexpr int64_t EIG_NMAX = 8192;  // rows of the largest eigenproblem
+constexpr size_t BT_SMEM = 200 * 1024;
+
 // one warp per eigenvalue, the largest problem of n rows
 static int launch_bisect(Ctx* c, int64_t n, int64_t kt, const double* d, const double* e, const EBlk* dblk,
                          const int2* deig, const int64_t* nr, double* ev) {
   const size_t smem = sizeof(double) * 2 * (size_t)n;
-  TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_bisect, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  TNT_TRY(func_smem(c, (const void*)k_bisect, sizeof(double) * 2 * EIG_NMAX));
   k_bisect<<<(unsigned)kt, 32, smem, c->stream>>>(d, e, dblk, deig, nr, ev);
   return TNT_OK;
 }
@@ -1482,7 +1485,7 @@ int heig_finish(Ctx* c, int64_t n, int64_t k, const z* Hv, const z* tau, const d
     return set_err(c, TNT_E_ALLOC, "scratch exhausted (eigenvectors n=%lld k=%lld)", (long long)n, (long long)k);
   }
   cudaStream_t st = c->stream;
-  const int cols = (sizeof(z) * n * BT_COLS <= (size_t)200 * 1024) ? BT_COLS : 1;
+  const int cols = (sizeof(z) * n * BT_COLS <= BT_SMEM) ? BT_COLS : 1;
   const int64_t nbt = (k + cols - 1) / cols;
   {  // one problem: the block table and the (eigenvalue, back-transformation) index tables
     const EBlk hb{n, k, 0, 0, 0, 0, 0};
@@ -1503,7 +1506,7 @@ int heig_finish(Ctx* c, int64_t n, int64_t k, const z* Hv, const z* tau, const d
   {
     ProfScope ps(c, "heig_backtransform", 8.0 * (double)n * (double)n * (double)k);
     const size_t smem = sizeof(z) * n * cols;
-    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_backtransform, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    TNT_TRY(func_smem(c, (const void*)k_backtransform, BT_SMEM));
     k_backtransform<<<(unsigned)nbt, 256, smem, st>>>(Y, Hv, tau, dblk, deig + k, cols, U0);
     c->launches++;
     TNT_CHECK_LAUNCH(c);
@@ -1547,7 +1550,7 @@ int heig_finish(Ctx* c, int64_t n, int64_t k, const z* Hv, const z* tau, const d
 // eigenvectors of the k largest eigenvalues, in descending order; ev (device, k).
 int heig_top(Ctx* c, z* G, int64_t n, int64_t k, z* U, int64_t ldu, double* ev) {
   if (k < 1 || k > n) return set_err(c, TNT_E_INVALID, "heig_top: k = %lld of n = %lld", (long long)k, (long long)n);
-  if (n > 8192) return set_err(c, TNT_E_UNSUPPORTED, "heig_top: n = %lld > 8192", (long long)n);
+  if (n > EIG_NMAX) return set_err(c, TNT_E_UNSUPPORTED, "heig_top: n = %lld > %lld", (long long)n, (long long)EIG_NMAX);
   const size_t top = c->ws.top;
   z* Hv = (z*)ws_alloc(c, ws_round(sizeof(z) * n * n));
   z* tau = (z*)ws_alloc(c, ws_round(sizeof(z) * n));
@@ -1568,22 +1571,15 @@ int heig_top(Ctx* c, z* G, int64_t n, int64_t k, z* U, int64_t ldu, double* ev) 
     // multiply-add, two rank-2 updates of the trailing block and its matrix-vector product)
     ProfScope ps(c, "heig_tridiag", 16.0 / 3.0 * nn * nn * nn);
     const size_t tri_smem = 4 * TRI_CACHE * sizeof(z);
-    static int nsm = 0, occ = 0;
-    if (!nsm) {
-      int v = 0;
-      TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_tridiag_persistent,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri_smem));
-      TNT_CUDA_TRY(c, cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, c->device));
-      TNT_CUDA_TRY(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tridiag_persistent,
-                                                                    TRI_THREADS, tri_smem));
-      nsm = v;
-    }
+    int occ = 0;
+    TNT_TRY(func_smem(c, (const void*)k_tridiag_persistent, tri_smem));
+    TNT_CUDA_TRY(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tridiag_persistent, TRI_THREADS, tri_smem));
     if (occ < 1) return set_err(c, TNT_E_UNSUPPORTED, "tridiagonal kernel cannot be resident");
     TNT_CUDA_TRY(c, cudaMemsetAsync(bar, 0, 256, st));
     TriArgs ta{G, n, Hv, tau, d, e, p, part, (unsigned*)bar, (int*)(bar + 16), c->d_status,
                gws};
     void* args[] = {&ta};
-    const int nb = std::min(nsm, TRI_MAX_BLOCKS);
+    const int nb = std::min(c->nsm, TRI_MAX_BLOCKS);
     TNT_CUDA_TRY(c, cudaLaunchCooperativeKernel((void*)k_tridiag_persistent, dim3(nb),
                                                 dim3(TRI_THREADS), args, tri_smem, st));
     c->launches += 1;
@@ -1776,18 +1772,17 @@ int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& all, z* U, double* ev
   if (blocks.empty()) return TNT_OK;
   std::stable_sort(blocks.begin(), blocks.end(), [](const SmallEig& a, const SmallEig& b) { return a.n > b.n; });
   const int nb = (int)blocks.size();
-  static int nsm = 0;
-  static size_t smem_max = 0;
-  if (!nsm) {
-    int v = 0, optin = 0;
+  if (!c->tri_smem) {
+    int optin = 0;
     cudaFuncAttributes fa{};
-    TNT_CUDA_TRY(c, cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, c->device));
     TNT_CUDA_TRY(c, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
     TNT_CUDA_TRY(c, cudaFuncGetAttributes(&fa, k_tridiag_group));
-    smem_max = (size_t)optin - fa.sharedSizeBytes;
-    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_tridiag_group, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
-    nsm = v;
+    const size_t most = (size_t)optin - fa.sharedSizeBytes;
+    TNT_TRY(func_smem(c, (const void*)k_tridiag_group, most));
+    c->tri_smem = most;
   }
+  const int nsm = c->nsm;
+  const size_t smem_max = c->tri_smem;
   // large blocks (the first nl): back-transformation by panels of reflectors
   int nl = 0;
   while (nl < nb && blocks[(size_t)nl].n > WY_MIN) ++nl;
@@ -1917,7 +1912,7 @@ int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& all, z* U, double* ev
     ProfScope ps(c, "heig_backtransform", fl);
     if (!hbt.empty()) {
       const size_t smem = sizeof(z) * (size_t)blocks[(size_t)nl].n * cols;
-      TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_backtransform, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      TNT_TRY(func_smem(c, (const void*)k_backtransform, BT_SMEM));
       k_backtransform<<<(unsigned)hbt.size(), 256, smem, st>>>(Y, G, tau, dblk, dbt, cols, U0);
       c->launches++;
     }

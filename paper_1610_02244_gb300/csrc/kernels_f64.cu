@@ -140,9 +140,7 @@ int zgemm(Ctx* c, const ZGemm& g) {
   }
   if (ozgemm_eligible(c, g)) return ozgemm(c, g);
   {
-    static int nsm = 0;
-    if (!nsm && (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || nsm < 1))
-      nsm = 152;
+    const int nsm = c->nsm;
     const int64_t tiles64 = ((g.M + GM - 1) / GM) * ((g.N + GN - 1) / GN) * g.batch;
     if (tiles64 < nsm && (g.M + 15) / 16 <= 65535 && g.batch <= 65535) {
       const int64_t tiles16 = ((g.M + 15) / 16) * ((g.N + 15) / 16) * g.batch;
@@ -219,7 +217,7 @@ int zgemm_fma_tasks(Ctx* c, const GemmTask* const* tasks, int n) {
   int64_t t16 = 0;
   for (int i = 0; i < n; ++i)
     t16 += ((tasks[i]->g.M + 15) / 16) * ((tasks[i]->g.N + 15) / 16) / (tasks[i]->herm ? 2 : 1);
-  const int R = tile_rows(t16, 152);
+  const int R = tile_rows(t16, c->nsm);
   for (int i0 = 0; i0 < n; i0 += FT_MAX) {
     FmaTasks T;
     T.n = std::min(FT_MAX, n - i0);
@@ -1298,13 +1296,8 @@ int vec_gs_reset(Ctx* c) {
 
 int vec_gs_step(Ctx* c, const z* V, int k, const z* w, int64_t n, z* vnext, double* d_alpha, double* d_beta) {
   if (k < 1 || k > 64) return set_err(c, TNT_E_UNSUPPORTED, "Gram-Schmidt step with k = %d", k);
-  static int nsm = 0;
-  if (!nsm) {
-    int v = 0;
-    TNT_CUDA_TRY(c, cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, c->device));
-    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_gs_step, cudaFuncAttributeMaxDynamicSharedMemorySize, GS_SMEM));
-    nsm = v;
-  }
+  const int nsm = c->nsm;
+  TNT_TRY(func_smem(c, (const void*)k_gs_step, GS_SMEM));
   const size_t top = c->ws.top;
   z* part = (z*)ws_alloc(c, ws_round(sizeof(z) * 2 * 64 * (size_t)nsm));
   double* npart = (double*)ws_alloc(c, ws_round(sizeof(double) * 2 * (size_t)nsm));

@@ -701,28 +701,20 @@ OzDeal oz_deal(int64_t tiles, int64_t nkb, int nsm) {
 // 30 us however small the product.  Measured with 16 x 16 tiles (FP64 / slices, us):
 // 128 x 512 x 32 35 / 30, 64 x 512 x 64 18 / 27, 256 x 256 x 64 36 / 30,
 // 256 x 1024 x 64 125 / 32, 64 x 64 x 1024 280 / 39.
-static double fma_rounds(double k, double tiles) { return k * std::max(0.3, tiles / 152.0); }
+static double fma_rounds(const Ctx* c, double k, double tiles) { return k * std::max(0.3, tiles / c->nsm); }
 bool ozgemm_eligible(const Ctx* c, const ZGemm& g) {
   if (c->oz_mode == 0 || g.batch != 1 || g.alpha.x != 1.0 || g.alpha.y != 0.0 || g.beta.x != 0.0 ||
       g.beta.y != 0.0 || g.M < 16 || g.N < 16 || g.K < 16 || g.M >= (1LL << 31) || g.N >= (1LL << 31))
     return false;
   const double tiles = (double)cdiv(g.M, 16) * (double)cdiv(g.N, 16) * (g.lower_only ? 0.5 : 1.0);
-  return fma_rounds((double)g.K, tiles) >= 110.0;
+  return fma_rounds(c, (double)g.K, tiles) >= 110.0;
 }
 
 namespace {
-int oz_sm_count(Ctx* c, int* sm) {
-  static int v = 0;
-  if (!v) {
-    int n = 0;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || n < 1) n = 152;
-    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_oz_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
-    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_oz_gemm<OZ_MAXT>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
-    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_oz_gemm<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
-    v = n;
-  }
-  *sm = v;
-  return TNT_OK;
+int oz_setup(Ctx* c) {
+  TNT_TRY(func_smem(c, (const void*)k_oz_gemm<1>, OZ_SMEM));
+  TNT_TRY(func_smem(c, (const void*)k_oz_gemm<OZ_MAXT>, OZ_SMEM));
+  return func_smem(c, (const void*)k_oz_gemm<0>, OZ_SMEM);
 }
 
 // tables of the products tk[0..n): T's head and tasks, and the bytes of buffer they use
@@ -820,8 +812,8 @@ unsigned oz_prep_grid(const OzTasks<CAP>& T) {
 // products, separate / one launch, us: 256 x 256 x 128 63.5 / 58.6, 1024 x 1024 x 64 86.7 / 81.8,
 // 1024 x 1024 x 512 189.7 / 186.1 (256 groups), 1024 x 4096 x 256 333.6 / 333.8 (640),
 // 2048 x 2048 x 512 536.7 / 539.1 (512), 256 x 8192 x 512 356.5 / 364.2 (1056).
-bool oz_one_prep(const OzHead& h, const OzTask* t, int n) {
-  if (h.groups[0] + h.groups[1] > 2 * 152) return false;
+bool oz_one_prep(const OzHead& h, const OzTask* t, int n, int sm) {
+  if (h.groups[0] + h.groups[1] > 2 * sm) return false;
   for (int i = 0; i < n; ++i)
     if (t[i].K > OZ_SCALE_K) return false;
   return true;
@@ -848,7 +840,7 @@ int oz_launch(Ctx* c, const GemmTask* const* tk, int n, int sm) {
   T.h.buf = (uint8_t*)c->oz_buf;
   {
     ProfScope ps(c, "oz_slice", bytes);
-    if (oz_one_prep(T.h, T.t, n)) {
+    if (oz_one_prep(T.h, T.t, n, sm)) {
       k_oz_prep<CAP><<<oz_prep_grid(T), 256, 0, c->stream>>>(T);
       c->launches++;
     } else {
@@ -875,8 +867,8 @@ int oz_launch(Ctx* c, const GemmTask* const* tk, int n, int sm) {
 
 // ---------------------------------------------------------------- repeated products
 size_t oz_plan_bytes(Ctx* c, const std::vector<GemmTask>& tasks) {
-  int sm = 0;
-  if (tasks.empty() || oz_sm_count(c, &sm) != TNT_OK) return 0;
+  if (tasks.empty()) return 0;
+  const int sm = c->nsm;
   std::vector<const GemmTask*> tk;
   for (const GemmTask& t : tasks) tk.push_back(&t);
   std::vector<OzTask> t(tasks.size());
@@ -887,8 +879,8 @@ size_t oz_plan_bytes(Ctx* c, const std::vector<GemmTask>& tasks) {
 }
 
 int oz_plan_build(Ctx* c, const std::vector<GemmTask>& tasks, int fixed_sides, OzPlan* p) {
-  int sm = 0;
-  TNT_TRY(oz_sm_count(c, &sm));
+  TNT_TRY(oz_setup(c));
+  const int sm = c->nsm;
   std::vector<const GemmTask*> tk;
   for (const GemmTask& t : tasks) {
     tk.push_back(&t);
@@ -907,7 +899,7 @@ int oz_plan_build(Ctx* c, const std::vector<GemmTask>& tasks, int fixed_sides, O
   T.h.buf = buf;
   T.h.status = c->d_status;
   T.t = dt;
-  const bool one = oz_one_prep(T.h, t.data(), (int)t.size());
+  const bool one = oz_one_prep(T.h, t.data(), (int)t.size(), sm);
   auto inputs = [&](OzNode* node) {  // the launches that read the operands of T.h.sides
     if (one) {
       node[0] = OzNode{(void*)k_oz_prep<0>, oz_prep_grid(T), 256, 0};
@@ -958,8 +950,8 @@ int oz_plan_run(Ctx* c, const OzPlan& p, const z* add_b) {
 }
 
 int ozgemm(Ctx* c, const ZGemm& g) {
-  int sm = 0;
-  TNT_TRY(oz_sm_count(c, &sm));
+  TNT_TRY(oz_setup(c));
+  const int sm = c->nsm;
   const GemmTask t{g, 0, 0};
   const GemmTask* p = &t;
   return oz_launch<1>(c, &p, 1, sm);
@@ -970,13 +962,13 @@ int ozgemm(Ctx* c, const ZGemm& g) {
 // FP64 tiles, dealt to the SMs, would take longer than the slice launches' 30 us (the rule of
 // ozgemm_eligible for the whole set); products with a side below 16 stay on FP64 units.
 int zgemm_tasks(Ctx* c, const std::vector<GemmTask>& tasks) {
-  int sm = 0;
-  TNT_TRY(oz_sm_count(c, &sm));
+  TNT_TRY(oz_setup(c));
+  const int sm = c->nsm;
   double rounds = 0, longest = 0;
   for (const GemmTask& t : tasks) {
     const double k = (double)t.g.K;
     rounds += k * (double)cdiv(t.g.M, 16) * (double)cdiv(t.g.N, 16) * (t.herm ? 0.5 : 1.0) / sm;
-    longest = std::max(longest, fma_rounds(k, 0.0));
+    longest = std::max(longest, fma_rounds(c, k, 0.0));
   }
   const bool slices = c->oz_mode != 0 && std::max(rounds, longest) >= 110.0;
   std::vector<const GemmTask*> oz, fma;

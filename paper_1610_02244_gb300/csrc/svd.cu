@@ -838,7 +838,7 @@ int svd_trunc_impl(Ctx* c, const z* M, int64_t m, int64_t n, const int64_t* h_rq
     auto select = ntot_vals <= 4096 ? k_select<4> : k_select<8>;  // 8192 candidates at most
     unsigned threads = 64;
     while (threads < 1024 && 4 * (int64_t)threads < ntot_vals) threads *= 2;
-    TNT_CUDA_TRY(c, cudaFuncSetAttribute(select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    TNT_TRY(func_smem(c, (const void*)select, 8192 * (sizeof(double) + 2 * sizeof(int))));
     // never more than the blocks' rank bounds (at most min(m, n), the callers' capacity),
     // whatever the number of candidates formed
     int64_t rank_total = 0;

@@ -336,12 +336,7 @@ int make_map(Ctx* c, CUtensorMap* tm, float* base, int64_t rows, int64_t K, int 
 
 int launch_cgemm(Ctx* c, const CUtensorMap& tA, const CUtensorMap& tB, int64_t M, int64_t N,
                  int64_t Kp, int split, float* C, int64_t ldc, int64_t K_true) {
-  static bool attr = false;
-  if (!attr) {
-    TNT_CUDA_TRY(c, cudaFuncSetAttribute(k_cgemm_tf32x3, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         SMEM_BYTES));
-    attr = true;
-  }
+  TNT_TRY(func_smem(c, (const void*)k_cgemm_tf32x3, SMEM_BYTES));
   CG g;
   g.M = M;
   g.N = N;

@@ -109,6 +109,9 @@ void dev_free(const DevAlloc& a, void* p);
 
 struct Ctx {
   int device = 0;
+  int nsm = 152;                          // SMs of the device
+  size_t tri_smem = 0;                    // dynamic shared memory a CTA of k_tridiag_group can have
+  std::map<const void*, size_t> smem_of;  // kernels whose shared-memory limit this context raised
   DevAlloc dalloc;
   cudaStream_t stream = 0;
   tnt_params params;
@@ -194,6 +197,11 @@ void* ws_alloc(Ctx* c, size_t bytes);
 inline void ws_reset(Ctx* c) { c->ws.top = 0; }
 inline size_t ws_round(size_t b) { return (b + 255) & ~size_t(255); }
 int pinned_reserve(Ctx* c, size_t bytes);
+// Raises a kernel's dynamic shared-memory limit to `bytes`, once per context: the limit belongs
+// to the device, so a guard for the process would leave a second device without it.  `bytes`
+// is the most that kernel is ever launched with, the same in every call, since contexts of
+// one device share the limit.
+int func_smem(Ctx* c, const void* fn, size_t bytes);
 // copies a host table to the device on the context's stream; src may go or change at return
 int to_device(Ctx* c, void* dst, const void* src, size_t bytes);
 
