@@ -20,6 +20,7 @@
 
 #include "heff_plan.cuh"
 #include "f32conv.cuh"
+#include "tri_deal.cuh"
 
 namespace tnt {
 
@@ -409,10 +410,8 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tridiag_persistent(TriArgs a) {
 // 4.5 ms, 1024 rows 24.4 ms).
 static_assert(TRI_WARPS == 16, "the flattened row split divides by 16 with shifts");
 constexpr int TRI_VEC = 3;              // vector entries per thread
-constexpr int64_t TRI_ROWS_NMAX = 1216; // <= TRI_VEC * TRI_THREADS; (8 + 3) n entries fit
-constexpr int TRI_RMAX = 128;           // rows per CTA
+static_assert(TRI_ROWS_NMAX <= TRI_VEC * TRI_THREADS, "every vector entry has a thread");
 constexpr int TRI_GTHREADS = TRI_THREADS + 32;
-constexpr int TRI_MAXB = 48;            // blocks of one launch
 
 struct TriBlk {
   z* G;          // the block, n x n; its rows become the reflectors
@@ -1599,48 +1598,6 @@ int heig_top(Ctx* c, z* G, int64_t n, int64_t k, z* U, int64_t ldu, double* ev) 
   return r;
 }
 
-namespace {
-// CTAs of each block's group (in the order of `n`, descending) for one launch on nsm SMs of
-// smem bytes: the shortest common time by the model
-//   t(n, nb) = n t_col + (2 n^3 / nb + 4 n^2) / f,
-// 12 FP64 operations per trailing entry of a CTA's rows and 16 per entry of its vectors at two
-// per SM and clock, and a column's latency t_col (scalars, loads, barrier: 4 us in a group
-// of one CTA, 5 us and 0.01 us per CTA with a barrier).  Returns how many of the blocks fit the launch.
-int tri_deal(const std::vector<int64_t>& n, int nsm, size_t smem, std::vector<int>* nb) {
-  auto fits = [&](int64_t m, int64_t q) {
-    const int64_t rows = (m + q - 1) / q;
-    return rows <= TRI_RMAX && (size_t)(rows + 3 + (q == 1)) * m * sizeof(z) <= smem;
-  };
-  auto time = [](double m, double q) { return m * (q > 1 ? 5.0 + 0.01 * q : 4.0) + (2.0 * m * m * m / q + 4.0 * m * m) / 2070.0; };
-  std::vector<int> lo;
-  int used = 0;
-  for (int64_t m : n) {  // the least group that holds each block
-    int q = 1;
-    while (q < m && !fits(m, q)) ++q;
-    if (!fits(m, q) || used + q > nsm || (int)lo.size() == TRI_MAXB) break;
-    lo.push_back(q);
-    used += q;
-  }
-  const int cnt = (int)lo.size();
-  // more CTAs to the block that takes longest, as long as that shortens it
-  std::vector<int> q = lo;
-  while (cnt > 0) {
-    int w = 0;
-    for (int i = 1; i < cnt; ++i)
-      if (time((double)n[(size_t)i], q[(size_t)i]) > time((double)n[(size_t)w], q[(size_t)w])) w = i;
-    const double m = (double)n[(size_t)w], now = time(m, q[(size_t)w]);
-    // the next size worth having: a second CTA brings the barrier's cost with it
-    int next = q[(size_t)w] + 1;
-    while (next - q[(size_t)w] <= nsm - used && next < (int)m && time(m, next) >= now) ++next;
-    if (next - q[(size_t)w] > nsm - used || next > (int)m || time(m, next) >= now) break;
-    used += next - q[(size_t)w];
-    q[(size_t)w] = next;
-  }
-  *nb = q;
-  return cnt;
-}
-}  // namespace
-
 // Above this many rows the panels' products are the faster back-transformation: a set of
 // grouped products costs about 35 us, so a 128-reflector panel about 70 and the T factors
 // 150 in all, where the one-CTA form takes about 2.5 us per reflector (two vectors a CTA:
@@ -1750,7 +1707,8 @@ size_t heig_blocks_scratch(int64_t n, int64_t k) {
 }
 
 // Eigenvectors of the k largest eigenvalues of many Hermitian blocks: every stage of the
-// eigensolve is one launch (or a few) over all blocks of up to TRI_ROWS_NMAX rows.
+// eigensolve is one launch (or a few) over all blocks that a group of CTAs can hold (tri_holds:
+// 1216 rows on 152 SMs); larger ones take heig_top one after the other.
 // blocks[i] = {offset of the n x n block in G (and of its eigenvector columns in U, leading
 // dimension n), n, k}; the reflectors replace the blocks' rows.  ev (device) receives
 // the eigenvalues of all blocks back to back.
@@ -1758,20 +1716,6 @@ int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& all, z* U, double* ev
   if (all.empty()) return TNT_OK;
   const size_t top = c->ws.top;
   cudaStream_t st = c->stream;
-  std::vector<SmallEig> blocks;
-  for (const SmallEig& b : all) {
-    if (b.n < 1 || b.k < 1 || b.k > b.n)
-      return set_err(c, TNT_E_INVALID, "eigensolve block n=%lld k=%lld", (long long)b.n, (long long)b.k);
-    if (b.n <= TRI_ROWS_NMAX) {
-      blocks.push_back(b);
-      continue;
-    }
-    TNT_TRY(heig_top(c, G + b.goff, b.n, b.k, U + b.goff, b.n, ev));
-    ev += b.k;
-  }
-  if (blocks.empty()) return TNT_OK;
-  std::stable_sort(blocks.begin(), blocks.end(), [](const SmallEig& a, const SmallEig& b) { return a.n > b.n; });
-  const int nb = (int)blocks.size();
   if (!c->tri_smem) {
     int optin = 0;
     cudaFuncAttributes fa{};
@@ -1783,6 +1727,20 @@ int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& all, z* U, double* ev
   }
   const int nsm = c->nsm;
   const size_t smem_max = c->tri_smem;
+  std::vector<SmallEig> blocks;
+  for (const SmallEig& b : all) {
+    if (b.n < 1 || b.k < 1 || b.k > b.n)
+      return set_err(c, TNT_E_INVALID, "eigensolve block n=%lld k=%lld", (long long)b.n, (long long)b.k);
+    if (tri_holds(b.n, nsm, smem_max)) {
+      blocks.push_back(b);
+      continue;
+    }
+    TNT_TRY(heig_top(c, G + b.goff, b.n, b.k, U + b.goff, b.n, ev));
+    ev += b.k;
+  }
+  if (blocks.empty()) return TNT_OK;
+  std::stable_sort(blocks.begin(), blocks.end(), [](const SmallEig& a, const SmallEig& b) { return a.n > b.n; });
+  const int nb = (int)blocks.size();
   // large blocks (the first nl): back-transformation by panels of reflectors
   int nl = 0;
   while (nl < nb && blocks[(size_t)nl].n > WY_MIN) ++nl;
