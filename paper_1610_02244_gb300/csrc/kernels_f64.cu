@@ -6,6 +6,7 @@
 #include <cstdarg>
 #include <cmath>
 
+#include "gs_split.cuh"
 #include "tnt_internal.cuh"
 #include "f32conv.cuh"
 
@@ -937,11 +938,6 @@ int vec_normalize(Ctx* c, const z* x, z* y, int64_t n, const double* d_norm2) {
 // reducing 16 sums per thread), 115 us at n = 5000.
 namespace {
 constexpr int GS_THREADS = 256, GS_WARPS = GS_THREADS / 32;
-constexpr int GS_SMEM = 204 * 1024;
-// Above this the slice of w alone nears the shared memory of an SM, and both forms are bound
-// by the FP64 pipe.  FP64 solves of this size, fused (then with two passes over all of V) /
-// separate launches: n = 2^12 9.7 / 27 ms, 2^16 28 / 50, 2^18 60 / 80, 2^20 232 / 239.
-constexpr int64_t GS_MAX_N = 1 << 20;
 
 struct GsArgs {  // part: 64 vectors' sums, npart: the norm's
   const z* V;
@@ -1284,9 +1280,7 @@ __global__ void __launch_bounds__(GS_THREADS, 1) k_gs_step(GsArgs a) {
 }
 }  // namespace
 
-// Elements of w per CTA, and whether the basis slice is kept: as many CTAs as SMs, down to 64
-// elements each
-bool vec_gs_eligible(int64_t n) { return n <= GS_MAX_N; }
+bool vec_gs_eligible(const Ctx* c, int64_t n) { return gs_fits(n, c->nsm); }
 
 int vec_gs_reset(Ctx* c) {
   TNT_CUDA_TRY(c, cudaMemsetAsync(c->d_count + 16, 0, sizeof(unsigned), c->stream));
@@ -1310,7 +1304,7 @@ int vec_gs_step(Ctx* c, const z* V, int k, const z* w, int64_t n, z* vnext, doub
   a.bar = c->d_count + 16;
   a.base = c->gs_arrivals;
   a.status = c->d_status;
-  a.S = (int)std::max<int64_t>(64, (n + nsm - 1) / nsm);
+  a.S = (int)gs_slice(n, nsm);
   const int grid = (int)((n + a.S - 1) / a.S);
   c->gs_arrivals += 4u * (unsigned)grid;
   const size_t sw = sizeof(z) * (size_t)a.S, all = sw * (size_t)(k + 1);

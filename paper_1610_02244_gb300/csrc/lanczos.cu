@@ -81,7 +81,7 @@ static int lanczos_cycle_loop(Ctx* c, const MatVec& A, z* theta, int precision,
   // u_32 |V c|, stays below the matvec's own ~2^-22 error); the Ritz vector is assembled
   // in FP64, as its norm enters the FP64 Rayleigh quotient
   const bool f32_gs = (precision == TNT_PREC_MIXED);
-  const bool fused_gs = !f32_gs && vec_gs_eligible(n);
+  const bool fused_gs = !f32_gs && vec_gs_eligible(c, n);
   if (fused_gs) TNT_TRY(vec_gs_reset(c));
   double* hp = c->h_pinned;
   // v_0 = theta / |theta| (a zero or non-finite start vector is reported, not iterated)

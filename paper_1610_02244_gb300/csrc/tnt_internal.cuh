@@ -308,12 +308,12 @@ int vec_normalize(Ctx* c, const z* x, z* y, int64_t n, const double* d_norm2);
 int vec_norm2(Ctx* c, const z* x, int64_t n, double* d_norm2);
 int vec_dot(Ctx* c, const z* x, const z* y, int64_t n, z* d_dot);
 
-// The FP64 Gram-Schmidt work of one Krylov step in one launch (n up to the bound of
+// The FP64 Gram-Schmidt work of one Krylov step in one launch (where
 // vec_gs_eligible): w = A V_{k-1} against V_{k-2} and V_{k-1}, then against V[0..k) (leading
 // dimension n), alpha[k-1] = Re <V_{k-1}|w> at first, beta[k-1] = |w| at last, vnext = w / |w|
 // (none if null); w itself is left as it was.  vec_gs_reset before the first step of a solve: the grid barrier's
 // count (a barrier whose wait expired leaves it behind).
-bool vec_gs_eligible(int64_t n);
+bool vec_gs_eligible(const Ctx* c, int64_t n);
 int vec_gs_reset(Ctx* c);
 int vec_gs_step(Ctx* c, const z* V, int k, const z* w, int64_t n, z* vnext, double* d_alpha,
                 double* d_beta);
