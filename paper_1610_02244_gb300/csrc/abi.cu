@@ -420,6 +420,7 @@ int tnt_ctx_destroy(tnt_ctx* ctx) {
   dev_free(ctx->c.dalloc, ctx->c.d_status);
   dev_free(ctx->c.dalloc, ctx->c.d_count);
   dev_free(ctx->c.dalloc, ctx->c.oz_buf);
+  for (void* b : ctx->c.oz_kept) dev_free(ctx->c.dalloc, b);
   delete ctx;
   return TNT_OK;
 }

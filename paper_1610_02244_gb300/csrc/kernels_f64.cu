@@ -139,7 +139,10 @@ int zgemm(Ctx* c, const ZGemm& g) {
     // C = beta C (or zero): not needed by the library; reject to keep the kernel simple
     return set_err(c, TNT_E_INVALID, "zgemm with K = 0");
   }
-  if (ozgemm_eligible(c, g)) return ozgemm(c, g);
+  if (ozgemm_eligible(c, g)) {
+    const int r = ozgemm(c, g);
+    if (r != OZ_NOROOM) return r;
+  }
   {
     const int nsm = c->nsm;
     const int64_t tiles64 = ((g.M + GM - 1) / GM) * ((g.N + GN - 1) / GN) * g.batch;

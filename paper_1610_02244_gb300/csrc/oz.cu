@@ -819,8 +819,18 @@ bool oz_one_prep(const OzHead& h, const OzTask* t, int n, int sm) {
   return true;
 }
 
+bool oz_capturing(Ctx* c) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream beside another stream's capture
+    return false;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
 // products tk[0..n) in one set of launches; slices and partial sums live in the context's own
-// buffer (grown between calls, never inside a capture)
+// buffer, grown between calls, never inside a capture (OZ_NOROOM); a buffer that a captured
+// graph refers to is kept until the context goes
 template <int CAP>
 int oz_launch(Ctx* c, const GemmTask* const* tk, int n, int sm) {
   OzTasks<CAP> T;
@@ -828,9 +838,14 @@ int oz_launch(Ctx* c, const GemmTask* const* tk, int n, int sm) {
   const size_t need = oz_layout(tk, n, sm, &T.h, T.t, &flop, &bytes);
   if (!need) return set_err(c, TNT_E_UNSUPPORTED, "FP64 products too large for one launch");
   T.h.status = c->d_status;
+  const bool capture = oz_capturing(c);
+  if (capture && need > c->oz_cap) return OZ_NOROOM;
+  if (capture) c->oz_captured = true;
   if (need > c->oz_cap) {
     TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    dev_free(c->dalloc, c->oz_buf);
+    if (c->oz_captured) c->oz_kept.push_back(c->oz_buf);
+    else dev_free(c->dalloc, c->oz_buf);
+    c->oz_captured = false;
     c->oz_buf = nullptr;
     c->oz_cap = 0;
     if (dev_alloc(c->dalloc, &c->oz_buf, need) != 0)
@@ -994,8 +1009,9 @@ int zgemm_tasks(Ctx* c, const std::vector<GemmTask>& tasks) {
   std::stable_sort(oz.begin(), oz.end(), [](const GemmTask* a, const GemmTask* b) { return a->g.K > b->g.K; });
   for (size_t i = 0; i < oz.size(); i += OZ_MAXT) {
     const int n = (int)std::min<size_t>(OZ_MAXT, oz.size() - i);
-    if (n == 1) TNT_TRY(oz_launch<1>(c, oz.data() + i, 1, sm));
-    else TNT_TRY(oz_launch<OZ_MAXT>(c, oz.data() + i, n, sm));
+    const int r = n == 1 ? oz_launch<1>(c, oz.data() + i, 1, sm) : oz_launch<OZ_MAXT>(c, oz.data() + i, n, sm);
+    if (r == OZ_NOROOM) fma.insert(fma.end(), oz.begin() + (long)i, oz.begin() + (long)i + n);
+    else TNT_TRY(r);
   }
   return fma.empty() ? TNT_OK : zgemm_fma_tasks(c, fma.data(), (int)fma.size());
 }

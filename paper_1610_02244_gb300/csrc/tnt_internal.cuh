@@ -148,6 +148,8 @@ struct Ctx {
   bool fp64_finish = false;
   void* oz_buf = nullptr;
   size_t oz_cap = 0;
+  bool oz_captured = false;        // a stream capture holds a pointer to it
+  std::vector<void*> oz_kept;      // earlier ones that a captured graph may still use
   // second stream for the Lanczos T_k eigenproblem, one Krylov step behind the vector
   // work on `stream`, and the events that order the two (created on first use)
   cudaStream_t side = nullptr;
@@ -227,6 +229,9 @@ int tile_rows(int64_t tiles, int nsm);
 // FP64-accurate C = A B on the tensor cores by exact integer slicing (oz.cu); zgemm routes
 // large products with alpha = 1, beta = 0, batch = 1 there when the context allows it
 bool ozgemm_eligible(const Ctx* c, const ZGemm& g);
+// OZ_NOROOM: the slice buffer is too small and the stream is being captured, so that it cannot
+// grow; nothing was launched, the FP64 units do the product
+constexpr int OZ_NOROOM = -1;
 int ozgemm(Ctx* c, const ZGemm& g);
 // One of a set of independent products run in grouped launches: herm, the result is
 // Hermitian (its lower triangle is computed and mirrored); sub, C -= A B instead of C = A B
