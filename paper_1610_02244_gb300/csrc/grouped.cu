@@ -784,23 +784,25 @@ int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
     const P1Info& i1 = info1[pi];
     const P4Info& i4 = info4[pi];
     // W12[(s1' s2' w2), (w s1 s2)] = sum_w1 W1[w,w1,s1',s1] W2[w1,w2,s2',s2]  (host, FP64),
-    // from the non-zero entries of the two tensors; per row its non-zero columns in order
+    // from the non-zero entries of the two tensors (from all where one is not finite); per row
+    // its non-zero columns in order
     const z* W1 = s.hW1 ? s.hW1 : hW[2 * pi].data();
     const z* W2 = s.hW2 ? s.hW2 : hW[2 * pi + 1].data();
     const int64_t nI = d * d * D, nJ = D * d * d;
+    const bool all = !finite_entries(W1, (size_t)(D * D * d * d)) || !finite_entries(W2, (size_t)(D * D * d * d));
     W12.assign((size_t)(nI * nJ), zmk(0, 0));
     nz2.assign((size_t)D, {});
     for (int64_t w1 = 0; w1 < D; ++w1)
       for (int64_t e = 0; e < D * d * d; ++e) {  // e = (w2, s2', s2)
         const z v = W2[w1 * D * d * d + e];
-        if (v.x != 0.0 || v.y != 0.0) nz2[(size_t)w1].push_back((int)e);
+        if (all || v.x != 0.0 || v.y != 0.0) nz2[(size_t)w1].push_back((int)e);
       }
     for (int64_t w1 = 0; w1 < D; ++w1)
       for (int64_t w = 0; w < D; ++w)
         for (int64_t s1o = 0; s1o < d; ++s1o)
           for (int64_t s1 = 0; s1 < d; ++s1) {
             const z u = W1[((w * D + w1) * d + s1o) * d + s1];
-            if (u.x == 0.0 && u.y == 0.0) continue;
+            if (!all && u.x == 0.0 && u.y == 0.0) continue;
             for (int e : nz2[(size_t)w1]) {
               const int64_t w2 = e / (d * d), s2o = (e / d) % d, s2 = e % d;
               zfma(W12[(size_t)(((s1o * d + s2o) * D + w2) * nJ + (w * d + s1) * d + s2)], u, W2[w1 * D * d * d + e]);

@@ -3,6 +3,7 @@
 // library performs before its matrix products (App. B.1.1) is folded into GEMM strides or
 // the operator offset tables here; nothing is permuted in memory.
 #include <algorithm>
+#include <cmath>
 
 #include "heff_plan.cuh"
 
@@ -31,23 +32,30 @@ size_t heff_scratch_bound(int64_t chl, int64_t d, int64_t D, int64_t chr, int pr
   return b;
 }
 
+bool finite_entries(const z* v, size_t n) {
+  for (size_t i = 0; i < n; ++i)
+    if (!std::isfinite(v[i].x) || !std::isfinite(v[i].y)) return false;
+  return true;
+}
+
 // W12[(s1',s2',w2),(w,s1,s2)] = sum_w1 W1[w,w1,s1',s1] W2[w1,w2,s2',s2]  (host, tiny; from the
-// non-zero entries of the two tensors, w1 ascending)
+// non-zero entries of the two tensors, w1 ascending; from all of them where one is not finite)
 static void build_w12(const std::vector<z>& W1, const std::vector<z>& W2, int64_t d, int64_t D,
                       std::vector<z>* W12) {
   const int64_t nI = d * d * D, nJ = D * d * d, slab = D * d * d;
   W12->assign((size_t)(nI * nJ), zmk(0, 0));
   std::vector<int> nz;
+  const bool all = !finite_entries(W1.data(), W1.size()) || !finite_entries(W2.data(), W2.size());
   for (int64_t w1 = 0; w1 < D; ++w1) {
     const z* v2 = W2.data() + w1 * slab;  // (w2, s2', s2)
     nz.clear();
     for (int64_t e = 0; e < slab; ++e)
-      if (v2[e].x != 0.0 || v2[e].y != 0.0) nz.push_back((int)e);
+      if (all || v2[e].x != 0.0 || v2[e].y != 0.0) nz.push_back((int)e);
     for (int64_t w = 0; w < D; ++w)
       for (int64_t s1o = 0; s1o < d; ++s1o)
         for (int64_t s1 = 0; s1 < d; ++s1) {
           const z u = W1[(size_t)(((w * D + w1) * d + s1o) * d + s1)];
-          if (u.x == 0.0 && u.y == 0.0) continue;
+          if (!all && u.x == 0.0 && u.y == 0.0) continue;
           for (int e : nz) {
             const int64_t w2 = e / (d * d), s2o = (e / d) % d, s2 = e % d;
             zfma((*W12)[(size_t)(((s1o * d + s2o) * D + w2) * nJ + (w * d + s1) * d + s2)], u, v2[e]);

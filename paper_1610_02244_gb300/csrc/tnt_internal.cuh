@@ -370,6 +370,8 @@ int heff_mixed(Ctx* c, const z* L, const z* W1, const z* W2, const z* R, const z
 // host copies of MPO tensors are needed to build the CSR ops: read back W (tiny)
 int read_small(Ctx* c, const void* dsrc, void* hdst, size_t bytes);
 int read_small2(Ctx* c, const void* d1, void* h1, size_t b1, const void* d2, void* h2, size_t b2);
+// whether every entry is finite: only then may products skip the zeros of the other factor
+bool finite_entries(const z* v, size_t n);
 
 int bh_mpo_site_host(int n_max, double J, double U, double mu, double V, double j, double jc,
                      z* W);
