@@ -392,12 +392,15 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tridiag_persistent(TriArgs a) {
 //   group barrier.
 // Reflector j replaces row j of the block in global memory (columns 0 .. n-j-2), the layout
 // the back-transformation reads: no CTA reads row j after its barrier j.
-// A Gram matrix is positive semidefinite, so its trailing block is bounded by the block's
-// trace, which is what the diagonal entries found so far leave of the whole trace.  Once an
-// entry and what is left are both at most SPLIT_TOL / 4 times the largest entry, so is the
-// coupling (the square root of their product), and the reduction stops: the rest is the
-// negligible range that k_split takes off (d = e = 0, no reflectors).  A 5 : 1 block of a
-// centre move has a fifth of its columns left to do, theta of a truncated state about half.
+// A Gram matrix is positive semidefinite, so its trailing block is bounded by that block's
+// trace.  Once an entry and the trace of what follows are both at most SPLIT_TOL / 4 times the
+// largest entry, so is the coupling (the square root of their product), and the reduction
+// stops: the rest is the negligible range that k_split takes off (d = e = 0, no reflectors).
+// What the entries found so far leave of the whole trace is only the hint: where many entries
+// are of the largest one's size that difference is off by thousands of eps of them (its own
+// rounding, and the drift of the trace under the reflectors).  At a hint the group sums the
+// trailing diagonal as it stands, with a barrier of its own (6 us, as a rule once per block).  A 5 : 1
+// block of a centre move has a fifth of its columns left to do, theta of a truncated state about half.
 // Vectors are indexed by row of the block.  Per column a CTA spends 16 FP64 operations per
 // trailing entry on the shared vectors and 12 per entry of its rows: that work bounds large
 // blocks (two operations per SM and clock); small ones are bound by the sequence of about 60
@@ -419,25 +422,25 @@ struct TriBlk {
   double* d;
   double* e;
   z* p;          // 2 x n: p of even / odd columns
-  double* part;  // 2 x nb parts of v^H T v
+  double* part;  // 2 x nb parts of v^H T v (even / odd columns), then nb of the trailing trace
   int n, c0, nb; // CTAs [c0, c0 + nb)
 };
 struct TriGroup {
   int nblk;
-  unsigned* bar;   // 32 words per block: arrivals (zero before the launch)
+  unsigned* bar;   // 32 words per block: arrivals (words 0 and 16, zero before the launch)
   int* status;
   TriBlk b[TRI_MAXB];
 };
 
-// Barrier j of a group of nb CTAs: each adds one to the group's counter (release: its threads'
+// Barrier j of a group of nb CTAs on its counter `word` (0: columns, 16: hints): each adds one to the group's counter (release: its threads'
 // stores before the CTA barrier are visible to whoever sees the sum) and waits until all
 // have.  false: the wait expired, the CTA must stop (and so will the others of its group).
-__device__ bool group_barrier(const TriGroup& t, int grp, int nb, int j) {
+__device__ bool group_barrier(const TriGroup& t, int grp, int nb, int j, int word) {
   __shared__ int s_ok;
   __syncthreads();
   if (nb == 1) return true;
   if (threadIdx.x == 0) {
-    unsigned* bar = t.bar + 32 * grp;
+    unsigned* bar = t.bar + 32 * grp + word;
     const unsigned want = (unsigned)nb * (unsigned)(j + 1);
     unsigned seen;
     int ok = 1;
@@ -502,8 +505,9 @@ struct RowsShared {
   GroupRefl rf[2];               // reflectors of even / odd columns
   z alpha;
   double cf, part;
-  double trace, dmax;            // of the trailing block; largest diagonal entry so far
-  int done;                      // the rest of the block is negligible
+  double left, dmax;             // what is left of the trace; largest diagonal entry so far
+  double limit, tailp;           // at a hint: the trace that would be negligible; one CTA's sum
+  int done, hints;               // the rest of the block may be, and then is, negligible; hints so far
 };
 
 // Reflector parameters (refl_params) by one warp
@@ -664,6 +668,34 @@ __device__ __forceinline__ double nrm_total(const RowsShared& S) {
   return nr;
 }
 
+// At a hint: S.done from the trace of rows j+1 and on, summed over the group before this column's
+// update, which leaves it.  false: the wait expired.
+__device__ __noinline__ bool trailing_trace(const TriGroup& T, int grp, const z* rows, int R, int b, int j,
+                                            RowsShared& S) {
+  const TriBlk& a = T.b[grp];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double* tails = a.nb == 1 ? &S.tailp : a.part + 2 * a.nb;
+  if (warp == 0) {
+    double tr = 0;
+    for (int i = lane; i < R; i += 32)
+      if (b + a.nb * i > j) tr += rows[(int64_t)i * a.n + b + a.nb * i].x;
+    tr = warp_sum_d(tr);
+    if (lane == 0) tails[b] = tr;
+  }
+  if (!group_barrier(T, grp, a.nb, S.hints, 16)) return false;
+  if (warp == 0) {
+    double tr = 0;
+    for (int q = lane; q < a.nb; q += 32) tr += a.nb == 1 ? tails[q] : __ldcg(tails + q);
+    tr = warp_sum_d(tr);
+    if (lane == 0) {
+      S.done = tr <= S.limit;
+      ++S.hints;
+    }
+  }
+  __syncthreads();
+  return true;
+}
+
 __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_constant__ TriGroup T) {
   extern __shared__ z sm_tri[];
   __shared__ RowsShared S;
@@ -688,9 +720,9 @@ __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
       const double d0 = __ldcg(a.G).x;
-      S.trace = s - d0;
+      S.left = s - d0;
       S.dmax = d0;
-      S.done = 0;
+      S.done = S.hints = 0;
     }
   }
   for (int i = 0; i < R; ++i) {
@@ -731,7 +763,7 @@ __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_
     if (warp == 0) rows_finish(rows, R, b, nb, n, 1, sx, S.rf[0], one ? sp : a.p, one ? &S.part : a.part + b, S);
   }
   for (int j = 0; j + 1 < n; ++j) {
-    if (!group_barrier(T, grp, nb, j)) return;
+    if (!group_barrier(T, grp, nb, j, 0)) return;
     const z* pj = one ? sp : a.p + (j & 1) * n;
     z* pn = one ? sp : a.p + ((j + 1) & 1) * n;
     const double* partj = one ? &S.part : a.part + (j & 1) * nb;
@@ -788,10 +820,12 @@ __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_
           sw[c] = zmk(fma(cf, vc[k].x, pc[k].x), fma(cf, vc[k].y, pc[k].y));
           if (c == j + 1) {  // thread 0
             if (b == 0) a.d[j + 1] = xn.x;
-            const double left = S.trace - xn.x, top = fmax(S.dmax, xn.x), tol = 0.25 * SPLIT_TOL * top;
-            S.trace = left;
+            const double left = S.left - xn.x, top = fmax(S.dmax, xn.x), tol = 0.25 * SPLIT_TOL * top;
+            S.left = left;
             S.dmax = top;
-            S.done = xn.x <= tol && left <= tol;
+            const bool hint = xn.x <= tol && left <= tol;
+            S.done = hint;
+            if (hint) S.limit = tol + xn.x;
           } else if (c == j + 2) {
             S.alpha = zconj(xn);
             sx[c] = zmk(0, 0);
@@ -806,6 +840,9 @@ __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_
     }
     __syncthreads();
     if (S.done) {  // the same decision in every CTA of the group
+      if (!trailing_trace(T, grp, rows, R, b, j, S)) return;
+    }
+    if (S.done) {
       if (b == 0)
         for (int i = j + 1 + tid; i < n; i += TRI_GTHREADS) {
           a.tau[i] = zmk(0, 0);
@@ -1774,7 +1811,7 @@ int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& all, z* U, double* ev
   double* e = (double*)ws_alloc(c, ws_round(sizeof(double) * tot));
   z* tau = (z*)ws_alloc(c, ws_round(sizeof(z) * tot));
   z* p = (z*)ws_alloc(c, ws_round(sizeof(z) * 2 * tot));
-  double* part = (double*)ws_alloc(c, ws_round(sizeof(double) * 2 * (size_t)nsm));
+  double* part = (double*)ws_alloc(c, ws_round(sizeof(double) * 3 * (size_t)nsm));
   unsigned* bar = (unsigned*)ws_alloc(c, ws_round(sizeof(unsigned) * 32 * TRI_MAXB));
   double* tn = (double*)ws_alloc(c, ws_round(sizeof(double) * nb));
   int64_t* nr = (int64_t*)ws_alloc(c, ws_round(sizeof(int64_t) * nb));
@@ -1842,7 +1879,7 @@ int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& all, z* U, double* ev
         const SmallEig& b = blocks[(size_t)(i0 + i)];
         const EBlk& E = he[(size_t)(i0 + i)];
         const int64_t rows = (b.n + q[(size_t)i] - 1) / q[(size_t)i];
-        T.b[i] = TriBlk{G + b.goff, tau + E.off, d + E.off, e + E.off, p + 2 * E.off, part + 2 * ctas,
+        T.b[i] = TriBlk{G + b.goff, tau + E.off, d + E.off, e + E.off, p + 2 * E.off, part + 3 * ctas,
                         (int)b.n, ctas, q[(size_t)i]};
         ctas += q[(size_t)i];
         smem = std::max(smem, (size_t)(rows + 3 + (q[(size_t)i] == 1)) * b.n * sizeof(z));
