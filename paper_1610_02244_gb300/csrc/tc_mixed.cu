@@ -246,7 +246,8 @@ __device__ __forceinline__ void op_mixed_rows(const OpApply& a, int i0, int i1, 
     }
   }
 }
-__global__ void __launch_bounds__(256) k_op_mixed(OpApply a, int rows, const float* __restrict__ t1,
+__global__ void __launch_bounds__(256) k_op_mixed(OpApply a, int rows, int D, int64_t kp4,
+                                                  const float* __restrict__ t1,
                                                   int64_t t1_plane, float* __restrict__ t3,
                                                   int64_t t3_plane) {
   __shared__ int s_row[257];
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(256) k_op_mixed(OpApply a, int rows, const flo
   const int i0 = blockIdx.y * rows, i1 = min(a.nI, i0 + rows);
   for (int t = threadIdx.x; t <= a.nI; t += blockDim.x) s_row[t] = a.row_ptr[t];
   for (int t = threadIdx.x; t < a.nJ; t += blockDim.x) s_in[t] = a.in_off[t];
-  for (int t = threadIdx.x; t < a.nI; t += blockDim.x) s_out[t] = a.out_off[t];
+  for (int t = threadIdx.x; t < a.nI; t += blockDim.x) s_out[t] = (t / D) * kp4 + (t % D) * a.B2;
   __syncthreads();
   int cplx = 0;
   for (int t = s_row[i0] + threadIdx.x; t < s_row[i1]; t += blockDim.x) {
@@ -419,18 +420,10 @@ int heff_mixed_prepare(Ctx* c, HeffPlan* p) {
   TNT_TRY(make_map(c, &m.tmTh, m.Thp, m.Np1, m.Kp1, BN));
   TNT_TRY(make_map(c, &m.tmT3, m.T3p, m.Mp4, m.Kp4, BM));
   TNT_TRY(make_map(c, &m.tmR, m.Rp, m.Np4, m.Kp4, BN));
-  // W12 with output offsets in T3-plane units: row (a' s1' s2'), column (w2 b)
+  // W12 from T1 to T3 planes: row (a' s1' s2'), column (w2 b); the kernel makes the offsets of
+  // (s1' s2' w2) itself (a table of its own cost a copy between kernels, 10 us a plan)
   m.op = p->op;
-  const int nI = (int)(d * d * D);
-  std::vector<int64_t> out_off(nI);
-  for (int64_t s1 = 0; s1 < d; ++s1)
-    for (int64_t s2 = 0; s2 < d; ++s2)
-      for (int64_t w2 = 0; w2 < D; ++w2)
-        out_off[(size_t)((s1 * d + s2) * D + w2)] = (s1 * d + s2) * m.Kp4 + w2 * chr;
-  int64_t* d_out = (int64_t*)ws_alloc(c, ws_round(sizeof(int64_t) * nI));
-  if (!d_out) return set_err(c, TNT_E_ALLOC, "scratch exhausted (mixed op table)");
-  TNT_TRY(to_device(c, d_out, out_off.data(), sizeof(int64_t) * nI));
-  m.op.out_off = d_out;
+  m.op.out_off = nullptr;
   m.op.B0 = chl;
   m.op.B1 = 1;
   m.op.B2 = chr;
@@ -460,7 +453,7 @@ int heff_run_mixed(Ctx* c, const HeffPlan& p, const z* theta, z* y) {
     const int64_t want = std::min<int64_t>(m.op.nI, (152 * 8 + blocks - 1) / blocks);
     const int rows = (int)((m.op.nI + want - 1) / want);
     k_op_mixed<<<dim3((unsigned)blocks, (unsigned)((m.op.nI + rows - 1) / rows)), 256, 0, c->stream>>>(
-        m.op, rows, m.T1, m.M1 * m.N1, m.T3p, m.Mp4 * m.Kp4);
+        m.op, rows, (int)p.D, m.Kp4, m.T1, m.M1 * m.N1, m.T3p, m.Mp4 * m.Kp4);
   }
   c->launches++;
   TNT_CHECK_LAUNCH(c);
