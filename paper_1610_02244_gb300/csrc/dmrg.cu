@@ -87,7 +87,7 @@ static int dmrg_update(Ctx* c, tnt_dmrg* g, int i, int dir, tnt_lanczos_result* 
     z* x = (z*)ws_alloc(c, ws_round(sizeof(z) * up.n));
     if (!x) return set_err(c, TNT_E_ALLOC, "scratch exhausted (compact theta)");
     TNT_TRY(u1_convert(c, spec[0], theta, x, 1));
-    TNT_TRY(u1_prepare(c, spec, &up));
+    TNT_TRY(u1_prepare(c, spec, &up, c->params.precision));
     if (marks) cudaEventRecord(g->ev[1], c->stream);
     c->fp64_finish = true;  // the sweep's energies and states are FP64-accurate
     int r = lanczos_run(c, U1MatVec(up), x, lz);
@@ -462,7 +462,7 @@ static int batched_update(Ctx* c, const std::vector<tnt_dmrg*>& gs, int i, int d
                             th[(size_t)p]));
     TNT_TRY(u1_convert(c, specs[(size_t)p], th[(size_t)p], x + up.x_off[(size_t)p], 1));
   }
-  TNT_TRY(u1_prepare(c, specs, &up));
+  TNT_TRY(u1_prepare(c, specs, &up, c->params.precision));
   std::vector<int64_t> off(up.x_off);
   off.push_back(up.n);
   c->fp64_finish = true;

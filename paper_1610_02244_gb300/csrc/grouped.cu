@@ -1042,7 +1042,34 @@ int autotune(Ctx* c, U1Plan* p) {
 }
 }  // namespace
 
-int u1_prepare(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
+// FP64 operands of a plan: zero padding (K columns beyond a task's K, and the T3 entries no pair
+// writes; up to gigabytes, so set while the host still builds the tables),
+static int u1_zero_f64(Ctx* c, U1Plan* p) {
+  TNT_CUDA_TRY(c, cudaMemsetAsync(p->A1z, 0, sizeof(z) * p->rowsA1 * p->KA1, c->stream));
+  TNT_CUDA_TRY(c, cudaMemsetAsync(p->A4z, 0, sizeof(z) * p->rowsA4 * p->KA4, c->stream));
+  TNT_CUDA_TRY(c, cudaMemsetAsync(p->B4z, 0, sizeof(z) * p->rowsB4 * p->KA4, c->stream));
+  return TNT_OK;
+}
+// environments into FP64 packs,
+static int u1_pack_f64(Ctx* c, U1Plan* p) {
+  const int nA = (int)p->segA1.size(), nB = (int)p->segB4.size();
+  k_pack_segs<false><<<cap_grid((nA + 7) / 8, 152 * 8), 256, 0, c->stream>>>(p->d_segA1, nA, nullptr, 0, p->A1z);
+  k_pack_segs<false><<<cap_grid((nB + 7) / 8, 152 * 8), 256, 0, c->stream>>>(p->d_segB4, nB, nullptr, 0, p->B4z);
+  c->launches += 2;
+  TNT_CHECK_LAUNCH(c);
+  return TNT_OK;
+}
+// and their slices
+static int u1_slice_f64(Ctx* c, U1Plan* p) {
+  if (p->oz) {
+    TNT_TRY(oz_plan_fix(c, p->oz1));
+    TNT_TRY(oz_plan_fix(c, p->oz4));
+  }
+  p->f64_ready = true;
+  return TNT_OK;
+}
+
+int u1_prepare(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p, int precision) {
   (void)probs;
   c->tune.emplace(p->sig, std::vector<int>());  // known; its tiles are chosen when first needed
   const size_t f = sizeof(float);
@@ -1062,10 +1089,8 @@ int u1_prepare(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
   if (!p->A1p || !p->B1p || !p->T1f || !p->A4p || !p->B4p || !p->Yf || !p->A1z || !p->T1z ||
       !p->A4z || !p->B4z || !p->Yz)
     return set_err(c, TNT_E_ALLOC, "scratch exhausted (grouped matvec buffers)");
-  // zero padding (K columns beyond a task's K, and the T3 entries no pair writes)
-  TNT_CUDA_TRY(c, cudaMemsetAsync(p->A1z, 0, sizeof(z) * p->rowsA1 * p->KA1, c->stream));
-  TNT_CUDA_TRY(c, cudaMemsetAsync(p->A4z, 0, sizeof(z) * p->rowsA4 * p->KA4, c->stream));
-  TNT_CUDA_TRY(c, cudaMemsetAsync(p->B4z, 0, sizeof(z) * p->rowsB4 * p->KA4, c->stream));
+  const bool f64 = precision == TNT_PREC_FP64;
+  if (f64) TNT_TRY(u1_zero_f64(c, p));
   // tables
   TNT_TRY(upload(c, &p->d_segA1, p->segA1));
   TNT_TRY(upload(c, &p->d_segB4, p->segB4));
@@ -1114,16 +1139,12 @@ int u1_prepare(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
   TNT_TRY(upload(c, &p->d_g4, none, p->s4.size()));
   TNT_TRY(upload(c, &p->d_g1tiles, none4, (size_t)p->cap_g1tiles));
   TNT_TRY(upload(c, &p->d_g4tiles, none4, (size_t)p->cap_g4tiles));
-  // constant operands: environments into FP64 packs
-  const int nA = (int)p->segA1.size(), nB = (int)p->segB4.size();
-  k_pack_segs<false><<<cap_grid((nA + 7) / 8, 152 * 8), 256, 0, c->stream>>>(p->d_segA1, nA, nullptr, 0, p->A1z);
-  k_pack_segs<false><<<cap_grid((nB + 7) / 8, 152 * 8), 256, 0, c->stream>>>(p->d_segB4, nB, nullptr, 0, p->B4z);
-  c->launches += 2;
-  TNT_CHECK_LAUNCH(c);
+  if (f64) TNT_TRY(u1_pack_f64(c, p));
   if (p->oz) {
     TNT_TRY(oz_plan_build(c, oz_stage(*p, 1), 1, &p->oz1));
     TNT_TRY(oz_plan_build(c, oz_stage(*p, 4), 2, &p->oz4));
   }
+  if (f64) TNT_TRY(u1_slice_f64(c, p));
   // arguments of the nodes whose pointers change per matvec
   p->in_tp = TPArgs{nullptr, p->d_slabs, p->d_ttiles, p->n_ttiles, p->B1p, p->KA1, p->rowsB1 * p->KA1};
   p->in_zg = ZGArgs{p->d_z1, p->d_z1tiles, p->n_z1tiles, p->A1z, nullptr, p->T1z};
@@ -1158,7 +1179,7 @@ int u1_tune(Ctx* c, const std::vector<U1Spec>& probs) {
   U1Plan p;
   TNT_TRY(u1_layout(c, probs, &p));
   TNT_TRY(ws_reserve(c, p.bytes));
-  TNT_TRY(u1_prepare(c, probs, &p));
+  TNT_TRY(u1_prepare(c, probs, &p, TNT_PREC_MIXED));
   TNT_TRY(u1_prepare_mixed(c, &p));
   TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   return TNT_OK;
@@ -1341,6 +1362,11 @@ int run_direct(Ctx* c, U1Plan& p, const z* x, z* y, int mixed) {
 int u1_run(Ctx* c, U1Plan& p, const z* x, z* y, int precision) {
   const int mixed = (precision == TNT_PREC_MIXED) ? 1 : 0;
   if (mixed && !p.mixed_ready) TNT_TRY(u1_prepare_mixed(c, &p));
+  if (!mixed && !p.f64_ready) {
+    TNT_TRY(u1_zero_f64(c, &p));
+    TNT_TRY(u1_pack_f64(c, &p));
+    TNT_TRY(u1_slice_f64(c, &p));
+  }
   // a plan used once needs no graph (its instantiation costs more than the launches it saves)
   if (!c->use_graphs || !c->prof_cls.empty() || p.runs[mixed]++ == 0) return run_direct(c, p, x, y, mixed);
   if (!p.exec[mixed]) TNT_TRY(build_graph(c, p, mixed));

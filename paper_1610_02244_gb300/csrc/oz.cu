@@ -924,15 +924,11 @@ int oz_plan_build(Ctx* c, const std::vector<GemmTask>& tasks, int fixed_sides, O
     node[1] = OzNode{(void*)k_oz_slice<0>, oz_slice_grid(T), 256, 0};
     return 2;
   };
+  p->fixed = 0;
   if (fixed_sides) {
     T.h.sides = fixed_sides;
-    OzNode node[2];
-    const int n = inputs(node);
-    void* args[] = {&T};
-    for (int i = 0; i < n; ++i) {
-      TNT_CUDA_TRY(c, cudaLaunchKernel(node[i].fn, dim3(node[i].grid), dim3(node[i].block), args, 0, c->stream));
-      c->launches++;
-    }
+    p->fixed = inputs(p->fix);
+    memcpy(p->fix_args, &T, sizeof(T));
   }
   T.h.sides = 3 & ~fixed_sides;
   memcpy(p->args, &T, sizeof(T));
@@ -941,6 +937,17 @@ int oz_plan_build(Ctx* c, const std::vector<GemmTask>& tasks, int fixed_sides, O
   p->node[p->inputs] = OzNode{(void*)k_oz_gemm<0>, (unsigned)std::min(T.h.items, sm), OZ_THREADS, OZ_SMEM};
   p->node[p->inputs + 1] = OzNode{(void*)k_oz_finish<0>, (unsigned)std::min(T.h.fin_blocks, 152 * 8), 256, 0};
   p->nodes = p->inputs + 2;
+  return TNT_OK;
+}
+
+int oz_plan_fix(Ctx* c, OzPlan& p) {
+  void* args[] = {p.fix_args};
+  for (int i = 0; i < p.fixed; ++i) {
+    const OzNode& n = p.fix[i];
+    TNT_CUDA_TRY(c, cudaLaunchKernel(n.fn, dim3(n.grid), dim3(n.block), args, n.smem, c->stream));
+    c->launches++;
+  }
+  TNT_CHECK_LAUNCH(c);
   return TNT_OK;
 }
 

@@ -244,7 +244,7 @@ int zgemm_tasks(Ctx* c, const std::vector<GemmTask>& tasks);
 int zgemm_fma_tasks(Ctx* c, const GemmTask* const* tasks, int n);
 // Products that repeat with the same shapes (oz.cu): tables and buffers from the scratch arena,
 // laid out once; the sides of fixed_sides (bit 0 A, bit 1 B) hold operands that do not change
-// and are sliced when the plan is built.  A task's B may be an offset from the vector given
+// and are sliced once, by oz_plan_fix before the first run.  A task's B may be an offset from the vector given
 // at each run (add_b; null for absolute pointers).  The kernels (the first `inputs` of them read
 // the operands) take one argument, for graph nodes: oz_plan_args writes it.
 struct OzNode {
@@ -255,10 +255,14 @@ struct OzPlan {
   alignas(16) unsigned char args[128];
   OzNode node[4];
   int nodes = 0, inputs = 0;
+  alignas(16) unsigned char fix_args[128];
+  OzNode fix[2];
+  int fixed = 0;
   double flop = 0;
 };
 size_t oz_plan_bytes(Ctx* c, const std::vector<GemmTask>& tasks);
 int oz_plan_build(Ctx* c, const std::vector<GemmTask>& tasks, int fixed_sides, OzPlan* p);
+int oz_plan_fix(Ctx* c, OzPlan& p);
 void oz_plan_args(const OzPlan& p, const z* add_b, void* out);
 int oz_plan_run(Ctx* c, const OzPlan& p, const z* add_b);
 // FP64 FMA GEMMs only while the guard lives (paths that must not allocate)

@@ -178,6 +178,7 @@ struct U1Plan {
   bool oz = false;
   OzPlan oz1, oz4;
   bool mixed_ready = false;  // split-TF32 operands packed and tiles chosen (on first use)
+  bool f64_ready = false;    // FP64 operands packed and sliced (on first use)
   int runs[2] = {0, 0};      // matvecs so far per precision: the graph is built at the second
   // tile choice (autotuned): N tile of stage 1 and stage 4, split-K of stage 4
   int bn1 = 128, bn4 = 128, split4 = 1;
@@ -199,9 +200,10 @@ struct U1Plan {
 
 // host layout of the grouped matvec (no device work); sets p->bytes
 int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p);
-// device buffers from the scratch arena (p->bytes must fit), tables and packed FP64 operands;
-// the split-TF32 operands and the autotuned tile choice follow at the first such matvec
-int u1_prepare(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p);
+// device buffers from the scratch arena (p->bytes must fit) and tables; the packed operands of
+// `precision` are made here where it is FP64; the others, and the autotuned split-TF32 tiles,
+// at their first matvec
+int u1_prepare(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p, int precision);
 // chooses the split-TF32 tiles of these problems' block structure
 int u1_tune(Ctx* c, const std::vector<U1Spec>& probs);
 int u1_run(Ctx* c, U1Plan& p, const z* x, z* y, int precision);
