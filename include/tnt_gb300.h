@@ -480,10 +480,14 @@ enum { TNT_FP64_GEMM_FMA = 0, TNT_FP64_GEMM_TC = 1 };
  * to below 1, rounded to 55 bits and cut into 8 integer slices (balanced base-128 digits);
  * slice products run as FP16 MMAs whose FP32 sums over K chunks of 256 stay within 2^24
  * and so are exact; the sums of the 36 slice pairs p + q <= 9 are combined in 64-bit
- * integers and rounded once.  The error is below 3 * 2^-53 * K * sigma_i * tau_j, sigma_i and
- * tau_j the powers of two just above max_k|A_ik| and max_k|B_kj|: the size of FP64's own
- * rounding bound.  A row of A or column of B with an infinity or NaN gives NaN.
- * Small products (and calls that must not allocate) use FMA. */
+ * integers and rounded once.  The error is below 3 * 2^-53 * K * sigma_i * tau_j and that
+ * rounding, sigma_i and tau_j the powers of two just above max_k|A_ik| and max_k|B_kj| (of the
+ * real and imaginary parts): the size of FP64's own rounding bound where the entries of a row
+ * are of a size.  An entry 2^-s below its row's or column's largest keeps 55 - s bits; where
+ * results that rest on such entries must have FP64's relative accuracy, choose FMA.
+ * A row of A or column of B with an infinity or NaN gives NaN.
+ * Small products (K times the 16 x 16 output tiles per SM below 110, or a side below 16:
+ * 256 x 1024 x 64 is sliced, 64 x 512 x 64 is not) and calls that must not allocate use FMA. */
 int tnt_set_fp64_gemm(tnt_ctx* ctx, int engine);
 
 /* ------------------------------------------------------------------ U(1) blocks, grouped */
