@@ -75,7 +75,8 @@ __host__ __device__ __forceinline__ double f64_of(float f) {
   return double_of_bits(((uint64_t)hi << 32) | lo);
 }
 
-// F = floor(|v| 2^(54 - esc)) for |v| < 2^esc: the 53-bit mantissa shifted (exact)
+// F = floor(|v| 2^(54 - esc)) for |v| < 2^esc: the 53-bit mantissa shifted (exact).  Only its host
+// check uses it now; the slices of the FP64-accurate GEMM come from oz_fixed (oz.cuh).
 __host__ __device__ __forceinline__ uint64_t fixed54(double v, int esc) {
   const uint64_t u = bits_of(v);
   const int eb = (int)((u >> 52) & 0x7ff);
@@ -87,10 +88,15 @@ __host__ __device__ __forceinline__ uint64_t fixed54(double v, int esc) {
 }
 
 #ifdef __CUDACC__
-// 1 / sqrt(s) and 1 / d for normal positive s, d != 0: an FP32 seed (relative error e0 of about
-// 2^-22), one step of third order, y (1 + e/2 + 3/8 e^2) with e = 1 - s y^2, and
-// r (1 + e + e^2) with e = 1 - d r: the error left is of order e0^3, below FP64 rounding.
-// The arguments are scaled to [1, 4) and [1, 2) by exponent arithmetic.
+// 1 / sqrt(s) for normal positive s and 1 / d for normal d, |d| < 2^923, from an FP32 seed (relative
+// error below 2^-21) by one step of third order: Householder's iteration for s y^2 = 1 (A. S.
+// Householder, The Numerical Treatment of a Single Nonlinear Equation, 1970),
+// y (1 + e/2 + 3/8 e^2) with e = 1 - s y^2, and the hyperpower iteration (M. Altman, Pacific J.
+// Math. 10, 1960), r (1 + e + e^2) with e = 1 - d r.  The series' rest is of order e^3 = 2^-60.
+// Rounding: the reciprocal's e is exact to its own last bit, so that one rounding, 2^-53,
+// is left; the root's e carries the rounding of s y, in all 1.5 2^-53, against 2 2^-53 of
+// 1.0 / sqrt(s) (tests/newton_gpu.cu).  The arguments are scaled to [1, 4) and [1, 2) by exponent
+// arithmetic.
 __device__ __forceinline__ double rsqrt_newton(double s) {
   const int hi = __double2hiint(s), ex = (hi >> 20) - 1023, h = ex >> 1;
   const double m = __hiloint2double((hi & 0xfffff) | ((1023 + (ex & 1)) << 20), __double2loint(s));
