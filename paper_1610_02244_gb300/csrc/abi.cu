@@ -26,6 +26,7 @@ int dev_alloc(const DevAlloc& a, void** p, size_t bytes) {
     return *p ? 0 : 1;
   }
   if (cudaMalloc(p, bytes) != cudaSuccess) {
+    cudaGetLastError();  // (the caller reports it, or does without)
     *p = nullptr;
     return 1;
   }

@@ -75,8 +75,10 @@ static int dmrg_update(Ctx* c, tnt_dmrg* g, int i, int dir, tnt_lanczos_result* 
     s.hW1 = g->mpo->hW[(size_t)i].data(); s.hW2 = g->mpo->hW[(size_t)i + 1].data();
     TNT_TRY(u1_layout(c, spec, &up));
     if (c->ws.top == 0)
-      TNT_TRY(ws_reserve(c, std::max(g->scratch, ws_round(sizeof(z) * n) + ws_round(sizeof(z) * up.n) + up.bytes +
-                                                     lanczos_scratch_bound(up.n, c->params.krylov_cap) + (4 << 20))));
+      TNT_TRY(u1_fit(&up, [&] {
+        return ws_reserve(c, std::max(g->scratch, ws_round(sizeof(z) * n) + ws_round(sizeof(z) * up.n) + up.bytes +
+                                                      lanczos_scratch_bound(up.n, c->params.krylov_cap) + (4 << 20)));
+      }));
   }
   const size_t top = c->ws.top;
   z* theta = (z*)ws_alloc(c, ws_round(sizeof(z) * n));
@@ -444,10 +446,12 @@ static int batched_update(Ctx* c, const std::vector<tnt_dmrg*>& gs, int i, int d
   }
   U1Plan up;
   TNT_TRY(u1_layout(c, specs, &up));
-  const size_t eig_bytes = ws_round(sizeof(z) * up.n) + up.bytes +
-                           lanczos_batched_scratch_bound(up.n, P, c->params.krylov_cap);
   ws_reset(c);
-  TNT_TRY(ws_reserve(c, std::max(scratch, th_bytes + std::max(eig_bytes, svd_bytes) + (size_t)(8 << 20))));
+  TNT_TRY(u1_fit(&up, [&] {
+    const size_t eig_bytes = ws_round(sizeof(z) * up.n) + up.bytes +
+                             lanczos_batched_scratch_bound(up.n, P, c->params.krylov_cap);
+    return ws_reserve(c, std::max(scratch, th_bytes + std::max(eig_bytes, svd_bytes) + (size_t)(8 << 20)));
+  }));
   std::vector<z*> th((size_t)P);
   for (int p = 0; p < P; ++p) {
     th[(size_t)p] = (z*)ws_alloc(c, ws_round(sizeof(z) * nth[(size_t)p]));

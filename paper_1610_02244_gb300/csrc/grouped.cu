@@ -944,7 +944,7 @@ int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
   p->oz = c && c->oz_mode != 0 && p->flops >= U1_OZ_MIN_FLOPS && k1 <= 512;
   if (p->oz) {
     const size_t o1 = oz_plan_bytes(c, oz_stage(*p, 1)), o4 = oz_plan_bytes(c, oz_stage(*p, 4));
-    if (o1 && o4) p->bytes += o1 + o4 + (size_t)(1 << 16);
+    if (o1 && o4) p->bytes += p->oz_bytes = o1 + o4 + (size_t)(1 << 16);
     else p->oz = false;
   }
   return TNT_OK;
@@ -1178,7 +1178,7 @@ int u1_tune(Ctx* c, const std::vector<U1Spec>& probs) {
   Scope sc(c);
   U1Plan p;
   TNT_TRY(u1_layout(c, probs, &p));
-  TNT_TRY(ws_reserve(c, p.bytes));
+  TNT_TRY(u1_fit(&p, [&] { return ws_reserve(c, p.bytes); }));
   TNT_TRY(u1_prepare(c, probs, &p, TNT_PREC_MIXED));
   TNT_TRY(u1_prepare_mixed(c, &p));
   TNT_CUDA_TRY(c, cudaStreamSynchronize(c->stream));

@@ -838,8 +838,8 @@ bool oz_capturing(Ctx* c) {
 }
 
 // products tk[0..n) in one set of launches; slices and partial sums live in the context's own
-// buffer, grown between calls, never inside a capture (OZ_NOROOM); a buffer that a captured
-// graph refers to is kept until the context goes
+// buffer, grown between calls, never inside a capture; a buffer that a captured graph refers to
+// is kept until the context goes.  OZ_NOROOM: the buffer cannot grow as needed
 template <int CAP>
 int oz_launch(Ctx* c, const GemmTask* const* tk, int n, int sm) {
   OzTasks<CAP> T;
@@ -857,8 +857,7 @@ int oz_launch(Ctx* c, const GemmTask* const* tk, int n, int sm) {
     c->oz_captured = false;
     c->oz_buf = nullptr;
     c->oz_cap = 0;
-    if (dev_alloc(c->dalloc, &c->oz_buf, need) != 0)
-      return set_err(c, TNT_E_ALLOC, "device allocation of %zu bytes (FP64 product slices) failed", need);
+    if (dev_alloc(c->dalloc, &c->oz_buf, need) != 0) return OZ_NOROOM;
     c->oz_cap = need;
   }
   T.h.buf = (uint8_t*)c->oz_buf;

@@ -229,8 +229,8 @@ int tile_rows(int64_t tiles, int nsm);
 // FP64-accurate C = A B on the tensor cores by exact integer slicing (oz.cu); zgemm routes
 // large products with alpha = 1, beta = 0, batch = 1 there when the context allows it
 bool ozgemm_eligible(const Ctx* c, const ZGemm& g);
-// OZ_NOROOM: the slice buffer is too small and the stream is being captured, so that it cannot
-// grow; nothing was launched, the FP64 units do the product
+// OZ_NOROOM: the slice buffer is too small and cannot grow (the stream is being captured, or there
+// is no memory for it); nothing was launched, the FP64 units do the product
 constexpr int OZ_NOROOM = -1;
 int ozgemm(Ctx* c, const ZGemm& g);
 // One of a set of independent products run in grouped launches: herm, the result is

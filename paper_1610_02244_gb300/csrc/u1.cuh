@@ -149,6 +149,7 @@ struct U1Plan {
   std::vector<int2> wtiles;
   std::vector<GRow> rows;
   size_t bytes = 0;                 // device scratch the plan takes
+  size_t oz_bytes = 0;              // of which for the slice products
   int nprob = 0;
   int64_t n = 0;                    // compact length over all problems
   std::vector<int64_t> x_off;       // per problem
@@ -200,6 +201,18 @@ struct U1Plan {
 
 // host layout of the grouped matvec (no device work); sets p->bytes
 int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p);
+// reserve() the scratch for a plan (it reads p->bytes); where that fails, once more for FP64 stages
+// on the FP64 units, which need none for slices
+template <typename F>
+int u1_fit(U1Plan* p, F reserve) {
+  int r = reserve();
+  if (r == TNT_E_ALLOC && p->oz) {
+    p->oz = false;
+    p->bytes -= p->oz_bytes;
+    r = reserve();
+  }
+  return r;
+}
 // device buffers from the scratch arena (p->bytes must fit) and tables; the packed operands of
 // `precision` are made here where it is FP64; the others, and the autotuned split-TF32 tiles,
 // at their first matvec

@@ -95,7 +95,7 @@ int tnt_heff_apply_u1(tnt_ctx* ctx, int nprob, const tnt_u1_problem* probs, cons
   Scope sc(c);
   U1Plan p;
   TNT_TRY(u1_layout(c, specs, &p));
-  TNT_TRY(ws_reserve(c, p.bytes));
+  TNT_TRY(u1_fit(&p, [&] { return ws_reserve(c, p.bytes); }));
   TNT_TRY(u1_prepare(c, specs, &p, precision));
   if (h_flops) *h_flops = p.flops;
   TNT_TRY(u1_run(c, p, (const z*)d_x, (z*)d_y, precision));
@@ -112,7 +112,7 @@ int tnt_lanczos_ground_u1(tnt_ctx* ctx, const tnt_u1_problem* prob, tnt_cplx* d_
   Scope sc(c);
   U1Plan p;
   TNT_TRY(u1_layout(c, specs, &p));
-  TNT_TRY(ws_reserve(c, p.bytes + lanczos_scratch_bound(p.n, c->params.krylov_cap)));
+  TNT_TRY(u1_fit(&p, [&] { return ws_reserve(c, p.bytes + lanczos_scratch_bound(p.n, c->params.krylov_cap)); }));
   TNT_TRY(u1_prepare(c, specs, &p, c->params.precision));
   const int r = lanczos_run(c, U1MatVec(p), (z*)d_x, res);
   TNT_TRY(status_check(c));
@@ -129,7 +129,9 @@ int tnt_lanczos_ground_u1_batched(tnt_ctx* ctx, int nprob, const tnt_u1_problem*
   Scope sc(c);
   U1Plan p;
   TNT_TRY(u1_layout(c, specs, &p));
-  TNT_TRY(ws_reserve(c, p.bytes + lanczos_batched_scratch_bound(p.n, nprob, c->params.krylov_cap)));
+  TNT_TRY(u1_fit(&p, [&] {
+    return ws_reserve(c, p.bytes + lanczos_batched_scratch_bound(p.n, nprob, c->params.krylov_cap));
+  }));
   TNT_TRY(u1_prepare(c, specs, &p, c->params.precision));
   std::vector<int64_t> off(p.x_off);
   off.push_back(p.n);
