@@ -527,7 +527,8 @@ CLASSES = {
     "op_mixed": ("hbm", "byte"), "split_theta": ("hbm", "byte"), "multidot": ("alu", "flop"),
     "multiaxpy": ("alu", "flop"), "multidot_cond": ("alu", None), "multiaxpy_cond": ("alu", None),
     "multidot32": ("hbm", "byte"), "multiaxpy32": ("hbm", "byte"), "heig_tridiag": ("alu", "flop"),
-    "heig_tridiag_eig": ("alu", None), "heig_backtransform": ("alu", "flop"),
+    "heig_tridiag_eig": ("alu", None),
+    "heig_backtransform": ("tensor_fp64", "flop"),  # above 192 rows, where its work is: slice products
     "cgemm_grouped": ("tensor", "flop"), "zgemm_grouped": ("alu", "flop"),
     "u1_wop": ("hbm", "byte"), "u1_pack_theta": ("hbm", "byte"), "u1_gather": ("hbm", "byte"),
     "oz_gemm": ("tensor_fp64", "flop"), "oz_slice": ("hbm", "byte"),

@@ -938,7 +938,11 @@ int u1_layout(Ctx* c, const std::vector<U1Spec>& probs, U1Plan* p) {
        ws_round(sizeof(ZTask) * (p->s1.size() + p->s4.size()));
   p->bytes = b + (size_t)(1 << 20);
   // FP64 stages as slice products: eight launches of about 50 us in all, against the FP64
-  // units' 1 TFLOP/s (32 chains at chi = 256, d = 5: 13 GFLOP, 28 ms)
+  // units' 1 TFLOP/s (32 chains at chi = 256, d = 5: 13 GFLOP, 28 ms).  Only up to left sectors of
+  // 512: theta is strided along K, beyond OZ_SCALE_K the column maxima come from several CTAs, and
+  // nothing in a plan's launches zeroes them between runs (oz_plan_build refuses such a
+  // product).  Two left sectors of 512, d = 3 (89 GFLOP): 2.6 ms against 79 ms on the FP64 units;
+  // of 520, on the FP64 units: 89 ms.
   int64_t k1 = 0;
   for (const TaskDesc& t : p->s1) k1 = std::max(k1, t.K);
   p->oz = c && c->oz_mode != 0 && p->flops >= U1_OZ_MIN_FLOPS && k1 <= 512;

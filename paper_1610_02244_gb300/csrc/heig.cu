@@ -1747,8 +1747,9 @@ size_t heig_blocks_scratch(int64_t n, int64_t k) {
 // eigensolve is one launch (or a few) over all blocks that a group of CTAs can hold (tri_holds:
 // 1216 rows on 152 SMs); larger ones take heig_top one after the other.
 // blocks[i] = {offset of the n x n block in G (and of its eigenvector columns in U, leading
-// dimension n), n, k}; the reflectors replace the blocks' rows.  ev (device) receives
-// the eigenvalues of all blocks back to back.
+// dimension n), n, k}; the reflectors replace the blocks' rows.  ev (device) receives the
+// eigenvalues: of the blocks that no group holds in the order given, then of the others, largest
+// block first.
 int heig_blocks(Ctx* c, z* G, const std::vector<SmallEig>& all, z* U, double* ev) {
   if (all.empty()) return TNT_OK;
   const size_t top = c->ws.top;
