@@ -432,9 +432,10 @@ struct TriGroup {
   TriBlk b[TRI_MAXB];
 };
 
-// Barrier j of a group of nb CTAs on its counter `word` (0: columns, 16: hints): each adds one to the group's counter (release: its threads'
-// stores before the CTA barrier are visible to whoever sees the sum) and waits until all
-// have.  false: the wait expired, the CTA must stop (and so will the others of its group).
+// Barrier j of a group of nb CTAs on its counter `word` (0: columns, 16: hints): each adds one
+// (release: its threads' stores before the CTA barrier are visible to whoever sees the sum) and
+// waits until all have.  false: the wait expired, the CTA must stop (and so will the others of
+// its group).
 __device__ bool group_barrier(const TriGroup& t, int grp, int nb, int j, int word) {
   __shared__ int s_ok;
   __syncthreads();
