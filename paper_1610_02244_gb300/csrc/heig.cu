@@ -507,7 +507,7 @@ struct RowsShared {
   z alpha;
   double cf, part;
   double left, dmax;             // what is left of the trace; largest diagonal entry so far
-  double limit, tailp;           // at a hint: the trace that would be negligible; one CTA's sum
+  double entry, tailp;           // the column's diagonal entry; at a hint: one CTA's trace
   int done, hints;               // the rest of the block may be, and then is, negligible; hints so far
 };
 
@@ -669,31 +669,67 @@ __device__ __forceinline__ double nrm_total(const RowsShared& S) {
   return nr;
 }
 
-// At a hint: S.done from the trace of rows j+1 and on, summed over the group before this column's
-// update, which leaves it.  false: the wait expired.
-__device__ __noinline__ bool trailing_trace(const TriGroup& T, int grp, const z* rows, int R, int b, int j,
-                                            RowsShared& S) {
+// Column j of a group's CTA after its scalars and vectors: reflector j+1, the update of the rows,
+// p_{j+1} and the CTA's part of K_{j+1}
+__device__ __forceinline__ void column_update(const TriBlk& a, z* rows, int R, int b, int j, const z* sv, const z* sw,
+                                              const z* sx, z* pn, double* partn, RowsShared& S) {
+  const int n = a.n, nb = a.nb, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool empty = n - j - 2 <= 0;  // length of reflector j+1
+  if (warp == TRI_WARPS) {
+    const GroupRefl rf = refl_warp(empty ? zmk(0, 0) : S.alpha, nrm_total(S), empty);
+    if (lane == 0) {
+      S.rf[(j + 1) & 1] = rf;
+      if (b == 0) {
+        a.tau[j + 1] = rf.tau;
+        if (!empty) a.e[j + 1] = rf.beta;
+      }
+    }
+  } else {
+    rows_update<true>(rows, R, b, nb, n, j + 2, sv, sw, sx, nb == 1 ? nullptr : a.G + (int64_t)(j + 2) * n, S);
+  }
+  __syncthreads();
+  if (warp == 0) rows_finish(rows, R, b, nb, n, j + 2, sx, S.rf[(j + 1) & 1], pn, partn, S);
+}
+
+// Column j at a hint: the trace of rows j+1 and on, summed over the group before the column's update,
+// which leaves it, says whether the reduction ends.  If not, the column goes on as usual.
+// true: the CTA is done (or the wait expired).  A call of its own, so that the loop over the
+// columns keeps its registers (with the sum inside it a column took 2.4% longer).
+__device__ __noinline__ bool hint_column(const TriGroup& T, int grp, z* rows, z* sv, int j, RowsShared& S) {
   const TriBlk& a = T.b[grp];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double* tails = a.nb == 1 ? &S.tailp : a.part + 2 * a.nb;
+  const int n = a.n, nb = a.nb, b = (int)blockIdx.x - a.c0, R = (b < n) ? (n - b + nb - 1) / nb : 0;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool one = nb == 1;
+  double* tails = one ? &S.tailp : a.part + 2 * nb;
   if (warp == 0) {
     double tr = 0;
     for (int i = lane; i < R; i += 32)
-      if (b + a.nb * i > j) tr += rows[(int64_t)i * a.n + b + a.nb * i].x;
+      if (b + nb * i > j) tr += rows[(int64_t)i * n + b + nb * i].x;
     tr = warp_sum_d(tr);
     if (lane == 0) tails[b] = tr;
   }
-  if (!group_barrier(T, grp, a.nb, S.hints, 16)) return false;
+  if (!group_barrier(T, grp, nb, S.hints, 16)) return true;
   if (warp == 0) {
     double tr = 0;
-    for (int q = lane; q < a.nb; q += 32) tr += a.nb == 1 ? tails[q] : __ldcg(tails + q);
+    for (int q = lane; q < nb; q += 32) tr += one ? tails[q] : __ldcg(tails + q);
     tr = warp_sum_d(tr);
     if (lane == 0) {
-      S.done = tr <= S.limit;
+      S.done = tr - S.entry <= 0.25 * SPLIT_TOL * S.dmax;
       ++S.hints;
     }
   }
   __syncthreads();
+  if (!S.done) {
+    column_update(a, rows, R, b, j, sv, sv + n, sv + 2 * n, one ? sv + 3 * n : a.p + ((j + 1) & 1) * n,
+                  one ? &S.part : a.part + ((j + 1) & 1) * nb + b, S);
+    return false;
+  }
+  if (b == 0)
+    for (int i = j + 1 + tid; i < n; i += TRI_GTHREADS) {
+      a.tau[i] = zmk(0, 0);
+      a.e[i] = 0.0;
+      if (i > j + 1) a.d[i] = 0.0;
+    }
   return true;
 }
 
@@ -824,9 +860,8 @@ __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_
             const double left = S.left - xn.x, top = fmax(S.dmax, xn.x), tol = 0.25 * SPLIT_TOL * top;
             S.left = left;
             S.dmax = top;
-            const bool hint = xn.x <= tol && left <= tol;
-            S.done = hint;
-            if (hint) S.limit = tol + xn.x;
+            S.done = xn.x <= tol && left <= tol;
+            S.entry = xn.x;
           } else if (c == j + 2) {
             S.alpha = zconj(xn);
             sx[c] = zmk(0, 0);
@@ -840,33 +875,11 @@ __global__ void __launch_bounds__(TRI_GTHREADS, 1) k_tridiag_group(const __grid_
       if (lane == 0) S.nrm[warp] = acc;
     }
     __syncthreads();
-    if (S.done) {  // the same decision in every CTA of the group
-      if (!trailing_trace(T, grp, rows, R, b, j, S)) return;
+    if (S.done) {  // the same in every CTA of the group
+      if (hint_column(T, grp, rows, sv, j, S)) return;
+      continue;
     }
-    if (S.done) {
-      if (b == 0)
-        for (int i = j + 1 + tid; i < n; i += TRI_GTHREADS) {
-          a.tau[i] = zmk(0, 0);
-          a.e[i] = 0.0;
-          if (i > j + 1) a.d[i] = 0.0;
-        }
-      return;
-    }
-    const bool empty = n - j - 2 <= 0;  // length of reflector j+1
-    if (scalar) {
-      const GroupRefl rf = refl_warp(empty ? zmk(0, 0) : S.alpha, nrm_total(S), empty);
-      if (lane == 0) {
-        S.rf[(j + 1) & 1] = rf;
-        if (b == 0) {
-          a.tau[j + 1] = rf.tau;
-          if (!empty) a.e[j + 1] = rf.beta;
-        }
-      }
-    } else {
-      rows_update<true>(rows, R, b, nb, n, j + 2, sv, sw, sx, one ? nullptr : a.G + (int64_t)(j + 2) * n, S);
-    }
-    __syncthreads();
-    if (warp == 0) rows_finish(rows, R, b, nb, n, j + 2, sx, S.rf[(j + 1) & 1], pn, partn, S);
+    column_update(a, rows, R, b, j, sv, sw, sx, pn, partn, S);
   }
 }
 
