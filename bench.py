@@ -539,7 +539,15 @@ OZ_TENSOR_PER_USEFUL = 36.0  # slice pairs per complex product: 36 x 4 real MMAs
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
 # capture per kernel class, valid while the class's source file is unchanged: class ->
 # (bytes per launch, source file under csrc/, sha256 prefix of that file, capture).
-TRAFFIC = {}  # (tc_mixed.cu and heig.cu changed since their captures)
+TRAFFIC = {
+    # both launches of one matvec (T1 = L theta: 21.01 + 0.02 MB; y = T3 R^T: 71.34 + 3.13 MB),
+    # averaged: profiles/cgemm_tf32x3_heff_cfg2.md
+    "cgemm_tf32x3": (47.75e6, "tc_mixed.cu", "ce9d3fcdce61e0c1", "ncu, test_heff_mixed 256-4-256"),
+    # two launches per update: the 1024-row Gram block (17.20 MB, ncu; the matrix read once)
+    # and the ~231-row tail block (its entries x the same 16.4 B per entry: 0.88 MB), averaged:
+    # profiles/tridiag_rows_gram1024.md
+    "heig_tridiag": (9.04e6, "heig.cu", "299ed51b98a26f98", "ncu, svd_large_block_cfg2_shape"),
+}
 
 
 def traffic_for(cls):
