@@ -540,13 +540,13 @@ OZ_TENSOR_PER_USEFUL = 36.0  # slice pairs per complex product: 36 x 4 real MMAs
 # capture per kernel class, valid while the class's source file is unchanged: class ->
 # (bytes per launch, source file under csrc/, sha256 prefix of that file, capture).
 TRAFFIC = {
-    # both launches of one matvec (T1 = L theta: 21.01 + 0.02 MB; y = T3 R^T: 71.34 + 3.13 MB),
+    # both launches of one matvec (T1 = L theta: 21.02 + 0.03 MB; y = T3 R^T: 71.34 + 3.22 MB),
     # averaged: profiles/cgemm_tf32x3_heff_cfg2.md
-    "cgemm_tf32x3": (47.75e6, "tc_mixed.cu", "ce9d3fcdce61e0c1", "ncu, test_heff_mixed 256-4-256"),
-    # two launches per update: the 1024-row Gram block (17.20 MB, ncu; the matrix read once)
-    # and the ~231-row tail block (its entries x the same 16.4 B per entry: 0.88 MB), averaged:
+    "cgemm_tf32x3": (47.80e6, "tc_mixed.cu", "ce9d3fcdce61e0c1", "ncu, test_heff_mixed 256-4-256"),
+    # two launches per update: the 1024-row Gram block (16.97 MB, ncu; the matrix read once)
+    # and the ~231-row tail block (its entries x the same 16.2 B per entry: 0.86 MB), averaged:
     # profiles/tridiag_rows_gram1024.md
-    "heig_tridiag": (9.04e6, "heig.cu", "299ed51b98a26f98", "ncu, svd_large_block_cfg2_shape"),
+    "heig_tridiag": (8.92e6, "heig.cu", "4cadece3b2cf64a2", "ncu, svd_large_block_cfg2_shape"),
 }
 
 

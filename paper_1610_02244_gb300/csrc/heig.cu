@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tridiag_persistent(TriArgs a) {
 // What the entries found so far leave of the whole trace is only the hint: where many entries
 // are of the largest one's size that difference is off by thousands of eps of them (its own
 // rounding, and the drift of the trace under the reflectors).  At a hint the group sums the
-// trailing diagonal as it stands, with a barrier of its own (6 us, as a rule once per block).  A 5 : 1
+// trailing diagonal as it stands, with a barrier of its own (as a rule once per block).  A 5 : 1
 // block of a centre move has a fifth of its columns left to do, theta of a truncated state about half.
 // Vectors are indexed by row of the block.  Per column a CTA spends 16 FP64 operations per
 // trailing entry on the shared vectors and 12 per entry of its rows: that work bounds large
