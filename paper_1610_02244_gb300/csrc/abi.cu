@@ -429,6 +429,7 @@ int tnt_ctx_destroy(tnt_ctx* ctx) {
 int tnt_set_stream(tnt_ctx* ctx, void* stream) {
   CTX_CHECK(ctx);
   ctx->c.stream = (cudaStream_t)stream;
+  ctx->c.up.detach();
   return TNT_OK;
 }
 

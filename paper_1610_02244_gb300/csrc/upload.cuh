@@ -17,6 +17,10 @@ struct UploadRing {
   bool busy[2] = {false, false};
   const void* stream = nullptr;
 
+  // The stream was replaced: the next copies open the other half even if the new stream has the old
+  // one's handle (the half's event was recorded on a stream that may be gone).
+  void detach() { stream = this; }
+
   // Offset for `bytes` (at most half) on stream st; *wait = the half whose event must pass
   // before the bytes are written, or -1.  After the copy the caller records event `cur`.
   size_t place(size_t bytes, const void* st, int* wait) {

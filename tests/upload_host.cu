@@ -1,6 +1,7 @@
 // Host check of csrc/upload.cuh: copies queued per stream and carried out only when something
 // waits for them (an event, or the end), the latest that CUDA allows, must still find the bytes
-// they were given.  Random sizes (empty, one byte, up to a whole half) and stream changes.
+// they were given.  Random sizes (empty, one byte, up to a whole half), stream changes, and streams
+// replaced by new ones of the same handle.
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
@@ -40,16 +41,22 @@ int main() {
           queue[i].want.clear();
         }
     };
-    int stream = 1;
+    int stream = 1, handle = 1, streams_made = 3;  // handles 1..3 at first stand for streams 1..3
+    int of_handle[4] = {0, 1, 2, 3};
     for (int k = 0; k < 400; ++k) {
       if (next_u64() % 16 == 0) {
-        stream = 1 + (int)(next_u64() % 3);
+        handle = 1 + (int)(next_u64() % 3);
+        if (next_u64() % 4 == 0) {
+          of_handle[handle] = ++streams_made;
+          r.detach();
+        }
+        stream = of_handle[handle];
         ++streams;
       }
       const uint64_t kind = next_u64() % 8;
       const size_t bytes = kind == 0 ? 1 : kind == 1 ? r.half : kind == 2 ? r.half - 1 : 1 + next_u64() % (r.half / 4);
       int wait;
-      const size_t at = r.place(bytes, (const void*)(intptr_t)stream, &wait);
+      const size_t at = r.place(bytes, (const void*)(intptr_t)handle, &wait);
       if (wait >= 0) {
         ++waits;
         carry_out(ev_stream[wait], upto[wait]);
@@ -62,7 +69,7 @@ int main() {
       upto[r.cur] = done + queue.size();
       ev_stream[r.cur] = stream;
     }
-    for (int st = 1; st <= 3; ++st) carry_out(st, (size_t)-1);
+    for (int st = 1; st <= streams_made; ++st) carry_out(st, (size_t)-1);
   }
   std::printf("waits %ld stream changes %ld mismatches %d\n", waits, streams, bad);
   return bad || !waits ? 1 : 0;
